@@ -1,0 +1,99 @@
+// Double-single arithmetic: FP64-like precision from FP32 instructions, for
+// the per-vertex work of kernels that would otherwise wait on the FP64 pipe.
+#pragma once
+
+#include <stdint.h>
+
+namespace gr {
+
+// Double-single numbers: an unevaluated sum hi + lo of two floats with
+// |lo| <= ulp(hi) / 2, about 48 significant bits (Dekker's extended
+// precision arithmetic; Knuth's TwoSum for exact sums, the product's error
+// from one FMA). FP32 instructions issue many times faster than FP64 on this
+// GPU, so BC's per-vertex finish (a reciprocal, a product and sums per lane)
+// runs in this form (uint64 path counts keep every value within FP32's
+// exponent range): on R-MAT s23 x 64 sources it took the finalize from
+// 16.2 to 10.8 ms. The backward's per-edge sums stay in FP64: in this form
+// its warp-serial loop became issue-bound (75.7 against 53.5 ms). The _rn
+// intrinsics keep the compiler from contracting or reassociating the error
+// terms.
+struct DS {
+  float hi, lo;
+};
+
+__device__ __forceinline__ DS ds_two_sum(float a, float b) {  // exact: hi + lo = a + b
+  const float s = __fadd_rn(a, b);
+  const float bb = __fsub_rn(s, a);
+  const float err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+  return {s, err};
+}
+
+__device__ __forceinline__ DS ds_fast_two_sum(float a, float b) {  // |a| >= |b|
+  const float s = __fadd_rn(a, b);
+  return {s, __fsub_rn(b, __fsub_rn(s, a))};
+}
+
+__device__ __forceinline__ DS ds_add(DS a, DS b) {
+  DS s = ds_two_sum(a.hi, b.hi);
+  const DS t = ds_two_sum(a.lo, b.lo);
+  s = ds_fast_two_sum(s.hi, __fadd_rn(s.lo, t.hi));
+  return ds_fast_two_sum(s.hi, __fadd_rn(s.lo, t.lo));
+}
+
+__device__ __forceinline__ DS ds_add_f(DS a, float b) {
+  const DS s = ds_two_sum(a.hi, b);
+  return ds_fast_two_sum(s.hi, __fadd_rn(s.lo, a.lo));
+}
+
+__device__ __forceinline__ DS ds_mul(DS a, DS b) {
+  const float p = __fmul_rn(a.hi, b.hi);
+  float e = __fmaf_rn(a.hi, b.hi, -p);  // the product's rounding error, exactly
+  e = __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, e));
+  return ds_fast_two_sum(p, e);
+}
+
+// 1 / a: the FP32 reciprocal refined by one Newton step in double-single,
+// r + r (1 - a r), which squares its relative error (2^-24 -> about 2^-48).
+__device__ __forceinline__ DS ds_rcp(DS a) {
+  const float r = __frcp_rn(a.hi);
+  const DS ar = ds_mul(a, DS{r, 0.f});
+  const DS res = ds_add(DS{1.f, 0.f}, DS{-ar.hi, -ar.lo});
+  return ds_add_f(ds_mul(DS{r, 0.f}, res), r);
+}
+
+// A 16-bit integer as a float without a conversion instruction: 2^23 + p
+// is a float whose low mantissa bits are p.
+__device__ __forceinline__ float u16_to_float(uint32_t p) {
+  return __fsub_rn(__int_as_float(0x4B000000 | (int)p), 8388608.f);
+}
+
+// A uint64 path count as double-single (its four 16-bit pieces, each exact
+// as a float, summed without losing more than the last of 64 bits' worth).
+__device__ __forceinline__ DS ds_from_u64(unsigned long long c) {
+  DS r{__fmul_rn(u16_to_float((uint32_t)(c >> 48)), 281474976710656.f), 0.f};  // 2^48
+  r = ds_add_f(r, __fmul_rn(u16_to_float((uint32_t)(c >> 32) & 0xFFFFu), 4294967296.f));
+  r = ds_add_f(r, __fmul_rn(u16_to_float((uint32_t)(c >> 16) & 0xFFFFu), 65536.f));
+  return ds_add_f(r, u16_to_float((uint32_t)c & 0xFFFFu));
+}
+
+__device__ __forceinline__ DS ds_from_double(double x) {
+  const float hi = __double2float_rn(x);
+  return {hi, __double2float_rn(x - (double)hi)};
+}
+
+__device__ __forceinline__ double ds_to_double(DS a) { return (double)a.hi + (double)a.lo; }
+
+__device__ __forceinline__ DS shfl_xor_ds(DS a, int o) {
+  return {__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
+}
+
+// r += x, both of any sign and size.
+__device__ __forceinline__ void ds_acc(DS &r, DS x) { r = ds_add(r, x); }
+
+// |a - b| exactly, as hi + lo.
+__device__ __forceinline__ DS ds_abs_diff(float a, float b) {
+  const DS d = ds_two_sum(a, -b);
+  return d.hi < 0.f ? DS{-d.hi, -d.lo} : d;
+}
+
+}  // namespace gr

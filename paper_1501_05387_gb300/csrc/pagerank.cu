@@ -5,15 +5,17 @@
 // iteration gathers over in-neighbourhoods instead (the neighbourhood
 // gather-reduce of Sec. 7), which computes the same sums without a scatter:
 //
-//   k_pr_gather  sum[v] = sum over edges (v, u) of contrib[u], contrib[u] =
-//                rank[u] / deg(u), FP32 (merge-path chunks, segmented warp
-//                sums, one atomicAdd per owner run)
-//   k_pr_update  rank'[v] = (1 - d)/n + d * (sum[v] + D/n), D = rank mass on
-//                degree-0 vertices; writes contrib' and clears sum; the
-//                dangling mass of rank' and the L1 change sum |rank' - rank|
-//                are reduced in FP64
-//   k_pr_end     one thread: stops after max_iter iterations or once the L1
-//                change is below tol
+//   gather  sum[v] = sum over edges (v, u) of contrib[u], contrib[u] =
+//           rank[u] / deg(u), FP32 (gather_reduce_tiles)
+//   update  rank'[v] = (1 - d)/n + d * (sum[v] + D/n), D = rank mass on
+//           degree-0 vertices; writes contrib' and clears sum; the dangling
+//           mass of rank' and the L1 change sum |rank' - rank| are reduced
+//           in double-single and FP64
+//
+// k_pr_do runs the whole iteration loop as one cooperative kernel, a grid
+// barrier after each of the two; every block takes the same stop decision
+// (max_iter iterations, or the L1 change below tol). GR_MODE_LAUNCH enqueues
+// the two as kernels of their own, with k_pr_end deciding.
 //
 // In-neighbours equal out-neighbours only for a symmetric CSR; a directed
 // CSR is transposed once on the device (counting sort by column) and the
@@ -21,41 +23,36 @@
 #include <algorithm>
 #include <cstring>
 
-#include "advance.cuh"
+#include "double_single.cuh"
+#include "gather.cuh"
 
 namespace gr {
 
-// Gather tiles: 20 items for each of 96 threads, 8 blocks per SM with the
-// L1 cache given the rest of the SM's shared-memory array. Long per-thread
-// runs of independent gathers and a large L1 for the hub values beat more,
-// smaller blocks (R-MAT s23, 50 iterations: 256 x 8 at 8 blocks per SM and
-// the default carveout 1.92 ms per iteration, this 1.47 ms).
-constexpr int kPrThreads = 96, kPrItems = 20, kPrBlocksPerSm = 8;
+// Gather: 8 entries per lane, 1536 threads per SM. R-MAT 2^21 (63.5 M
+// entries): 175 us; 207 us at 2048 threads (spills), 174 at 1280, 191 with
+// 16 entries per lane at 1024. The shared-memory tiles before it took 300 us.
+// Two blocks of 768 keep the grid barrier's arrivals few.
+constexpr int kPrThreads = 768, kPrBlocksPerSm = 2;
 
 struct PrCtl {
-  float *rank;           // output ranks (set per call, read by every kernel)
+  GridBarrier bar;
+  float *rank;           // output ranks (set per call)
+  double red[2][2];      // L1 change and dangling mass of the ranks being produced, by parity
   double dangling;       // D of the current ranks
-  double dangling_next;  // D of the ranks being produced
-  double delta;          // L1 change of the last iteration
   double tol;
   float damping;
   int32_t iter;
   int32_t max_iter;
   int32_t done;
+  int32_t error;
 };
 
 struct PrWorkspace {
   DevMem contrib, sum, ctl;
-  DevMem cb;  // chunk bounds of the gather's merge path (fixed per graph)
-  int gather_blocks = 0;  // resident gather blocks (all SMs)
+  GatherPlan plan;  // of the gather structure (fixed per graph)
+  int blocks = 0;  // resident blocks of k_pr_do and k_pr_gather (all SMs)
   DevMem tr_off, tr_col;  // transpose (directed graphs only)
   bool has_transpose = false;
-  cudaGraphExec_t exec = nullptr;
-  cudaGraph_t graph = nullptr;
-  ~PrWorkspace() {
-    if (exec) cudaGraphExecDestroy(exec);
-    if (graph) cudaGraphDestroy(graph);
-  }
 };
 
 void free_pr(PrWorkspace *ws) { delete ws; }
@@ -65,14 +62,14 @@ GR_GUARD_REPORTER(guard_report_pr)
 namespace {
 
 struct PrArgs {
-  const int32_t *R;   // gather structure (CSR or its transpose)
-  const int32_t *C;
+  const int32_t *C;   // gather structure's columns (the CSR's or its transpose's)
   const int32_t *deg; // out-degrees
   int32_t n;
   float *contrib;
   float *sum;
   PrCtl *ctl;
-  const int32_t *cb;  // chunk bounds of the gather
+  int32_t m;
+  GatherPlanArgs plan;
 };
 
 __global__ void k_pr_init(PrArgs a, float *rank, float damping, int32_t max_iter, double tol,
@@ -87,67 +84,118 @@ __global__ void k_pr_init(PrArgs a, float *rank, float damping, int32_t max_iter
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     PrCtl *c = a.ctl;
+    grid_barrier_reset(&c->bar);
     c->rank = rank;
     c->dangling = (double)num_dangling / (double)a.n;
-    c->dangling_next = 0.0;
-    c->delta = 0.0;
+    c->red[0][0] = c->red[0][1] = c->red[1][0] = c->red[1][1] = 0.0;
     c->tol = tol;
     c->damping = damping;
     c->iter = 0;
     c->max_iter = max_iter;
     c->done = max_iter <= 0;
+    c->error = kDevOk;
   }
 }
 
+// plain loads: k_pr_do rewrites contrib between its gathers
 struct ContribG {
+  static constexpr bool kWeighted = false;
   const float *contrib;
-  __device__ __forceinline__ float operator()(int32_t u, int32_t) const { return __ldg(contrib + u); }
+  __device__ __forceinline__ float operator()(int32_t u, int32_t) const { return contrib[u]; }
 };
 
-__global__ void __launch_bounds__(kPrThreads, kPrBlocksPerSm) k_pr_gather(PrArgs a) {
-  if (a.ctl->done) return;
-  ContribG g{a.contrib};
-  lb_neighbor_reduce<kPrThreads, kPrItems, float>(a.R, a.C, a.n, g, a.sum, a.cb);
+__device__ __forceinline__ void pr_gather(const PrArgs &a) {
+  const ContribG g{a.contrib};
+  gather_reduce_tiles<1, float, ReduceSum<float>>(a.plan, a.C, nullptr, 0, a.m, g, a.sum,
+                                                  spread_warp(), grid_warps());
 }
 
-__global__ void __launch_bounds__(256) k_pr_update(PrArgs a) {
-  PrCtl *c = a.ctl;
-  if (c->done) return;
-  const double d = c->damping;
-  const double base = (1.0 - d) / a.n + d * c->dangling / a.n;
-  float *rank = c->rank;
-  double dang = 0.0, delta = 0.0;
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < a.n;
-       v += (int64_t)gridDim.x * blockDim.x) {
-    const float rn = (float)(base + d * (double)a.sum[v]);
-    const float ro = rank[v];
+// The part of an iteration's new rank that all vertices share.
+__device__ __forceinline__ double pr_base(float damping, int32_t n, double dangling) {
+  const double d = damping;
+  return (1.0 - d) / n + d * dangling / n;
+}
+
+// New ranks from the sums, their contributions, the block's share of the L1
+// change (red[0]) and of the dangling mass (red[1]). base + d * sum is formed
+// in double-single and rounded once: the FP64 form (two conversions and an
+// FMA per vertex, two more operations for the change, and the base's
+// divisions in every thread) kept the FP64 pipe busy for 50 us of a 245 us
+// iteration at R-MAT 2^21.
+__device__ __forceinline__ void pr_update(const PrArgs &a, float *rank, float damping, double base,
+                                          double *smem, double *red) {
+  const float bh = (float)base, bl = (float)(base - (double)bh);
+  DS dang{0.f, 0.f}, delta{0.f, 0.f};
+  const int lane = threadIdx.x & 31;
+  for (int64_t v = spread_warp() * 32 + lane; v < a.n; v += grid_warps() * 32) {
+    const float s = a.sum[v], ro = rank[v];
     const int32_t dg = a.deg[v];
+    const float p = __fmul_rn(damping, s);  // p + e = damping * s exactly
+    const float e = __fmaf_rn(damping, s, -p);
+    const DS t = ds_two_sum(bh, p);
+    const float rn = __fadd_rn(t.hi, __fadd_rn(t.lo, __fadd_rn(e, bl)));
     rank[v] = rn;
     a.contrib[v] = dg ? rn / (float)dg : 0.0f;
     a.sum[v] = 0.0f;
-    if (!dg) dang += rn;
-    delta += fabs((double)rn - (double)ro);
+    if (!dg) dang = ds_add_f(dang, rn);
+    delta = ds_add(delta, ds_abs_diff(rn, ro));
   }
-  __shared__ double s_red[33];
-  dang = block_sum(dang, s_red);
-  delta = block_sum(delta, s_red);
-  if (threadIdx.x == 0) {
-    if (dang != 0.0) atomicAdd(&c->dangling_next, dang);
-    atomicAdd(&c->delta, delta);
+  block_add_f64<kPrThreads>(ds_to_double(delta), smem, red);
+  block_add_f64<kPrThreads>(ds_to_double(dang), smem, red + 1);
+}
+
+__device__ __forceinline__ double read_f64(const double *p) { return *(const volatile double *)p; }
+
+__global__ void __launch_bounds__(kPrThreads, kPrBlocksPerSm) k_pr_do(PrArgs a) {
+  __shared__ double smem[kPrThreads];
+  __shared__ double s_base;
+  PrCtl *c = a.ctl;
+  float *rank = c->rank;
+  const float damping = c->damping;
+  const int32_t max_iter = c->max_iter;
+  double dangling = c->dangling;
+  int32_t it = 0, gen = 0;
+  while (it < max_iter) {
+    pr_gather(a);
+    if (threadIdx.x == 0) s_base = pr_base(damping, a.n, dangling);
+    if (!grid_sync(&c->bar, &c->error, gen)) return;
+    // the other parity was read by every block before this barrier
+    double *red = c->red[it & 1];
+    if (blockIdx.x == 0 && threadIdx.x < 2) c->red[(it + 1) & 1][threadIdx.x] = 0.0;
+    pr_update(a, rank, damping, s_base, smem, red);
+    if (!grid_sync(&c->bar, &c->error, gen)) return;
+    ++it;
+    dangling = read_f64(red + 1);
+    if (read_f64(red) < c->tol) break;
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    c->iter = it;
+    c->done = 1;
   }
 }
 
-__global__ void k_pr_end(PrArgs a, cudaGraphConditionalHandle h, int32_t use_cond) {
-  if (threadIdx.x != 0) return;
+// GR_MODE_LAUNCH: one iteration as three kernels.
+__global__ void __launch_bounds__(kPrThreads, kPrBlocksPerSm) k_pr_gather(PrArgs a) {
+  if (!a.ctl->done) pr_gather(a);
+}
+
+__global__ void __launch_bounds__(kPrThreads, kPrBlocksPerSm) k_pr_update(PrArgs a) {
+  __shared__ double smem[kPrThreads];
+  __shared__ double s_base;
   PrCtl *c = a.ctl;
-  if (!c->done) {
-    c->iter += 1;
-    c->dangling = c->dangling_next;
-    c->dangling_next = 0.0;
-    if (c->iter >= c->max_iter || c->delta < c->tol) c->done = 1;
-    else c->delta = 0.0;
-  }
-  if (use_cond) cudaGraphSetConditional(h, c->done ? 0u : 1u);
+  if (c->done) return;
+  if (threadIdx.x == 0) s_base = pr_base(c->damping, a.n, c->dangling);
+  __syncthreads();
+  pr_update(a, c->rank, c->damping, s_base, smem, c->red[0]);
+}
+
+__global__ void k_pr_end(PrArgs a) {
+  PrCtl *c = a.ctl;
+  if (c->done) return;
+  c->iter += 1;
+  if (c->iter >= c->max_iter || c->red[0][0] < c->tol) c->done = 1;
+  c->dangling = c->red[0][1];
+  c->red[0][0] = c->red[0][1] = 0.0;
 }
 
 // ---- transpose for directed graphs: counting sort of (u, v) by v
@@ -199,7 +247,8 @@ static gr_status ensure_pr_ws(gr_graph *g, cudaStream_t s) {
     GR_TRY(ws->ctl.alloc(sizeof(PrCtl), "PageRank control"));
     int per_sm = 1;
     GR_TRY(fit_carveout(k_pr_gather, kPrThreads, kPrBlocksPerSm, g->device, &per_sm));
-    ws->gather_blocks = per_sm * g->num_sms;
+    GR_TRY(fit_carveout(k_pr_do, kPrThreads, kPrBlocksPerSm, g->device, &per_sm));
+    ws->blocks = per_sm * g->num_sms;
     g->pr = ws.release();
   }
   PrWorkspace *ws = g->pr;
@@ -221,69 +270,29 @@ static gr_status ensure_pr_ws(gr_graph *g, cudaStream_t s) {
     GR_CUDA(cudaStreamSynchronize(s));
     ws->has_transpose = true;
   }
-  if (!ws->cb.p) {
-    // the gather's merge path over all vertices is the same every
-    // iteration: its chunk bounds are found once
-    const int32_t *R = g->symmetric ? g->row_off.as<int32_t>() : ws->tr_off.as<int32_t>();
-    const int32_t chunks = merge_chunks(g->n, g->m, kPrThreads * kPrItems);
-    GR_TRY(ws->cb.alloc(sizeof(int32_t) * ((size_t)chunks + 1), "PageRank chunk bounds"));
-    k_chunk_bounds<<<(chunks + 256) / 256, 256, 0, s>>>(R, g->n, kPrThreads * kPrItems, chunks,
-                                                         ws->cb.as<int32_t>());
-    GR_CUDA(cudaGetLastError());
-  }
-  return GR_OK;
+  const int32_t *R = g->symmetric ? g->row_off.as<int32_t>() : ws->tr_off.as<int32_t>();
+  return gather_plan_build(&ws->plan, R, g->n, g->m, s);
 }
 
 static PrArgs pr_args(gr_graph *g) {
   PrWorkspace *ws = g->pr;
   PrArgs a;
-  a.R = g->symmetric ? g->row_off.as<int32_t>() : ws->tr_off.as<int32_t>();
   a.C = g->symmetric ? g->col.as<int32_t>() : ws->tr_col.as<int32_t>();
   a.deg = g->degree.as<int32_t>();
   a.n = g->n;
   a.contrib = ws->contrib.as<float>();
   a.sum = ws->sum.as<float>();
   a.ctl = ws->ctl.as<PrCtl>();
-  a.cb = ws->cb.as<int32_t>();
+  a.m = (int32_t)g->m;
+  a.plan = ws->plan.a;
   return a;
 }
 
-static gr_status pr_enqueue_iter(gr_graph *g, const PrArgs &a, cudaStream_t s,
-                                 cudaGraphConditionalHandle h, int use_cond) {
-  k_pr_gather<<<g->pr->gather_blocks, kPrThreads, 0, s>>>(a);
-  k_pr_update<<<g->num_sms * 4, 256, 0, s>>>(a);
-  k_pr_end<<<1, 32, 0, s>>>(a, h, use_cond);
+static gr_status pr_enqueue_iter(gr_graph *g, const PrArgs &a, cudaStream_t s) {
+  k_pr_gather<<<g->pr->blocks, kPrThreads, 0, s>>>(a);
+  k_pr_update<<<g->pr->blocks, kPrThreads, 0, s>>>(a);
+  k_pr_end<<<1, 1, 0, s>>>(a);
   GR_CUDA(cudaGetLastError());
-  return GR_OK;
-}
-
-static gr_status build_pr_graph(gr_graph *g) {
-  PrWorkspace *ws = g->pr;
-  if (ws->exec) return GR_OK;
-  cudaGraph_t graph;
-  GR_CUDA(cudaGraphCreate(&graph, 0));
-  cudaGraphConditionalHandle h;
-  GR_CUDA(cudaGraphConditionalHandleCreate(&h, graph, 1, cudaGraphCondAssignDefault));
-  cudaGraphNodeParams cp = {};
-  cp.type = cudaGraphNodeTypeConditional;
-  cp.conditional.handle = h;
-  cp.conditional.type = cudaGraphCondTypeWhile;
-  cp.conditional.size = 1;
-  cudaGraphNode_t node;
-  GR_CUDA(cudaGraphAddNode(&node, graph, nullptr, nullptr, 0, &cp));
-  cudaGraph_t body = cp.conditional.phGraph_out[0];
-  cudaStream_t cs;
-  GR_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
-  GR_CUDA(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0,
-                                        cudaStreamCaptureModeThreadLocal));
-  gr_status st = pr_enqueue_iter(g, pr_args(g), cs, h, 1);
-  cudaGraph_t captured;
-  cudaError_t e = cudaStreamEndCapture(cs, &captured);
-  cudaStreamDestroy(cs);
-  if (st != GR_OK) return st;
-  GR_CUDA(e);
-  GR_CUDA(cudaGraphInstantiate(&ws->exec, graph, 0));
-  ws->graph = graph;
   return GR_OK;
 }
 
@@ -318,15 +327,15 @@ gr_status gr_pagerank(gr_graph *g, float damping, int32_t max_iter, double tol, 
       PrCtl h;
       for (int32_t it = 0; it < max_iter;) {
         const int32_t batch = std::min<int32_t>(8, max_iter - it);
-        for (int32_t i = 0; i < batch; ++i) GR_TRY(pr_enqueue_iter(g, a, s, 0, 0));
+        for (int32_t i = 0; i < batch; ++i) GR_TRY(pr_enqueue_iter(g, a, s));
         it += batch;
         GR_CUDA(cudaMemcpyAsync(&h, a.ctl, sizeof(h), cudaMemcpyDeviceToHost, s));
         GR_CUDA(cudaStreamSynchronize(s));
         if (h.done) break;
       }
     } else {
-      GR_TRY(build_pr_graph(g));
-      GR_CUDA(cudaGraphLaunch(g->pr->exec, s));
+      void *args[] = {&a};
+      GR_CUDA(cudaLaunchCooperativeKernel((void *)k_pr_do, g->pr->blocks, kPrThreads, args, 0, s));
     }
   }
   if (cp_rank)
@@ -336,6 +345,7 @@ gr_status gr_pagerank(gr_graph *g, float damping, int32_t max_iter, double tol, 
     PrCtl h;
     GR_CUDA(cudaMemcpyAsync(&h, a.ctl, sizeof(h), cudaMemcpyDeviceToHost, s));
     GR_CUDA(cudaStreamSynchronize(s));
+    if (h.error == kDevTimeout) return fail(GR_ETIMEOUT, "a device-side wait timed out");
     *iters = h.iter;
   }
   GR_TRY(end_call(g, s));

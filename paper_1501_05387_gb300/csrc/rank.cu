@@ -4,15 +4,19 @@
 // computation the paper cites).
 //
 //   gr_neighbor_reduce  out[v] = sum / weighted sum / min / max of x[u] over
-//                the entries (v, u) of v's row, for every vertex or for the
-//                vertices of a frontier list (lb_gather_reduce; a frontier's
-//                degree scan is computed first, three kernels).
+//                the entries (v, u) of v's row, for every vertex
+//                (gather_reduce_tiles) or for the vertices of a frontier list
+//                (lb_gather_reduce; the frontier's degree scan is computed
+//                first, three kernels).
 //   gr_hits, gr_salsa   on a bipartite graph stored symmetrically (hubs
 //                [0, n_left), authorities [n_left, n)): one iteration is the
 //                2-hop traversal hub -> authority -> hub, two gather-reduce
 //                passes over the two vertex ranges (each authority gathers
-//                from its hubs, then each hub from its authorities), with a
-//                normalisation sweep after each pass.
+//                from its hubs, then each hub from its authorities), each
+//                followed by a sweep over its range. HITS sums the
+//                authorities' squares while the hubs already gather the
+//                unscaled sums, and the hubs' while the authorities are
+//                scaled: four grid barriers an iteration.
 //   gr_ppr       personalized PageRank: per iteration one gather-reduce over
 //                all vertices and one update sweep (teleport and dangling
 //                mass to the seeds).
@@ -27,16 +31,24 @@
 #include <cmath>
 #include <cstring>
 
-#include "advance.cuh"
+#include "gather.cuh"
 
 namespace gr {
 
-// Gather tiles of 12 items for each of 96 threads, 8 blocks per SM, the
-// rest of the SM's shared-memory array left to L1 (R-MAT s23 gather-reduce,
-// FP64 sum: 256 x 8 at 4 blocks per SM with the default carveout 3.48 ms,
-// with the fitted carveout 1.96 ms, this tile 1.57 ms).
+// A frontier's gather tiles: 12 items for each of 96 threads, 8 blocks per
+// SM, the rest of the SM's shared-memory array left to L1.
 constexpr int kRkThreads = 96, kRkItems = 12;
 constexpr int kRkBlocksPerSm = 8;
+// Gathers over vertex ranges: two groups of 8 FP64 entries per lane and 1024
+// threads per SM (FP64 adds are scarce: a lane's 16 share one scan over the
+// warp). R-MAT 2^21, 63.5 M entries: 197 us; 207 us with one group at 1280
+// threads, 234 at 2048; int32 values take one group at 1536 threads. The
+// shared-memory tiles before took 275 us for 45 M entries, this 162.
+constexpr int kRgThreads = 256;
+constexpr int kRgBlocksF64 = 4, kRgBlocksI32 = 6;
+// The rankings' persistent kernels: the same 1024 threads per SM in one
+// block, so that a grid barrier has one arrival per SM.
+constexpr int kRkDoThreads = 1024;
 
 struct RankCtl {
   GridBarrier bar;
@@ -47,13 +59,10 @@ struct RankCtl {
 };
 
 struct RankWorkspace {
-  DevMem cur, tmp, dv, tele, ctl, seeds;
+  DevMem cur, tmp, dv, idg, tele, ctl, seeds;
   DevMem fscan, part;   // gr_neighbor_reduce: a frontier's degree scan, block partials
   int32_t bip_left = -1;  // n_left the graph was last checked to be bipartite for
-  // chunk bounds of the gather's merge paths: all vertices (fixed per
-  // graph), and the hub and authority ranges of the last n_left
-  DevMem cb_all, cb_hub, cb_auth;
-  int32_t cb_left = -1;
+  GatherPlan plan;  // row structure of the gathers over vertex ranges
 };
 
 void free_rank(RankWorkspace *ws) { delete ws; }
@@ -61,7 +70,10 @@ void free_rank(RankWorkspace *ws) { delete ws; }
 namespace {
 
 // ------------------------------------------------------ gather functors
+// operator()(u, e): the value an entry e = (v, u) brings; with kWeighted a
+// gather over a vertex range passes w(e) itself (wt), a frontier's the entry
 struct GatherF64 {
+  static constexpr bool kWeighted = false;
   const double *x;
   __device__ __forceinline__ double operator()(int32_t u, int32_t) const { return x[u]; }
 };
@@ -72,7 +84,15 @@ struct GatherWF64 {
     return (double)w[e] * x[u];
   }
 };
+struct GatherWtF64 {
+  static constexpr bool kWeighted = true;
+  const double *x;
+  __device__ __forceinline__ double operator()(int32_t u, int32_t wt) const {
+    return (double)(uint32_t)wt * x[u];
+  }
+};
 struct GatherI32 {
+  static constexpr bool kWeighted = false;
   const int32_t *x;
   __device__ __forceinline__ int32_t operator()(int32_t u, int32_t) const { return x[u]; }
 };
@@ -145,12 +165,22 @@ __global__ void k_scan_apply(const int32_t *R, const int32_t *Q, int32_t q, cons
   }
 }
 
-template <class T, class OP, bool FRONTIER, class G>
-__global__ void __launch_bounds__(kRkThreads, kRkBlocksPerSm) k_nr_gather(const int32_t *R, const int32_t *C,
-                                                           const int32_t *Q, const int32_t *S,
-                                                           int32_t q, G g, T *out,
-                                                           const int32_t *cb) {
-  lb_gather_reduce<kRkThreads, kRkItems, T, OP, FRONTIER>(R, C, Q, S, q, 0, g, out, cb);
+template <class T, class OP, class G>
+__global__ void __launch_bounds__(kRkThreads, kRkBlocksPerSm) k_nr_frontier(
+    const int32_t *R, const int32_t *C, const int32_t *Q, const int32_t *S, int32_t q, G g, T *out) {
+  lb_gather_reduce<kRkThreads, kRkItems, T, OP>(R, C, Q, S, q, g, out);
+}
+
+template <class T>
+constexpr int range_groups() { return sizeof(T) == 8 ? 2 : 1; }
+template <class T>
+constexpr int range_blocks() { return sizeof(T) == 8 ? kRgBlocksF64 : kRgBlocksI32; }
+
+template <class T, class OP, class G>
+__global__ void __launch_bounds__(kRgThreads, range_blocks<T>()) k_nr_all(
+    GatherPlanArgs plan, const int32_t *C, const int32_t *W, int32_t m, G g, T *out) {
+  gather_reduce_tiles<range_groups<T>(), T, OP>(
+      plan, C, W, 0, m, g, out, spread_warp(), grid_warps());
 }
 
 // ------------------------------------------------------ ranking kernels
@@ -162,95 +192,111 @@ struct RankArgs {
   double *cur;   // scores
   double *tmp;   // gathered sums (zero before each gather)
   double *dv;    // score / degree (SALSA, PPR)
+  double *idg;   // 1 / degree, 0 where there is none (SALSA, PPR)
   const double *tele;  // teleport vector (PPR)
   double damping;
   double tol;
   int32_t max_iter;
   RankCtl *ctl;
-  const int32_t *cb_all, *cb_hub, *cb_auth;  // chunk bounds of the gathers' ranges
+  GatherPlanArgs plan;
 };
 
-// Block-wide FP64 sum, added to *dst by thread 0.
-__device__ __forceinline__ void block_add(double v, double *smem, double *dst) {
-  const double t = block_sum(v, smem);
-  if (threadIdx.x == 0 && t != 0.0) atomicAdd(dst, t);
+// out[v] += sum of x over the rows of the vertices [v0, v1), the grid's warps
+// sharing their entries.
+__device__ __forceinline__ void range_sum(const RankArgs &a, int32_t v0, int32_t v1,
+                                          const double *x, double *out) {
+  const GatherF64 g{x};
+  const int32_t eb = a.R[v0], ee = a.R[v1];
+  // tiles of 512 entries, of 256 where those would leave warps without one
+  if (ee - eb >= grid_warps() * 512)
+    gather_reduce_tiles<2, double, ReduceSum<double>>(a.plan, a.C, nullptr, eb, ee, g, out,
+                                                      spread_warp(), grid_warps());
+  else
+    gather_reduce_tiles<1, double, ReduceSum<double>>(a.plan, a.C, nullptr, eb, ee, g, out,
+                                                      spread_warp(), grid_warps());
 }
 
 __device__ __forceinline__ double read_slot(const double *p) { return *(const volatile double *)p; }
 
+// x / deg from idg = 1 / deg (0 where deg is 0), correctly rounded by one
+// remainder step (Markstein, "Computation of elementary functions on the IBM
+// RISC System/6000 processor", 1990): three FP64 operations where a division
+// takes some twenty, which at R-MAT 2^21 was 80 us of a PPR iteration.
+__device__ __forceinline__ double over_degree(double x, int32_t deg, double idg) {
+  const double q = x * idg;
+  return fma(fma(-q, (double)deg, x), idg, q);
+}
+
+// 1 / |x| of a vector with the given sum of squares (1 for a zero vector),
+// by one thread: every thread's own square root and division would hold the
+// FP64 pipe for 12 us.
+__device__ __forceinline__ void block_inv_norm(const double *slot, double *s_inv) {
+  if (threadIdx.x == 0) {
+    const double t = read_slot(slot);
+    *s_inv = t > 0.0 ? 1.0 / sqrt(t) : 1.0;
+  }
+  __syncthreads();
+}
+
 template <int KIND>  // 0: HITS, 1: SALSA
-__global__ void __launch_bounds__(kRkThreads, kRkBlocksPerSm) k_bipartite_do(RankArgs a) {
-  __shared__ double red[33];
+__global__ void __launch_bounds__(kRkDoThreads, 1) k_bipartite_do(RankArgs a) {
+  __shared__ double smem[kRkDoThreads];
+  __shared__ double s_inv;
   RankCtl *c = a.ctl;
-  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const int64_t tid = spread_warp() * 32 + (threadIdx.x & 31);
+  const int64_t stride = grid_warps() * 32;
   const int32_t nl = a.n_left, n = a.n;
   int32_t gen = 0;
   int32_t it = 0;
   while (it < a.max_iter) {
-    double *slot = c->red[it & 1];
+    double *slot = c->red[it & 1];  // authorities' squares, hubs' squares, L1 change
     // authorities gather from their hubs: h[l] (HITS) or h[l] / deg(l) (SALSA)
-    {
-      GatherF64 gf{KIND == 0 ? a.cur : a.dv};
-      lb_gather_reduce<kRkThreads, kRkItems, double, ReduceSum<double>, false>(
-          a.R, a.C, nullptr, a.R + nl, n - nl, nl, gf, a.tmp, a.cb_auth);
-    }
+    range_sum(a, nl, n, KIND == 0 ? a.cur : a.dv, a.tmp);
     if (!grid_sync(&c->bar, &c->error, gen)) return;
     if (blockIdx.x == 0 && threadIdx.x < 4) c->red[(it + 1) & 1][threadIdx.x] = 0.0;
-    double inv = 1.0;
+    double delta = 0.0;
     if (KIND == 0) {
+      // hubs gather the unscaled sums of their authorities
       double ss = 0.0;
       for (int64_t r = nl + tid; r < n; r += stride) ss += a.tmp[r] * a.tmp[r];
-      block_add(ss, red, &slot[0]);
+      block_add_f64<kRkDoThreads>(ss, smem, &slot[0]);
+      range_sum(a, 0, nl, a.tmp, a.tmp);
       if (!grid_sync(&c->bar, &c->error, gen)) return;
-      const double t = read_slot(&slot[0]);
-      inv = t > 0.0 ? 1.0 / sqrt(t) : 1.0;
-    }
-    {
-      double delta = 0.0;
+      block_inv_norm(&slot[0], &s_inv);
+      const double inv = s_inv;
       for (int64_t r = nl + tid; r < n; r += stride) {
         const double x = a.tmp[r] * inv;
         delta += fabs(x - a.cur[r]);
         a.cur[r] = x;
-        if (KIND == 1) {
-          const int32_t d = a.R[r + 1] - a.R[r];
-          a.dv[r] = d ? x / d : 0.0;
-        }
         a.tmp[r] = 0.0;
       }
-      block_add(delta, red, &slot[2]);
-    }
-    if (!grid_sync(&c->bar, &c->error, gen)) return;
-    // hubs gather from the new authorities
-    {
-      GatherF64 gf{KIND == 0 ? a.cur : a.dv};
-      lb_gather_reduce<kRkThreads, kRkItems, double, ReduceSum<double>, false>(
-          a.R, a.C, nullptr, a.R, nl, 0, gf, a.tmp, a.cb_hub);
-    }
-    if (!grid_sync(&c->bar, &c->error, gen)) return;
-    inv = 1.0;
-    if (KIND == 0) {
-      double ss = 0.0;
+      ss = 0.0;
       for (int64_t l = tid; l < nl; l += stride) ss += a.tmp[l] * a.tmp[l];
-      block_add(ss, red, &slot[1]);
+      block_add_f64<kRkDoThreads>(ss, smem, &slot[1]);
       if (!grid_sync(&c->bar, &c->error, gen)) return;
-      const double t = read_slot(&slot[1]);
-      inv = t > 0.0 ? 1.0 / sqrt(t) : 1.0;
-    }
-    {
-      double delta = 0.0;
-      for (int64_t l = tid; l < nl; l += stride) {
-        const double x = a.tmp[l] * inv;
-        delta += fabs(x - a.cur[l]);
-        a.cur[l] = x;
-        if (KIND == 1) {
-          const int32_t d = a.R[l + 1] - a.R[l];
-          a.dv[l] = d ? x / d : 0.0;
-        }
-        a.tmp[l] = 0.0;
+      block_inv_norm(&slot[1], &s_inv);  // of the unscaled sums: their scale falls out
+    } else {
+      for (int64_t r = nl + tid; r < n; r += stride) {
+        const double x = a.tmp[r];
+        delta += fabs(x - a.cur[r]);
+        a.cur[r] = x;
+        a.dv[r] = over_degree(x, a.R[r + 1] - a.R[r], a.idg[r]);
+        a.tmp[r] = 0.0;
       }
-      block_add(delta, red, &slot[2]);
+      if (!grid_sync(&c->bar, &c->error, gen)) return;
+      // hubs gather from the new authorities
+      range_sum(a, 0, nl, a.dv, a.tmp);
+      if (!grid_sync(&c->bar, &c->error, gen)) return;
     }
+    const double inv = KIND == 0 ? s_inv : 1.0;
+    for (int64_t l = tid; l < nl; l += stride) {
+      const double x = KIND == 0 ? a.tmp[l] * inv : a.tmp[l];
+      delta += fabs(x - a.cur[l]);
+      a.cur[l] = x;
+      if (KIND == 1) a.dv[l] = over_degree(x, a.R[l + 1] - a.R[l], a.idg[l]);
+      a.tmp[l] = 0.0;
+    }
+    block_add_f64<kRkDoThreads>(delta, smem, &slot[2]);
     if (!grid_sync(&c->bar, &c->error, gen)) return;
     ++it;
     if (read_slot(&slot[2]) < a.tol) break;
@@ -258,11 +304,11 @@ __global__ void __launch_bounds__(kRkThreads, kRkBlocksPerSm) k_bipartite_do(Ran
   if (blockIdx.x == 0 && threadIdx.x == 0) c->iters = it;
 }
 
-__global__ void __launch_bounds__(kRkThreads, kRkBlocksPerSm) k_ppr_do(RankArgs a) {
-  __shared__ double red[33];
+__global__ void __launch_bounds__(kRkDoThreads, 1) k_ppr_do(RankArgs a) {
+  __shared__ double smem[kRkDoThreads];
   RankCtl *c = a.ctl;
-  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const int64_t tid = spread_warp() * 32 + (threadIdx.x & 31);
+  const int64_t stride = grid_warps() * 32;
   const double d = a.damping;
   int32_t gen = 0;
   int32_t it = 0;
@@ -270,26 +316,23 @@ __global__ void __launch_bounds__(kRkThreads, kRkBlocksPerSm) k_ppr_do(RankArgs 
   double dangling = read_slot(&c->red[1][3]);
   while (it < a.max_iter) {
     double *slot = c->red[it & 1];
-    {
-      GatherF64 gf{a.dv};
-      lb_gather_reduce<kRkThreads, kRkItems, double, ReduceSum<double>, false>(
-          a.R, a.C, nullptr, a.R, a.n, 0, gf, a.tmp, a.cb_all);
-    }
+    range_sum(a, 0, a.n, a.dv, a.tmp);
     if (!grid_sync(&c->bar, &c->error, gen)) return;
     if (blockIdx.x == 0 && threadIdx.x < 4) c->red[(it + 1) & 1][threadIdx.x] = 0.0;
     double delta = 0.0, dang = 0.0;
     for (int64_t v = tid; v < a.n; v += stride) {
-      const double t = a.tele[v];
-      const double x = (1.0 - d) * t + d * (a.tmp[v] + dangling * t);
+      const double t = a.tele[v], s = a.tmp[v];
+      // most vertices are not seeds: their teleport terms are zero
+      const double x = t == 0.0 ? d * s : (1.0 - d) * t + d * (s + dangling * t);
       delta += fabs(x - a.cur[v]);
       a.cur[v] = x;
       const int32_t deg = a.R[v + 1] - a.R[v];
-      a.dv[v] = deg ? x / deg : 0.0;
+      a.dv[v] = over_degree(x, deg, a.idg[v]);
       if (!deg) dang += x;
       a.tmp[v] = 0.0;
     }
-    block_add(delta, red, &slot[2]);
-    block_add(dang, red, &slot[3]);
+    block_add_f64<kRkDoThreads>(delta, smem, &slot[2]);
+    block_add_f64<kRkDoThreads>(dang, smem, &slot[3]);
     if (!grid_sync(&c->bar, &c->error, gen)) return;
     ++it;
     dangling = read_slot(&slot[3]);
@@ -318,7 +361,11 @@ __global__ void k_rank_init(RankArgs a, int32_t kind) {
     else x = a.tele[v];
     a.cur[v] = x;
     a.tmp[v] = 0.0;
-    if (a.dv) a.dv[v] = deg ? x / deg : 0.0;
+    if (kind != 0) {
+      const double idg = deg ? 1.0 / deg : 0.0;
+      a.idg[v] = idg;
+      a.dv[v] = over_degree(x, deg, idg);
+    }
   }
   if (tid == 0) {
     RankCtl *c = a.ctl;
@@ -370,63 +417,53 @@ __global__ void k_check_bipartite(const int32_t *R, const int32_t *C, int32_t n,
 
 }  // namespace
 
-static gr_status rank_ws(gr_graph *g, RankWorkspace **out) {
+static gr_status rank_ws(gr_graph *g, bool by_degree, RankWorkspace **out) {
   if (!g->rank) g->rank = new RankWorkspace();
   RankWorkspace *ws = g->rank;
   const size_t bytes = sizeof(double) * (size_t)g->n;
-  if (!ws->cur.p) {
+  if (!ws->ctl.p) {  // the last of them: an earlier call may have failed half way
     GR_TRY(ws->cur.alloc(bytes, "ranking scores"));
     GR_TRY(ws->tmp.alloc(bytes, "ranking sums"));
     GR_TRY(ws->dv.alloc(bytes, "ranking scores per degree"));
     GR_TRY(ws->ctl.alloc(sizeof(RankCtl), "ranking control"));
   }
+  if (by_degree && !ws->idg.p) GR_TRY(ws->idg.alloc(bytes, "ranking inverse degrees"));
   *out = ws;
   return GR_OK;
 }
 
-// Chunk bounds of the gather's merge path over the vertex range [v0, v1)
-// into buf (one search per chunk, on `s`).
-static gr_status range_bounds(gr_graph *g, int32_t v0, int32_t v1, DevMem &buf, cudaStream_t s) {
-  const int32_t *R = g->row_off.as<int32_t>();
-  int32_t r[2] = {0, 0};
-  // the range's entry count: two offsets, read once per call
-  GR_CUDA(cudaMemcpyAsync(&r[0], R + v0, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-  GR_CUDA(cudaMemcpyAsync(&r[1], R + v1, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-  GR_CUDA(cudaStreamSynchronize(s));
-  const int32_t chunks = merge_chunks(v1 - v0, (long long)r[1] - r[0], kRkThreads * kRkItems);
-  if (buf.bytes < sizeof(int32_t) * ((size_t)chunks + 1))
-    GR_TRY(buf.alloc(sizeof(int32_t) * ((size_t)chunks + 1), "gather chunk bounds"));
-  k_chunk_bounds<<<(chunks + 256) / 256, 256, 0, s>>>(R + v0, v1 - v0, kRkThreads * kRkItems,
-                                                       chunks, buf.as<int32_t>());
+// One gather-reduce over all vertices or a frontier, at the resident blocks
+// per SM its launch bounds ask for, the rest of the SM's shared-memory array
+// left to L1.
+template <class T, class OP, class G>
+static gr_status nr_launch_all(gr_graph *g, RankWorkspace *ws, cudaStream_t s, G gf, T *out) {
+  GR_TRY(gather_plan_build(&ws->plan, g->row_off.as<int32_t>(), g->n, g->m, s));
+  auto kern = k_nr_all<T, OP, G>;
+  int per_sm = 1;
+  GR_TRY(fit_carveout(kern, kRgThreads, range_blocks<T>(), g->device, &per_sm));
+  kern<<<per_sm * g->num_sms, kRgThreads, 0, s>>>(ws->plan.a, g->col.as<int32_t>(),
+                                                  g->w.as<int32_t>(), (int32_t)g->m, gf, out);
   GR_CUDA(cudaGetLastError());
   return GR_OK;
 }
 
-static gr_status all_bounds(gr_graph *g, RankWorkspace *ws, cudaStream_t s) {
-  if (!ws->cb_all.p) GR_TRY(range_bounds(g, 0, g->n, ws->cb_all, s));
-  return GR_OK;
-}
-
-// One gather-reduce over a range or a frontier, at the tile's resident
-// blocks per SM with the rest of the shared-memory array left to L1.
-template <class T, class OP, bool FRONTIER, class G>
-static gr_status nr_launch(gr_graph *g, cudaStream_t s, const int32_t *R, const int32_t *C,
-                           const int32_t *Q, const int32_t *S, int32_t q, G gf, T *out,
-                           const int32_t *cb) {
-  auto kern = k_nr_gather<T, OP, FRONTIER, G>;
+template <class T, class OP, class G>
+static gr_status nr_launch_frontier(gr_graph *g, cudaStream_t s, const int32_t *Q,
+                                    const int32_t *S, int32_t q, G gf, T *out) {
+  auto kern = k_nr_frontier<T, OP, G>;
   int per_sm = 1;
   GR_TRY(fit_carveout(kern, kRkThreads, kRkBlocksPerSm, g->device, &per_sm));
-  kern<<<per_sm * g->num_sms, kRkThreads, 0, s>>>(R, C, Q, S, q, gf, out, cb);
+  kern<<<per_sm * g->num_sms, kRkThreads, 0, s>>>(g->row_off.as<int32_t>(), g->col.as<int32_t>(),
+                                                  Q, S, q, gf, out);
   GR_CUDA(cudaGetLastError());
   return GR_OK;
 }
 
 static gr_status rank_launch(gr_graph *g, void *kern, RankArgs &a, cudaStream_t s) {
   int per_sm = 1;
-  GR_TRY(fit_carveout(kern, kRkThreads, kRkBlocksPerSm, g->device, &per_sm));
-  const int blocks = per_sm * g->num_sms;
+  GR_TRY(fit_carveout(kern, kRkDoThreads, 1, g->device, &per_sm));
   void *args[] = {&a};
-  GR_CUDA(cudaLaunchCooperativeKernel(kern, blocks, kRkThreads, args, 0, s));
+  GR_CUDA(cudaLaunchCooperativeKernel(kern, per_sm * g->num_sms, kRkDoThreads, args, 0, s));
   return GR_OK;
 }
 
@@ -459,7 +496,7 @@ static gr_status bipartite_run(gr_graph *g, int kind, int32_t n_left, int32_t ma
   cudaStream_t s = (cudaStream_t)stream;
   GR_TRY(begin_call(g, s));
   RankWorkspace *ws;
-  GR_TRY(rank_ws(g, &ws));
+  GR_TRY(rank_ws(g, kind == 1, &ws));
   if (ws->bip_left != n_left) {
     DevMem bad;
     GR_TRY(bad.alloc(sizeof(int32_t), "bipartite check"));
@@ -475,22 +512,18 @@ static gr_status bipartite_run(gr_graph *g, int kind, int32_t n_left, int32_t ma
   }
   bool host = false;
   GR_TRY(output_on_host(g, score, &host));
-  if (ws->cb_left != n_left) {
-    GR_TRY(range_bounds(g, 0, n_left, ws->cb_hub, s));
-    GR_TRY(range_bounds(g, n_left, g->n, ws->cb_auth, s));
-    ws->cb_left = n_left;
-  }
+  GR_TRY(gather_plan_build(&ws->plan, g->row_off.as<int32_t>(), g->n, g->m, s));
   RankArgs a;
   std::memset(&a, 0, sizeof(a));
   a.R = g->row_off.as<int32_t>();
   a.C = g->col.as<int32_t>();
   a.n = g->n;
   a.n_left = n_left;
-  a.cb_hub = ws->cb_hub.as<int32_t>();
-  a.cb_auth = ws->cb_auth.as<int32_t>();
+  a.plan = ws->plan.a;
   a.cur = ws->cur.as<double>();
   a.tmp = ws->tmp.as<double>();
   a.dv = ws->dv.as<double>();
+  a.idg = ws->idg.as<double>();
   a.tol = tol;
   a.max_iter = max_iter;
   a.ctl = ws->ctl.as<RankCtl>();
@@ -555,30 +588,22 @@ gr_status gr_neighbor_reduce(gr_graph *g, int32_t op, const int32_t *frontier, i
     GR_CUDA(cudaGetLastError());
   }
   if (count > 0) {
-    const int32_t *cb = nullptr;
-    if (!frontier) {
-      if (!g->rank) g->rank = new RankWorkspace();
-      GR_TRY(all_bounds(g, g->rank, s));
-      cb = g->rank->cb_all.as<int32_t>();
-    }
+    if (!g->rank) g->rank = new RankWorkspace();
+    RankWorkspace *ws = g->rank;
+    const double *xd = (const double *)x;
+    const int32_t *xi = (const int32_t *)x;
+    double *od = (double *)d_out;
+    int32_t *oi = (int32_t *)d_out;
     if (!frontier) {
       if (op == GR_REDUCE_SUM)
-        GR_TRY((nr_launch<double, ReduceSum<double>, false>(
-            g, s, R, C, nullptr, R, count, GatherF64{(const double *)x}, (double *)d_out, cb)));
+        GR_TRY((nr_launch_all<double, ReduceSum<double>>(g, ws, s, GatherF64{xd}, od)));
       else if (op == GR_REDUCE_WSUM)
-        GR_TRY((nr_launch<double, ReduceSum<double>, false>(
-            g, s, R, C, nullptr, R, count, GatherWF64{(const double *)x, g->w.as<uint32_t>()},
-            (double *)d_out, cb)));
+        GR_TRY((nr_launch_all<double, ReduceSum<double>>(g, ws, s, GatherWtF64{xd}, od)));
       else if (op == GR_REDUCE_MIN)
-        GR_TRY((nr_launch<int32_t, ReduceMinI32, false>(
-            g, s, R, C, nullptr, R, count, GatherI32{(const int32_t *)x}, (int32_t *)d_out, cb)));
+        GR_TRY((nr_launch_all<int32_t, ReduceMinI32>(g, ws, s, GatherI32{xi}, oi)));
       else
-        GR_TRY((nr_launch<int32_t, ReduceMaxI32, false>(
-            g, s, R, C, nullptr, R, count, GatherI32{(const int32_t *)x}, (int32_t *)d_out, cb)));
+        GR_TRY((nr_launch_all<int32_t, ReduceMaxI32>(g, ws, s, GatherI32{xi}, oi)));
     } else {
-      RankWorkspace *ws;
-      if (!g->rank) g->rank = new RankWorkspace();
-      ws = g->rank;
       const int32_t tiles = (count + kScanTile - 1) / kScanTile;
       if (ws->fscan.bytes < sizeof(int32_t) * ((size_t)g->n + 1)) {
         GR_CUDA(cudaStreamSynchronize(s));
@@ -593,21 +618,17 @@ gr_status gr_neighbor_reduce(gr_graph *g, int32_t op, const int32_t *frontier, i
       k_scan_parts<<<1, 256, 0, s>>>(part, tiles);
       k_scan_apply<<<tiles, 256, 0, s>>>(R, frontier, count, part, S);
       if (op == GR_REDUCE_SUM)
-        GR_TRY((nr_launch<double, ReduceSum<double>, true>(
-            g, s, R, C, frontier, S, count, GatherF64{(const double *)x}, (double *)d_out,
-            nullptr)));
+        GR_TRY((nr_launch_frontier<double, ReduceSum<double>>(g, s, frontier, S, count,
+                                                              GatherF64{xd}, od)));
       else if (op == GR_REDUCE_WSUM)
-        GR_TRY((nr_launch<double, ReduceSum<double>, true>(
-            g, s, R, C, frontier, S, count, GatherWF64{(const double *)x, g->w.as<uint32_t>()},
-            (double *)d_out, nullptr)));
+        GR_TRY((nr_launch_frontier<double, ReduceSum<double>>(
+            g, s, frontier, S, count, GatherWF64{xd, g->w.as<uint32_t>()}, od)));
       else if (op == GR_REDUCE_MIN)
-        GR_TRY((nr_launch<int32_t, ReduceMinI32, true>(
-            g, s, R, C, frontier, S, count, GatherI32{(const int32_t *)x}, (int32_t *)d_out,
-            nullptr)));
+        GR_TRY((nr_launch_frontier<int32_t, ReduceMinI32>(g, s, frontier, S, count,
+                                                          GatherI32{xi}, oi)));
       else
-        GR_TRY((nr_launch<int32_t, ReduceMaxI32, true>(
-            g, s, R, C, frontier, S, count, GatherI32{(const int32_t *)x}, (int32_t *)d_out,
-            nullptr)));
+        GR_TRY((nr_launch_frontier<int32_t, ReduceMaxI32>(g, s, frontier, S, count,
+                                                          GatherI32{xi}, oi)));
     }
   }
   if (cp) GR_CUDA(cudaMemcpyAsync(out, d_out, elem * (size_t)g->n, cudaMemcpyDeviceToHost, s));
@@ -647,7 +668,7 @@ gr_status gr_ppr(gr_graph *g, const int32_t *seeds, int32_t num_seeds, double da
   cudaStream_t s = (cudaStream_t)stream;
   GR_TRY(begin_call(g, s));
   RankWorkspace *ws;
-  GR_TRY(rank_ws(g, &ws));
+  GR_TRY(rank_ws(g, true, &ws));
   if (!ws->tele.p) GR_TRY(ws->tele.alloc(sizeof(double) * (size_t)g->n, "PPR teleport"));
   if (ws->seeds.bytes < sizeof(int32_t) * (size_t)num_seeds) {
     GR_CUDA(cudaStreamSynchronize(s));  // the old buffer may still be read
@@ -658,7 +679,7 @@ gr_status gr_ppr(gr_graph *g, const int32_t *seeds, int32_t num_seeds, double da
                           cudaMemcpyHostToDevice, s));
   bool host = false;
   GR_TRY(output_on_host(g, rank, &host));
-  GR_TRY(all_bounds(g, ws, s));
+  GR_TRY(gather_plan_build(&ws->plan, g->row_off.as<int32_t>(), g->n, g->m, s));
   RankArgs a;
   std::memset(&a, 0, sizeof(a));
   a.R = g->row_off.as<int32_t>();
@@ -667,8 +688,9 @@ gr_status gr_ppr(gr_graph *g, const int32_t *seeds, int32_t num_seeds, double da
   a.cur = ws->cur.as<double>();
   a.tmp = ws->tmp.as<double>();
   a.dv = ws->dv.as<double>();
+  a.idg = ws->idg.as<double>();
   a.tele = ws->tele.as<double>();
-  a.cb_all = ws->cb_all.as<int32_t>();
+  a.plan = ws->plan.a;
   a.damping = damping;
   a.tol = tol;
   a.max_iter = max_iter;
