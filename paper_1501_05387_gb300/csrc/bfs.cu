@@ -106,6 +106,7 @@ struct BfsArgs {
   BfsCtl *ctl;
   int32_t do_bitmap;
   int32_t low_degree;   // push-only on a graph of small maximum degree: per-thread expansion
+  const int4 *adj;      // low-degree graphs: first four neighbours per vertex (low_adjacency)
   // persistent kernel: per-block segments of the vertices a pull level
   // found (and their degrees), compacted into a queue by the next level
   // when it pushes; null in the other drivers
@@ -125,9 +126,8 @@ constexpr int kLvWarps = kLvThreads / 32;
 // at 3, 0.1815 at 5, 0.1806 at 8, 0.1811 at 12, 0.1809 at 20)
 constexpr int kPullLane = 8;
 constexpr int kLvBlocksPerSm = 6;
-// Largest maximum degree for which push levels expand one frontier vertex per
-// thread (mesh-like graphs), and the neighbours a thread loads at once.
-constexpr int32_t kLowDegreeMax = 16;
+// On graphs of at most kLowDegreeMax push levels expand one frontier vertex
+// per thread; the neighbours a thread loads at once.
 constexpr int kTpvItems = 4;
 
 struct BfsWorkspace {
@@ -944,8 +944,170 @@ __global__ void __launch_bounds__(kLvThreads, kDoBlocksPerSm) k_bfs_do(BfsArgs a
   }
 }
 
+// ------------------------------------------------------- one-block driver
+// A mesh's levels hold a few hundred vertices: what they cost is the way from
+// one level to the next. The one-cluster driver below takes 3.5-4.3 us for it
+// (the cluster fence waits 0.6 us for the level's stores, the visited test and
+// claim are two L2 round trips, row bounds and columns two more). A single
+// block separates its levels with __syncthreads and keeps the visited bitmap
+// and the frontier in shared memory (a claim takes 20 ns instead of 270), and
+// a vertex's row comes as one 16-byte load (low_adjacency), the only L2 round
+// trip of a level. What bounds it is then that one SM takes about one random
+// L2 access per clock, some 1.5 ns a vertex. 1024 x 1024 grid: 6.44 ms for
+// 1505 levels with the cluster.
+//
+// n is limited by the bitmap (1.58 M vertices). A frontier of more than
+// kSoloHandoff vertices goes to the grid kernel, with the bitmap and the list
+// in global memory, as from the cluster driver.
+constexpr int kSoloThreads = 1024;
+constexpr int32_t kSoloQueue = 4096;  // frontier vertices kept in shared memory, per parity
+constexpr int32_t kSoloHandoff = kSoloQueue;
+
+__global__ void __launch_bounds__(kSoloThreads, 1) k_bfs_solo(BfsArgs a) {
+  extern __shared__ uint32_t solo_smem[];
+  __shared__ int32_t s_cnt[2];        // frontier sizes by parity
+  __shared__ unsigned long long s_mf;  // edges of the frontier (traced levels, hand-over)
+  BfsCtl *c = a.ctl;
+  int32_t *qs[2] = {(int32_t *)solo_smem, (int32_t *)solo_smem + kSoloQueue};
+  uint32_t *bits = solo_smem + 2 * kSoloQueue;  // visited
+  int32_t *depth = c->depth;
+  int32_t *parent = c->parent;
+  const int32_t src = c->src, max_levels = c->max_levels;
+  const int lane = threadIdx.x & 31;
+  const uint32_t lt = (1u << lane) - 1u;
+  for (int32_t w = threadIdx.x; w < a.nwords; w += kSoloThreads)
+    bits[w] = w == (src >> 5) ? 1u << (src & 31) : 0u;
+  if (threadIdx.x == 0) {
+    qs[0][0] = src;
+    s_cnt[0] = 1;
+    s_cnt[1] = 0;
+    s_mf = 0ull;
+  }
+  __syncthreads();
+  int32_t L = 0;
+  for (;; ++L) {
+    const int p = L & 1;
+    const int32_t q = s_cnt[p];
+    if (q == 0 || q > kSoloHandoff || L >= max_levels) break;
+    const int32_t *Q = p ? qs[1] : qs[0];
+    int32_t *Qn = p ? qs[0] : qs[1], *Qg = p ? a.q[0] : a.q[1];
+    const bool trace = L < kTraceLevels;
+    uint32_t deg = 0u;
+    for (int32_t i0 = 0; i0 < q; i0 += kSoloThreads) {
+      const int32_t i = i0 + (int32_t)threadIdx.x;
+      if (__all_sync(0xffffffffu, i >= q)) break;
+      int32_t u = 0, e = 0, e1 = 0;  // [e, e1): what is left of a row longer than four
+      int32_t v[kTpvItems] = {-1, -1, -1, -1};
+      if (i < q) {
+        u = Q[i];
+        const int4 row = __ldg(a.adj + u);
+        if (row.x == -2) {
+          e = row.y;
+          e1 = row.z;
+        } else {
+          v[0] = row.x; v[1] = row.y; v[2] = row.z; v[3] = row.w;
+        }
+      }
+      for (;;) {
+        if (e < e1) {
+#pragma unroll
+          for (int j = 0; j < kTpvItems; ++j) v[j] = e + j < e1 ? a.C[e + j] : -1;
+          e += kTpvItems;
+        }
+        uint32_t won[kTpvItems];
+        bool mine[kTpvItems];
+        int32_t total = 0;
+#pragma unroll
+        for (int j = 0; j < kTpvItems; ++j) {
+          mine[j] = false;
+          if (v[j] >= 0 && GR_IN(v[j], a.n, 195)) {
+            const uint32_t bit = 1u << (v[j] & 31);
+            mine[j] = !(atomicOr(&bits[v[j] >> 5], bit) & bit);
+            deg += 1u;
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < kTpvItems; ++j) {
+          won[j] = __ballot_sync(0xffffffffu, mine[j]);
+          total += __popc(won[j]);
+        }
+        if (total) {
+          int32_t k = 0;
+          if (lane == 0) k = atomicAdd(&s_cnt[p ^ 1], total);
+          k = __shfl_sync(0xffffffffu, k, 0);
+#pragma unroll
+          for (int j = 0; j < kTpvItems; ++j) {
+            if (mine[j]) {
+              const int32_t at = k + __popc(won[j] & lt);
+              if (at < kSoloQueue) Qn[at] = v[j];
+              else Qg[at] = v[j];
+              depth[v[j]] = L + 1;
+              if (parent) parent[v[j]] = u;
+            }
+            k += __popc(won[j]);
+          }
+        }
+        if (!__any_sync(0xffffffffu, e < e1)) break;
+#pragma unroll
+        for (int j = 0; j < kTpvItems; ++j) v[j] = -1;
+      }
+    }
+    if (trace) {
+      const uint32_t wdeg = __reduce_add_sync(0xffffffffu, deg);
+      if (lane == 0 && wdeg) atomicAdd(&s_mf, (unsigned long long)wdeg);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      s_cnt[p] = 0;  // what level L + 1 counts
+      if (trace) {
+        c->tr_dir[L] = kPush;
+        c->tr_q[L] = q;
+        c->tr_mf[L] = (long long)s_mf;
+        c->tr_t[L] = globaltimer();
+        s_mf = 0ull;
+      }
+    }
+    __syncthreads();
+  }
+  const int p = L & 1;
+  const int32_t q = s_cnt[p];
+  const bool over = q > 0 && L >= max_levels;
+  if (q == 0 || over) {
+    if (threadIdx.x == 0) {
+      c->level = L;
+      c->pull_levels = 0;
+      if (over) c->error = kDevOverflow;
+      c->done = 1;
+    }
+    return;
+  }
+  // hand over: the visited bitmap and the frontier as one list
+  for (int32_t w = threadIdx.x; w < a.nwords; w += kSoloThreads) a.visited[w] = bits[w];
+  int32_t *Qg = p ? a.q[1] : a.q[0];
+  const int32_t *Q = p ? qs[1] : qs[0];
+  long long edges = 0;
+  for (int32_t i = threadIdx.x; i < q; i += kSoloThreads) {
+    const int32_t v = i < kSoloQueue ? Q[i] : Qg[i];
+    if (i < kSoloQueue) Qg[i] = v;
+    edges += a.R[v + 1] - a.R[v];
+  }
+  edges = warp_sum(edges);
+  __syncthreads();
+  if (threadIdx.x == 0) s_mf = 0ull;
+  __syncthreads();
+  if (lane == 0) atomicAdd(&s_mf, (unsigned long long)edges);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    c->level = L;
+    c->parity = p;
+    c->q_len = q;
+    c->mf = (long long)s_mf;
+  }
+}
+
 // ------------------------------------------------------ one-cluster driver
-// On graphs of small maximum degree (meshes) a BFS has thousands of levels
+// On graphs of small maximum degree (meshes) too large for the one-block
+// driver a BFS has thousands of levels
 // of a few thousand vertices each, and a grid-wide barrier per level costs
 // more than the level's work. This driver runs those levels in ONE thread
 // block cluster: the CTAs meet at the hardware cluster barrier, and each
@@ -1322,13 +1484,21 @@ __global__ void __launch_bounds__(kPersThreads) k_bfs_persistent(BfsArgs a) {
 }  // namespace
 
 // ---------------------------------------------------------------- host
+// Shared memory the one-block driver needs on this graph, 0 where the graph
+// is not a mesh or does not fit.
+static size_t solo_smem(const gr_graph *g) {
+  if (g->max_degree > kLowDegreeMax) return 0;
+  const size_t bytes = sizeof(int32_t) * (2 * (size_t)kSoloQueue + (size_t)g->nwords);
+  return bytes + 64 <= kBlockSmemMax ? bytes : 0;
+}
+
 size_t bfs_ws_bytes(const gr_graph *g) {
   const size_t n = (size_t)g->n;
   const size_t seg = (size_t)g->nwords * 32 +
                      (size_t)g->num_sms * kDoBlocksPerSm * kLvWarps * kPullWords * 32;
   return 2 * sizeof(int32_t) * (n + 1) + 2 * sizeof(int32_t) * (n + 2) +
          4 * sizeof(uint32_t) * (size_t)g->nwords + 2 * sizeof(int32_t) * seg +
-         sizeof(BfsCtl);
+         sizeof(BfsCtl) + (solo_smem(g) ? 16 * n : 0);
 }
 
 gr_status bfs_ws_create(gr_graph *g, cudaStream_t s, BfsWorkspace **out) {
@@ -1353,6 +1523,7 @@ gr_status bfs_ws_create(gr_graph *g, cudaStream_t s, BfsWorkspace **out) {
   GR_TRY(ws->ctl.alloc(sizeof(BfsCtl), "BFS control"));
   GR_TRY(ws->h_ctl.alloc(sizeof(BfsCtl), "BFS control mirror"));
   GR_CUDA(cudaMemsetAsync(ws->ctl.p, 0, sizeof(BfsCtl), s));
+  if (solo_smem(g)) GR_TRY(low_adjacency(g, false, s));
   GR_CUDA(cudaStreamSynchronize(s));
   *out = ws.release();
   return GR_OK;
@@ -1376,6 +1547,7 @@ static BfsArgs make_args(gr_graph *g, BfsWorkspace *ws, int32_t do_bitmap) {
   a.ctl = ws->ctl.as<BfsCtl>();
   a.do_bitmap = do_bitmap;
   a.low_degree = (!do_bitmap && g->max_degree <= kLowDegreeMax) ? 1 : 0;
+  a.adj = g->adj4.as<int4>();
   a.seg_v = nullptr;
   a.seg_d = nullptr;
   a.seg_cnt = nullptr;
@@ -1517,8 +1689,17 @@ gr_status bfs_run(gr_graph *g, BfsWorkspace *ws, int32_t src, int32_t *depth, in
     a.seg_v = ws->seg_v.as<int32_t>();
     a.seg_d = ws->seg_d.as<int32_t>();
     a.seg_cnt = ws->seg_cnt.as<unsigned long long>();
-    // low-degree graphs: the small-frontier levels in one cluster first
-    if (a.low_degree) GR_TRY(launch_cluster_bfs(a, s));
+    // low-degree graphs: the small-frontier levels in one block or, when
+    // their visited bitmap does not fit it, in one cluster first
+    const size_t solo = a.low_degree ? solo_smem(g) : 0;
+    if (solo) {
+      GR_CUDA(cudaFuncSetAttribute(k_bfs_solo, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)solo));
+      k_bfs_solo<<<1, kSoloThreads, solo, s>>>(a);
+      GR_CUDA(cudaGetLastError());
+    } else if (a.low_degree) {
+      GR_TRY(launch_cluster_bfs(a, s));
+    }
     void *args[] = {&a};
     GR_CUDA(cudaLaunchCooperativeKernel((void *)k_bfs_do, blocks, kLvThreads, args, 0, s));
   } else {

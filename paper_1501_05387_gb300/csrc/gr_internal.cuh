@@ -93,6 +93,10 @@ struct gr_graph {
   gr::DevMem isolated_bits;  // bit v set iff deg(v) == 0
   gr::DevMem first_col;      // first neighbour of v (C[R[v]]), -1 if deg(v) == 0
   gr::DevMem degree;         // int32 deg(v), used by PageRank
+  // Graphs of small maximum degree, per vertex: its first four neighbours
+  // (-1: none), the same with their weights behind them; a longer row has -2,
+  // its start and its end there. Built by low_adjacency.
+  gr::DevMem adj4, adjw4;
   int32_t max_degree = 0;
   int32_t num_isolated = 0;
   bool symmetric = false;
@@ -156,6 +160,16 @@ gr_status resolve_output(gr_graph *g, int slot, void *user, size_t bytes,
                          void **dev, bool *needs_copy);
 
 const gr_opts &default_opts();
+
+// Largest maximum degree of a mesh-like graph: its traversals take one
+// frontier vertex per thread.
+constexpr int32_t kLowDegreeMax = 16;
+// Shared memory one block may take.
+constexpr size_t kBlockSmemMax = 232448;
+
+// Builds g->adj4 (g->adjw4 if weighted) on `s` unless it is there already.
+// The caller synchronises `s` before another stream may read it.
+gr_status low_adjacency(gr_graph *g, bool weighted, cudaStream_t s);
 
 // Internal primitive entry points with explicit workspaces (device outputs,
 // no locking, no staging); used by the C ABI wrappers and the server.

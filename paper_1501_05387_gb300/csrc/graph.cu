@@ -211,6 +211,25 @@ __global__ void k_symmetric(const int32_t *R, const int32_t *C, int32_t n,
   }
 }
 
+__global__ void k_low_adjacency(const int32_t *R, const int32_t *C, const uint32_t *W, int32_t n,
+                                int4 *adj, int32_t stride) {
+  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
+       v += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t r0 = R[v], r1 = R[v + 1];
+    int32_t u[4];
+    uint32_t w[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const bool in = r0 + j < r1;
+      u[j] = in ? C[r0 + j] : -1;
+      w[j] = in && W ? W[r0 + j] : 0u;
+    }
+    adj[v * stride] = r1 - r0 > 4 ? make_int4(-2, r0, r1, 0) : make_int4(u[0], u[1], u[2], u[3]);
+    if (W)
+      adj[v * stride + 1] = make_int4((int32_t)w[0], (int32_t)w[1], (int32_t)w[2], (int32_t)w[3]);
+  }
+}
+
 __global__ void k_weight_sum(const uint32_t *W, int64_t m, unsigned long long *sum) {
   unsigned long long local = 0;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m;
@@ -221,6 +240,21 @@ __global__ void k_weight_sum(const uint32_t *W, int64_t m, unsigned long long *s
 }
 
 }  // namespace
+
+gr_status low_adjacency(gr_graph *g, bool weighted, cudaStream_t s) {
+  DevMem &m = weighted ? g->adjw4 : g->adj4;
+  if (m.p) return GR_OK;
+  GR_TRY(m.alloc((weighted ? 32 : 16) * (size_t)g->n, "low-degree adjacency"));
+  k_low_adjacency<<<g->num_sms * 8, 256, 0, s>>>(
+      g->row_off.as<int32_t>(), g->col.as<int32_t>(), weighted ? g->w.as<uint32_t>() : nullptr,
+      g->n, m.as<int4>(), weighted ? 2 : 1);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) {
+    m.reset();
+    return cuda_fail(e, "low-degree adjacency");
+  }
+  return GR_OK;
+}
 
 gr_status validate_host_csr(int32_t n, int64_t m, const int32_t *R,
                             const int32_t *C) {

@@ -108,6 +108,8 @@ struct SsspArgs {
   int32_t *far_stamp;
   SsspCtl *ctl;
   int32_t low_degree;  // graph of small maximum degree: per-thread relaxation
+  const int4 *adjw;    // first four neighbours and weights per vertex (low_adjacency)
+  int32_t far_in_smem;  // k_sssp_solo keeps the far pile's membership bits in shared memory
   const int32_t *cb;   // chunk bounds of the pull relaxation's all-vertex merge path
   int32_t *qcb;        // room for the chunk bounds of a dense near frontier (or null)
 };
@@ -115,15 +117,21 @@ struct SsspArgs {
 constexpr int kSsspThreads = 256, kSsspItems = 4;
 constexpr int kSsspChunk = kSsspThreads * kSsspItems;
 constexpr int kSsspBlocksPerSm = 5;
-// Largest maximum degree for which relaxation takes one frontier vertex per
-// thread (mesh-like graphs), and the neighbours a thread loads at once.
-constexpr int32_t kSsspLowDegreeMax = 16;
+// On graphs of at most kLowDegreeMax relaxation takes one frontier vertex
+// per thread; the neighbours a thread loads at once.
 constexpr int kSsspTpvItems = 4;
 // A persistent relaxation first finds every chunk's bounds in one pass once
 // its frontier has at least this many chunks per block.
 constexpr int kSsspBoundsChunksPerBlock = 4;
 // Most sources one batched run takes.
 constexpr int32_t kSsspMaxLanes = 64;
+// k_sssp_solo: threads of the block that runs a search, frontier vertices it
+// keeps in shared memory per parity, and the frontier size from which the
+// search goes on as k_sssp_do. A block expands about one vertex in 3 ns, so
+// 2560 take it as long (8 us) as a grid barrier and its frontier on all SMs.
+constexpr int kSoloThreads = 1024;
+constexpr int32_t kSoloQueue = 4096;
+constexpr int32_t kSoloHandoff = 2560;
 
 struct SsspWorkspace {
   int32_t lanes = 1;  // copies of the graph the buffers hold (batched form)
@@ -157,9 +165,11 @@ struct SsspSources {
   int32_t s[kSsspMaxLanes];
 };
 
+// solo: k_sssp_solo runs the searches from their sources; the control block
+// then starts out as what its lanes hand over: nothing.
 __global__ void k_sssp_init(SsspArgs a, SsspSources src, uint32_t *dist, int32_t *pred,
                             unsigned long long delta, int32_t max_iters,
-                            long long pull_min_edges) {
+                            long long pull_min_edges, int32_t solo) {
   const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t v = tid; v < a.nv; v += stride) {
@@ -186,7 +196,7 @@ __global__ void k_sssp_init(SsspArgs a, SsspSources src, uint32_t *dist, int32_t
     c->mode = kSsspRelax;
     c->near_parity = 0;
     c->far_parity = 0;
-    c->near_len = src.k;
+    c->near_len = solo ? 0 : src.k;
     c->far_len = 0;
     c->far_next_len = 0;
     c->done = 0;
@@ -200,9 +210,9 @@ __global__ void k_sssp_init(SsspArgs a, SsspSources src, uint32_t *dist, int32_t
     c->far_min_next = 0xFFFFFFFFu;
     c->near_next_packed = 0ull;
     c->delta = delta;
-    c->T = delta;
+    c->T = solo ? ~0ull : delta;
     c->T_old = 0;
-    c->near_edges = edges;
+    c->near_edges = solo ? 0 : edges;
     c->relaxations = 0;
     c->pull_min_edges = pull_min_edges;
     c->pulls = 0;
@@ -823,6 +833,256 @@ __global__ void __launch_bounds__(kSsspThreads, kSsspBlocksPerSm)
   }
 }
 
+// ------------------------------------------------------- one block per search
+// On a mesh a search is a thousand iterations of a few hundred vertices, and
+// each iteration of the grid kernel costs two microseconds of barrier and a
+// chain of L2 round trips from queue to queue (9 us in all). Here one block
+// runs a search by itself, so a batch runs its searches side by side on SMs of
+// their own: iterations are separated by __syncthreads, the frontier and the
+// near and far membership bits live in shared memory, a vertex's row comes as
+// one 32-byte load (low_adjacency), and the only L2 chain left is row and
+// distance, then atomicMin: 0.6 us. On the 511 x 511 grid an iteration went
+// from 8.8 to 1.1 us.
+//
+// A lane whose frontier outgrows kSoloHandoff vertices writes it and its far
+// pile to the control block's queues (parity 0) and stops; k_sssp_do, next on
+// the stream, goes on with all lanes handed over, under the smallest of their
+// thresholds (a far entry is never below its own lane's, so none is dropped).
+// Per lane, the ids [lane * n, (lane + 1) * n) of nearq[1] hold what the
+// shared-memory queue cannot, and those of nearS[0] and nearS[1] the far pile
+// by parity (both are free: per-thread relaxations use no degree scan).
+struct SoloState {
+  int32_t near[2];   // frontier sizes by parity
+  int32_t far[2];    // far pile sizes by parity
+  uint32_t far_min;  // lower bound of the far pile's distances
+  int32_t near_at, far_at;  // hand-over positions
+  unsigned long long relaxed;
+};
+
+// Appends the entries of a warp (code 1: near, 2: far) of item j to the
+// queues: one shared-memory atomic per queue.
+template <int ITEMS>
+__device__ __forceinline__ void solo_append(const int32_t (&v)[ITEMS], const int (&code)[ITEMS],
+                                            int32_t *near_cnt, int32_t *far_cnt, int32_t *near_s,
+                                            int32_t *near_g, int32_t *far) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t lt = (1u << lane) - 1u;
+  uint32_t nb[ITEMS], fb[ITEMS];
+  int32_t nt = 0, ft = 0;
+#pragma unroll
+  for (int j = 0; j < ITEMS; ++j) {
+    nb[j] = __ballot_sync(0xffffffffu, code[j] == 1);
+    fb[j] = __ballot_sync(0xffffffffu, code[j] == 2);
+    nt += __popc(nb[j]);
+    ft += __popc(fb[j]);
+  }
+  int32_t at = 0;
+  if (lane == 0 && nt) at = atomicAdd(near_cnt, nt);
+  if (lane == 1 && ft) at = atomicAdd(far_cnt, ft);
+  int32_t kn = __shfl_sync(0xffffffffu, at, 0), kf = __shfl_sync(0xffffffffu, at, 1);
+#pragma unroll
+  for (int j = 0; j < ITEMS; ++j) {
+    if (code[j] == 1) {
+      const int32_t k = kn + __popc(nb[j] & lt);
+      if (k < kSoloQueue) near_s[k] = v[j];
+      else near_g[k] = v[j];
+    } else if (code[j] == 2) {
+      far[kf + __popc(fb[j] & lt)] = v[j];
+    }
+    kn += __popc(nb[j]);
+    kf += __popc(fb[j]);
+  }
+}
+
+__global__ void __launch_bounds__(kSoloThreads, 1) k_sssp_solo(SsspArgs a, SsspSources src) {
+  extern __shared__ uint32_t solo_smem[];
+  __shared__ SoloState st;
+  SsspCtl *c = a.ctl;
+  const int32_t nwords = (a.n + 31) >> 5;
+  int32_t *qs[2] = {(int32_t *)solo_smem, (int32_t *)solo_smem + kSoloQueue};
+  uint32_t *nbits = solo_smem + 2 * kSoloQueue;  // on the next frontier
+  uint32_t *fbits = nbits + nwords;              // in the far pile (far_in_smem)
+  const int32_t base = (int32_t)blockIdx.x * a.n;
+  uint32_t *dist = c->dist + base;
+  int32_t *near_g = a.nearq[1] + base;
+  int32_t *far_stamp = a.far_stamp + base;  // -1: not in the far pile (far not in smem)
+  int32_t *far0 = a.nearS[0] + base, *far1 = a.nearS[1] + base;
+  const unsigned long long delta = c->delta;
+  const int32_t max_iters = c->max_iters;
+  const bool fsm = a.far_in_smem;
+  const int lane = threadIdx.x & 31;
+  for (int32_t w = threadIdx.x; w < nwords * (fsm ? 2 : 1); w += kSoloThreads) nbits[w] = 0u;
+  if (threadIdx.x == 0) {
+    qs[0][0] = src.s[blockIdx.x];
+    st.near[0] = 1;
+    st.near[1] = 0;
+    st.far[0] = st.far[1] = 0;
+    st.far_min = 0xFFFFFFFFu;
+    st.relaxed = 0ull;
+  }
+  unsigned long long T = delta;
+  int32_t p = 0, fp = 0, iter = 0, phases = 0;
+  uint32_t relaxed = 0u;
+  __syncthreads();
+  for (;;) {
+    // every thread reads the same sizes; what they count next is cleared
+    // before the barrier that opens the appends
+    const int32_t q = st.near[p], len = st.far[fp];
+    const uint32_t far_min = st.far_min;
+    const bool split = q == 0;
+    if ((split && len == 0) || q > kSoloHandoff || iter >= max_iters) break;
+    int32_t *far = fp ? far1 : far0;
+    int32_t *Qn = p ? qs[0] : qs[1];
+    uint32_t local_min = 0xFFFFFFFFu;
+    if (!split) {
+      const int32_t *Q = p ? qs[1] : qs[0];
+      // off the frontier: from here on a lowered vertex joins the next one
+      for (int32_t i = threadIdx.x; i < q; i += kSoloThreads)
+        atomicAnd(&nbits[Q[i] >> 5], ~(1u << (Q[i] & 31)));
+      if (threadIdx.x == 0) st.near[p ^ 1] = 0;
+      __syncthreads();
+      for (int32_t i0 = 0; i0 < q; i0 += kSoloThreads) {
+        const int32_t i = i0 + (int32_t)threadIdx.x;
+        if (__all_sync(0xffffffffu, i >= q)) break;
+        int32_t v[4] = {-1, -1, -1, -1};
+        uint32_t w[4] = {0u, 0u, 0u, 0u};
+        uint32_t du = 0xFFFFFFFFu;
+        int32_t e = 0, e1 = 0;  // what is left of a row longer than four
+        if (i < q) {
+          const int32_t u = Q[i];
+          const int4 *row = a.adjw + 2 * (int64_t)u;
+          const int4 rv = __ldg(row), rw = __ldg(row + 1);
+          du = __ldcg(dist + u);  // lowered by atomics: not from L1
+          if (rv.x == -2) {
+            e = rv.y;
+            e1 = rv.z;
+          } else {
+            v[0] = rv.x; v[1] = rv.y; v[2] = rv.z; v[3] = rv.w;
+            w[0] = (uint32_t)rw.x; w[1] = (uint32_t)rw.y; w[2] = (uint32_t)rw.z; w[3] = (uint32_t)rw.w;
+          }
+        }
+        for (;;) {
+          if (e < e1) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const bool in = e + j < e1;
+              v[j] = in ? a.C[e + j] : -1;
+              w[j] = in ? a.W[e + j] : 0u;
+            }
+            e += 4;
+          }
+          uint32_t nd[4], old[4];
+          int code[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const unsigned long long t = (unsigned long long)du + w[j];
+            const bool ok = v[j] >= 0 && t < 0xFFFFFFFFull && GR_IN(v[j], a.n, 340);
+            relaxed += v[j] >= 0;
+            nd[j] = (uint32_t)t;
+            old[j] = ok ? atomicMin(dist + v[j], nd[j]) : 0u;
+          }
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            code[j] = 0;
+            if (nd[j] < old[j]) {  // this thread lowered dist[v]
+              const uint32_t bit = 1u << (v[j] & 31);
+              if (nd[j] < T) {
+                code[j] = atomicOr(&nbits[v[j] >> 5], bit) & bit ? 0 : 1;
+              } else {
+                local_min = min(local_min, nd[j]);
+                if (fsm) code[j] = atomicOr(&fbits[v[j] >> 5], bit) & bit ? 0 : 2;
+                else code[j] = atomicExch(far_stamp + v[j], 0) == 0 ? 0 : 2;
+              }
+            }
+          }
+          solo_append<4>(v, code, &st.near[p ^ 1], &st.far[fp], Qn, near_g, far);
+          if (!__any_sync(0xffffffffu, e < e1)) break;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) v[j] = -1;
+        }
+      }
+      p ^= 1;
+    } else {
+      // the far pile by the raised threshold; entries that fell below the
+      // old one were expanded already
+      const unsigned long long T_old = T, t = T + delta, b = bucket_end(far_min, delta);
+      T = t > b ? t : b;
+      int32_t *far_n = fp ? far0 : far1;
+      __syncthreads();  // every thread has read far_min
+      if (threadIdx.x == 0) {
+        st.near[p ^ 1] = 0;
+        st.far[fp ^ 1] = 0;
+        st.far_min = 0xFFFFFFFFu;
+      }
+      __syncthreads();
+      for (int32_t i0 = 0; i0 < len; i0 += kSoloThreads) {
+        const int32_t i = i0 + (int32_t)threadIdx.x;
+        if (__all_sync(0xffffffffu, i >= len)) break;
+        int32_t v[1] = {0};
+        int code[1] = {0};
+        if (i < len) {
+          v[0] = far[i];
+          const uint32_t d = __ldcg(dist + v[0]);
+          const uint32_t bit = 1u << (v[0] & 31);
+          if ((unsigned long long)d >= T) {
+            code[0] = 2;
+            local_min = min(local_min, d);
+          } else {
+            if (fsm) atomicAnd(&fbits[v[0] >> 5], ~bit);
+            else far_stamp[v[0]] = -1;
+            if ((unsigned long long)d >= T_old) {
+              code[0] = 1;
+              atomicOr(&nbits[v[0] >> 5], bit);
+            }
+          }
+        }
+        solo_append<1>(v, code, &st.near[p ^ 1], &st.far[fp ^ 1], Qn, near_g, far_n);
+      }
+      p ^= 1;
+      fp ^= 1;
+      phases += 1;
+    }
+    local_min = __reduce_min_sync(0xffffffffu, local_min);
+    if (lane == 0 && local_min != 0xFFFFFFFFu) atomicMin(&st.far_min, local_min);
+    iter += 1;
+    __syncthreads();
+  }
+  const uint32_t wsum = __reduce_add_sync(0xffffffffu, relaxed);
+  if (lane == 0) atomicAdd(&st.relaxed, (unsigned long long)wsum);
+  __syncthreads();
+  const int32_t q = st.near[p], len = st.far[fp];
+  const bool over = (q > 0 || len > 0) && iter >= max_iters;
+  const bool handoff = !over && q > kSoloHandoff;
+  if (threadIdx.x == 0) {
+    atomicMax(&c->iter, iter);
+    atomicMax(&c->phases, phases);
+    atomicAdd((unsigned long long *)&c->relaxations, st.relaxed);
+    if (over) atomicExch(&c->error, kDevOverflow);
+    if (handoff) {
+      st.near_at = atomicAdd(&c->near_len, q);
+      st.far_at = atomicAdd(&c->far_len, len);
+      atomicMin(&c->far_min, st.far_min);
+      atomicMin(&c->T, T);
+    }
+  }
+  __syncthreads();
+  if (!handoff) return;
+  const int32_t *Q = p ? qs[1] : qs[0];
+  const int32_t *far = fp ? far1 : far0;
+  long long edges = 0;
+  for (int32_t i = threadIdx.x; i < q; i += kSoloThreads) {
+    const int32_t v = i < kSoloQueue ? Q[i] : near_g[i];
+    a.nearq[0][st.near_at + i] = base + v;
+    edges += a.R[v + 1] - a.R[v];
+  }
+  edges = warp_sum(edges);
+  if (lane == 0 && edges) atomicAdd((unsigned long long *)&c->near_edges, (unsigned long long)edges);
+  for (int32_t i = threadIdx.x; i < len; i += kSoloThreads) {
+    a.farq[0][st.far_at + i] = base + far[i];
+    far_stamp[far[i]] = 0;  // k_sssp_do's first far epoch
+  }
+}
+
 // Persistent form: the whole SSSP in one cooperative kernel, one grid
 // barrier per iteration. After the barrier every block reads the
 // iteration's counters and recomputes the same next state in registers; the
@@ -840,12 +1100,16 @@ __global__ void __launch_bounds__(kSsspThreads, kSsspBlocksPerSm) k_sssp_do(Sssp
   uint32_t *dist = c->dist;
   const unsigned long long delta = c->delta;
   const int32_t max_iters = c->max_iters;
-  int32_t mode = kSsspRelax, near_parity = 0, far_parity = 0, near_len = c->near_len, far_len = 0;
-  long long near_edges = c->near_edges, relaxations = 0;
+  // the sources, or what k_sssp_solo handed over (no near frontier: it
+  // finished every search)
+  int32_t mode = kSsspRelax, near_parity = 0, far_parity = 0, near_len = c->near_len,
+          far_len = c->far_len;
+  if (near_len == 0) return;
+  long long near_edges = c->near_edges, relaxations = c->relaxations;
   const long long pull_min_edges = c->pull_min_edges;
-  int32_t iter = 0, far_epoch = 0, phases = 0, gen = 0, pulls = 0;
-  uint32_t far_min = 0xFFFFFFFFu;
-  unsigned long long T = delta, T_old = 0;
+  int32_t iter = c->iter, far_epoch = 0, phases = c->phases, gen = 0, pulls = 0;
+  uint32_t far_min = c->far_min;
+  unsigned long long T = c->T, T_old = 0;
   for (;;) {
     const int32_t slot = iter % 3, clear = (iter + 1) % 3;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -970,14 +1234,24 @@ __global__ void k_sssp_pred_fin(int32_t *pred, int32_t n, int32_t src) {
 
 }  // namespace
 
+// Shared memory k_sssp_solo needs on this graph with the far pile's bits in
+// it or not; 0 where the graph is not a mesh or does not fit.
+static size_t solo_smem(const gr_graph *g, bool far_bits) {
+  if (g->max_degree > kLowDegreeMax) return 0;
+  const size_t bytes = sizeof(int32_t) * (2 * (size_t)kSoloQueue +
+                                          (size_t)g->nwords * (far_bits ? 2 : 1));
+  return bytes + sizeof(SoloState) <= kBlockSmemMax ? bytes : 0;
+}
+
 size_t sssp_ws_bytes(const gr_graph *g, int32_t lanes) {
   const size_t n = (size_t)g->n * (size_t)std::max(lanes, 1);
-  const size_t qcb = g->max_degree > kSsspLowDegreeMax
+  const size_t qcb = g->max_degree > kLowDegreeMax
                          ? sizeof(int32_t) * ((n + (size_t)std::max(lanes, 1) * (size_t)g->m) /
                                                   kSsspChunk + 3)
                          : 0;
   return 4 * sizeof(int32_t) * (n + 1) + 2 * sizeof(int32_t) * (n + 2) +
-         2 * sizeof(int32_t) * n + sizeof(SsspCtl) + qcb;
+         2 * sizeof(int32_t) * n + sizeof(SsspCtl) + qcb +
+         (solo_smem(g, false) ? 32 * (size_t)g->n : 0);
 }
 
 int32_t sssp_batch_max_lanes(const gr_graph *g) {
@@ -1003,7 +1277,7 @@ gr_status sssp_ws_create(gr_graph *g, cudaStream_t s, SsspWorkspace **out, int32
   GR_TRY(ws->stamp.alloc(sizeof(int32_t) * n, "SSSP near stamps"));
   GR_TRY(ws->far_stamp.alloc(sizeof(int32_t) * n, "SSSP far stamps"));
   GR_TRY(ws->ctl.alloc(sizeof(SsspCtl), "SSSP control"));
-  if (g->max_degree > kSsspLowDegreeMax) {
+  if (g->max_degree > kLowDegreeMax) {
     // a frontier holds at most n vertices of each lane and their edges
     const long long chunks = ((long long)n + (long long)lanes * g->m) / kSsspChunk + 2;
     GR_TRY(ws->qcb.alloc(sizeof(int32_t) * ((size_t)chunks + 1), "SSSP frontier chunk bounds"));
@@ -1017,6 +1291,7 @@ gr_status sssp_ws_create(gr_graph *g, cudaStream_t s, SsspWorkspace **out, int32
     GR_CUDA(cudaGetLastError());
   }
   GR_CUDA(cudaMemsetAsync(ws->ctl.p, 0, sizeof(SsspCtl), s));
+  if (solo_smem(g, false)) GR_TRY(low_adjacency(g, true, s));
   GR_CUDA(cudaStreamSynchronize(s));
   *out = ws.release();
   return GR_OK;
@@ -1038,7 +1313,9 @@ static SsspArgs sssp_args(gr_graph *g, SsspWorkspace *ws, int32_t lanes = 1) {
   a.stamp = ws->stamp.as<int32_t>();
   a.far_stamp = ws->far_stamp.as<int32_t>();
   a.ctl = ws->ctl.as<SsspCtl>();
-  a.low_degree = g->max_degree <= kSsspLowDegreeMax ? 1 : 0;
+  a.low_degree = g->max_degree <= kLowDegreeMax ? 1 : 0;
+  a.adjw = g->adjw4.as<int4>();
+  a.far_in_smem = 0;
   a.cb = ws->cb.as<int32_t>();  // null for batched workspaces, which never pull
   a.qcb = ws->qcb.as<int32_t>();  // null on low-degree graphs
   return a;
@@ -1052,7 +1329,7 @@ static SsspArgs sssp_args(gr_graph *g, SsspWorkspace *ws, int32_t lanes = 1) {
 // never pulls, GR_DIR_PULL pulls every relaxation. Only a symmetric CSR
 // (rows = in-neighbours) and a single search can pull.
 static long long sssp_pull_min_edges(const gr_graph *g, const gr_opts &o, int32_t lanes) {
-  if (!g->symmetric || lanes != 1 || g->max_degree <= kSsspLowDegreeMax || g->m == 0 ||
+  if (!g->symmetric || lanes != 1 || g->max_degree <= kLowDegreeMax || g->m == 0 ||
       o.direction == GR_DIR_PUSH)
     return LLONG_MAX;
   if (o.direction == GR_DIR_PULL) return 1;
@@ -1122,9 +1399,35 @@ gr_status sssp_check(const gr_graph *g, int32_t src, const gr_opts &o) {
   return GR_OK;
 }
 
-// Runs the device-side loop of an initialised search with the given driver.
-static gr_status sssp_drive(gr_graph *g, SsspWorkspace *ws, SsspArgs a, int32_t mode,
-                            const gr_opts &o, int32_t max_iters, cudaStream_t s) {
+static unsigned long long sssp_delta_of(const gr_graph *g, const gr_opts &o) {
+  return o.delta == UINT32_MAX ? (1ull << 40) : (o.delta ? o.delta : g->sssp_delta);
+}
+
+static int32_t sssp_max_iters_of(const gr_graph *g, const gr_opts &o) {
+  return o.max_iters > 0 ? o.max_iters
+                         : (int32_t)std::min<long long>(INT32_MAX, 8ll * g->n + 1024);
+}
+
+// Initialises the searches and runs their device-side loop with the given
+// driver.
+static gr_status sssp_drive(gr_graph *g, SsspWorkspace *ws, SsspArgs a, const SsspSources &src,
+                            uint32_t *dist, int32_t *pred, int32_t mode, const gr_opts &o,
+                            cudaStream_t s) {
+  const int32_t max_iters = sssp_max_iters_of(g, o);
+  // meshes whose membership bits fit one block's shared memory: one block
+  // per search, up to the frontier size where the grid takes over
+  const size_t near_only = mode == GR_MODE_PERSISTENT ? solo_smem(g, false) : 0;
+  k_sssp_init<<<g->num_sms * 8, 256, 0, s>>>(a, src, dist, pred, sssp_delta_of(g, o), max_iters,
+                                             sssp_pull_min_edges(g, o, src.k), near_only > 0);
+  GR_CUDA(cudaGetLastError());
+  if (near_only) {
+    const size_t both = solo_smem(g, true);
+    a.far_in_smem = both > 0;
+    GR_CUDA(cudaFuncSetAttribute(k_sssp_solo, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(both ? both : near_only)));
+    k_sssp_solo<<<src.k, kSoloThreads, both ? both : near_only, s>>>(a, src);
+    GR_CUDA(cudaGetLastError());
+  }
   if (mode == GR_MODE_PERSISTENT) {
     void *kern = a.low_degree ? (void *)k_sssp_do<true> : (void *)k_sssp_do<false>;
     const int32_t want = o.block > 0 ? o.block : g->tuned_sssp_blocks_per_sm;
@@ -1154,30 +1457,16 @@ static gr_status sssp_drive(gr_graph *g, SsspWorkspace *ws, SsspArgs a, int32_t 
   return GR_OK;
 }
 
-static unsigned long long sssp_delta_of(const gr_graph *g, const gr_opts &o) {
-  return o.delta == UINT32_MAX ? (1ull << 40) : (o.delta ? o.delta : g->sssp_delta);
-}
-
-static int32_t sssp_max_iters_of(const gr_graph *g, const gr_opts &o) {
-  return o.max_iters > 0 ? o.max_iters
-                         : (int32_t)std::min<long long>(INT32_MAX, 8ll * g->n + 1024);
-}
-
 // SSSP into device outputs with an explicit workspace (no locking, no
 // staging): the public gr_sssp and the query server both call this.
 gr_status sssp_run(gr_graph *g, SsspWorkspace *ws, int32_t src, uint32_t *dist, int32_t *pred,
                    const gr_opts &o, cudaStream_t s) {
-  const unsigned long long delta = sssp_delta_of(g, o);
-  const int32_t max_iters = sssp_max_iters_of(g, o);
   SsspArgs a = sssp_args(g, ws);
   SsspSources one;
   one.k = 1;
   one.s[0] = src;
-  k_sssp_init<<<g->num_sms * 8, 256, 0, s>>>(a, one, dist, pred, delta, max_iters,
-                                             sssp_pull_min_edges(g, o, 1));
-  GR_CUDA(cudaGetLastError());
   const int32_t mode = o.mode != GR_MODE_AUTO ? o.mode : g->tuned_sssp_mode;
-  GR_TRY(sssp_drive(g, ws, a, mode, o, max_iters, s));
+  GR_TRY(sssp_drive(g, ws, a, one, dist, pred, mode, o, s));
   if (pred) {
     const int grid = g->num_sms * 8;
     k_sssp_pred_init<<<grid, 256, 0, s>>>(pred, g->n);
@@ -1194,15 +1483,10 @@ gr_status sssp_run(gr_graph *g, SsspWorkspace *ws, int32_t src, uint32_t *dist, 
 gr_status sssp_batch_run(gr_graph *g, SsspWorkspace *ws, const int32_t *h_srcs, int32_t k,
                          uint32_t *dist, const gr_opts &o, cudaStream_t s) {
   if (k < 1 || k > ws->lanes) return fail(GR_EINVAL, "batched SSSP: k exceeds the workspace");
-  const unsigned long long delta = sssp_delta_of(g, o);
-  const int32_t max_iters = sssp_max_iters_of(g, o);
   SsspArgs a = sssp_args(g, ws, k);
   SsspSources srcs;
   srcs.k = k;
   for (int32_t l = 0; l < kSsspMaxLanes; ++l) srcs.s[l] = l < k ? h_srcs[l] : 0;
-  k_sssp_init<<<g->num_sms * 8, 256, 0, s>>>(a, srcs, dist, nullptr, delta, max_iters,
-                                             LLONG_MAX);
-  GR_CUDA(cudaGetLastError());
   int32_t mode = o.mode != GR_MODE_AUTO ? o.mode : g->tuned_sssp_mode;
   if (mode != GR_MODE_PERSISTENT) mode = GR_MODE_LAUNCH;
   gr_opts ob = o;
@@ -1211,7 +1495,7 @@ gr_status sssp_batch_run(gr_graph *g, SsspWorkspace *ws, const int32_t *h_srcs, 
   // sources on the 4096^2 mesh: 282 ms at 2 blocks per SM, 321 at 1, 297 at
   // 3, 335 at 5)
   if (k > 1 && ob.block == 0 && g->tuned_sssp_blocks_per_sm == 1) ob.block = 2;
-  return sssp_drive(g, ws, a, mode, ob, max_iters, s);
+  return sssp_drive(g, ws, a, srcs, dist, nullptr, mode, ob, s);
 }
 
 }  // namespace gr
