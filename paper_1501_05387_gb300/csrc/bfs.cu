@@ -949,117 +949,117 @@ __global__ void __launch_bounds__(kLvThreads, kDoBlocksPerSm) k_bfs_do(BfsArgs a
 // one level to the next. The one-cluster driver below takes 3.5-4.3 us for it
 // (the cluster fence waits 0.6 us for the level's stores, the visited test and
 // claim are two L2 round trips, row bounds and columns two more). A single
-// block separates its levels with __syncthreads and keeps the visited bitmap
-// and the frontier in shared memory (a claim takes 20 ns instead of 270), and
-// a vertex's row comes as one 16-byte load (low_adjacency), the only L2 round
-// trip of a level. What bounds it is then that one SM takes about one random
-// L2 access per clock, some 1.5 ns a vertex. 1024 x 1024 grid: 6.44 ms for
-// 1505 levels with the cluster.
+// block separates its levels with one __syncthreads and keeps the visited
+// bitmap and the frontier in shared memory (a claim takes 20 ns instead of
+// 270), and a vertex's row comes as one 16-byte load (low_adjacency): the only
+// L2 round trip of a level. A thread makes the four claims of its vertex
+// without a branch (a missing neighbour claims a word of its lane's own), so
+// that they overlap: 1.55 us a level on the 1024 x 1024 grid where claims one
+// after another took 1.67, 0.75 against 0.94 on 300 x 300. A thread per edge
+// (0.6 us a level at 64 x 64, 2.2 at 1024 x 1024), testing a word before
+// claiming it (1.93) and more or fewer threads (1.55 at 1024, 1.66 at 512)
+// were no better. One SM takes about one random L2 access per clock, two a
+// vertex here: that bounds the large levels, instruction latency the small.
 //
 // n is limited by the bitmap (1.58 M vertices). A frontier of more than
 // kSoloHandoff vertices goes to the grid kernel, with the bitmap and the list
 // in global memory, as from the cluster driver.
-constexpr int kSoloThreads = 1024;
+constexpr int kSoloThreads = 768;
 constexpr int32_t kSoloQueue = 4096;  // frontier vertices kept in shared memory, per parity
 constexpr int32_t kSoloHandoff = kSoloQueue;
 
+// LONG: the graph has rows of more than four entries (the code for them costs
+// the others instruction fetches on every level)
+template <bool LONG>
 __global__ void __launch_bounds__(kSoloThreads, 1) k_bfs_solo(BfsArgs a) {
   extern __shared__ uint32_t solo_smem[];
-  __shared__ int32_t s_cnt[2];        // frontier sizes by parity
+  __shared__ int32_t s_cnt[3];         // frontier sizes, ring by level
   __shared__ unsigned long long s_mf;  // edges of the frontier (traced levels, hand-over)
   BfsCtl *c = a.ctl;
-  int32_t *qs[2] = {(int32_t *)solo_smem, (int32_t *)solo_smem + kSoloQueue};
+  int32_t *const q0 = (int32_t *)solo_smem, *const q1 = q0 + kSoloQueue;
   uint32_t *bits = solo_smem + 2 * kSoloQueue;  // visited
+  uint32_t *spare = bits + a.nwords;            // a word per lane for claims of nothing
   int32_t *depth = c->depth;
   int32_t *parent = c->parent;
   const int32_t src = c->src, max_levels = c->max_levels;
   const int lane = threadIdx.x & 31;
   const uint32_t lt = (1u << lane) - 1u;
-  for (int32_t w = threadIdx.x; w < a.nwords; w += kSoloThreads)
+  for (int32_t w = threadIdx.x; w < a.nwords + 32; w += kSoloThreads)
     bits[w] = w == (src >> 5) ? 1u << (src & 31) : 0u;
   if (threadIdx.x == 0) {
-    qs[0][0] = src;
+    q0[0] = src;
     s_cnt[0] = 1;
     s_cnt[1] = 0;
     s_mf = 0ull;
   }
   __syncthreads();
-  int32_t L = 0;
+  int32_t L = 0, ring = 0;
   for (;; ++L) {
-    const int p = L & 1;
-    const int32_t q = s_cnt[p];
+    const int32_t next = ring == 2 ? 0 : ring + 1, after = next == 2 ? 0 : next + 1;
+    const int32_t q = s_cnt[ring];
     if (q == 0 || q > kSoloHandoff || L >= max_levels) break;
-    const int32_t *Q = p ? qs[1] : qs[0];
-    int32_t *Qn = p ? qs[0] : qs[1], *Qg = p ? a.q[0] : a.q[1];
-    const bool trace = L < kTraceLevels;
+    if (threadIdx.x == 0) s_cnt[after] = 0;  // last read a level ago
+    const int32_t *Q = L & 1 ? q1 : q0;
+    int32_t *Qn = L & 1 ? q0 : q1, *Qg = L & 1 ? a.q[0] : a.q[1];
     uint32_t deg = 0u;
-    for (int32_t i0 = 0; i0 < q; i0 += kSoloThreads) {
-      const int32_t i = i0 + (int32_t)threadIdx.x;
-      if (__all_sync(0xffffffffu, i >= q)) break;
-      int32_t u = 0, e = 0, e1 = 0;  // [e, e1): what is left of a row longer than four
-      int32_t v[kTpvItems] = {-1, -1, -1, -1};
+    for (int32_t i = threadIdx.x; i - lane < q; i += kSoloThreads) {  // warp-uniform
+      int32_t u = 0;
+      int4 row = make_int4(-1, -1, -1, -1);
       if (i < q) {
         u = Q[i];
-        const int4 row = __ldg(a.adj + u);
-        if (row.x == -2) {
-          e = row.y;
-          e1 = row.z;
-        } else {
-          v[0] = row.x; v[1] = row.y; v[2] = row.z; v[3] = row.w;
-        }
+        row = __ldg(a.adj + u);
+      }
+      int32_t e = 0, e1 = 0;  // [e, e1): what is left of a row longer than four
+      if (LONG && row.x == -2) {
+        e = row.y;
+        e1 = row.z;
+        row = make_int4(-1, -1, -1, -1);
       }
       for (;;) {
-        if (e < e1) {
+        int32_t v[kTpvItems] = {row.x, row.y, row.z, row.w};
+        if (LONG && e < e1) {
 #pragma unroll
           for (int j = 0; j < kTpvItems; ++j) v[j] = e + j < e1 ? a.C[e + j] : -1;
           e += kTpvItems;
         }
-        uint32_t won[kTpvItems];
-        bool mine[kTpvItems];
+        uint32_t old[kTpvItems], won[kTpvItems];
         int32_t total = 0;
 #pragma unroll
         for (int j = 0; j < kTpvItems; ++j) {
-          mine[j] = false;
-          if (v[j] >= 0 && GR_IN(v[j], a.n, 195)) {
-            const uint32_t bit = 1u << (v[j] & 31);
-            mine[j] = !(atomicOr(&bits[v[j] >> 5], bit) & bit);
-            deg += 1u;
-          }
+          if (v[j] >= 0 && !GR_IN(v[j], a.n, 195)) v[j] = -1;
+          old[j] = atomicOr(v[j] >= 0 ? bits + (v[j] >> 5) : spare + lane,
+                            v[j] >= 0 ? 1u << (v[j] & 31) : 0u);
         }
 #pragma unroll
         for (int j = 0; j < kTpvItems; ++j) {
-          won[j] = __ballot_sync(0xffffffffu, mine[j]);
+          deg += v[j] >= 0;
+          won[j] = __ballot_sync(0xffffffffu, v[j] >= 0 && !((old[j] >> (v[j] & 31)) & 1u));
           total += __popc(won[j]);
         }
-        if (total) {
-          int32_t k = 0;
-          if (lane == 0) k = atomicAdd(&s_cnt[p ^ 1], total);
-          k = __shfl_sync(0xffffffffu, k, 0);
+        int32_t at = 0;
+        if (lane == 0) at = atomicAdd(&s_cnt[next], total);
+        at = __shfl_sync(0xffffffffu, at, 0);
+        const bool fits = at + total <= kSoloQueue;
 #pragma unroll
-          for (int j = 0; j < kTpvItems; ++j) {
-            if (mine[j]) {
-              const int32_t at = k + __popc(won[j] & lt);
-              if (at < kSoloQueue) Qn[at] = v[j];
-              else Qg[at] = v[j];
-              depth[v[j]] = L + 1;
-              if (parent) parent[v[j]] = u;
-            }
-            k += __popc(won[j]);
+        for (int j = 0; j < kTpvItems; ++j) {
+          if ((won[j] >> lane) & 1u) {
+            const int32_t k = at + __popc(won[j] & lt);
+            depth[v[j]] = L + 1;
+            if (parent) parent[v[j]] = u;
+            if (fits || k < kSoloQueue) Qn[k] = v[j];
+            else Qg[k] = v[j];
           }
+          at += __popc(won[j]);
         }
-        if (!__any_sync(0xffffffffu, e < e1)) break;
-#pragma unroll
-        for (int j = 0; j < kTpvItems; ++j) v[j] = -1;
+        if (!LONG || !__any_sync(0xffffffffu, e < e1)) break;
+        row = make_int4(-1, -1, -1, -1);
       }
     }
-    if (trace) {
+    if (__builtin_expect(L < kTraceLevels, 0)) {
       const uint32_t wdeg = __reduce_add_sync(0xffffffffu, deg);
       if (lane == 0 && wdeg) atomicAdd(&s_mf, (unsigned long long)wdeg);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      s_cnt[p] = 0;  // what level L + 1 counts
-      if (trace) {
+      __syncthreads();
+      if (threadIdx.x == 0) {
         c->tr_dir[L] = kPush;
         c->tr_q[L] = q;
         c->tr_mf[L] = (long long)s_mf;
@@ -1068,9 +1068,9 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_bfs_solo(BfsArgs a) {
       }
     }
     __syncthreads();
+    ring = next;
   }
-  const int p = L & 1;
-  const int32_t q = s_cnt[p];
+  const int32_t q = s_cnt[ring];
   const bool over = q > 0 && L >= max_levels;
   if (q == 0 || over) {
     if (threadIdx.x == 0) {
@@ -1083,8 +1083,9 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_bfs_solo(BfsArgs a) {
   }
   // hand over: the visited bitmap and the frontier as one list
   for (int32_t w = threadIdx.x; w < a.nwords; w += kSoloThreads) a.visited[w] = bits[w];
+  const int p = L & 1;
   int32_t *Qg = p ? a.q[1] : a.q[0];
-  const int32_t *Q = p ? qs[1] : qs[0];
+  const int32_t *Q = p ? q1 : q0;
   long long edges = 0;
   for (int32_t i = threadIdx.x; i < q; i += kSoloThreads) {
     const int32_t v = i < kSoloQueue ? Q[i] : Qg[i];
@@ -1092,7 +1093,6 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_bfs_solo(BfsArgs a) {
     edges += a.R[v + 1] - a.R[v];
   }
   edges = warp_sum(edges);
-  __syncthreads();
   if (threadIdx.x == 0) s_mf = 0ull;
   __syncthreads();
   if (lane == 0) atomicAdd(&s_mf, (unsigned long long)edges);
@@ -1488,7 +1488,7 @@ __global__ void __launch_bounds__(kPersThreads) k_bfs_persistent(BfsArgs a) {
 // is not a mesh or does not fit.
 static size_t solo_smem(const gr_graph *g) {
   if (g->max_degree > kLowDegreeMax) return 0;
-  const size_t bytes = sizeof(int32_t) * (2 * (size_t)kSoloQueue + (size_t)g->nwords);
+  const size_t bytes = sizeof(int32_t) * (2 * (size_t)kSoloQueue + (size_t)g->nwords + 32);
   return bytes + 64 <= kBlockSmemMax ? bytes : 0;
 }
 
@@ -1693,9 +1693,9 @@ gr_status bfs_run(gr_graph *g, BfsWorkspace *ws, int32_t src, int32_t *depth, in
     // their visited bitmap does not fit it, in one cluster first
     const size_t solo = a.low_degree ? solo_smem(g) : 0;
     if (solo) {
-      GR_CUDA(cudaFuncSetAttribute(k_bfs_solo, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)solo));
-      k_bfs_solo<<<1, kSoloThreads, solo, s>>>(a);
+      auto kern = g->max_degree > 4 ? k_bfs_solo<true> : k_bfs_solo<false>;
+      GR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)solo));
+      kern<<<1, kSoloThreads, solo, s>>>(a);
       GR_CUDA(cudaGetLastError());
     } else if (a.low_degree) {
       GR_TRY(launch_cluster_bfs(a, s));
