@@ -68,11 +68,12 @@ enum {
   GR_MODE_GRAPH = 2,      /* one CUDA graph whose device-side while loop
                              runs one level per iteration */
   GR_MODE_PERSISTENT = 3  /* one cooperative kernel runs every level with a
-                             bounded-spin grid barrier between levels; for a
-                             BFS on a graph of maximum degree <= 16 one
-                             thread-block cluster runs the levels first and
-                             hands a frontier of more than 32768 vertices to
-                             that kernel */
+                             bounded-spin grid barrier between levels; on a
+                             graph of maximum degree <= 16 one thread block
+                             (above 1.58 M vertices, for a BFS, one
+                             thread-block cluster) runs the levels first and
+                             hands a frontier of more than 4096 (32768)
+                             vertices to that kernel */
 };
 
 /* Options; pass NULL for tuned defaults. Zero in a field means "tuned". */
@@ -150,11 +151,15 @@ gr_status gr_bfs_stats(gr_graph *g, int32_t *levels, int32_t *pull_levels);
  * near/far bucket width (0: tuned, UINT32_MAX: a single bucket); the
  * distances do not depend on it. Direction (the pull form of Sec. 4.5
  * applied to the relaxation, which the paper leaves to future work): on a
- * symmetric CSR a relaxation whose near frontier holds at least m /
- * opts->alpha edges (opts->alpha 0: the tuned threshold, by default never)
- * runs as a pull, every vertex taking the minimum over its in-edges;
- * opts->direction GR_DIR_PUSH never pulls, GR_DIR_PULL (symmetric CSR
- * only, else GR_EINVAL) pulls every relaxation. Distances do not depend on
+ * symmetric CSR whose weights are equal in both directions a relaxation whose
+ * near frontier holds at least m / opts->alpha edges (opts->alpha 0: the
+ * tuned threshold, by default a third of the edges of a graph with enough of
+ * them to fill the GPU) runs as a pull, every vertex taking the minimum over
+ * its in-edges; opts->direction GR_DIR_PUSH never pulls, GR_DIR_PULL
+ * (symmetric CSR only, else GR_EINVAL) pulls every relaxation that can be.
+ * On a graph of maximum degree <= 16 the persistent mode runs a search by one
+ * thread block (a batch's by one each) and hands a near frontier of more than
+ * 4096 vertices to the grid. Distances do not depend on
  * the direction. */
 gr_status gr_sssp(gr_graph *g, int32_t src, uint32_t *dist, int32_t *pred,
                   const gr_opts *opts, void *stream);

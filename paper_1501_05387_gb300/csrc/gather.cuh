@@ -22,6 +22,13 @@
 // so a lane takes 16 FP64 values to a scan), and the two pieces that reach
 // over a tile's ends go out as atomics. out[v] must therefore hold OP's
 // identity beforehand; vertices without entries are not touched.
+//
+// Which warp takes which tile is the caller's: neighbouring tiles on
+// different SMs (spread_warp) suit the rankings and PageRank, whose loops also
+// meet small graphs (PageRank 2^21 3.84 ms, 4.05 with a block's tiles
+// together; HITS 512k x 128k 1.61, 1.69), tiles of a block together
+// (block_warp) the single gather over FP64 values (1.5 M vertices, 45 M
+// entries: 167 us, 172 spread).
 #pragma once
 
 #include "advance.cuh"
@@ -46,6 +53,11 @@ struct GatherPlan {
   GatherPlanArgs a = {nullptr, nullptr, nullptr};
 };
 
+// Device memory of a plan.
+inline size_t gather_plan_bytes(int32_t n, int64_t m) {
+  return (size_t)m / 4 + (size_t)m / 64 + 4 * (size_t)n + 4096;
+}
+
 // Builds the plan of the CSR row offsets R (n vertices, m entries) on `s`
 // unless it is there already; nothing is synchronised. In gather.cu.
 gr_status gather_plan_build(GatherPlan *p, const int32_t *R, int32_t n, int64_t m, cudaStream_t s);
@@ -60,13 +72,26 @@ __device__ __forceinline__ void ld_stream8(const int32_t *p, int32_t (&v)[8]) {
                : "l"(p));
 }
 
+// Where a row's value goes: whole rows are stored, pieces of a row that
+// crosses a tile combined atomically.
+template <class T, class OP>
+struct StoreReduced {
+  T *out;
+  __device__ __forceinline__ void operator()(int32_t v, T x, bool whole) const {
+    if (whole) out[v] = x;
+    else OP::atomic(out + v, x);
+  }
+};
+
 // One warp's share (tiles gw, gw + nw, ...) of the entries [eb, ee), which
 // begin and end with whole rows. F: value_type operator()(u, weight) and
-// F::kWeighted (whether it reads w[e], then non-null).
-template <int G8, class T, class OP, class F>
+// F::kWeighted (whether it reads w[e], then non-null). E: operator()(v,
+// value, whole), once per whole row and once per piece of the others.
+template <int G8, class T, class OP, class F, class E>
 __device__ __forceinline__ void gather_reduce_tiles(const GatherPlanArgs &p, const int32_t *C,
                                                     const int32_t *W, int32_t eb, int32_t ee,
-                                                    const F &f, T *out, int64_t gw, int64_t nw) {
+                                                    const F &f, const E &emit, int64_t gw,
+                                                    int64_t nw) {
   constexpr int ITEMS = 8 * G8;
   constexpr int TILE = 32 * ITEMS;
   static_assert(TILE % kGpTile == 0, "a warp's tile is whole rank_base tiles");
@@ -130,7 +155,7 @@ __device__ __forceinline__ void gather_reduce_tiles(const GatherPlanArgs &p, con
     for (int i = 0; i < ITEMS; ++i) {
       if (i) acc = (ends >> (i - 1)) & 1u ? v[i] : OP::op(acc, v[i]);
       if ((ends >> i) & 1u) {
-        if (any) out[p.rows[rank]] = acc;
+        if (any) emit(p.rows[rank], acc, true);
         else head = acc;
         any = true;
         ++rank;
@@ -152,13 +177,11 @@ __device__ __forceinline__ void gather_reduce_tiles(const GatherPlanArgs &p, con
     const bool opens = tb < eb || (p.rank_base[tb / kGpTile] >> 31);
     if (any) {
       if (lane) head = OP::op(carry, head);
-      T *dst = out + p.rows[rank_head];
-      if (!(em & lt) && !opens) OP::atomic(dst, head);
-      else *dst = head;
+      emit(p.rows[rank_head], head, (em & lt) || opens);
     }
     // the row that reaches into the next tile
     if (lane == 31 && tb + TILE < ee && !((ends >> (ITEMS - 1)) & 1u))
-      OP::atomic(out + p.rows[rank], s);
+      emit(p.rows[rank], s, false);
   }
 }
 
@@ -169,6 +192,10 @@ __device__ __forceinline__ int64_t spread_warp() {
 }
 __device__ __forceinline__ int64_t grid_warps() {
   return (int64_t)gridDim.x * (blockDim.x >> 5);
+}
+// This thread's warp, a block's warps together.
+__device__ __forceinline__ int64_t block_warp() {
+  return (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
 }
 
 // Block-wide FP64 sum, added to *dst by thread 0. Block-uniform call of

@@ -94,12 +94,13 @@ struct gr_graph {
   gr::DevMem first_col;      // first neighbour of v (C[R[v]]), -1 if deg(v) == 0
   gr::DevMem degree;         // int32 deg(v), used by PageRank
   // Graphs of small maximum degree, per vertex: its first four neighbours
-  // (-1: none), the same with their weights behind them; a longer row has -2,
-  // its start and its end there. Built by low_adjacency.
+  // (-1: none), or four (neighbour, weight) pairs; a longer row has -2, its
+  // start and its end there instead. Built by low_adjacency.
   gr::DevMem adj4, adjw4;
   int32_t max_degree = 0;
   int32_t num_isolated = 0;
   bool symmetric = false;
+  bool weights_symmetric = false;  // and (u, v) weighs what (v, u) does
   bool rows_sorted = false;
   bool has_weights = false;
   uint32_t sssp_delta = 1;    // tuned near/far bucket width

@@ -174,59 +174,93 @@ __global__ void k_graph_stats(const int32_t *R, int32_t n, int32_t nwords,
   }
 }
 
-// rows_sorted: every row's columns are non-decreasing (one warp per row)
-__global__ void k_rows_sorted(const int32_t *R, const int32_t *C, int32_t n,
-                              int32_t *unsorted) {
+// What the symmetry check needs to know of the rows (one warp per row):
+// whether every row's columns are non-decreasing, whether one has the same
+// column twice, and the entries above and below the diagonal.
+struct RowFlags {
+  int32_t unsorted, repeated;
+  unsigned long long above, below;
+};
+
+__global__ void k_rows_sorted(const int32_t *R, const int32_t *C, int32_t n, RowFlags *out) {
   int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   int lane = threadIdx.x & 31;
+  bool bad = false, twice = false;
+  unsigned long long above = 0, below = 0;
   for (int64_t v = gw; v < n; v += nwarps) {
-    bool bad = false;
-    for (int32_t e = R[v] + 1 + lane; e < R[v + 1]; e += 32)
-      bad |= C[e - 1] > C[e];
-    if (__any_sync(0xffffffffu, bad) && lane == 0) *unsorted = 1;
+    const int32_t r0 = R[v];
+    for (int32_t e = r0 + lane; e < R[v + 1]; e += 32) {
+      const int32_t c = C[e];
+      above += c > v;
+      below += c < v;
+      if (e > r0) {
+        const int32_t prev = C[e - 1];
+        bad |= prev > c;
+        twice |= prev == c;
+      }
+    }
   }
+  if (__any_sync(0xffffffffu, bad) && lane == 0) out->unsorted = 1;
+  if (__any_sync(0xffffffffu, twice) && lane == 0) out->repeated = 1;
+  above = warp_sum(above);
+  below = warp_sum(below);
+  if (lane == 0 && above) atomicAdd(&out->above, above);
+  if (lane == 0 && below) atomicAdd(&out->below, below);
 }
 
-// symmetric: for each entry (u, v) the row of v contains u (binary search;
-// rows sorted). One warp per row u, lanes over its entries.
-__global__ void k_symmetric(const int32_t *R, const int32_t *C, int32_t n,
-                            int32_t *asym) {
+// asym[0]: an entry (u, v) has no (v, u); asym[1]: it has, with another
+// weight, or an end's row has the other more than once (then the pairs are
+// not told apart). Rows sorted; binary search, one warp per row u, lanes over
+// its entries. With half only the entries above the diagonal are looked up:
+// rows without repeated columns and as many entries below it as above have
+// each of those below as the partner of one above.
+__global__ void k_symmetric(const int32_t *R, const int32_t *C, const uint32_t *W, int32_t n,
+                            int32_t half, int32_t *asym) {
   int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   int lane = threadIdx.x & 31;
+  bool bad = false, other = false;
   for (int64_t uu = gw; uu < n; uu += nwarps) {
     int32_t u = (int32_t)uu;
-    bool bad = false;
     for (int32_t e = R[u] + lane; e < R[u + 1]; e += 32) {
       int32_t v = C[e];
+      if (half && v <= u) continue;
       int32_t a = R[v], b = R[v + 1], end = b;
       while (a < b) {
         int32_t mid = a + (b - a) / 2;
         if (C[mid] < u) a = mid + 1; else b = mid;
       }
-      bad |= (a >= end || C[a] != u);
+      const bool found = a < end && C[a] == u;
+      bad |= !found;
+      if (W && found)
+        other |= W[a] != W[e] || (!half && a + 1 < end && C[a + 1] == u);
     }
-    if (__any_sync(0xffffffffu, bad) && lane == 0) *asym = 1;
   }
+  if (__any_sync(0xffffffffu, bad) && lane == 0) asym[0] = 1;
+  if (__any_sync(0xffffffffu, other) && lane == 0) asym[1] = 1;
 }
 
+// adj: 4 neighbours per vertex, or 4 (neighbour, weight) pairs with W.
 __global__ void k_low_adjacency(const int32_t *R, const int32_t *C, const uint32_t *W, int32_t n,
-                                int4 *adj, int32_t stride) {
+                                int4 *adj) {
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
        v += (int64_t)gridDim.x * blockDim.x) {
     const int32_t r0 = R[v], r1 = R[v + 1];
-    int32_t u[4];
-    uint32_t w[4];
+    int32_t u[4], w[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const bool in = r0 + j < r1;
       u[j] = in ? C[r0 + j] : -1;
-      w[j] = in && W ? W[r0 + j] : 0u;
+      w[j] = in && W ? (int32_t)W[r0 + j] : 0;
     }
-    adj[v * stride] = r1 - r0 > 4 ? make_int4(-2, r0, r1, 0) : make_int4(u[0], u[1], u[2], u[3]);
-    if (W)
-      adj[v * stride + 1] = make_int4((int32_t)w[0], (int32_t)w[1], (int32_t)w[2], (int32_t)w[3]);
+    const bool is_long = r1 - r0 > 4;
+    if (!W) {
+      adj[v] = is_long ? make_int4(-2, r0, r1, 0) : make_int4(u[0], u[1], u[2], u[3]);
+    } else {
+      adj[2 * v] = is_long ? make_int4(-2, r0, r1, 0) : make_int4(u[0], w[0], u[1], w[1]);
+      adj[2 * v + 1] = is_long ? make_int4(-1, 0, -1, 0) : make_int4(u[2], w[2], u[3], w[3]);
+    }
   }
 }
 
@@ -247,7 +281,7 @@ gr_status low_adjacency(gr_graph *g, bool weighted, cudaStream_t s) {
   GR_TRY(m.alloc((weighted ? 32 : 16) * (size_t)g->n, "low-degree adjacency"));
   k_low_adjacency<<<g->num_sms * 8, 256, 0, s>>>(
       g->row_off.as<int32_t>(), g->col.as<int32_t>(), weighted ? g->w.as<uint32_t>() : nullptr,
-      g->n, m.as<int4>(), weighted ? 2 : 1);
+      g->n, m.as<int4>());
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     m.reset();
@@ -340,9 +374,12 @@ gr_status gr_graph_create(int32_t n, int64_t m, const int32_t *row_off,
   if (m) GR_CUDA(cudaMemcpyAsync(g->col.p, col, sizeof(int32_t) * (size_t)m, kind, s));
   if (w && m) GR_CUDA(cudaMemcpyAsync(g->w.p, w, sizeof(uint32_t) * (size_t)m, kind, s));
 
+  // [0] CSR validity, [1] maximum degree, [2] isolated vertices, [4..5]
+  // symmetry, [8..] RowFlags
+  constexpr int kFlags = 8 + sizeof(RowFlags) / sizeof(int32_t);
   DevMem flags;
-  GR_TRY(flags.alloc(sizeof(int32_t) * 8, "flags"));
-  GR_CUDA(cudaMemsetAsync(flags.p, 0, sizeof(int32_t) * 8, s));
+  GR_TRY(flags.alloc(sizeof(int32_t) * kFlags, "flags"));
+  GR_CUDA(cudaMemsetAsync(flags.p, 0, flags.bytes, s));
   int32_t *f = flags.as<int32_t>();
   int grid = g->num_sms * 4;
   if (inputs_on_device) {
@@ -350,7 +387,7 @@ gr_status gr_graph_create(int32_t n, int64_t m, const int32_t *row_off,
                                         n, m, f + 0);
     GR_CUDA(cudaGetLastError());
   }
-  int32_t hf[8];
+  alignas(8) int32_t hf[kFlags];
   GR_CUDA(cudaMemcpyAsync(hf, f, sizeof(hf), cudaMemcpyDeviceToHost, s));
   GR_CUDA(cudaStreamSynchronize(s));
   if (hf[0]) return fail(GR_EINVAL, "invalid CSR (device check flags " + std::to_string(hf[0]) + ")");
@@ -361,7 +398,8 @@ gr_status gr_graph_create(int32_t n, int64_t m, const int32_t *row_off,
                                      g->isolated_bits.as<uint32_t>(),
                                      g->degree.as<int32_t>(), f + 1, f + 2);
   GR_CUDA(cudaGetLastError());
-  k_rows_sorted<<<grid, 256, 0, s>>>(g->row_off.as<int32_t>(), g->col.as<int32_t>(), n, f + 3);
+  RowFlags *rf = (RowFlags *)(f + 8);
+  k_rows_sorted<<<grid * 2, 256, 0, s>>>(g->row_off.as<int32_t>(), g->col.as<int32_t>(), n, rf);
   GR_CUDA(cudaGetLastError());
   GR_TRY(g->first_col.alloc(sizeof(int32_t) * (size_t)n, "first neighbours"));
   k_first_col<<<grid, 256, 0, s>>>(g->row_off.as<int32_t>(), g->col.as<int32_t>(), n,
@@ -369,17 +407,21 @@ gr_status gr_graph_create(int32_t n, int64_t m, const int32_t *row_off,
   GR_CUDA(cudaGetLastError());
   GR_CUDA(cudaMemcpyAsync(hf, f, sizeof(hf), cudaMemcpyDeviceToHost, s));
   GR_CUDA(cudaStreamSynchronize(s));
+  RowFlags hr;
+  std::memcpy(&hr, hf + 8, sizeof(hr));
   g->max_degree = hf[1];
   g->num_isolated = hf[2];
-  g->rows_sorted = hf[3] == 0;
+  g->rows_sorted = !hr.unsorted;
   g->symmetric = false;
-  if (g->rows_sorted) {
+  if (g->rows_sorted && hr.above == hr.below) {
     k_symmetric<<<grid * 2, 256, 0, s>>>(g->row_off.as<int32_t>(), g->col.as<int32_t>(),
-                                          n, f + 4);
+                                          w ? g->w.as<uint32_t>() : nullptr, n, !hr.repeated,
+                                          f + 4);
     GR_CUDA(cudaGetLastError());
     GR_CUDA(cudaMemcpyAsync(hf, f, sizeof(hf), cudaMemcpyDeviceToHost, s));
     GR_CUDA(cudaStreamSynchronize(s));
     g->symmetric = hf[4] == 0;
+    g->weights_symmetric = g->symmetric && hf[5] == 0;
   }
   if (w && m) {
     GR_CUDA(cudaMemsetAsync(flags.p, 0, sizeof(unsigned long long), s));

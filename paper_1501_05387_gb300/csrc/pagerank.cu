@@ -106,7 +106,8 @@ struct ContribG {
 
 __device__ __forceinline__ void pr_gather(const PrArgs &a) {
   const ContribG g{a.contrib};
-  gather_reduce_tiles<1, float, ReduceSum<float>>(a.plan, a.C, nullptr, 0, a.m, g, a.sum,
+  const StoreReduced<float, ReduceSum<float>> to{a.sum};
+  gather_reduce_tiles<1, float, ReduceSum<float>>(a.plan, a.C, nullptr, 0, a.m, g, to,
                                                   spread_warp(), grid_warps());
 }
 

@@ -179,8 +179,10 @@ constexpr int range_blocks() { return sizeof(T) == 8 ? kRgBlocksF64 : kRgBlocksI
 template <class T, class OP, class G>
 __global__ void __launch_bounds__(kRgThreads, range_blocks<T>()) k_nr_all(
     GatherPlanArgs plan, const int32_t *C, const int32_t *W, int32_t m, G g, T *out) {
-  gather_reduce_tiles<range_groups<T>(), T, OP>(
-      plan, C, W, 0, m, g, out, spread_warp(), grid_warps());
+  constexpr int G8 = range_groups<T>();
+  gather_reduce_tiles<G8, T, OP>(plan, C, W, 0, m, g, StoreReduced<T, OP>{out},
+                                 m < grid_warps() * (256 * G8) ? spread_warp() : block_warp(),
+                                 grid_warps());
 }
 
 // ------------------------------------------------------ ranking kernels
@@ -208,11 +210,12 @@ __device__ __forceinline__ void range_sum(const RankArgs &a, int32_t v0, int32_t
   const GatherF64 g{x};
   const int32_t eb = a.R[v0], ee = a.R[v1];
   // tiles of 512 entries, of 256 where those would leave warps without one
+  const StoreReduced<double, ReduceSum<double>> to{out};
   if (ee - eb >= grid_warps() * 512)
-    gather_reduce_tiles<2, double, ReduceSum<double>>(a.plan, a.C, nullptr, eb, ee, g, out,
+    gather_reduce_tiles<2, double, ReduceSum<double>>(a.plan, a.C, nullptr, eb, ee, g, to,
                                                       spread_warp(), grid_warps());
   else
-    gather_reduce_tiles<1, double, ReduceSum<double>>(a.plan, a.C, nullptr, eb, ee, g, out,
+    gather_reduce_tiles<1, double, ReduceSum<double>>(a.plan, a.C, nullptr, eb, ee, g, to,
                                                       spread_warp(), grid_warps());
 }
 
@@ -402,17 +405,16 @@ __global__ void k_count_linked(const int32_t *R, int32_t n_left, int32_t *linked
   if (threadIdx.x == 0 && t) atomicAdd(linked, t);
 }
 
-// Every entry joins a hub and an authority.
-__global__ void k_check_bipartite(const int32_t *R, const int32_t *C, int32_t n, int32_t nl,
+// Every entry joins a hub and an authority: the hubs' rows, the entries
+// before R[nl], hold authorities only, the others hubs only.
+__global__ void k_check_bipartite(const int32_t *R, const int32_t *C, int32_t m, int32_t nl,
                                   int32_t *bad) {
-  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t v = tid; v < n; v += stride)
-    for (int32_t e = R[v]; e < R[v + 1]; ++e)
-      if ((v < nl) == (C[e] < nl)) {
-        atomicOr(bad, 1);
-        break;
-      }
+  const int32_t split = R[nl];
+  bool found = false;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m;
+       e += (int64_t)gridDim.x * blockDim.x)
+    found |= (e < split) == (C[e] < nl);
+  if (found) atomicOr(bad, 1);
 }
 
 }  // namespace
@@ -502,7 +504,7 @@ static gr_status bipartite_run(gr_graph *g, int kind, int32_t n_left, int32_t ma
     GR_TRY(bad.alloc(sizeof(int32_t), "bipartite check"));
     GR_CUDA(cudaMemsetAsync(bad.p, 0, sizeof(int32_t), s));
     k_check_bipartite<<<g->num_sms * 8, 256, 0, s>>>(g->row_off.as<int32_t>(),
-                                                     g->col.as<int32_t>(), g->n, n_left,
+                                                     g->col.as<int32_t>(), (int32_t)g->m, n_left,
                                                      bad.as<int32_t>());
     int32_t h = 0;
     GR_CUDA(cudaMemcpyAsync(&h, bad.p, sizeof(int32_t), cudaMemcpyDeviceToHost, s));

@@ -15,11 +15,12 @@
 //          otherwise (deduplicated by a per-phase stamp)
 //   pull   the relaxation in pull form (direction-optimising SSSP, which
 //          the paper names for future work in Sec. 4.5 and Sec. 7), for
-//          near frontiers holding most of the edges on a symmetric graph:
+//          near frontiers holding much of the edges on a symmetric graph:
 //          every vertex takes the minimum of dist[u] + w(e) over its
-//          in-edges (= its row) and keeps it if lower, so no atomic is
-//          needed except for vertices whose row is split between threads;
-//          the improved vertices go to near / far exactly as in relax
+//          in-edges (= its row; gather_reduce_tiles) and keeps it if lower,
+//          so no atomic is needed except for rows split between tiles; a
+//          sweep over the marks of the lowered vertices then sends them to
+//          near / far as in relax
 //   split  only when the near frontier is empty: the far pile is split by
 //          the raised threshold into near and far; entries whose distance
 //          fell below the old threshold were already expanded and are
@@ -48,11 +49,12 @@
 #include <climits>
 #include <cstring>
 
-#include "advance.cuh"
+#include "gather.cuh"
 
 namespace gr {
 
-enum : int32_t { kSsspRelax = 0, kSsspSplit = 1, kSsspPull = 2 };
+// kSsspSweep: the second half of a pull, its lowered vertices to near / far
+enum : int32_t { kSsspRelax = 0, kSsspSplit = 1, kSsspPull = 2, kSsspSweep = 3 };
 
 struct SsspCtl {
   uint32_t *dist;
@@ -108,15 +110,18 @@ struct SsspArgs {
   int32_t *far_stamp;
   SsspCtl *ctl;
   int32_t low_degree;  // graph of small maximum degree: per-thread relaxation
-  const int4 *adjw;    // first four neighbours and weights per vertex (low_adjacency)
-  int32_t far_in_smem;  // k_sssp_solo keeps the far pile's membership bits in shared memory
-  const int32_t *cb;   // chunk bounds of the pull relaxation's all-vertex merge path
+  const int4 *adjw;    // four (neighbour, weight) pairs per vertex (low_adjacency)
+  GatherPlanArgs plan;  // row structure of the pull relaxation
+  uint32_t *lowered;    // marks of the vertices a pull lowered (zero between pulls)
   int32_t *qcb;        // room for the chunk bounds of a dense near frontier (or null)
 };
 
 constexpr int kSsspThreads = 256, kSsspItems = 4;
-constexpr int kSsspChunk = kSsspThreads * kSsspItems;
 constexpr int kSsspBlocksPerSm = 5;
+// Items per thread of the persistent kernel that may pull: its pushes have
+// the smaller frontiers, and half the shared memory leaves the pull's random
+// distance loads the L1.
+constexpr int kSsspPullItems = 2;
 // On graphs of at most kLowDegreeMax relaxation takes one frontier vertex
 // per thread; the neighbours a thread loads at once.
 constexpr int kSsspTpvItems = 4;
@@ -127,16 +132,19 @@ constexpr int kSsspBoundsChunksPerBlock = 4;
 constexpr int32_t kSsspMaxLanes = 64;
 // k_sssp_solo: threads of the block that runs a search, frontier vertices it
 // keeps in shared memory per parity, and the frontier size from which the
-// search goes on as k_sssp_do. A block expands about one vertex in 3 ns, so
-// 2560 take it as long (8 us) as a grid barrier and its frontier on all SMs.
+// search goes on as k_sssp_do. A block expands a vertex in 5 ns, so 4096 take
+// it twice as long as a grid barrier and their expansion on all SMs (9 us);
+// but the grid keeps the search once it has it, and meshes pass 2560 for a
+// few iterations only (700 x 700, 12 mean weights: 7.6 ms handed over there).
 constexpr int kSoloThreads = 1024;
 constexpr int32_t kSoloQueue = 4096;
-constexpr int32_t kSoloHandoff = 2560;
+constexpr int32_t kSoloHandoff = 4096;
 
 struct SsspWorkspace {
   int32_t lanes = 1;  // copies of the graph the buffers hold (batched form)
   DevMem nearq[2], nearS[2], farq[2], stamp, far_stamp, ctl;
-  DevMem cb;  // chunk bounds of the pull relaxation (single search; fixed per graph)
+  GatherPlan plan;  // of the pull relaxation (single search on a symmetric graph)
+  DevMem lowered;
   DevMem qcb;  // chunk bounds of a dense near frontier (persistent driver)
   cudaGraphExec_t exec = nullptr;
   cudaGraph_t graph = nullptr;
@@ -179,6 +187,8 @@ __global__ void k_sssp_init(SsspArgs a, SsspSources src, uint32_t *dist, int32_t
     a.stamp[v] = -1;
     a.far_stamp[v] = -1;
   }
+  if (a.lowered)
+    for (int64_t w = tid; w < (a.n + 31) / 32; w += stride) a.lowered[w] = 0u;
   if (tid == 0) {
     SsspCtl *c = a.ctl;
     // the initial near frontier: every lane's source with its degree scan
@@ -225,13 +235,15 @@ __global__ void k_sssp_init(SsspArgs a, SsspSources src, uint32_t *dist, int32_t
   }
 }
 
+template <int ITEMS>
 struct SsspSmem {
-  int32_t off[kSsspChunk + 1];
-  uint32_t du[kSsspChunk + 1];
-  int32_t row[kSsspChunk + 1];
-  int32_t base[kSsspChunk + 1];  // first id of the vertex's graph copy
-  ScannedBuf<kSsspChunk> nearb;
-  AppendBuf<kSsspChunk> farb;
+  static constexpr int kChunk = kSsspThreads * ITEMS;
+  int32_t off[kChunk + 1];
+  uint32_t du[kChunk + 1];
+  int32_t row[kChunk + 1];
+  int32_t base[kChunk + 1];  // first id of the vertex's graph copy
+  ScannedBuf<kChunk> nearb;
+  AppendBuf<kChunk> farb;
   int32_t i[2];
   int32_t sred[kSsspThreads / 32];
   int32_t last;
@@ -257,7 +269,8 @@ struct SsspStep {
 // The merge-path chunk bounds of a near frontier (q members, exclusive
 // degree scan S[0..q), s_q entries in all: S[q] itself is not stored),
 // grid-stride: cb[c] = the members whose end marker S[i + 1] + i lies before
-// c * kSsspChunk, cb[nchunks] = q.
+// c * CHUNK, cb[nchunks] = q.
+template <int CHUNK>
 __device__ void frontier_chunk_bounds(const int32_t *S, int32_t q, int32_t s_q,
                                       long long nchunks, int32_t *cb) {
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c <= nchunks;
@@ -266,7 +279,7 @@ __device__ void frontier_chunk_bounds(const int32_t *S, int32_t q, int32_t s_q,
       cb[c] = q;
       continue;
     }
-    const long long d = c * kSsspChunk;
+    const long long d = c * CHUNK;
     int32_t lo = 0, hi = q;  // first member whose end marker is not before d
     while (lo < hi) {
       const int32_t mid = (int32_t)(((long long)lo + hi) >> 1);
@@ -280,8 +293,10 @@ __device__ void frontier_chunk_bounds(const int32_t *S, int32_t q, int32_t s_q,
 
 // qcb (may be null): the frontier's chunk bounds, computed for this
 // iteration by frontier_chunk_bounds, so a chunk needs no search.
-__device__ void relax_body(const SsspArgs &a, uint32_t *dist, SsspSmem &sm, const SsspStep &st,
-                           const int32_t *qcb = nullptr) {
+template <int ITEMS>
+__device__ void relax_body(const SsspArgs &a, uint32_t *dist, SsspSmem<ITEMS> &sm,
+                           const SsspStep &st, const int32_t *qcb = nullptr) {
+  constexpr int CHUNK = kSsspThreads * ITEMS;
   const int32_t np = st.near_parity;
   const int32_t *Q = pick(a.nearq, np);
   const int32_t *S = pick(a.nearS, np);
@@ -290,17 +305,18 @@ __device__ void relax_body(const SsspArgs &a, uint32_t *dist, SsspSmem &sm, cons
   const int32_t q = st.q;
   const unsigned long long T = st.T;
   const int32_t iter = st.iter, epoch = st.far_epoch;
+  uint32_t local_min = 0xFFFFFFFFu;
   const long long total = (long long)q + st.q_edges;
-  const long long nchunks = (total + kSsspChunk - 1) / kSsspChunk;
+  const long long nchunks = (total + CHUNK - 1) / CHUNK;
   for (long long chunk = blockIdx.x; chunk < nchunks; chunk += gridDim.x) {
-    const long long d0 = chunk * kSsspChunk;
-    const long long d1 = min(d0 + kSsspChunk, total);
+    const long long d0 = chunk * CHUNK;
+    const long long d1 = min(d0 + CHUNK, total);
     int32_t i0, i1;
     if (qcb) {
       i0 = qcb[chunk];
       i1 = qcb[chunk + 1];
     } else {
-      block_chunk_bounds<kSsspThreads>(S, q, st.q_edges, d0, d1, kSsspChunk, sm.sred, &i0, &i1);
+      block_chunk_bounds<kSsspThreads>(S, q, st.q_edges, d0, d1, CHUNK, sm.sred, &i0, &i1);
     }
     const long long j0 = d0 - i0, j1 = d1 - i1;
     const int32_t nv = (i0 <= q - 1) ? (min(i1, q - 1) - i0 + 1) : 0;
@@ -317,16 +333,16 @@ __device__ void relax_body(const SsspArgs &a, uint32_t *dist, SsspSmem &sm, cons
       sm.du[k] = dist[u];
     }
     __syncthreads();
-    // each thread takes kSsspItems edges (ranks tid, tid + T, ...) and issues
+    // each thread takes ITEMS edges (ranks tid, tid + T, ...) and issues
     // each step's loads (heads and weights, head distances, atomicMin, stamps,
     // degrees) for all of them before using any, so the latency chains of the
     // items overlap
-    const int32_t ne = (int32_t)(j1 - j0);  // <= kSsspChunk: one pass
-    int32_t e[kSsspItems], v[kSsspItems], vl[kSsspItems], vb[kSsspItems], code[kSsspItems],
-        dv[kSsspItems];
-    uint32_t wt[kSsspItems], du[kSsspItems], nd[kSsspItems], cur[kSsspItems];
+    const int32_t ne = (int32_t)(j1 - j0);  // <= CHUNK: one pass
+    int32_t e[ITEMS], v[ITEMS], vl[ITEMS], vb[ITEMS], code[ITEMS],
+        dv[ITEMS];
+    uint32_t wt[ITEMS], du[ITEMS], nd[ITEMS], cur[ITEMS];
 #pragma unroll
-    for (int j = 0; j < kSsspItems; ++j) {
+    for (int j = 0; j < ITEMS; ++j) {
       const int32_t k = j * kSsspThreads + threadIdx.x;
       e[j] = -1;
       vb[j] = 0;
@@ -348,12 +364,12 @@ __device__ void relax_body(const SsspArgs &a, uint32_t *dist, SsspSmem &sm, cons
       }
     }
 #pragma unroll
-    for (int j = 0; j < kSsspItems; ++j) {
+    for (int j = 0; j < ITEMS; ++j) {
       vl[j] = e[j] >= 0 ? a.C[e[j]] : -1;
       wt[j] = e[j] >= 0 ? a.W[e[j]] : 0u;
     }
 #pragma unroll
-    for (int j = 0; j < kSsspItems; ++j) {
+    for (int j = 0; j < ITEMS; ++j) {
       nd[j] = 0xFFFFFFFFu;  // not representable below 0xFFFFFFFF: no improvement
       if (vl[j] >= 0 && !GR_IN(vl[j], a.n, 305)) vl[j] = -1;
       v[j] = vl[j] >= 0 ? vb[j] + vl[j] : -1;  // the neighbour in the same copy
@@ -363,36 +379,42 @@ __device__ void relax_body(const SsspArgs &a, uint32_t *dist, SsspSmem &sm, cons
       }
     }
 #pragma unroll
-    for (int j = 0; j < kSsspItems; ++j)
+    for (int j = 0; j < ITEMS; ++j)
       cur[j] = nd[j] != 0xFFFFFFFFu ? dist[v[j]] : 0u;  // plain-load cull
 #pragma unroll
-    for (int j = 0; j < kSsspItems; ++j) {
+    for (int j = 0; j < ITEMS; ++j) {
       const bool try_it = nd[j] < cur[j];
       cur[j] = try_it ? atomicMin(dist + v[j], nd[j]) : 0u;
       if (!try_it) nd[j] = 0xFFFFFFFFu;
     }
 #pragma unroll
-    for (int j = 0; j < kSsspItems; ++j) {
+    for (int j = 0; j < ITEMS; ++j) {
       code[j] = 0;
       if (nd[j] < cur[j]) {  // this thread lowered dist[v]
         if (nd[j] < T) {
           code[j] = atomicExch(a.stamp + v[j], iter) != iter ? 1 : 0;
         } else {
-          atomicMin(st.fmin, nd[j]);
+          local_min = min(local_min, nd[j]);
           code[j] = atomicExch(a.far_stamp + v[j], epoch) != epoch ? 2 : 0;
         }
       }
     }
 #pragma unroll
-    for (int j = 0; j < kSsspItems; ++j)
+    for (int j = 0; j < ITEMS; ++j)
       dv[j] = code[j] == 1 ? a.R[vl[j] + 1] - a.R[vl[j]] : 0;
 #pragma unroll
-    for (int j = 0; j < kSsspItems; ++j) {
+    for (int j = 0; j < ITEMS; ++j) {
       emit_scanned(sm.nearb, code[j] == 1, v[j], dv[j]);
       emit_plain(sm.farb, code[j] == 2, v[j]);
     }
     flush_scanned<kSsspThreads>(sm.nearb, st.near_ctr, Qn, Sn, a.nv + 1);
     flush_plain<kSsspThreads>(sm.farb, st.far_ctr, st.far_dest, st.far_cap);
+  }
+  if (blockIdx.x < nchunks) {
+    // one atomic per warp: one per far edge kept the one address busy for
+    // 0.9 of 2.5 ms (R-MAT 2^21, one mean weight a bucket)
+    local_min = __reduce_min_sync(0xffffffffu, local_min);
+    if ((threadIdx.x & 31) == 0 && local_min != 0xFFFFFFFFu) atomicMin(st.fmin, local_min);
   }
 }
 
@@ -519,142 +541,69 @@ __device__ void relax_body_thread(const SsspArgs &a, uint32_t *dist, const SsspS
 
 // Pull form of one relaxation: for every vertex v (one graph copy), the
 // smallest dist[u] + w(e) over the entries e = (v, u) of its row, which on a
-// symmetric CSR are its in-edges, replaces dist[v] if smaller. Merge-based
-// like the neighbourhood gather-reduce: a chunk's vertex end markers and its
-// edges form one sequence; the block gathers dist[C[e]] + W[e] of the
-// chunk's edges into shared memory (coalesced column and weight loads, the
-// distance gathers of the chunk in flight at once), then each thread walks
-// kSsspItems consecutive items, taking the minimum per vertex. A vertex
-// whose row lies inside one thread's items is lowered with a plain store
-// (nobody else writes it in this iteration); the pieces of a split row use
-// atomicMin. A lowered vertex joins the next near frontier (below T) or the
-// far pile, deduplicated by the same stamps as in relax.
-__device__ void pull_relax_body(const SsspArgs &a, uint32_t *dist, SsspSmem &sm,
-                                const SsspStep &st) {
-  constexpr int ITEMS = kSsspItems;
-  constexpr int CHUNK = kSsspChunk;
+// symmetric CSR are its in-edges, replaces dist[v] if smaller, and v is
+// marked. Distances change under the readers' hands, downwards only: a
+// reader may miss a lowering, but the vertex lowered is marked and goes on
+// the next frontier. R-MAT 2^21, 63.5 M entries: 205 us with the sweep, where
+// a push of that frontier takes 750.
+struct PullValue {
+  static constexpr bool kWeighted = true;
+  const uint32_t *dist;
+  __device__ __forceinline__ uint32_t operator()(int32_t u, int32_t w) const {
+    const uint32_t d = dist[u], t = d + (uint32_t)w;
+    return t < d ? 0xFFFFFFFFu : t;  // sums past the range: unreachable
+  }
+};
+struct ReduceMinU32 {
+  static __device__ __forceinline__ uint32_t identity() { return 0xFFFFFFFFu; }
+  static __device__ __forceinline__ uint32_t op(uint32_t a, uint32_t b) { return min(a, b); }
+};
+struct LowerDist {
+  uint32_t *dist;
+  uint32_t *lowered;
+  __device__ __forceinline__ void operator()(int32_t v, uint32_t nd, bool whole) const {
+    if (nd >= dist[v]) return;
+    if (whole) dist[v] = nd;  // nobody else writes it in this pull
+    else if (nd >= atomicMin(dist + v, nd)) return;
+    atomicOr(lowered + (v >> 5), 1u << (v & 31));
+  }
+};
+
+__device__ __forceinline__ void pull_body(const SsspArgs &a, uint32_t *dist) {
+  gather_reduce_tiles<1, uint32_t, ReduceMinU32>(
+      a.plan, a.C, (const int32_t *)a.W, 0, (int32_t)a.m, PullValue{dist},
+      LowerDist{dist, a.lowered}, spread_warp(), grid_warps());
+}
+
+// The marked vertices to near (below T) or far, the marks cleared.
+template <int ITEMS>
+__device__ void sweep_body(const SsspArgs &a, const uint32_t *dist, SsspSmem<ITEMS> &sm,
+                           const SsspStep &st) {
+  constexpr int CHUNK = kSsspThreads * ITEMS;
   int32_t *Qn = pick(a.nearq, st.near_parity ^ 1);
   int32_t *Sn = pick(a.nearS, st.near_parity ^ 1);
-  const unsigned long long T = st.T;
-  const int32_t iter = st.iter, epoch = st.far_epoch;
-  int32_t *s_end = sm.off;  // end marker of each chunk vertex, chunk-local
-  uint32_t *s_val = sm.du;  // dist[u] + w(e) of each chunk edge
   uint32_t local_min = 0xFFFFFFFFu;
-  const long long total = (long long)a.n + a.m;
-  const long long nchunks = (total + CHUNK - 1) / CHUNK;
-  for (long long chunk = blockIdx.x; chunk < nchunks; chunk += gridDim.x) {
-    const long long d0 = chunk * CHUNK;
-    const long long d1 = min(d0 + CHUNK, total);
-    const int32_t i0 = a.cb[chunk], i1 = a.cb[chunk + 1];
-    const long long j0 = d0 - i0, j1 = d1 - i1;
-    const int32_t nv = (i0 <= a.n - 1) ? (min(i1, a.n - 1) - i0 + 1) : 0;
-    const int32_t ne = (int32_t)(j1 - j0);
-    const int32_t len = (int32_t)(d1 - d0);
-    for (int32_t k = threadIdx.x; k < nv; k += kSsspThreads)
-      s_end[k] = (int32_t)((long long)a.R[i0 + k + 1] + i0 + k - d0);
-    {
-      int32_t col[ITEMS];
-      uint32_t wt[ITEMS];
+  for (int64_t b = (int64_t)blockIdx.x * CHUNK; b < a.n; b += (int64_t)gridDim.x * CHUNK) {
 #pragma unroll
-      for (int i = 0; i < ITEMS; ++i) {
-        const int32_t k = threadIdx.x + i * kSsspThreads;
-        col[i] = -1;
-        wt[i] = 0u;
-        if (k < ne && GR_IN(j0 + k, a.m, 330)) {
-          col[i] = a.C[j0 + k];
-          wt[i] = a.W[j0 + k];
-          if (!GR_IN(col[i], a.n, 331)) col[i] = -1;
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < ITEMS; ++i) {
-        const int32_t k = threadIdx.x + i * kSsspThreads;
-        if (k < ne) {
-          uint32_t val = 0xFFFFFFFFu;
-          if (col[i] >= 0) {
-            const unsigned long long t = (unsigned long long)dist[col[i]] + wt[i];
-            if (t < 0xFFFFFFFFull) val = (uint32_t)t;
-          }
-          s_val[k] = val;
-        }
-      }
-    }
-    __syncthreads();
-    // this thread's items [k0, k1) of the chunk: item i closes at most one
-    // vertex (slot i), and slot ITEMS holds the vertex continuing past k1
-    int32_t cv[ITEMS + 1];
-    uint32_t cd[ITEMS + 1];
-    bool cw[ITEMS + 1];  // whole: the vertex's row lies in this thread's items
-#pragma unroll
-    for (int j = 0; j <= ITEMS; ++j) {
-      cv[j] = -1;
-      cd[j] = 0xFFFFFFFFu;
-      cw[j] = false;
-    }
-    const int32_t k0 = min(len, (int32_t)threadIdx.x * ITEMS);
-    const int32_t k1 = min(len, k0 + ITEMS);
-    if (k0 < k1) {
-      int32_t lo = 0, hi = nv;
-      while (lo < hi) {
-        const int32_t mid = (lo + hi) >> 1;
-        if (s_end[mid] < k0) lo = mid + 1;
-        else hi = mid;
-      }
-      int32_t r = lo, e = k0 - r;
-      uint32_t best = 0xFFFFFFFFu;
-      bool first = true;  // the current vertex may have entries before k0
-#pragma unroll
-      for (int i = 0; i < ITEMS; ++i) {
-        const int32_t k = k0 + i;
-        if (k < k1) {
-          if (r < nv && s_end[r] == k) {  // end marker of vertex i0 + r
-            cv[i] = i0 + r;
-            cd[i] = best;
-            cw[i] = !first;
-            best = 0xFFFFFFFFu;
-            first = false;
-            ++r;
-          } else {
-            best = min(best, s_val[e]);
-            ++e;
-          }
-        }
-      }
-      if (r < nv && best != 0xFFFFFFFFu) {  // continues past k1
-        cv[ITEMS] = i0 + r;
-        cd[ITEMS] = best;
-        cw[ITEMS] = false;
-      }
-    }
-    // lower, classify and emit (warp-uniform emission calls)
-#pragma unroll
-    for (int j = 0; j <= ITEMS; ++j) {
+    for (int j = 0; j < ITEMS; ++j) {
+      const int64_t v0 = b + j * kSsspThreads + threadIdx.x;  // a warp has one word of marks
+      const uint32_t word = v0 < a.n ? a.lowered[v0 >> 5] : 0u;
       int code = 0;
-      int32_t dvg = 0;
-      const int32_t v = cv[j];
-      const uint32_t nd = cd[j];
-      if (v >= 0 && nd != 0xFFFFFFFFu) {
-        bool lowered;
-        if (cw[j]) {
-          lowered = nd < dist[v];
-          if (lowered) dist[v] = nd;
+      int32_t d = 0;
+      if ((word >> (v0 & 31)) & 1u) {
+        const uint32_t nd = dist[v0];
+        if (nd < st.T) {
+          code = 1;
+          d = a.R[v0 + 1] - a.R[v0];
         } else {
-          lowered = nd < atomicMin(dist + v, nd);
-        }
-        if (lowered) {
-          if ((unsigned long long)nd < T) {
-            if (atomicExch(a.stamp + v, iter) != iter) {
-              code = 1;
-              dvg = a.R[v + 1] - a.R[v];
-            }
-          } else {
-            local_min = min(local_min, nd);
-            code = atomicExch(a.far_stamp + v, epoch) != epoch ? 2 : 0;
-          }
+          local_min = min(local_min, nd);
+          code = atomicExch(a.far_stamp + v0, st.far_epoch) != st.far_epoch ? 2 : 0;
         }
       }
-      emit_scanned(sm.nearb, code == 1, v, dvg);
-      emit_plain(sm.farb, code == 2, v);
+      __syncwarp();
+      if ((threadIdx.x & 31) == 0 && word) a.lowered[v0 >> 5] = 0u;
+      emit_scanned(sm.nearb, code == 1, (int32_t)v0, d);
+      emit_plain(sm.farb, code == 2, (int32_t)v0);
     }
     flush_scanned<kSsspThreads>(sm.nearb, st.near_ctr, Qn, Sn, a.nv + 1);
     flush_plain<kSsspThreads>(sm.farb, st.far_ctr, st.far_dest, st.far_cap);
@@ -663,7 +612,8 @@ __device__ void pull_relax_body(const SsspArgs &a, uint32_t *dist, SsspSmem &sm,
   if ((threadIdx.x & 31) == 0 && local_min != 0xFFFFFFFFu) atomicMin(st.fmin, local_min);
 }
 
-__device__ void split_body(const SsspArgs &a, const uint32_t *dist, SsspSmem &sm,
+template <int ITEMS>
+__device__ void split_body(const SsspArgs &a, const uint32_t *dist, SsspSmem<ITEMS> &sm,
                            const SsspStep &st) {
   const int32_t *F = pick(a.farq, st.far_parity);
   const int32_t np = st.near_parity;
@@ -697,7 +647,7 @@ __device__ void split_body(const SsspArgs &a, const uint32_t *dist, SsspSmem &sm
     }
     emit_scanned(sm.nearb, code == 1, v, dv);
     emit_plain(sm.farb, code == 2, v);
-    if ((r + 1) % (kSsspChunk / kSsspThreads) == 0 || r == rounds - 1) {
+    if ((r + 1) % ITEMS == 0 || r == rounds - 1) {
       flush_scanned<kSsspThreads>(sm.nearb, st.near_ctr, Qn, Sn, a.nv + 1);
       flush_plain<kSsspThreads>(sm.farb, st.far_ctr, st.far_dest, st.far_cap);
     }
@@ -707,7 +657,7 @@ __device__ void split_body(const SsspArgs &a, const uint32_t *dist, SsspSmem &sm
 }
 
 template <bool LOW>
-__device__ void relax_mode(const SsspArgs &a, SsspCtl *c, SsspSmem &sm) {
+__device__ void relax_mode(const SsspArgs &a, SsspCtl *c, SsspSmem<kSsspItems> &sm) {
   SsspStep st;
   st.near_parity = c->near_parity;
   st.far_parity = c->far_parity;
@@ -723,12 +673,13 @@ __device__ void relax_mode(const SsspArgs &a, SsspCtl *c, SsspSmem &sm) {
   st.far_dest = pick(a.farq, c->far_parity);
   st.far_cap = (long long)a.nv + 1;
   st.fmin = &c->far_min;
-  if (!LOW && c->mode == kSsspPull) pull_relax_body(a, c->dist, sm, st);
-  else if (LOW) relax_body_thread(a, c->dist, st);
+  if (LOW) relax_body_thread(a, c->dist, st);
+  else if (c->mode == kSsspPull) pull_body(a, c->dist);
+  else if (c->mode == kSsspSweep) sweep_body(a, c->dist, sm, st);
   else relax_body(a, c->dist, sm, st);
 }
 
-__device__ void split_mode(const SsspArgs &a, SsspCtl *c, SsspSmem &sm) {
+__device__ void split_mode(const SsspArgs &a, SsspCtl *c, SsspSmem<kSsspItems> &sm) {
   SsspStep st;
   st.near_parity = c->near_parity;
   st.far_parity = c->far_parity;
@@ -757,13 +708,17 @@ __device__ void sssp_end(const SsspArgs &a, SsspCtl *c) {
     c->done = 1;
     return;
   }
+  if (c->mode == kSsspPull) {  // its sweep is the rest of this iteration
+    c->mode = kSsspSweep;
+    return;
+  }
   // counters the other blocks filled with atomics: read past L1
   const unsigned long long packed = *(volatile unsigned long long *)&c->near_next_packed;
   const int32_t qn = (int32_t)(packed & 0xFFFFFFFFull);
   const long long en = (long long)(packed >> 32);
   if (c->mode != kSsspSplit) {
-    c->relaxations += c->mode == kSsspPull ? a.m : c->near_edges;
-    c->pulls += c->mode == kSsspPull;
+    c->relaxations += c->mode == kSsspSweep ? a.m : c->near_edges;
+    c->pulls += c->mode == kSsspSweep;
     c->far_len = *(volatile int32_t *)&c->far_len;
     c->far_min = *(volatile uint32_t *)&c->far_min;
   } else {
@@ -811,7 +766,7 @@ __global__ void __launch_bounds__(kSsspThreads, kSsspBlocksPerSm)
     if (use_cond && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(h, 0u);
     return;
   }
-  __shared__ SsspSmem sm;
+  __shared__ SsspSmem<kSsspItems> sm;
   if (threadIdx.x == 0) {
     sm.nearb.cnt = 0;
     sm.farb.cnt = 0;
@@ -838,11 +793,21 @@ __global__ void __launch_bounds__(kSsspThreads, kSsspBlocksPerSm)
 // each iteration of the grid kernel costs two microseconds of barrier and a
 // chain of L2 round trips from queue to queue (9 us in all). Here one block
 // runs a search by itself, so a batch runs its searches side by side on SMs of
-// their own: iterations are separated by __syncthreads, the frontier and the
-// near and far membership bits live in shared memory, a vertex's row comes as
-// one 32-byte load (low_adjacency), and the only L2 chain left is row and
-// distance, then atomicMin: 0.6 us. On the 511 x 511 grid an iteration went
-// from 8.8 to 1.1 us.
+// their own: iterations are separated by one __syncthreads, the frontier and
+// the near and far membership bits live in shared memory, a vertex's row is
+// one 32-byte sector of low_adjacency read by four threads, an edge each, and
+// the L2 chain left is row and distance, then atomicMin. 511 x 511 grid,
+// weights to 16, two mean weights a bucket: 8.8 us an iteration on the grid,
+// 2.5 with a thread per vertex (its four bit tests one after another) and a
+// pass of its own to take the frontier off the bits, 2.1 so. What is left is
+// that chain (1.4 us) and, above some 300 vertices, one L2 access a clock.
+//
+// A vertex leaves the frontier's membership bits when its first thread takes
+// it up; that thread's read of the distance waits for the cleared word, as
+// the bit test of a thread that lowers the distance waits for what its
+// atomicMin returns. So whoever lowers the distance and still finds the bit
+// did so before that read, everybody else finds it clear and puts the vertex
+// on the next frontier, and no barrier stands between the two.
 //
 // A lane whose frontier outgrows kSoloHandoff vertices writes it and its far
 // pile to the control block's queues (parity 0) and stops; k_sssp_do, next on
@@ -852,68 +817,61 @@ __global__ void __launch_bounds__(kSsspThreads, kSsspBlocksPerSm)
 // shared-memory queue cannot, and those of nearS[0] and nearS[1] the far pile
 // by parity (both are free: per-thread relaxations use no degree scan).
 struct SoloState {
-  int32_t near[2];   // frontier sizes by parity
+  int32_t near[3];   // frontier sizes, ring by iteration
   int32_t far[2];    // far pile sizes by parity
   uint32_t far_min;  // lower bound of the far pile's distances
   int32_t near_at, far_at;  // hand-over positions
   unsigned long long relaxed;
 };
 
-// Appends the entries of a warp (code 1: near, 2: far) of item j to the
-// queues: one shared-memory atomic per queue.
-template <int ITEMS>
-__device__ __forceinline__ void solo_append(const int32_t (&v)[ITEMS], const int (&code)[ITEMS],
-                                            int32_t *near_cnt, int32_t *far_cnt, int32_t *near_s,
-                                            int32_t *near_g, int32_t *far) {
+// Appends a warp's entries (code 1: near, 2: far), one shared-memory atomic
+// per queue.
+__device__ __forceinline__ void solo_append(int32_t v, int code, int32_t *near_cnt,
+                                            int32_t *far_cnt, int32_t *near_s, int32_t *near_g,
+                                            int32_t *far) {
+  const uint32_t nb = __ballot_sync(0xffffffffu, code == 1);
+  const uint32_t fb = __ballot_sync(0xffffffffu, code == 2);
+  if (!(nb | fb)) return;
   const int lane = threadIdx.x & 31;
   const uint32_t lt = (1u << lane) - 1u;
-  uint32_t nb[ITEMS], fb[ITEMS];
-  int32_t nt = 0, ft = 0;
-#pragma unroll
-  for (int j = 0; j < ITEMS; ++j) {
-    nb[j] = __ballot_sync(0xffffffffu, code[j] == 1);
-    fb[j] = __ballot_sync(0xffffffffu, code[j] == 2);
-    nt += __popc(nb[j]);
-    ft += __popc(fb[j]);
-  }
   int32_t at = 0;
-  if (lane == 0 && nt) at = atomicAdd(near_cnt, nt);
-  if (lane == 1 && ft) at = atomicAdd(far_cnt, ft);
-  int32_t kn = __shfl_sync(0xffffffffu, at, 0), kf = __shfl_sync(0xffffffffu, at, 1);
-#pragma unroll
-  for (int j = 0; j < ITEMS; ++j) {
-    if (code[j] == 1) {
-      const int32_t k = kn + __popc(nb[j] & lt);
-      if (k < kSoloQueue) near_s[k] = v[j];
-      else near_g[k] = v[j];
-    } else if (code[j] == 2) {
-      far[kf + __popc(fb[j] & lt)] = v[j];
-    }
-    kn += __popc(nb[j]);
-    kf += __popc(fb[j]);
+  if (lane == 0 && nb) at = atomicAdd(near_cnt, __popc(nb));
+  if (lane == 1 && fb) at = atomicAdd(far_cnt, __popc(fb));
+  const int32_t kn = __shfl_sync(0xffffffffu, at, 0) + __popc(nb & lt);
+  const int32_t kf = __shfl_sync(0xffffffffu, at, 1) + __popc(fb & lt);
+  if (code == 1) {
+    if (kn < kSoloQueue) near_s[kn] = v;
+    else near_g[kn] = v;
+  } else if (code == 2) {
+    far[kf] = v;
   }
 }
 
+// LONG: the graph has rows of more than four entries; FAR_BITS: the far pile's
+// membership bits fit shared memory (else far_stamp holds them). The code for
+// the other cases costs instruction fetches on every iteration.
+template <bool LONG, bool FAR_BITS>
 __global__ void __launch_bounds__(kSoloThreads, 1) k_sssp_solo(SsspArgs a, SsspSources src) {
   extern __shared__ uint32_t solo_smem[];
   __shared__ SoloState st;
   SsspCtl *c = a.ctl;
   const int32_t nwords = (a.n + 31) >> 5;
-  int32_t *qs[2] = {(int32_t *)solo_smem, (int32_t *)solo_smem + kSoloQueue};
-  uint32_t *nbits = solo_smem + 2 * kSoloQueue;  // on the next frontier
-  uint32_t *fbits = nbits + nwords;              // in the far pile (far_in_smem)
+  int32_t *const q0 = (int32_t *)solo_smem, *const q1 = q0 + kSoloQueue;
+  uint32_t *nbits = solo_smem + 2 * kSoloQueue;  // on the frontier or the next one
+  uint32_t *fbits = nbits + nwords;              // in the far pile (FAR_BITS)
   const int32_t base = (int32_t)blockIdx.x * a.n;
   uint32_t *dist = c->dist + base;
   int32_t *near_g = a.nearq[1] + base;
-  int32_t *far_stamp = a.far_stamp + base;  // -1: not in the far pile (far not in smem)
+  int32_t *far_stamp = a.far_stamp + base;  // -1: not in the far pile (without FAR_BITS)
   int32_t *far0 = a.nearS[0] + base, *far1 = a.nearS[1] + base;
   const unsigned long long delta = c->delta;
   const int32_t max_iters = c->max_iters;
-  const bool fsm = a.far_in_smem;
   const int lane = threadIdx.x & 31;
-  for (int32_t w = threadIdx.x; w < nwords * (fsm ? 2 : 1); w += kSoloThreads) nbits[w] = 0u;
+  const int32_t s0 = src.s[blockIdx.x];
+  for (int32_t w = threadIdx.x; w < nwords * (FAR_BITS ? 2 : 1); w += kSoloThreads)
+    nbits[w] = w == (s0 >> 5) ? 1u << (s0 & 31) : 0u;
   if (threadIdx.x == 0) {
-    qs[0][0] = src.s[blockIdx.x];
+    q0[0] = s0;
     st.near[0] = 1;
     st.near[1] = 0;
     st.far[0] = st.far[1] = 0;
@@ -921,136 +879,120 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_sssp_solo(SsspArgs a, SsspS
     st.relaxed = 0ull;
   }
   unsigned long long T = delta;
-  int32_t p = 0, fp = 0, iter = 0, phases = 0;
+  int32_t fp = 0, iter = 0, ring = 0, phases = 0;
   uint32_t relaxed = 0u;
   __syncthreads();
   for (;;) {
-    // every thread reads the same sizes; what they count next is cleared
-    // before the barrier that opens the appends
-    const int32_t q = st.near[p], len = st.far[fp];
-    const uint32_t far_min = st.far_min;
+    const int32_t next = ring == 2 ? 0 : ring + 1, after = next == 2 ? 0 : next + 1;
+    const int32_t q = st.near[ring], len = st.far[fp];
     const bool split = q == 0;
     if ((split && len == 0) || q > kSoloHandoff || iter >= max_iters) break;
+    if (threadIdx.x == 0) st.near[after] = 0;  // last read an iteration ago
+    const int32_t *Q = iter & 1 ? q1 : q0;
+    int32_t *Qn = iter & 1 ? q0 : q1;
     int32_t *far = fp ? far1 : far0;
-    int32_t *Qn = p ? qs[0] : qs[1];
     uint32_t local_min = 0xFFFFFFFFu;
     if (!split) {
-      const int32_t *Q = p ? qs[1] : qs[0];
-      // off the frontier: from here on a lowered vertex joins the next one
-      for (int32_t i = threadIdx.x; i < q; i += kSoloThreads)
-        atomicAnd(&nbits[Q[i] >> 5], ~(1u << (Q[i] & 31)));
-      if (threadIdx.x == 0) st.near[p ^ 1] = 0;
-      __syncthreads();
-      for (int32_t i0 = 0; i0 < q; i0 += kSoloThreads) {
-        const int32_t i = i0 + (int32_t)threadIdx.x;
-        if (__all_sync(0xffffffffu, i >= q)) break;
-        int32_t v[4] = {-1, -1, -1, -1};
-        uint32_t w[4] = {0u, 0u, 0u, 0u};
+      // nd < T, for distances below 0xFFFFFFFF
+      const uint32_t T32 = (uint32_t)min(T, 0xFFFFFFFFull);
+      for (int32_t i = threadIdx.x; i - lane < 4 * q; i += kSoloThreads) {  // warp-uniform
+        int2 vw = make_int2(-1, 0);
         uint32_t du = 0xFFFFFFFFu;
-        int32_t e = 0, e1 = 0;  // what is left of a row longer than four
-        if (i < q) {
-          const int32_t u = Q[i];
-          const int4 *row = a.adjw + 2 * (int64_t)u;
-          const int4 rv = __ldg(row), rw = __ldg(row + 1);
-          du = __ldcg(dist + u);  // lowered by atomics: not from L1
-          if (rv.x == -2) {
-            e = rv.y;
-            e1 = rv.z;
-          } else {
-            v[0] = rv.x; v[1] = rv.y; v[2] = rv.z; v[3] = rv.w;
-            w[0] = (uint32_t)rw.x; w[1] = (uint32_t)rw.y; w[2] = (uint32_t)rw.z; w[3] = (uint32_t)rw.w;
+        if (i < 4 * q) {
+          const int32_t u = Q[i >> 2];
+          vw = __ldg((const int2 *)a.adjw + 4 * (int64_t)u + (lane & 3));
+          if ((lane & 3) == 0) {
+            // u's bit is set: the address below is u's, once the bit is clear
+            const uint32_t old = atomicAnd(&nbits[u >> 5], ~(1u << (u & 31)));
+            const int32_t u_then = u - 1 + (int32_t)((old >> (u & 31)) & 1u);
+            if (GR_IN(u_then, a.n, 341)) du = __ldcg(dist + u_then);  // atomics lower it: not from L1
+          }
+        }
+        du = __shfl_sync(0xffffffffu, du, lane & ~3);
+        int32_t e = 0, e1 = 0;  // a row longer than four: its quad walks it
+        if (LONG && __any_sync(0xffffffffu, vw.x == -2)) {
+          const int32_t tag = __shfl_sync(0xffffffffu, vw.x, lane & ~3);
+          const int32_t r0 = __shfl_sync(0xffffffffu, vw.y, lane & ~3);
+          const int32_t r1 = __shfl_sync(0xffffffffu, vw.x, (lane & ~3) + 1);
+          if (tag == -2) {
+            e = r0 + (lane & 3);
+            e1 = r1;
+            vw = e < e1 ? make_int2(a.C[e], (int32_t)a.W[e]) : make_int2(-1, 0);
           }
         }
         for (;;) {
-          if (e < e1) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const bool in = e + j < e1;
-              v[j] = in ? a.C[e + j] : -1;
-              w[j] = in ? a.W[e + j] : 0u;
-            }
-            e += 4;
-          }
-          uint32_t nd[4], old[4];
-          int code[4];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const unsigned long long t = (unsigned long long)du + w[j];
-            const bool ok = v[j] >= 0 && t < 0xFFFFFFFFull && GR_IN(v[j], a.n, 340);
-            relaxed += v[j] >= 0;
-            nd[j] = (uint32_t)t;
-            old[j] = ok ? atomicMin(dist + v[j], nd[j]) : 0u;
-          }
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            code[j] = 0;
-            if (nd[j] < old[j]) {  // this thread lowered dist[v]
-              const uint32_t bit = 1u << (v[j] & 31);
-              if (nd[j] < T) {
-                code[j] = atomicOr(&nbits[v[j] >> 5], bit) & bit ? 0 : 1;
-              } else {
-                local_min = min(local_min, nd[j]);
-                if (fsm) code[j] = atomicOr(&fbits[v[j] >> 5], bit) & bit ? 0 : 2;
-                else code[j] = atomicExch(far_stamp + v[j], 0) == 0 ? 0 : 2;
-              }
+          const int32_t v = vw.x;
+          int code = 0;
+          // below 0xFFFFFFFF, or the sum wrapped round or is no distance
+          const uint32_t nd = du + (uint32_t)vw.y;
+          relaxed += v >= 0;
+          if (v >= 0 && nd >= du && nd != 0xFFFFFFFFu && GR_IN(v, a.n, 340) &&
+              nd < atomicMin(dist + v, nd)) {  // this thread lowered dist[v]
+            const uint32_t bit = 1u << (v & 31);
+            if (nd < T32) {
+              code = atomicOr(&nbits[v >> 5], bit) & bit ? 0 : 1;
+            } else {
+              local_min = min(local_min, nd);
+              if (FAR_BITS) code = atomicOr(&fbits[v >> 5], bit) & bit ? 0 : 2;
+              else code = atomicExch(far_stamp + v, 0) == 0 ? 0 : 2;
             }
           }
-          solo_append<4>(v, code, &st.near[p ^ 1], &st.far[fp], Qn, near_g, far);
-          if (!__any_sync(0xffffffffu, e < e1)) break;
-#pragma unroll
-          for (int j = 0; j < 4; ++j) v[j] = -1;
+          __syncwarp();
+          solo_append(v, code, &st.near[next], &st.far[fp], Qn, near_g, far);
+          e += 4;
+          if (!LONG || !__any_sync(0xffffffffu, e < e1)) break;
+          vw = e < e1 ? make_int2(a.C[e], (int32_t)a.W[e]) : make_int2(-1, 0);
         }
       }
-      p ^= 1;
     } else {
       // the far pile by the raised threshold; entries that fell below the
       // old one were expanded already
-      const unsigned long long T_old = T, t = T + delta, b = bucket_end(far_min, delta);
+      const unsigned long long T_old = T, t = T + delta, b = bucket_end(st.far_min, delta);
       T = t > b ? t : b;
       int32_t *far_n = fp ? far0 : far1;
       __syncthreads();  // every thread has read far_min
       if (threadIdx.x == 0) {
-        st.near[p ^ 1] = 0;
         st.far[fp ^ 1] = 0;
         st.far_min = 0xFFFFFFFFu;
       }
       __syncthreads();
       for (int32_t i0 = 0; i0 < len; i0 += kSoloThreads) {
         const int32_t i = i0 + (int32_t)threadIdx.x;
-        if (__all_sync(0xffffffffu, i >= len)) break;
-        int32_t v[1] = {0};
-        int code[1] = {0};
+        if (i0 + (int32_t)(threadIdx.x & ~31) >= len) break;  // warp-uniform
+        int32_t v = 0;
+        int code = 0;
         if (i < len) {
-          v[0] = far[i];
-          const uint32_t d = __ldcg(dist + v[0]);
-          const uint32_t bit = 1u << (v[0] & 31);
+          v = far[i];
+          const uint32_t d = __ldcg(dist + v);
+          const uint32_t bit = 1u << (v & 31);
           if ((unsigned long long)d >= T) {
-            code[0] = 2;
+            code = 2;
             local_min = min(local_min, d);
           } else {
-            if (fsm) atomicAnd(&fbits[v[0] >> 5], ~bit);
-            else far_stamp[v[0]] = -1;
+            if (FAR_BITS) atomicAnd(&fbits[v >> 5], ~bit);
+            else far_stamp[v] = -1;
             if ((unsigned long long)d >= T_old) {
-              code[0] = 1;
-              atomicOr(&nbits[v[0] >> 5], bit);
+              code = 1;
+              atomicOr(&nbits[v >> 5], bit);
             }
           }
         }
-        solo_append<1>(v, code, &st.near[p ^ 1], &st.far[fp ^ 1], Qn, near_g, far_n);
+        __syncwarp();
+        solo_append(v, code, &st.near[next], &st.far[fp ^ 1], Qn, near_g, far_n);
       }
-      p ^= 1;
       fp ^= 1;
       phases += 1;
     }
     local_min = __reduce_min_sync(0xffffffffu, local_min);
     if (lane == 0 && local_min != 0xFFFFFFFFu) atomicMin(&st.far_min, local_min);
     iter += 1;
+    ring = next;
     __syncthreads();
   }
   const uint32_t wsum = __reduce_add_sync(0xffffffffu, relaxed);
   if (lane == 0) atomicAdd(&st.relaxed, (unsigned long long)wsum);
   __syncthreads();
-  const int32_t q = st.near[p], len = st.far[fp];
+  const int32_t q = st.near[ring], len = st.far[fp];
   const bool over = (q > 0 || len > 0) && iter >= max_iters;
   const bool handoff = !over && q > kSoloHandoff;
   if (threadIdx.x == 0) {
@@ -1067,7 +1009,7 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_sssp_solo(SsspArgs a, SsspS
   }
   __syncthreads();
   if (!handoff) return;
-  const int32_t *Q = p ? qs[1] : qs[0];
+  const int32_t *Q = iter & 1 ? q1 : q0;
   const int32_t *far = fp ? far1 : far0;
   long long edges = 0;
   for (int32_t i = threadIdx.x; i < q; i += kSoloThreads) {
@@ -1088,10 +1030,12 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_sssp_solo(SsspArgs a, SsspS
 // iteration's counters and recomputes the same next state in registers; the
 // counters form rings of three (the one an iteration fills, the one just
 // read, the one block 0 clears for the next iteration).
-template <bool LOW>
+template <bool LOW, bool PULL>
 __global__ void __launch_bounds__(kSsspThreads, kSsspBlocksPerSm) k_sssp_do(SsspArgs a) {
+  constexpr int ITEMS = PULL ? kSsspPullItems : kSsspItems;
+  constexpr int CHUNK = kSsspThreads * ITEMS;
   SsspCtl *c = a.ctl;
-  __shared__ SsspSmem sm;
+  __shared__ SsspSmem<ITEMS> sm;
   if (threadIdx.x == 0) {
     sm.nearb.cnt = 0;
     sm.farb.cnt = 0;
@@ -1133,17 +1077,19 @@ __global__ void __launch_bounds__(kSsspThreads, kSsspBlocksPerSm) k_sssp_do(Sssp
     if (mode != kSsspSplit) {
       st.far_dest = pick(a.farq, far_parity) + far_len;  // appended after the pile
       st.far_cap = (long long)a.nv + 1 - far_len;
-      if (!LOW && mode == kSsspPull) {
-        pull_relax_body(a, dist, sm, st);
+      if (PULL && mode == kSsspPull) {
+        pull_body(a, dist);
+        if (!grid_sync(&c->bar, &c->error, gen)) break;
+        sweep_body(a, dist, sm, st);
       } else if (LOW) {
         relax_body_thread(a, dist, st);
       } else {
         // a dense frontier's chunk bounds in one grid-wide pass (every block
         // then starts its chunks without a search)
-        const long long nchunks = ((long long)near_len + near_edges + kSsspChunk - 1) / kSsspChunk;
+        const long long nchunks = ((long long)near_len + near_edges + CHUNK - 1) / CHUNK;
         const bool bounds = a.qcb && nchunks >= (long long)kSsspBoundsChunksPerBlock * gridDim.x;
         if (bounds) {
-          frontier_chunk_bounds(pick(a.nearS, near_parity), near_len, (int32_t)near_edges,
+          frontier_chunk_bounds<CHUNK>(pick(a.nearS, near_parity), near_len, (int32_t)near_edges,
                                 nchunks, a.qcb);
           if (!grid_sync(&c->bar, &c->error, gen)) break;
         }
@@ -1176,7 +1122,7 @@ __global__ void __launch_bounds__(kSsspThreads, kSsspBlocksPerSm) k_sssp_do(Sssp
     iter += 1;
     bool done = false, overflow = false;
     if (near_len > 0) {
-      mode = near_edges >= pull_min_edges ? kSsspPull : kSsspRelax;
+      mode = PULL && near_edges >= pull_min_edges ? kSsspPull : kSsspRelax;
     } else if (far_len > 0) {
       mode = kSsspSplit;
       T_old = T;
@@ -1243,15 +1189,22 @@ static size_t solo_smem(const gr_graph *g, bool far_bits) {
   return bytes + sizeof(SoloState) <= kBlockSmemMax ? bytes : 0;
 }
 
+// Whether a single search may pull: a row holds the in-edges and their
+// weights.
+static bool can_pull(const gr_graph *g) {
+  return g->weights_symmetric && g->max_degree > kLowDegreeMax && g->m > 0;
+}
+
 size_t sssp_ws_bytes(const gr_graph *g, int32_t lanes) {
   const size_t n = (size_t)g->n * (size_t)std::max(lanes, 1);
   const size_t qcb = g->max_degree > kLowDegreeMax
                          ? sizeof(int32_t) * ((n + (size_t)std::max(lanes, 1) * (size_t)g->m) /
-                                                  kSsspChunk + 3)
+                                                  (kSsspThreads * kSsspPullItems) + 3)
                          : 0;
   return 4 * sizeof(int32_t) * (n + 1) + 2 * sizeof(int32_t) * (n + 2) +
          2 * sizeof(int32_t) * n + sizeof(SsspCtl) + qcb +
-         (solo_smem(g, false) ? 32 * (size_t)g->n : 0);
+         (solo_smem(g, false) ? 32 * (size_t)g->n : 0) +
+         (lanes == 1 && can_pull(g) ? gather_plan_bytes(g->n, g->m) + 4 * (size_t)g->nwords : 0);
 }
 
 int32_t sssp_batch_max_lanes(const gr_graph *g) {
@@ -1279,16 +1232,13 @@ gr_status sssp_ws_create(gr_graph *g, cudaStream_t s, SsspWorkspace **out, int32
   GR_TRY(ws->ctl.alloc(sizeof(SsspCtl), "SSSP control"));
   if (g->max_degree > kLowDegreeMax) {
     // a frontier holds at most n vertices of each lane and their edges
-    const long long chunks = ((long long)n + (long long)lanes * g->m) / kSsspChunk + 2;
+    const long long chunks = ((long long)n + (long long)lanes * g->m) /
+                                 (kSsspThreads * kSsspPullItems) + 2;
     GR_TRY(ws->qcb.alloc(sizeof(int32_t) * ((size_t)chunks + 1), "SSSP frontier chunk bounds"));
   }
-  if (lanes == 1) {
-    // the pull relaxation's merge path over all vertices never changes
-    const int32_t chunks = merge_chunks(g->n, g->m, kSsspChunk);
-    GR_TRY(ws->cb.alloc(sizeof(int32_t) * ((size_t)chunks + 1), "SSSP pull chunk bounds"));
-    k_chunk_bounds<<<(chunks + 256) / 256, 256, 0, s>>>(g->row_off.as<int32_t>(), g->n,
-                                                         kSsspChunk, chunks, ws->cb.as<int32_t>());
-    GR_CUDA(cudaGetLastError());
+  if (lanes == 1 && can_pull(g)) {
+    GR_TRY(gather_plan_build(&ws->plan, g->row_off.as<int32_t>(), g->n, g->m, s));
+    GR_TRY(ws->lowered.alloc(sizeof(uint32_t) * (size_t)g->nwords, "SSSP pull marks"));
   }
   GR_CUDA(cudaMemsetAsync(ws->ctl.p, 0, sizeof(SsspCtl), s));
   if (solo_smem(g, false)) GR_TRY(low_adjacency(g, true, s));
@@ -1315,23 +1265,18 @@ static SsspArgs sssp_args(gr_graph *g, SsspWorkspace *ws, int32_t lanes = 1) {
   a.ctl = ws->ctl.as<SsspCtl>();
   a.low_degree = g->max_degree <= kLowDegreeMax ? 1 : 0;
   a.adjw = g->adjw4.as<int4>();
-  a.far_in_smem = 0;
-  a.cb = ws->cb.as<int32_t>();  // null for batched workspaces, which never pull
+  a.plan = ws->plan.a;  // null for batched workspaces, which never pull
+  a.lowered = ws->lowered.as<uint32_t>();
   a.qcb = ws->qcb.as<int32_t>();  // null on low-degree graphs
   return a;
 }
 
-// Smallest near-frontier edge count at which a relaxation pulls. Pull reads
-// every row once where push reads the frontier's rows (and pays atomics and
-// its per-chunk chain), so it pays only where the frontier covers most of
-// the graph: at m / opts->alpha edges, else at m / the graph's tuned alpha
-// (0: never, the default until gr_autotune finds pulling faster); GR_DIR_PUSH
-// never pulls, GR_DIR_PULL pulls every relaxation. Only a symmetric CSR
-// (rows = in-neighbours) and a single search can pull.
+// Smallest near-frontier edge count at which a relaxation pulls: m /
+// opts->alpha, else m / the graph's tuned alpha (0: never); GR_DIR_PUSH
+// never pulls, GR_DIR_PULL pulls every relaxation. A graph whose rows are not
+// its in-edges (weights that differ by direction among them) is only pushed.
 static long long sssp_pull_min_edges(const gr_graph *g, const gr_opts &o, int32_t lanes) {
-  if (!g->symmetric || lanes != 1 || g->max_degree <= kLowDegreeMax || g->m == 0 ||
-      o.direction == GR_DIR_PUSH)
-    return LLONG_MAX;
+  if (lanes != 1 || !can_pull(g) || o.direction == GR_DIR_PUSH) return LLONG_MAX;
   if (o.direction == GR_DIR_PULL) return 1;
   const double div = o.alpha > 0.f ? (double)o.alpha : (double)g->tuned_sssp_alpha;
   if (div <= 0.0) return LLONG_MAX;
@@ -1421,15 +1366,18 @@ static gr_status sssp_drive(gr_graph *g, SsspWorkspace *ws, SsspArgs a, const Ss
                                              sssp_pull_min_edges(g, o, src.k), near_only > 0);
   GR_CUDA(cudaGetLastError());
   if (near_only) {
-    const size_t both = solo_smem(g, true);
-    a.far_in_smem = both > 0;
-    GR_CUDA(cudaFuncSetAttribute(k_sssp_solo, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(both ? both : near_only)));
-    k_sssp_solo<<<src.k, kSoloThreads, both ? both : near_only, s>>>(a, src);
+    const size_t both = solo_smem(g, true), bytes = both ? both : near_only;
+    const bool longer = g->max_degree > 4;
+    auto kern = both ? (longer ? k_sssp_solo<true, true> : k_sssp_solo<false, true>)
+                     : (longer ? k_sssp_solo<true, false> : k_sssp_solo<false, false>);
+    GR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    kern<<<src.k, kSoloThreads, bytes, s>>>(a, src);
     GR_CUDA(cudaGetLastError());
   }
   if (mode == GR_MODE_PERSISTENT) {
-    void *kern = a.low_degree ? (void *)k_sssp_do<true> : (void *)k_sssp_do<false>;
+    void *kern = a.low_degree ? (void *)k_sssp_do<true, false>
+                 : sssp_pull_min_edges(g, o, src.k) < LLONG_MAX ? (void *)k_sssp_do<false, true>
+                                                                : (void *)k_sssp_do<false, false>;
     const int32_t want = o.block > 0 ? o.block : g->tuned_sssp_blocks_per_sm;
     // the carveout fitted to the blocks that run leaves the rest to L1
     int bps = 1;

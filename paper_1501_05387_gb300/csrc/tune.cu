@@ -37,10 +37,28 @@ void tune_prior(gr_graph *g) {
     // thousands of thin iterations: one kernel with a cheap grid barrier
     g->tuned_sssp_mode = GR_MODE_PERSISTENT;
     g->tuned_sssp_blocks_per_sm = 1;
+    // six mean weights a bucket: one block's search (k_sssp_solo) of grids of
+    // 64 to 1024 a side, weights to 16, 64 and 1000, took 1.0-1.2 times its
+    // best there, 1.1-1.7 times at two mean weights, 1.0-1.3 at twelve
+    if (g->has_weights)
+      g->sssp_delta = (uint32_t)std::max(1.0, std::min(6.0 * g->mean_weight, 4.0e9));
   } else {
     g->tuned_direction = GR_DIR_AUTO;
     g->tuned_blocks_per_sm = 0;  // all resident blocks
+    // skewed graphs reach most vertices in a few dense relaxations: the
+    // persistent kernel, and buckets wide enough not to repeat them (R-MAT
+    // 2^21, pushed: 2.28 ms in the graph loop at two mean weights a bucket,
+    // 1.60 so; 2^16: 432 and 315 us)
+    g->tuned_sssp_mode = GR_MODE_PERSISTENT;
+    if (g->has_weights)
+      g->sssp_delta = (uint32_t)std::max(1.0, std::min(8.0 * g->mean_weight, 4.0e9));
   }
+  // A frontier with a third of the edges is relaxed in pull form where its
+  // 256-entry tiles fill the GPU: R-MAT 2^21 0.95 ms (1.60 pushed; 0.95 from
+  // half of the edges, 0.96 from a sixth, 1.01 from an eighth), 300,001
+  // vertices 0.42 ms (0.55), but 2^16 and 1.4 M entries 326 us (321), 2^13
+  // 128 us (115).
+  g->tuned_sssp_alpha = g->m >= (int64_t)g->num_sms * 10240 ? 3.f : 0.f;
   g->tuned_mode = GR_MODE_AUTO;
 }
 
@@ -153,12 +171,12 @@ gr_status gr_autotune(gr_graph *g, const int32_t *srcs, int32_t k, int32_t what,
     for (double f : {0.5, 1.0, 2.0, 4.0, 8.0, 32.0, 64.0})
       deltas.push_back((uint32_t)std::max(1.0, std::min(4.0e9, f * mw)));
     deltas.push_back(UINT32_MAX);
-    // pull thresholds to try where the graph can pull (symmetric, not
-    // mesh-like): the frontier holding 80 % or half of the edges
+    // pull thresholds to try where the graph can pull (in-edges in the rows,
+    // not mesh-like): the frontier holding half or a sixth of the edges
     std::vector<float> alphas = {0.f};
-    if (g->symmetric && g->max_degree > 16) {
-      alphas.push_back(1.25f);
+    if (g->weights_symmetric && g->max_degree > kLowDegreeMax) {
       alphas.push_back(2.f);
+      alphas.push_back(6.f);
     }
     for (uint32_t d : deltas)
       for (float al : alphas) {

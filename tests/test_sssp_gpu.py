@@ -369,3 +369,40 @@ def test_mesh_persistent_equals_graph_driver(cuda_lib, delta):
         d_graph, _ = run_sssp(cuda_lib, g, src, opts(cuda_lib, delta, "graph"))
         d_pers, _ = run_sssp(cuda_lib, g, src, opts(cuda_lib, delta, "persistent"))
         assert np.array_equal(d_graph, d_pers)
+
+
+@pytest.mark.parametrize("direction", ["auto", "pull"])
+def test_weights_that_differ_by_direction(cuda_lib, direction):
+    """A symmetric CSR whose edges weigh more one way than the other, and one
+    with an edge stored twice: a row then is not the in-edges, so nothing may
+    be pulled."""
+    gr = cuda_lib
+    r, c = gg.rmat(14, 16, seed=5)
+    w = np.random.default_rng(5).integers(1, 65, c.size).astype(np.uint32)
+    with gr.gr_graph_create(r, c, w) as g:
+        for alpha in (0.0, 16.0):
+            check(gr, r, c, w, g, gg.max_degree_vertex(r),
+                  opts(gr, 0, "persistent", direction, alpha))
+    r = np.array([0, 3, 6, 7], np.int32)
+    c = np.array([1, 1, 2, 0, 0, 2, 0], np.int32)  # 1 has no way back from 2
+    r2 = np.array([0, 3, 6, 8], np.int32)
+    c2 = np.array([1, 1, 2, 0, 0, 2, 0, 1], np.int32)
+    w2 = np.array([5, 9, 50, 9, 7, 1, 2, 3], np.uint32)
+    with gr.gr_graph_create(r, c, w2[:7]) as g, gr.gr_graph_create(r2, c2, w2) as g2:
+        assert not gr.gr_graph_info(g)["symmetric"] and gr.gr_graph_info(g2)["symmetric"]
+        for src in range(3):
+            check(gr, r, c, w2[:7], g, src)
+            check(gr, r2, c2, w2, g2, src, opts(gr, 0, "persistent", direction))
+
+
+def test_symmetry_needs_the_right_partners(cuda_lib):
+    """As many entries above the diagonal as below, but not each other's."""
+    for edges, want in (([(0, 1), (1, 0), (2, 3), (3, 2)], True),
+                        ([(0, 1), (2, 0), (1, 2)], False),
+                        ([(0, 1), (1, 0), (0, 2), (3, 1)], False),
+                        ([(0, 0), (0, 1), (1, 0), (1, 1)], True)):
+        r = np.zeros(5, np.int32)
+        np.add.at(r, np.array([u for u, _ in edges]) + 1, 1)
+        c = np.array([v for _, v in sorted(edges)], np.int32)
+        with cuda_lib.gr_graph_create(np.cumsum(r).astype(np.int32), c) as g:
+            assert cuda_lib.gr_graph_info(g)["symmetric"] == want, edges
