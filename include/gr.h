@@ -205,8 +205,7 @@ gr_status gr_sssp_pull_stats(gr_graph *g, int32_t *pulls);
  * hooking pass is sampled: every vertex first hooks to its first two
  * neighbours, the trees are compressed, and only the vertices outside the
  * component most of a fixed sample of vertices falls in hook all their
- * edges (the labels are the same; the call synchronises once to read the
- * sample). opts is unused. */
+ * edges (the labels are the same). opts is unused. */
 gr_status gr_cc(gr_graph *g, int32_t *label, int32_t *num_components,
                 const gr_opts *opts, void *stream);
 

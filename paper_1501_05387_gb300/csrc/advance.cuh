@@ -98,7 +98,8 @@ __device__ __forceinline__ void warp_append(int code, int32_t v, int32_t *buf0,
   }
 }
 
-// Load-balanced advance over frontier Q[0..q) with scanned degrees S[0..q].
+// Load-balanced advance over frontier Q[0..q) with scanned degrees S[0..q),
+// s_q = S[q] (which need not be stored).
 // For every edge e = (u, v) of a frontier vertex, f(u, v, e) runs once and
 // returns 0 (drop), 1 (append v to out0) or 2 (append v to out1, only when
 // NOUT == 2); with NOUT == 0 nothing is appended and the output arguments
@@ -108,10 +109,10 @@ __device__ __forceinline__ void warp_append(int code, int32_t v, int32_t *buf0,
 // Q == nullptr means the all-vertex frontier (Q[i] = i, S = R, q = n).
 template <int THREADS, int ITEMS, int NOUT, class F>
 __device__ void lb_advance(const int32_t *R, const int32_t *C, const int32_t *Q, int32_t q,
-                           const int32_t *S, F &f, int32_t *out0, int32_t *len0,
+                           const int32_t *S, int32_t s_q, F &f, int32_t *out0, int32_t *len0,
                            int32_t *out1, int32_t *len1) {
   constexpr int CHUNK = THREADS * ITEMS;
-  const long long total = (long long)q + S[q];
+  const long long total = (long long)q + s_q;
   const long long nchunks = (total + CHUNK - 1) / CHUNK;
   __shared__ int32_t s_off[CHUNK + 1];
   __shared__ int32_t s_u[CHUNK + 1];
@@ -125,7 +126,7 @@ __device__ void lb_advance(const int32_t *R, const int32_t *C, const int32_t *Q,
     const long long d1 = min(d0 + CHUNK, total);
     if (threadIdx.x < 2) s_cnt[threadIdx.x] = 0;
     int32_t i0, i1;
-    block_chunk_bounds<THREADS>(S, q, S[q], d0, d1, CHUNK, s_red8, &i0, &i1);
+    block_chunk_bounds<THREADS>(S, q, s_q, d0, d1, CHUNK, s_red8, &i0, &i1);
     const long long j0 = d0 - i0, j1 = d1 - i1;
     const int32_t nv = (i0 <= q - 1) ? (min(i1, q - 1) - i0 + 1) : 0;
     for (int32_t k = threadIdx.x; k < nv; k += THREADS) {

@@ -1105,6 +1105,230 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_bfs_solo(BfsArgs a) {
   }
 }
 
+// ------------------------------------------------------------ small graphs
+// On a graph of a few thousand vertices a traversal is a handful of levels,
+// each a grid barrier (4-7 us) around a microsecond of work, after an init
+// kernel and a cooperative launch. Here one block does all of it in one
+// launch: depths, parents and the visited bits live in shared memory (16-bit:
+// at most 32768 vertices), so do the vertices in the order of their discovery,
+// in which a level is a range; the outputs are written once, in full rows.
+// Pushes deal the frontier's edges to the threads by a scan of its degrees
+// (1024 frontier vertices at a time); pulls give a warp a word of vertices, as
+// on the grid, and test a neighbour's depth instead of a frontier bitmap.
+//
+// One SM takes about one random access a clock, so the edges it may have to
+// push are limited: a direction-optimising traversal pushes at most a tenth
+// of the unexplored ones a level, a push-only one all of them.
+constexpr int kSmallThreads = 1024;
+constexpr int32_t kSmallMaxN = 32768;
+constexpr int64_t kSmallMaxM = 1 << 20, kSmallMaxPushM = 1 << 16;
+
+__host__ __device__ __forceinline__ size_t small_smem_bytes(int32_t n) {
+  return 3 * sizeof(uint16_t) * (size_t)((n + 31) & ~31) + sizeof(uint32_t) * (size_t)((n + 31) / 32);
+}
+
+struct SmallState {
+  int32_t pre[kSmallThreads];   // push: scan of a frontier chunk's degrees
+  int32_t row[kSmallThreads];   // and its row starts
+  uint16_t u[kSmallThreads];    // and its vertices
+  uint32_t red[33];
+  int32_t tail;                 // vertices discovered so far
+};
+
+// Appends the vertices of a warp (take) in their order of discovery.
+__device__ __forceinline__ void small_append(int32_t *tail, uint16_t *order, bool take, int32_t v) {
+  const uint32_t b = __ballot_sync(0xffffffffu, take);
+  if (!b) return;
+  const int lane = threadIdx.x & 31;
+  int32_t at = 0;
+  if (lane == 0) at = atomicAdd(tail, __popc(b));
+  at = __shfl_sync(0xffffffffu, at, 0);
+  if (take) order[at + __popc(b & ((1u << lane) - 1u))] = (uint16_t)v;
+}
+
+__global__ void __launch_bounds__(kSmallThreads, 1)
+    k_bfs_small(BfsArgs a, int32_t src, int32_t *depth, int32_t *parent, int32_t policy,
+                float alpha, float beta, int32_t max_levels, int32_t preset_iso) {
+  extern __shared__ uint32_t solo_smem[];
+  __shared__ SmallState st;
+  BfsCtl *c = a.ctl;
+  const int32_t npad = (a.n + 31) & ~31;
+  uint32_t *visited = solo_smem;
+  uint16_t *order = (uint16_t *)(visited + a.nwords);
+  uint16_t *dep = order + npad;  // 0xFFFF: unreached
+  uint16_t *par = dep + npad;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int32_t w = threadIdx.x; w < a.nwords; w += kSmallThreads)
+    visited[w] = (preset_iso ? a.iso[w] : 0u) | (w == (src >> 5) ? 1u << (src & 31) : 0u);
+  for (int32_t v = threadIdx.x; v < a.n; v += kSmallThreads) {
+    dep[v] = v == src ? 0 : 0xFFFF;
+    par[v] = v == src ? (uint16_t)src : 0xFFFF;
+  }
+  if (threadIdx.x == 0) {
+    order[0] = (uint16_t)src;
+    st.tail = 1;
+    c->t_start = globaltimer();
+  }
+  __syncthreads();
+  int32_t lo = 0, hi = 1, L = 0, pulls = 0, q_prev = 0, dir = kPush;
+  long long mu = a.m;
+  bool over = false;
+  for (;; ++L) {
+    const int32_t q = hi - lo;
+    if (L >= max_levels) {
+      over = true;
+      break;
+    }
+    // the frontier's edges; a frontier of one chunk is then scanned already
+    int32_t u = 0, r0 = 0;
+    uint32_t d = 0u;
+    for (int32_t i = lo + threadIdx.x; i < hi; i += kSmallThreads) {
+      u = order[i];
+      r0 = a.R[u];
+      d += (uint32_t)(a.R[u + 1] - r0);
+    }
+    uint32_t mf;
+    uint32_t ex = block_excl_sum(d, st.red, &mf);
+    mu -= mf;
+    if (L > 0)
+      dir = next_direction(policy, dir == kPull, q, q_prev, mf, mu, a.m, a.n, alpha, beta);
+    if (dir == kPull) {
+      ++pulls;
+      const int32_t groups = (a.nwords + kPullWords - 1) / kPullWords;
+      for (int32_t g = wid; g < groups; g += kSmallThreads / 32) {
+        uint32_t vis[kPullWords];
+        int32_t v[kPullWords], e0[kPullWords], e1[kPullWords], uf[kPullWords];
+        bool act[kPullWords];
+#pragma unroll
+        for (int j = 0; j < kPullWords; ++j) {
+          const int32_t w = g * kPullWords + j;
+          vis[j] = w < a.nwords ? visited[w] : 0xFFFFFFFFu;
+          v[j] = w * 32 + lane;
+          act[j] = v[j] < a.n && !((vis[j] >> lane) & 1u);
+          uf[j] = act[j] ? a.first[v[j]] : -1;
+          e0[j] = act[j] ? a.R[v[j]] + 1 : 0;
+          e1[j] = act[j] ? a.R[v[j] + 1] : 0;
+        }
+#pragma unroll
+        for (int j = 0; j < kPullWords; ++j) {
+          if (uf[j] >= 0 && !(GR_IN(uf[j], a.n, 196) && dep[uf[j]] == L)) uf[j] = -1;
+          // a lane alone for two steps of four neighbours
+#pragma unroll 1
+          for (int k = 0; k < 2; ++k) {
+            if (uf[j] < 0 && e0[j] < e1[j]) {
+              int32_t x[4];
+#pragma unroll
+              for (int i = 0; i < 4; ++i) x[i] = e0[j] + i < e1[j] ? a.C[e0[j] + i] : -1;
+#pragma unroll
+              for (int i = 3; i >= 0; --i)
+                if (x[i] >= 0 && GR_IN(x[i], a.n, 197) && dep[x[i]] == L) uf[j] = x[i];
+              e0[j] += 4;
+            }
+          }
+          // then the warp on what is left of each long list
+          uint32_t longm = __ballot_sync(0xffffffffu, uf[j] < 0 && e0[j] < e1[j]);
+          while (longm) {
+            const int leader = __ffs(longm) - 1;
+            longm &= longm - 1u;
+            const int32_t b1 = __shfl_sync(0xffffffffu, e1[j], leader);
+            for (int32_t b = __shfl_sync(0xffffffffu, e0[j], leader); b < b1; b += 128) {
+              int32_t hit = -1;
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                const int32_t e = b + 32 * i + lane;
+                const int32_t x = e < b1 ? a.C[e] : -1;
+                if (x >= 0 && GR_IN(x, a.n, 198) && dep[x] == L) hit = x;
+              }
+              const uint32_t hb = __ballot_sync(0xffffffffu, hit >= 0);
+              if (hb) {
+                const int32_t x = __shfl_sync(0xffffffffu, hit, __ffs(hb) - 1);
+                if (lane == leader) uf[j] = x;
+                break;
+              }
+            }
+          }
+          const bool found = act[j] && uf[j] >= 0;
+          const uint32_t fm = __ballot_sync(0xffffffffu, found);
+          if (fm) {
+            if (lane == 0) visited[g * kPullWords + j] = vis[j] | fm;
+            if (found) {
+              dep[v[j]] = (uint16_t)(L + 1);
+              par[v[j]] = (uint16_t)uf[j];
+            }
+            small_append(&st.tail, order, found, v[j]);
+          }
+        }
+      }
+    } else {
+      for (int32_t c0 = lo; c0 < hi; c0 += kSmallThreads) {
+        const int32_t cnt = min(kSmallThreads, hi - c0);
+        uint32_t edges = mf;
+        if (q > kSmallThreads) {  // block-uniform: this chunk's own scan
+          d = 0u;
+          if ((int32_t)threadIdx.x < cnt) {
+            u = order[c0 + threadIdx.x];
+            r0 = a.R[u];
+            d = (uint32_t)(a.R[u + 1] - r0);
+          }
+          ex = block_excl_sum(d, st.red, &edges);
+        }
+        st.pre[threadIdx.x] = (int32_t)ex;
+        st.row[threadIdx.x] = r0;
+        st.u[threadIdx.x] = (uint16_t)u;
+        __syncthreads();
+        for (uint32_t e = threadIdx.x; e - lane < edges; e += kSmallThreads) {  // warp-uniform
+          bool won = false;
+          int32_t v = 0;
+          if (e < edges) {
+            int32_t k = 0, top = cnt - 1;  // last member whose edges begin at or before e
+            while (k < top) {
+              const int32_t mid = (k + top + 1) >> 1;
+              if (st.pre[mid] <= (int32_t)e) k = mid;
+              else top = mid - 1;
+            }
+            v = a.C[st.row[k] + ((int32_t)e - st.pre[k])];
+            if (GR_IN(v, a.n, 199)) {
+              const uint32_t bit = 1u << (v & 31);
+              won = !(visited[v >> 5] & bit) && !(atomicOr(&visited[v >> 5], bit) & bit);
+              if (won) {
+                dep[v] = (uint16_t)(L + 1);
+                par[v] = st.u[k];
+              }
+            }
+          }
+          __syncwarp();
+          small_append(&st.tail, order, won, v);
+        }
+        if (q > kSmallThreads) __syncthreads();  // the tables are reused
+      }
+    }
+    if (threadIdx.x == 0 && L < kTraceLevels) {
+      c->tr_dir[L] = dir;
+      c->tr_q[L] = q;
+      c->tr_mf[L] = mf;
+      c->tr_t[L] = globaltimer();
+    }
+    __syncthreads();
+    q_prev = q;
+    lo = hi;
+    hi = st.tail;
+    if (lo == hi) {
+      ++L;
+      break;
+    }
+  }
+  if (threadIdx.x == 0) {
+    c->level = L;
+    c->pull_levels = pulls;
+    c->error = over ? kDevOverflow : kDevOk;
+    c->done = 1;
+  }
+  for (int32_t v = threadIdx.x; v < a.n; v += kSmallThreads) {
+    depth[v] = dep[v] == 0xFFFF ? -1 : (int32_t)dep[v];
+    if (parent) parent[v] = par[v] == 0xFFFF ? -1 : (int32_t)par[v];
+  }
+}
+
 // ------------------------------------------------------ one-cluster driver
 // On graphs of small maximum degree (meshes) too large for the one-block
 // driver a BFS has thousands of levels
@@ -1665,6 +1889,18 @@ gr_status bfs_run(gr_graph *g, BfsWorkspace *ws, int32_t src, int32_t *depth, in
   int32_t max_levels = g->n + 1;
   if (o.max_iters > 0) max_levels = std::min(max_levels, o.max_iters);
   BfsArgs a = make_args(g, ws, do_bitmap);
+  // small graphs in one block; a caller who asks for blocks per SM, or for
+  // pulls from the first level on, gets the grid
+  if (mode == GR_MODE_PERSISTENT && !a.low_degree && o.block == 0 && policy != GR_DIR_PULL &&
+      g->n <= kSmallMaxN && g->m <= (policy == GR_DIR_PUSH ? kSmallMaxPushM : kSmallMaxM)) {
+    const size_t bytes = small_smem_bytes(g->n);
+    GR_CUDA(cudaFuncSetAttribute(k_bfs_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)bytes));
+    k_bfs_small<<<1, kSmallThreads, bytes, s>>>(a, src, depth, parent, policy, alpha, beta,
+                                                max_levels, (g->symmetric && do_bitmap) ? 1 : 0);
+    GR_CUDA(cudaGetLastError());
+    return GR_OK;
+  }
   k_bfs_init<<<g->num_sms * 8, 256, 0, s>>>(a, src, depth, parent, policy, alpha, beta,
                                             max_levels, (g->symmetric && do_bitmap) ? 1 : 0);
   GR_CUDA(cudaGetLastError());

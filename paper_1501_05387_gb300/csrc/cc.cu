@@ -27,9 +27,6 @@
 // hooking under the smaller root makes every root its component's smallest
 // id whatever the order. For a directed CSR every arc hooks in one sweep,
 // giving weakly connected components (an arc is not visible from its head).
-#include <algorithm>
-#include <vector>
-
 #include "advance.cuh"
 
 namespace gr {
@@ -41,7 +38,7 @@ constexpr int kCcFrontierCap = 1024;
 
 struct CcWorkspace {
   DevMem counter;  // [0] components, [1] scratch; [2..3] packed frontier counter
-  DevMem q, sc, picks;
+  DevMem q, sc, skip;
 };
 
 void free_cc(CcWorkspace *ws) { delete ws; }
@@ -113,11 +110,29 @@ __global__ void k_cc_sample(const int32_t *R, const int32_t *C, int32_t n, int32
   }
 }
 
-// Roots (labels after compression) of kCcPicks vertices spread over the ids
-// by a multiplicative hash.
-__global__ void k_cc_pick(const int32_t *label, int32_t n, int32_t *picks) {
-  const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < kCcPicks) picks[i] = label[(int32_t)(((unsigned long long)i * 2654435761ull) % n)];
+// The component to skip: the root (label after compression) that most of
+// kCcPicks vertices have, spread over the ids by a multiplicative hash; the
+// smallest of equals. One block, a vertex per thread, each counting its root
+// among all: 3 us on the device, where fetching the roots to sort them on the
+// host stopped the stream for 60.
+__global__ void __launch_bounds__(kCcPicks) k_cc_pick(const int32_t *label, int32_t n,
+                                                      int32_t *skip) {
+  __shared__ int4 s_root[kCcPicks / 4];
+  __shared__ unsigned long long s_best;
+  const int32_t root = label[(int32_t)(((unsigned long long)threadIdx.x * 2654435761ull) % n)];
+  ((int32_t *)s_root)[threadIdx.x] = root;
+  if (threadIdx.x == 0) s_best = 0ull;
+  __syncthreads();
+  uint32_t same = 0;
+#pragma unroll 4
+  for (int i = 0; i < kCcPicks / 4; ++i) {
+    const int4 r = s_root[i];
+    same += (r.x == root) + (r.y == root) + (r.z == root) + (r.w == root);
+  }
+  const uint32_t most = __reduce_max_sync(0xffffffffu, same);
+  if (same == most) atomicMax(&s_best, ((unsigned long long)same << 32) | (0x7FFFFFFFu - (uint32_t)root));
+  __syncthreads();
+  if (threadIdx.x == 0) *skip = (int32_t)(0x7FFFFFFFu - (uint32_t)(s_best & 0xFFFFFFFFull));
 }
 
 // The vertices outside component `skip` that have edges, with their
@@ -125,10 +140,11 @@ __global__ void k_cc_pick(const int32_t *label, int32_t n, int32_t *picks) {
 // the frontier whose edges the last hooking pass visits.
 __global__ void __launch_bounds__(kCcThreads) k_cc_rest_frontier(const int32_t *R,
                                                                   const int32_t *label, int32_t n,
-                                                                  int32_t skip, int32_t *Q,
+                                                                  const int32_t *skip_p, int32_t *Q,
                                                                   int32_t *S,
                                                                   unsigned long long *packed) {
   __shared__ ScannedBuf<kCcFrontierCap> buf;
+  const int32_t skip = *skip_p;
   if (threadIdx.x == 0) buf.cnt = 0;
   __syncthreads();
   constexpr int PER = kCcFrontierCap / kCcThreads;
@@ -149,20 +165,15 @@ __global__ void __launch_bounds__(kCcThreads) k_cc_rest_frontier(const int32_t *
   }
 }
 
-// S[q] = the frontier's edge total (the advance reads it as the scan's end).
-__global__ void k_cc_close(const unsigned long long *packed, int32_t *S) {
-  const unsigned long long p = *packed;
-  S[(int32_t)(p & 0xFFFFFFFFull)] = (int32_t)(p >> 32);
-}
-
 // Hook every edge of the frontier Q (size and scan from k_cc_rest_frontier).
 __global__ void __launch_bounds__(kCcThreads) k_cc_hook_rest(const int32_t *R, const int32_t *C,
                                                               int32_t n, int32_t *label,
                                                               const int32_t *Q, const int32_t *S,
                                                               const unsigned long long *packed) {
   HookF f{label, 0, n};
-  const int32_t q = (int32_t)(*packed & 0xFFFFFFFFull);
-  lb_advance<kCcThreads, kCcItems, 0>(R, C, Q, q, S, f, nullptr, nullptr, nullptr, nullptr);
+  const unsigned long long p = *packed;
+  lb_advance<kCcThreads, kCcItems, 0>(R, C, Q, (int32_t)(p & 0xFFFFFFFFull), S, (int32_t)(p >> 32),
+                                      f, nullptr, nullptr, nullptr, nullptr);
 }
 
 __global__ void __launch_bounds__(kCcThreads) k_cc_hook(const int32_t *R, const int32_t *C,
@@ -171,7 +182,7 @@ __global__ void __launch_bounds__(kCcThreads) k_cc_hook(const int32_t *R, const 
   HookF f{label, only_lower, n};
   // every edge is settled in its visit: the edge frontier it would filter
   // into stays empty, so the advance appends nothing
-  lb_advance<kCcThreads, kCcItems, 0>(R, C, nullptr, n, R, f, nullptr, nullptr, nullptr,
+  lb_advance<kCcThreads, kCcItems, 0>(R, C, nullptr, n, R, R[n], f, nullptr, nullptr, nullptr,
                                       nullptr);
 }
 
@@ -192,7 +203,7 @@ __global__ void k_cc_jump(int32_t *label, int32_t n, int32_t *num_roots) {
 
 size_t cc_ws_bytes(const gr_graph *g) {
   return sizeof(int32_t) * 4 + sizeof(int32_t) * (2 * (size_t)g->n + 3) +
-         sizeof(int32_t) * kCcPicks;
+         sizeof(int32_t);
 }
 
 gr_status cc_ws_create(gr_graph *g, CcWorkspace **out) {
@@ -201,7 +212,7 @@ gr_status cc_ws_create(gr_graph *g, CcWorkspace **out) {
   if (g->symmetric) {
     GR_TRY(ws->q.alloc(sizeof(int32_t) * ((size_t)g->n + 1), "CC frontier"));
     GR_TRY(ws->sc.alloc(sizeof(int32_t) * ((size_t)g->n + 2), "CC frontier degree scan"));
-    GR_TRY(ws->picks.alloc(sizeof(int32_t) * kCcPicks, "CC root sample"));
+    GR_TRY(ws->skip.alloc(sizeof(int32_t), "CC skipped component"));
   }
   *out = ws.release();
   return GR_OK;
@@ -220,27 +231,11 @@ gr_status cc_run(gr_graph *g, CcWorkspace *ws, int32_t *label, cudaStream_t s) {
   } else {
     k_cc_sample<<<grid, 256, 0, s>>>(R, C, g->n, label);
     k_cc_jump<<<grid, 256, 0, s>>>(label, g->n, cnt + 1);  // compress (count unused)
-    k_cc_pick<<<(kCcPicks + 255) / 256, 256, 0, s>>>(label, g->n, ws->picks.as<int32_t>());
-    GR_CUDA(cudaGetLastError());
-    std::vector<int32_t> picks(kCcPicks);
-    GR_CUDA(cudaMemcpyAsync(picks.data(), ws->picks.p, sizeof(int32_t) * kCcPicks,
-                            cudaMemcpyDeviceToHost, s));
-    GR_CUDA(cudaStreamSynchronize(s));
-    std::sort(picks.begin(), picks.end());
-    int32_t skip = picks[0], best = 0;
-    for (size_t i = 0; i < picks.size();) {
-      size_t j = i;
-      while (j < picks.size() && picks[j] == picks[i]) ++j;
-      if ((int32_t)(j - i) > best) {
-        best = (int32_t)(j - i);
-        skip = picks[i];
-      }
-      i = j;
-    }
+    int32_t *skip = ws->skip.as<int32_t>();
+    k_cc_pick<<<1, kCcPicks, 0, s>>>(label, g->n, skip);
     unsigned long long *packed = ws->counter.as<unsigned long long>() + 1;
     int32_t *Q = ws->q.as<int32_t>(), *S = ws->sc.as<int32_t>();
     k_cc_rest_frontier<<<grid, kCcThreads, 0, s>>>(R, label, g->n, skip, Q, S, packed);
-    k_cc_close<<<1, 1, 0, s>>>(packed, S);
     k_cc_hook_rest<<<g->num_sms * 4, kCcThreads, 0, s>>>(R, C, g->n, label, Q, S, packed);
   }
   k_cc_jump<<<grid, 256, 0, s>>>(label, g->n, cnt);

@@ -185,6 +185,8 @@ gr_status sssp_ws_create(gr_graph *g, cudaStream_t s, SsspWorkspace **out, int32
 size_t sssp_ws_bytes(const gr_graph *g, int32_t lanes = 1);
 // most sources one batched SSSP run on this graph may take
 int32_t sssp_batch_max_lanes(const gr_graph *g);
+// blocks per SM the persistent SSSP kernel starts out with on m entries
+int32_t sssp_prior_blocks(int64_t m);
 // k searches (k <= the workspace's lanes) into dist[k][n] on the device
 gr_status sssp_batch_run(gr_graph *g, SsspWorkspace *ws, const int32_t *h_srcs, int32_t k,
                          uint32_t *dist, const gr_opts &o, cudaStream_t s);

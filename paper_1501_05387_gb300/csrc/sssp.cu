@@ -1344,6 +1344,11 @@ gr_status sssp_check(const gr_graph *g, int32_t src, const gr_opts &o) {
   return GR_OK;
 }
 
+// Blocks per SM of a search over m entries, measured in tune_prior (0: all).
+int32_t sssp_prior_blocks(int64_t m) {
+  return m < 150'000 ? 1 : m < 4'000'000 ? 3 : m < 16'000'000 ? 4 : 0;
+}
+
 static unsigned long long sssp_delta_of(const gr_graph *g, const gr_opts &o) {
   return o.delta == UINT32_MAX ? (1ull << 40) : (o.delta ? o.delta : g->sssp_delta);
 }
@@ -1439,10 +1444,12 @@ gr_status sssp_batch_run(gr_graph *g, SsspWorkspace *ws, const int32_t *h_srcs, 
   if (mode != GR_MODE_PERSISTENT) mode = GR_MODE_LAUNCH;
   gr_opts ob = o;
   // k lanes carry k times the frontier of one search per iteration: where
-  // the single search was tuned to one block per SM, two do better (16
-  // sources on the 4096^2 mesh: 282 ms at 2 blocks per SM, 321 at 1, 297 at
-  // 3, 335 at 5)
-  if (k > 1 && ob.block == 0 && g->tuned_sssp_blocks_per_sm == 1) ob.block = 2;
+  // one search runs on few blocks a batch takes more (16 sources on the 4096^2
+  // mesh: 282 ms at 2 blocks per SM, 321 at 1, 297 at 3, 335 at 5)
+  if (k > 1 && ob.block == 0 && g->tuned_sssp_blocks_per_sm > 0) {
+    const int32_t more = a.low_degree ? 2 : sssp_prior_blocks((int64_t)k * g->m);
+    ob.block = more == 0 ? kSsspBlocksPerSm : std::max(more, g->tuned_sssp_blocks_per_sm);
+  }
   return sssp_drive(g, ws, a, srcs, dist, nullptr, mode, ob, s);
 }
 

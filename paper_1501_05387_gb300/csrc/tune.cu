@@ -44,7 +44,16 @@ void tune_prior(gr_graph *g) {
       g->sssp_delta = (uint32_t)std::max(1.0, std::min(6.0 * g->mean_weight, 4.0e9));
   } else {
     g->tuned_direction = GR_DIR_AUTO;
-    g->tuned_blocks_per_sm = 0;  // all resident blocks
+    // Small graphs are bound by the grid barrier, whose cost grows with the
+    // blocks that meet at it. BFS at 1, 2, 3, 4 and 6 blocks per SM: R-MAT
+    // 2^12 (0.1 M entries) 42, 48, 48, 49, 55 us; 2^16 (1.8 M) 48, 54, 56, 59,
+    // 70; 2^18 (7.6 M) 87, 77, 78, 71, 77; 2^21 (64 M) 234, 158, 137, 123, 126;
+    // 2^22 (128 M) 426, 260, 211, 188, 180.
+    g->tuned_blocks_per_sm = g->m < 4'000'000 ? 1 : g->m < 96'000'000 ? 4 : 0;
+    // SSSP at 1 to 5: 2^12 101, 115, 123, 126, 141 us; 2^14 (0.4 M) 158, 143,
+    // 133, 141, 151; 2^16 195, 181, 181, 186, 198; 2^18 422, 292, 262, 243, 251;
+    // 2^20 (31 M) 1552, 914, 726, 629, 607.
+    g->tuned_sssp_blocks_per_sm = sssp_prior_blocks(g->m);
     // skewed graphs reach most vertices in a few dense relaxations: the
     // persistent kernel, and buckets wide enough not to repeat them (R-MAT
     // 2^21, pushed: 2.28 ms in the graph loop at two mean weights a bucket,
