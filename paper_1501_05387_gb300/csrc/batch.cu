@@ -254,6 +254,13 @@ __device__ __forceinline__ unsigned long long joined(const MbArgs &a, int32_t v)
   return 1ull | ((unsigned long long)(uint32_t)(a.R[v + 1] - a.R[v]) << 32);
 }
 
+// A warp's window of a lane-wise gather (below).
+struct LaneBuf {
+  int32_t u[32];
+  uint32_t bits[2][32];
+  uint8_t lane_of[2][32];
+};
+
 // Shared memory of the level forms (one at a time).
 union MbSmem {
   struct {
@@ -263,6 +270,7 @@ union MbSmem {
   struct {
     int32_t off[kMbChunk + 1];
     unsigned long long U[kMbChunk + 1];
+    LaneBuf lanes[kMbThreads / 32];
   } fwd;
   struct {
     int32_t off[kMbChunk + 1];
@@ -393,19 +401,143 @@ __device__ void mb_pull_level(const MbArgs &a, MbSmem &sm, int32_t *s_red8, int3
   if ((threadIdx.x & 31) == 0 && new_vertices) atomicAdd(counter, new_vertices);
 }
 
+// ------------------------------------------------------- lane-wise gathers
+// BC adds, for an edge (v, u) and every lane s set in its `bits`, one value of
+// u's row of 64 to v's sum of lane s. Few lanes are set, and they are much the
+// same along v's row (the lanes whose level v is on): R-MAT 2^17, 64 sources,
+// busiest level: 41.8 M (edge, lane) pairs on 2.9 M edges, 7.9 of 32 lanes in
+// a half row that has any. With lane s of a warp serving source s, edge after
+// edge, that is 5.3 M half-row adds of which three quarters do nothing, and
+// an FP64 add holds the SM's pipe for 16 cycles whatever its lanes.
+//
+// Here a warp takes a window of 32 edges, packs those of one vertex that have
+// bits into shared memory, and deals its threads to the vertex's lanes of a
+// half row: with a lanes in it, thread t serves the (t mod a)-th of them and
+// every (32 / a)-th edge. The partial sums of a lane meet in the atomics that
+// add them to v's row (done in L2, not in the FP64 pipe).
+// What a warp is summing: vertex `owner`, lanes `mask`; per half row the
+// thread's source, its first edge and edge step (step 0: none), its sum.
+template <class T>
+struct LaneSums {
+  int32_t owner;
+  uint32_t mask[2];
+  int32_t src[2], first[2], step[2];
+  T acc[2];
+};
+
+template <class T>
+__device__ __forceinline__ void lane_deal(LaneSums<T> &s, LaneBuf &b, int32_t owner, uint32_t m0,
+                                          uint32_t m1) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t lt = (1u << lane) - 1u;
+  s.owner = owner;
+  s.mask[0] = m0;
+  s.mask[1] = m1;
+  if ((m0 >> lane) & 1u) b.lane_of[0][__popc(m0 & lt)] = (uint8_t)lane;
+  if ((m1 >> lane) & 1u) b.lane_of[1][__popc(m1 & lt)] = (uint8_t)(lane + 32);
+  __syncwarp();
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int32_t a = __popc(s.mask[h]);
+    // 32 / a and lane / a, exact for these sizes
+    const float r = __frcp_rn((float)max(a, 1));
+    const int32_t groups = (int32_t)(32.5f * r), g = (int32_t)(((float)lane + 0.5f) * r);
+    s.src[h] = a ? b.lane_of[h][lane - g * a] : 0;
+    s.first[h] = g < groups ? g : 32;  // a left-over thread: no edge
+    s.step[h] = a ? groups : 0;
+    s.acc[h] = T(0);
+  }
+}
+
+// One window: lane i's edge (owner, u) with `bits` (0: no edge) of v's lanes
+// `of` (the same for all of v's edges; with OWN_MASK it is what the window's
+// edges have). add(x, y) adds, flush(s) takes the sums of an owner and mask.
+template <bool OWN_MASK, class T, class ADD, class FLUSH>
+__device__ __forceinline__ void lane_window(LaneSums<T> &s, LaneBuf &b, int32_t owner, int32_t u,
+                                            unsigned long long bits, unsigned long long of,
+                                            const T *val, ADD add, FLUSH flush) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t lt = (1u << lane) - 1u;
+  uint32_t act = __ballot_sync(0xffffffffu, bits != 0ull);
+  while (act) {  // warp-uniform
+    const int j0 = __ffs(act) - 1;
+    const int32_t ov = __shfl_sync(0xffffffffu, owner, j0);
+    const uint32_t seg = __ballot_sync(0xffffffffu, owner == ov) & act;
+    act &= ~seg;
+    const bool mine = (seg >> lane) & 1u;
+    uint32_t m0, m1;
+    if (OWN_MASK) {
+      m0 = __reduce_or_sync(0xffffffffu, mine ? (uint32_t)bits : 0u);
+      m1 = __reduce_or_sync(0xffffffffu, mine ? (uint32_t)(bits >> 32) : 0u);
+    } else {
+      m0 = __shfl_sync(0xffffffffu, (uint32_t)of, j0);
+      m1 = __shfl_sync(0xffffffffu, (uint32_t)(of >> 32), j0);
+    }
+    __syncwarp();  // the buffer's last readers are done
+    if (ov != s.owner || m0 != s.mask[0] || m1 != s.mask[1]) {
+      if (s.owner >= 0) flush(s);
+      lane_deal(s, b, ov, m0, m1);
+    }
+    if (mine) {
+      const int k = __popc(seg & lt);
+      b.u[k] = u;
+      b.bits[0][k] = (uint32_t)bits;
+      b.bits[1][k] = (uint32_t)(bits >> 32);
+    }
+    __syncwarp();
+    const int cnt = __popc(seg);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int step = s.step[h];
+      if (!step) continue;  // warp-uniform
+      const int bit = s.src[h] & 31;
+      for (int base = 0; base < cnt; base += 4 * step) {
+        T x[4];
+        bool has[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int j = base + k * step + s.first[h];
+          has[k] = j < cnt && ((b.bits[h][j & 31] >> bit) & 1u);
+          x[k] = has[k] ? val[(int64_t)b.u[j & 31] * 64 + s.src[h]] : T(0);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (base + k * step < cnt && has[k]) s.acc[h] = add(s.acc[h], x[k]);
+      }
+    }
+  }
+}
+
+// The windows of a chunk's ne edges that this warp takes: [*w0, *w1), together.
+__device__ __forceinline__ void chunk_windows(int32_t ne, int32_t *w0, int32_t *w1) {
+  const int32_t windows = (ne + 31) >> 5, wid = threadIdx.x >> 5;
+  *w0 = wid * windows / (kMbThreads / 32);
+  *w1 = (wid + 1) * windows / (kMbThreads / 32);
+}
+
 // A BC forward pull level: nxt[v] = OR over edges (v,u) of cur[u] &
 // ~seen(v), seen(v) = visit[v] | cur[v], and the path counts of the newly
 // reached lanes. The vertex loader of each chunk folds cur into visit
 // (idempotent, so chunks sharing a vertex may both do it).
 template <int SK>
-__device__ void mb_forward_level(const MbArgs &a, MbSmem &sm, int32_t *s_red8,
-                                 const unsigned long long *cur, unsigned long long *nxt,
-                                 unsigned long long *counter, bool &ovf) {
+__device__ void mb_forward_level(const MbArgs &a, MbSmem &sm, const unsigned long long *cur,
+                                 unsigned long long *nxt, unsigned long long *counter, bool &ovf) {
   using T = CountT<SK>;
   const int lane = threadIdx.x & 31;
   const long long total = (long long)a.n + a.R[a.n];
   const long long nchunks = (total + kMbChunk - 1) / kMbChunk;
   unsigned long long new_vertices = 0;
+  T *const sigma = (T *)a.sigma;
+  auto add = [&](T x, T y) { return count_add(x, y, ovf); };
+  LaneBuf &buf = sm.fwd.lanes[threadIdx.x >> 5];
+  auto flush = [&](const LaneSums<T> &s) {
+    T *sg = sigma + (int64_t)s.owner * 64;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (s.acc[h] != T(0)) count_atomic_add(sg + s.src[h], s.acc[h], ovf);
+    if (lane == 0 && !atomicOr(nxt + s.owner, ((unsigned long long)s.mask[1] << 32) | s.mask[0]))
+      new_vertices += joined(a, s.owner);
+  };
   for (long long chunk = blockIdx.x; chunk < nchunks; chunk += gridDim.x) {
     const long long d0 = chunk * kMbChunk;
     const long long d1 = min(d0 + kMbChunk, total);
@@ -422,8 +554,12 @@ __device__ void mb_forward_level(const MbArgs &a, MbSmem &sm, int32_t *s_red8,
     }
     __syncthreads();
     const int32_t ne = (int32_t)(j1 - j0);
-    for (int32_t kb = 0; kb < ne; kb += kMbThreads) {
-      const int32_t kk = kb + threadIdx.x;
+    int32_t w0, w1;
+    chunk_windows(ne, &w0, &w1);
+    LaneSums<T> sums = {};
+    sums.owner = -1;
+    for (int32_t w = w0; w < w1; ++w) {
+      const int32_t kk = w * 32 + lane;
       int32_t owner = -1, u = 0;
       unsigned long long bits = 0ull;
       if (kk < ne) {
@@ -442,45 +578,10 @@ __device__ void mb_forward_level(const MbArgs &a, MbSmem &sm, int32_t *s_red8,
           bits = GR_IN(u, a.n, 203) ? (cur[u] & U) : 0ull;
         }
       }
-      // the warp serves the edges with bits one at a time: lane l handles
-      // BFS lanes l and l + 32 of the predecessor's 64 path counts; a half
-      // with no bits set is skipped by the whole warp
-      T *const sigma = (T *)a.sigma;
-      uint32_t act = __ballot_sync(0xffffffffu, bits != 0ull);
-      int32_t cur_owner = -1;
-      unsigned long long orbits = 0ull;
-      T acc0 = T(0), acc1 = T(0);
-      while (act) {
-        const int j = __ffs(act) - 1;
-        act &= act - 1u;
-        const int32_t ov = __shfl_sync(0xffffffffu, owner, j);
-        const int32_t uj = __shfl_sync(0xffffffffu, u, j);
-        const unsigned long long bj = shfl_u64(bits, j);
-        if (ov != cur_owner) {
-          if (cur_owner >= 0) {
-            T *sg = sigma + (int64_t)cur_owner * 64;
-            if ((orbits >> lane) & 1ull) count_atomic_add(sg + lane, acc0, ovf);
-            if ((orbits >> (lane + 32)) & 1ull) count_atomic_add(sg + lane + 32, acc1, ovf);
-            if (lane == 0 && !atomicOr(nxt + cur_owner, orbits))
-              new_vertices += joined(a, cur_owner);
-          }
-          cur_owner = ov;
-          orbits = 0ull;
-          acc0 = acc1 = T(0);
-        }
-        orbits |= bj;
-        const T *su = sigma + (int64_t)uj * 64;
-        if ((uint32_t)bj && ((bj >> lane) & 1ull)) acc0 = count_add(acc0, su[lane], ovf);
-        if ((bj >> 32) && ((bj >> (lane + 32)) & 1ull))
-          acc1 = count_add(acc1, su[lane + 32], ovf);
-      }
-      if (cur_owner >= 0) {
-        T *sg = sigma + (int64_t)cur_owner * 64;
-        if ((orbits >> lane) & 1ull) count_atomic_add(sg + lane, acc0, ovf);
-        if ((orbits >> (lane + 32)) & 1ull) count_atomic_add(sg + lane + 32, acc1, ovf);
-        if (lane == 0 && !atomicOr(nxt + cur_owner, orbits)) new_vertices += joined(a, cur_owner);
-      }
+      __syncwarp();
+      lane_window<true>(sums, buf, owner, u, bits, 0ull, sigma, add, flush);
     }
+    if (sums.owner >= 0) flush(sums);
     __syncthreads();
   }
   for (int o = 16; o > 0; o >>= 1) new_vertices += __shfl_xor_sync(0xffffffffu, new_vertices, o);
@@ -633,7 +734,7 @@ __device__ void mb_depth_pass(const MbArgs &a, int32_t levels) {
 // for 64 sources on R-MAT s23 against 8.25 ms at 6), BC at 6 (116 ms
 // against 118 ms at 5).
 template <int SK>
-constexpr int mb_do_blocks_per_sm() { return SK == kSigNone ? 5 : 6; }
+constexpr int mb_do_blocks_per_sm() { return SK == kSigNone ? 5 : 4; }
 
 // The forward levels in one cooperative kernel. Every block runs every
 // level; levels are separated by one bounded grid barrier, after which each
@@ -727,7 +828,7 @@ __global__ void __launch_bounds__(kMbThreads, mb_do_blocks_per_sm<SK>()) k_mb_do
     } else if (SK == kSigNone) {
       mb_pull_level(a, sm, s_red8, L, cur, nxt, counter);
     } else {
-      mb_forward_level<SK == kSigNone ? kSigU64 : SK>(a, sm, s_red8, cur, nxt, counter, ovf);
+      mb_forward_level<SK == kSigNone ? kSigU64 : SK>(a, sm, cur, nxt, counter, ovf);
     }
     unsigned long long pk = 0ull;
     if (gridDim.x > kFlatBarrierBlocks) {
@@ -807,7 +908,7 @@ __global__ void k_list_bounds(const int32_t *S, const unsigned long long *fpacke
 
 // resident blocks per SM of the backward pass (its carveout is fitted to
 // them, the rest of the shared-memory array left to L1 for the children's rows)
-constexpr int kBcBackBlocksPerSm = 6;
+constexpr int kBcBackBlocksPerSm = 4;
 
 // Backward level L: q[v][s] += q[w][s] over edges (v, w) with v in lane s's
 // level L and w in its level L+1 (w's q is final: level L+1 was finished).
@@ -815,7 +916,7 @@ constexpr int kBcBackBlocksPerSm = 6;
 // visited, so the whole backward pass reads every edge about once instead of
 // once per level.
 
-__global__ void __launch_bounds__(kMbThreads) k_bc_backward(BcBackArgs a, const int32_t *Q,
+__global__ void __launch_bounds__(kMbThreads, kBcBackBlocksPerSm) k_bc_backward(BcBackArgs a, const int32_t *Q,
                                                              const int32_t *S,
                                                              const unsigned long long *fpacked,
                                                              const int32_t *cb) {
@@ -823,13 +924,21 @@ __global__ void __launch_bounds__(kMbThreads) k_bc_backward(BcBackArgs a, const 
   __shared__ int32_t s_row[kMbChunk + 1];
   __shared__ int32_t s_v[kMbChunk + 1];
   __shared__ unsigned long long s_A[kMbChunk + 1];
-  __shared__ int32_t s_red8[kMbThreads / 32];
+  __shared__ LaneBuf s_lanes[kMbThreads / 32];
   const int lane = threadIdx.x & 31;
   const unsigned long long fp = *fpacked;
   const int32_t q = (int32_t)(fp & 0xFFFFFFFFull);
   const int32_t qe = (int32_t)(fp >> 32);
   const long long total = (long long)q + qe;
   const long long nchunks = (total + kMbChunk - 1) / kMbChunk;
+  auto add = [](double x, double y) { return x + y; };
+  LaneBuf &buf = s_lanes[threadIdx.x >> 5];
+  auto flush = [&](const LaneSums<double> &s) {
+    double *qv = a.q + (int64_t)s.owner * 64;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (s.acc[h] != 0.0) atomicAdd(qv + s.src[h], s.acc[h]);
+  };
   for (long long chunk = blockIdx.x; chunk < nchunks; chunk += gridDim.x) {
     const long long d0 = chunk * kMbChunk;
     const long long d1 = min(d0 + kMbChunk, total);
@@ -847,10 +956,14 @@ __global__ void __launch_bounds__(kMbThreads) k_bc_backward(BcBackArgs a, const 
     }
     __syncthreads();
     const int32_t ne = (int32_t)(j1 - j0);
-    for (int32_t kb = 0; kb < ne; kb += kMbThreads) {
-      const int32_t k = kb + threadIdx.x;
+    int32_t w0, w1;
+    chunk_windows(ne, &w0, &w1);
+    LaneSums<double> sums = {};
+    sums.owner = -1;
+    for (int32_t win = w0; win < w1; ++win) {
+      const int32_t k = win * 32 + lane;
       int32_t owner = -1, w = 0;
-      unsigned long long bits = 0ull;
+      unsigned long long bits = 0ull, A = 0ull;
       if (k < ne) {
         const int32_t er = (int32_t)(j0 + k);
         int32_t lo = 0, hi = nv - 1;
@@ -861,44 +974,16 @@ __global__ void __launch_bounds__(kMbThreads) k_bc_backward(BcBackArgs a, const 
         }
         owner = s_v[lo];
         const long long e = (long long)s_row[lo] + (er - s_off[lo]);
-        const unsigned long long A = s_A[lo];
+        A = s_A[lo];
         if (owner >= 0 && A && GR_IN(e, a.m, 222)) {
           w = a.C[e];
           bits = GR_IN(w, a.n, 223) ? (A & a.lw[w]) : 0ull;
         }
       }
-      uint32_t act = __ballot_sync(0xffffffffu, bits != 0ull);
-      int32_t cur_owner = -1;
-      unsigned long long orbits = 0ull;
-      double acc0 = 0.0, acc1 = 0.0;
-      while (act) {
-        const int j = __ffs(act) - 1;
-        act &= act - 1u;
-        const int32_t ov = __shfl_sync(0xffffffffu, owner, j);
-        const int32_t wj = __shfl_sync(0xffffffffu, w, j);
-        const unsigned long long bj = shfl_u64(bits, j);
-        if (ov != cur_owner) {
-          if (cur_owner >= 0) {
-            double *qv = a.q + (int64_t)cur_owner * 64;
-            if ((orbits >> lane) & 1ull) atomicAdd(qv + lane, acc0);
-            if ((orbits >> (lane + 32)) & 1ull) atomicAdd(qv + lane + 32, acc1);
-          }
-          cur_owner = ov;
-          orbits = 0ull;
-          acc0 = acc1 = 0.0;
-        }
-        orbits |= bj;
-        const double *qw = a.q + (int64_t)wj * 64;
-        // a half with no bits set costs the warp no FP64 add
-        if ((uint32_t)bj && ((bj >> lane) & 1ull)) acc0 += qw[lane];
-        if ((bj >> 32) && ((bj >> (lane + 32)) & 1ull)) acc1 += qw[lane + 32];
-      }
-      if (cur_owner >= 0) {
-        double *qv = a.q + (int64_t)cur_owner * 64;
-        if ((orbits >> lane) & 1ull) atomicAdd(qv + lane, acc0);
-        if ((orbits >> (lane + 32)) & 1ull) atomicAdd(qv + lane + 32, acc1);
-      }
+      __syncwarp();
+      lane_window<false>(sums, buf, owner, w, bits, A, (const double *)a.q, add, flush);
     }
+    if (sums.owner >= 0) flush(sums);
     __syncthreads();
   }
 }

@@ -17,8 +17,9 @@
 // smallest vertex id, which is the canonical label.
 //
 // Symmetric graphs store each undirected edge twice, so most edges need no
-// visit at all: the sampling form of the hooking sweep first hooks every
-// vertex to its first kCcSample neighbours and compresses, which on graphs
+// visit at all: the sampling form of the hooking sweep starts every vertex
+// under its first neighbour (where that has the smaller id: no cycle, and no
+// atomic), hooks it to the second and compresses, which on graphs
 // with one giant component already places most vertices in it; the
 // component that most of a fixed sample of vertices lies in is then
 // skipped, and only the vertices outside it hook all their edges (an edge
@@ -32,7 +33,6 @@
 namespace gr {
 
 constexpr int kCcThreads = 256, kCcItems = 8;
-constexpr int kCcSample = 2;    // neighbours per vertex hooked before the skip
 constexpr int kCcPicks = 1024;  // vertices whose roots choose the skipped component
 constexpr int kCcFrontierCap = 1024;
 
@@ -47,10 +47,13 @@ GR_GUARD_REPORTER(guard_report_cc)
 
 namespace {
 
-__global__ void k_cc_init(int32_t *label, int32_t n) {
+// first (may be null): the vertices' first neighbours, -1 where there is none
+__global__ void k_cc_init(int32_t *label, const int32_t *first, int32_t n) {
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
-       v += (int64_t)gridDim.x * blockDim.x)
-    label[v] = (int32_t)v;
+       v += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t u = first ? first[v] : -1;
+    label[v] = u >= 0 && u < v ? u : (int32_t)v;
+  }
 }
 
 // root of x with path halving (pointers only ever decrease)
@@ -97,40 +100,67 @@ struct HookF {
   }
 };
 
-// Each vertex hooks to its first kCcSample neighbours.
-__global__ void k_cc_sample(const int32_t *R, const int32_t *C, int32_t n, int32_t *label) {
+// Each vertex hooks to its second neighbour, and to its first where
+// k_cc_init could not start it there. The trees are shallow by then and most
+// pairs share one already: R-MAT 2^22 143 us when all vertices hooked both
+// neighbours from themselves on, their roots' CASes in each other's way.
+__global__ void k_cc_sample(const int32_t *R, const int32_t *C, const int32_t *first, int32_t n,
+                            int32_t *label) {
   for (int64_t vv = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; vv < n;
        vv += (int64_t)gridDim.x * blockDim.x) {
     const int32_t v = (int32_t)vv;
-    const int32_t r0 = R[v], r1 = min(R[v + 1], r0 + kCcSample);
-    for (int32_t e = r0; e < r1; ++e) {
-      const int32_t u = C[e];
-      if (GR_IN(u, n, 403)) hook(label, v, u);
+    const int32_t u = first[v];
+    if (u < 0) continue;
+    const int32_t r = R[v] + 1;
+    if (u > v) hook(label, v, u);
+    if (r < R[v + 1]) {
+      const int32_t x = C[r];
+      if (GR_IN(x, n, 403)) hook(label, v, x);
     }
   }
 }
 
 // The component to skip: the root (label after compression) that most of
 // kCcPicks vertices have, spread over the ids by a multiplicative hash; the
-// smallest of equals. One block, a vertex per thread, each counting its root
-// among all: 3 us on the device, where fetching the roots to sort them on the
-// host stopped the stream for 60.
+// smallest of equals. One block, a vertex per thread; the roots are counted
+// warp by warp in a hash table in shared memory. Fetching them to sort them
+// on the host stopped the stream for 60 us; comparing each with all took 18.
 __global__ void __launch_bounds__(kCcPicks) k_cc_pick(const int32_t *label, int32_t n,
                                                       int32_t *skip) {
-  __shared__ int4 s_root[kCcPicks / 4];
+  constexpr uint32_t kSlots = 2 * kCcPicks;
+  __shared__ int32_t s_root[kSlots];
+  __shared__ uint32_t s_count[kSlots];
   __shared__ unsigned long long s_best;
-  const int32_t root = label[(int32_t)(((unsigned long long)threadIdx.x * 2654435761ull) % n)];
-  ((int32_t *)s_root)[threadIdx.x] = root;
-  if (threadIdx.x == 0) s_best = 0ull;
-  __syncthreads();
-  uint32_t same = 0;
-#pragma unroll 4
-  for (int i = 0; i < kCcPicks / 4; ++i) {
-    const int4 r = s_root[i];
-    same += (r.x == root) + (r.y == root) + (r.z == root) + (r.w == root);
+  for (uint32_t i = threadIdx.x; i < kSlots; i += kCcPicks) {
+    s_root[i] = -1;
+    s_count[i] = 0u;
   }
-  const uint32_t most = __reduce_max_sync(0xffffffffu, same);
-  if (same == most) atomicMax(&s_best, ((unsigned long long)same << 32) | (0x7FFFFFFFu - (uint32_t)root));
+  if (threadIdx.x == 0) s_best = 0ull;
+  const int32_t root = label[(int32_t)(((unsigned long long)threadIdx.x * 2654435761ull) % n)];
+  __syncthreads();
+  const uint32_t peers = __match_any_sync(0xffffffffu, root);
+  if ((threadIdx.x & 31) == (uint32_t)(__ffs(peers) - 1)) {
+    uint32_t i = ((uint32_t)root * 2654435761u) % kSlots;  // at most kCcPicks roots: one is free
+    for (;;) {
+      const int32_t there = atomicCAS(&s_root[i], -1, root);
+      if (there == -1 || there == root) break;
+      i = (i + 1) % kSlots;
+    }
+    atomicAdd(&s_count[i], (uint32_t)__popc(peers));
+  }
+  __syncthreads();
+  unsigned long long best = 0ull;
+  for (uint32_t i = threadIdx.x; i < kSlots; i += kCcPicks)
+    if (s_count[i]) {
+      const unsigned long long mine =
+          ((unsigned long long)s_count[i] << 32) | (0x7FFFFFFFu - (uint32_t)s_root[i]);
+      best = best > mine ? best : mine;
+    }
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long x = __shfl_xor_sync(0xffffffffu, best, o);
+    best = best > x ? best : x;
+  }
+  if ((threadIdx.x & 31) == 0 && best) atomicMax(&s_best, best);
   __syncthreads();
   if (threadIdx.x == 0) *skip = (int32_t)(0x7FFFFFFFu - (uint32_t)(s_best & 0xFFFFFFFFull));
 }
@@ -155,9 +185,9 @@ __global__ void __launch_bounds__(kCcThreads) k_cc_rest_frontier(const int32_t *
       const int64_t v = base + j * kCcThreads + threadIdx.x;
       int32_t d = 0;
       bool take = false;
-      if (v < n) {
+      if (v < n && label[v] != skip) {
         d = R[v + 1] - R[v];
-        take = d > 0 && label[v] != skip;
+        take = d > 0;
       }
       emit_scanned(buf, take, (int32_t)v, d);
     }
@@ -190,8 +220,8 @@ __global__ void k_cc_jump(int32_t *label, int32_t n, int32_t *num_roots) {
   int32_t roots = 0;
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
        v += (int64_t)gridDim.x * blockDim.x) {
-    int32_t r = label[v];
-    while (label[r] != r) r = label[r];
+    // halving on the way: a mesh's chains of first neighbours are long
+    const int32_t r = find_root(label, (int32_t)v);
     label[v] = r;
     roots += r == v;
   }
@@ -225,11 +255,12 @@ gr_status cc_run(gr_graph *g, CcWorkspace *ws, int32_t *label, cudaStream_t s) {
   const int grid = g->num_sms * 8;
   const int32_t *R = g->row_off.as<int32_t>(), *C = g->col.as<int32_t>();
   GR_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * 4, s));
-  k_cc_init<<<grid, 256, 0, s>>>(label, g->n);
+  const int32_t *first = g->symmetric ? g->first_col.as<int32_t>() : nullptr;
+  k_cc_init<<<grid, 256, 0, s>>>(label, first, g->n);
   if (!g->symmetric) {
     k_cc_hook<<<g->num_sms * 4, kCcThreads, 0, s>>>(R, C, g->n, label, 0);
   } else {
-    k_cc_sample<<<grid, 256, 0, s>>>(R, C, g->n, label);
+    k_cc_sample<<<grid, 256, 0, s>>>(R, C, first, g->n, label);
     k_cc_jump<<<grid, 256, 0, s>>>(label, g->n, cnt + 1);  // compress (count unused)
     int32_t *skip = ws->skip.as<int32_t>();
     k_cc_pick<<<1, kCcPicks, 0, s>>>(label, g->n, skip);

@@ -76,12 +76,40 @@ __device__ __forceinline__ DS ds_from_u64(unsigned long long c) {
   return ds_add_f(r, u16_to_float((uint32_t)c & 0xFFFFu));
 }
 
+// Conversions between FP64 and double-single take their turn in the FP64
+// pipe like arithmetic, three for each direction; for positive values well
+// inside FP32's exponent range the bits are moved with integers instead
+// (to_double keeps one FP64 addition). The high part is rounded to nearest,
+// the rest, a signed 29-bit integer, to FP32: as the conversions do it.
 __device__ __forceinline__ DS ds_from_double(double x) {
-  const float hi = __double2float_rn(x);
-  return {hi, __double2float_rn(x - (double)hi)};
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int e = (int)(b >> 52) - 1023;  // above 1023 for a negative x
+  if (b == 0ull) return {0.f, 0.f};     // a vertex without children, often
+  if (e < -70 || e > 120) {  // very small, very large, negative, not finite
+    const float hi = __double2float_rn(x);
+    return {hi, __double2float_rn(x - (double)hi)};
+  }
+  const unsigned long long up = (b + (1ull << 28)) >> 29;  // rounded to FP32's 23 bits
+  const int rest = (int)(b & 0x1FFFFFFFull) - (up != (b >> 29) ? 1 << 29 : 0);
+  const float hi = __uint_as_float((uint32_t)(up - ((unsigned long long)(1023 - 127) << 23)));
+  return {hi, __fmul_rn(__int2float_rn(rest), __uint_as_float((uint32_t)(e - 52 + 127) << 23))};
 }
 
-__device__ __forceinline__ double ds_to_double(DS a) { return (double)a.hi + (double)a.lo; }
+__device__ __forceinline__ double ds_to_double(DS a) {
+  const uint32_t h = __float_as_uint(a.hi), l = __float_as_uint(a.lo);
+  const uint32_t eh = (h >> 23) & 0xFFu, el = (l >> 23) & 0xFFu;
+  if (eh - 1u >= 0xFEu) return (double)a.hi + (double)a.lo;  // 0, subnormal, not finite
+  const double dh = __longlong_as_double(
+      (long long)(((unsigned long long)(h & 0x80000000u) << 32) |
+                  (((unsigned long long)(h & 0x7FFFFFFFu) << 29) + ((unsigned long long)(1023 - 127) << 52))));
+  // a subnormal low part is below 2^-126: next to nothing beside hi
+  const double dl = el == 0u ? 0.0
+                             : __longlong_as_double((long long)(
+                                   ((unsigned long long)(l & 0x80000000u) << 32) |
+                                   (((unsigned long long)(l & 0x7FFFFFFFu) << 29) +
+                                    ((unsigned long long)(1023 - 127) << 52))));
+  return dh + dl;
+}
 
 __device__ __forceinline__ DS shfl_xor_ds(DS a, int o) {
   return {__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
