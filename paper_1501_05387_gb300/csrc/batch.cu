@@ -63,6 +63,10 @@ constexpr long long kPushDiv = 16;
 // Graphs of at most this maximum degree (meshes) keep no level's masks.
 constexpr int32_t kLowDegreeMaxBatch = 16;
 constexpr int kMbChunk = kMbThreads * kMbItems;
+// BC's gathers take chunks of this many items per warp: with one per block
+// its warps waited for the slowest at every chunk (half of the forward's
+// stalls).
+constexpr int kMbWarpChunk = 128;
 // What the forward pass counts: nothing (batched BFS), path counts in uint64,
 // or path counts in FP64 (a batch whose uint64 counts overflowed).
 enum : int { kSigNone = 0, kSigU64 = 1, kSigF64 = 2 };
@@ -125,7 +129,7 @@ struct MbArgs {
   int32_t max_levels;
   MbCtl *ctl;
   // chunk bounds of the all-vertex merge paths of the pull levels (chunks of
-  // kMbPullChunk items for the batched BFS, kMbChunk for BC)
+  // kMbPullChunk items for the batched BFS, kMbWarpChunk for BC)
   const int32_t *cb_pull;
   const int32_t *cb_fwd;
 };
@@ -254,24 +258,16 @@ __device__ __forceinline__ unsigned long long joined(const MbArgs &a, int32_t v)
   return 1ull | ((unsigned long long)(uint32_t)(a.R[v + 1] - a.R[v]) << 32);
 }
 
-// A warp's window of a lane-wise gather (below).
-struct LaneBuf {
-  int32_t u[32];
-  uint32_t bits[2][32];
-  uint8_t lane_of[2][32];
-};
-
 // Shared memory of the level forms (one at a time).
 union MbSmem {
   struct {
     int32_t end[kMbPullChunk + 1];  // end marker of each vertex, chunk-local
     unsigned long long U[kMbPullChunk + 1];  // lanes the vertex still misses
   } pull;
-  struct {
-    int32_t off[kMbChunk + 1];
-    unsigned long long U[kMbChunk + 1];
-    LaneBuf lanes[kMbThreads / 32];
-  } fwd;
+  struct {  // per warp
+    int32_t off[kMbWarpChunk + 1];
+    unsigned long long U[kMbWarpChunk + 1];
+  } fwd[kMbThreads / 32];
   struct {
     int32_t off[kMbChunk + 1];
     int32_t row[kMbChunk + 1];
@@ -415,12 +411,17 @@ __device__ void mb_pull_level(const MbArgs &a, MbSmem &sm, int32_t *s_red8, int3
 // half row: with a lanes in it, thread t serves the (t mod a)-th of them and
 // every (32 / a)-th edge. The partial sums of a lane meet in the atomics that
 // add them to v's row (done in L2, not in the FP64 pipe).
-// What a warp is summing: vertex `owner`, lanes `mask`; per half row the
-// thread's source, its first edge and edge step (step 0: none), its sum.
+struct LaneBuf {
+  int32_t u[32];
+  uint32_t bits[2][32];
+  uint8_t lane_of[2][32];
+};
+
+// What a warp is summing: vertex `owner`; per half row the thread's source,
+// its first edge and edge step (step 0: none), its sum.
 template <class T>
 struct LaneSums {
   int32_t owner;
-  uint32_t mask[2];
   int32_t src[2], first[2], step[2];
   T acc[2];
 };
@@ -431,14 +432,12 @@ __device__ __forceinline__ void lane_deal(LaneSums<T> &s, LaneBuf &b, int32_t ow
   const int lane = threadIdx.x & 31;
   const uint32_t lt = (1u << lane) - 1u;
   s.owner = owner;
-  s.mask[0] = m0;
-  s.mask[1] = m1;
   if ((m0 >> lane) & 1u) b.lane_of[0][__popc(m0 & lt)] = (uint8_t)lane;
   if ((m1 >> lane) & 1u) b.lane_of[1][__popc(m1 & lt)] = (uint8_t)(lane + 32);
   __syncwarp();
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
-    const int32_t a = __popc(s.mask[h]);
+    const int32_t a = __popc(h ? m1 : m0);
     // 32 / a and lane / a, exact for these sizes
     const float r = __frcp_rn((float)max(a, 1));
     const int32_t groups = (int32_t)(32.5f * r), g = (int32_t)(((float)lane + 0.5f) * r);
@@ -450,12 +449,11 @@ __device__ __forceinline__ void lane_deal(LaneSums<T> &s, LaneBuf &b, int32_t ow
 }
 
 // One window: lane i's edge (owner, u) with `bits` (0: no edge) of v's lanes
-// `of` (the same for all of v's edges; with OWN_MASK it is what the window's
-// edges have). add(x, y) adds, flush(s) takes the sums of an owner and mask.
-template <bool OWN_MASK, class T, class ADD, class FLUSH>
+// `of` (the same for all of v's edges). flush(s) takes a vertex's sums.
+template <class T, class FLUSH>
 __device__ __forceinline__ void lane_window(LaneSums<T> &s, LaneBuf &b, int32_t owner, int32_t u,
                                             unsigned long long bits, unsigned long long of,
-                                            const T *val, ADD add, FLUSH flush) {
+                                            const T *val, FLUSH flush) {
   const int lane = threadIdx.x & 31;
   const uint32_t lt = (1u << lane) - 1u;
   uint32_t act = __ballot_sync(0xffffffffu, bits != 0ull);
@@ -465,18 +463,11 @@ __device__ __forceinline__ void lane_window(LaneSums<T> &s, LaneBuf &b, int32_t 
     const uint32_t seg = __ballot_sync(0xffffffffu, owner == ov) & act;
     act &= ~seg;
     const bool mine = (seg >> lane) & 1u;
-    uint32_t m0, m1;
-    if (OWN_MASK) {
-      m0 = __reduce_or_sync(0xffffffffu, mine ? (uint32_t)bits : 0u);
-      m1 = __reduce_or_sync(0xffffffffu, mine ? (uint32_t)(bits >> 32) : 0u);
-    } else {
-      m0 = __shfl_sync(0xffffffffu, (uint32_t)of, j0);
-      m1 = __shfl_sync(0xffffffffu, (uint32_t)(of >> 32), j0);
-    }
     __syncwarp();  // the buffer's last readers are done
-    if (ov != s.owner || m0 != s.mask[0] || m1 != s.mask[1]) {
+    if (ov != s.owner) {
       if (s.owner >= 0) flush(s);
-      lane_deal(s, b, ov, m0, m1);
+      lane_deal(s, b, ov, __shfl_sync(0xffffffffu, (uint32_t)of, j0),
+                __shfl_sync(0xffffffffu, (uint32_t)(of >> 32), j0));
     }
     if (mine) {
       const int k = __popc(seg & lt);
@@ -502,88 +493,126 @@ __device__ __forceinline__ void lane_window(LaneSums<T> &s, LaneBuf &b, int32_t 
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-          if (base + k * step < cnt && has[k]) s.acc[h] = add(s.acc[h], x[k]);
+          if (base + k * step < cnt && has[k]) s.acc[h] += x[k];
       }
     }
   }
 }
 
-// The windows of a chunk's ne edges that this warp takes: [*w0, *w1), together.
-__device__ __forceinline__ void chunk_windows(int32_t ne, int32_t *w0, int32_t *w1) {
-  const int32_t windows = (ne + 31) >> 5, wid = threadIdx.x >> 5;
-  *w0 = wid * windows / (kMbThreads / 32);
-  *w1 = (wid + 1) * windows / (kMbThreads / 32);
-}
-
 // A BC forward pull level: nxt[v] = OR over edges (v,u) of cur[u] &
 // ~seen(v), seen(v) = visit[v] | cur[v], and the path counts of the newly
 // reached lanes. The vertex loader of each chunk folds cur into visit
-// (idempotent, so chunks sharing a vertex may both do it).
+// (idempotent, so chunks sharing a vertex may both do it). Lane l of a warp
+// counts for the sources l and l + 32: uint64 adds cost little, so the edges
+// with bits are served one by one by all lanes, but four at a time, the rows of
+// all four loaded before any is added (dealing the threads to the lanes in
+// use, as the backward does, was slower: 1.79 against 1.48 ms on R-MAT 2^18
+// with 64 sources, before the chunks became the warps' own).
 template <int SK>
 __device__ void mb_forward_level(const MbArgs &a, MbSmem &sm, const unsigned long long *cur,
                                  unsigned long long *nxt, unsigned long long *counter, bool &ovf) {
   using T = CountT<SK>;
   const int lane = threadIdx.x & 31;
   const long long total = (long long)a.n + a.R[a.n];
-  const long long nchunks = (total + kMbChunk - 1) / kMbChunk;
+  const long long nchunks = (total + kMbWarpChunk - 1) / kMbWarpChunk;
   unsigned long long new_vertices = 0;
   T *const sigma = (T *)a.sigma;
-  auto add = [&](T x, T y) { return count_add(x, y, ovf); };
-  LaneBuf &buf = sm.fwd.lanes[threadIdx.x >> 5];
-  auto flush = [&](const LaneSums<T> &s) {
-    T *sg = sigma + (int64_t)s.owner * 64;
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-      if (s.acc[h] != T(0)) count_atomic_add(sg + s.src[h], s.acc[h], ovf);
-    if (lane == 0 && !atomicOr(nxt + s.owner, ((unsigned long long)s.mask[1] << 32) | s.mask[0]))
-      new_vertices += joined(a, s.owner);
+  int32_t *off = sm.fwd[threadIdx.x >> 5].off;
+  unsigned long long *U = sm.fwd[threadIdx.x >> 5].U;
+  // the vertex being summed, its lanes so far, its counts
+  int32_t sum_of = -1;
+  uint32_t got0 = 0u, got1 = 0u;
+  T a0 = T(0), a1 = T(0);
+  auto flush = [&]() {
+    if (sum_of < 0) return;
+    T *sg = sigma + (int64_t)sum_of * 64 + lane;
+    if ((got0 >> lane) & 1u) count_atomic_add(sg, a0, ovf);
+    if ((got1 >> lane) & 1u) count_atomic_add(sg + 32, a1, ovf);
+    if (lane == 0 && !atomicOr(nxt + sum_of, ((unsigned long long)got1 << 32) | got0))
+      new_vertices += joined(a, sum_of);
   };
-  for (long long chunk = blockIdx.x; chunk < nchunks; chunk += gridDim.x) {
-    const long long d0 = chunk * kMbChunk;
-    const long long d1 = min(d0 + kMbChunk, total);
+  const long long warps = (long long)gridDim.x * (kMbThreads / 32);
+  for (long long chunk = (long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; chunk < nchunks;
+       chunk += warps) {
+    const long long d0 = chunk * kMbWarpChunk;
+    const long long d1 = min(d0 + kMbWarpChunk, total);
     const int32_t i0 = a.cb_fwd[chunk], i1 = a.cb_fwd[chunk + 1];
     const long long j0 = d0 - i0, j1 = d1 - i1;
     const int32_t nv = (i0 <= a.n - 1) ? (min(i1, a.n - 1) - i0 + 1) : 0;
-    for (int32_t kk = threadIdx.x; kk < nv; kk += kMbThreads) {
+    bool any = false;
+    for (int32_t kk = lane; kk < nv; kk += 32) {
       const int32_t v = i0 + kk;
       const unsigned long long c = cur[v];
       const unsigned long long seen = a.visit[v] | c;
       if (c) a.visit[v] = seen;
-      sm.fwd.off[kk] = a.R[v];
-      sm.fwd.U[kk] = a.all & ~seen;
+      off[kk] = a.R[v];
+      U[kk] = a.all & ~seen;
+      any |= (a.all & ~seen) != 0ull;
     }
-    __syncthreads();
+    if (!__any_sync(0xffffffffu, any)) continue;  // every lane of these vertices is there
+    __syncwarp();
     const int32_t ne = (int32_t)(j1 - j0);
-    int32_t w0, w1;
-    chunk_windows(ne, &w0, &w1);
-    LaneSums<T> sums = {};
-    sums.owner = -1;
-    for (int32_t w = w0; w < w1; ++w) {
-      const int32_t kk = w * 32 + lane;
+    for (int32_t kb = 0; kb < ne; kb += 32) {
+      const int32_t kk = kb + lane;
       int32_t owner = -1, u = 0;
-      unsigned long long bits = 0ull;
+      uint32_t lo = 0u, hi = 0u;
       if (kk < ne) {
         const int32_t e = (int32_t)(j0 + kk);
-        int32_t lo = 0, hi = nv - 1;
-        while (lo < hi) {
-          const int32_t mid = (lo + hi + 1) >> 1;
-          if (sm.fwd.off[mid] <= e) lo = mid;
-          else hi = mid - 1;
+        int32_t k = 0, top = nv - 1;
+        while (k < top) {
+          const int32_t mid = (k + top + 1) >> 1;
+          if (off[mid] <= e) k = mid;
+          else top = mid - 1;
         }
-        owner = i0 + lo;
-        if (!GR_IN(owner, a.n, 201)) owner = -1;
-        const unsigned long long U = owner >= 0 ? sm.fwd.U[lo] : 0ull;
-        if (U && GR_IN(e, a.m, 202)) {
+        const unsigned long long miss = U[k];
+        if (miss && GR_IN(i0 + k, a.n, 201) && GR_IN(e, a.m, 202)) {
+          owner = i0 + k;
           u = a.C[e];
-          bits = GR_IN(u, a.n, 203) ? (cur[u] & U) : 0ull;
+          const unsigned long long bits = GR_IN(u, a.n, 203) ? (cur[u] & miss) : 0ull;
+          lo = (uint32_t)bits;
+          hi = (uint32_t)(bits >> 32);
         }
       }
-      __syncwarp();
-      lane_window<true>(sums, buf, owner, u, bits, 0ull, sigma, add, flush);
+      uint32_t act = __ballot_sync(0xffffffffu, (lo | hi) != 0u);
+      while (act) {  // warp-uniform: one owner's edges at a time
+        const int32_t ov = __shfl_sync(0xffffffffu, owner, __ffs(act) - 1);
+        uint32_t seg = __ballot_sync(0xffffffffu, owner == ov) & act;
+        act &= ~seg;
+        if (ov != sum_of) {
+          flush();
+          sum_of = ov;
+          got0 = got1 = 0u;
+          a0 = a1 = T(0);
+        }
+        while (seg) {
+          uint32_t l[4], h[4];
+          T x[4], y[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const bool has = seg != 0u;
+            const int j = has ? __ffs(seg) - 1 : 0;
+            seg &= seg - 1u;
+            const int32_t uj = __shfl_sync(0xffffffffu, u, j);
+            l[k] = __shfl_sync(0xffffffffu, lo, j);
+            h[k] = __shfl_sync(0xffffffffu, hi, j);
+            if (!has) l[k] = h[k] = 0u;
+            const T *su = sigma + (int64_t)uj * 64 + lane;
+            x[k] = (l[k] >> lane) & 1u ? su[0] : T(0);
+            y[k] = (h[k] >> lane) & 1u ? su[32] : T(0);
+          }
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            got0 |= l[k];
+            got1 |= h[k];
+            if (l[k]) a0 = count_add(a0, x[k], ovf);  // warp-uniform
+            if (h[k]) a1 = count_add(a1, y[k], ovf);
+          }
+        }
+      }
     }
-    if (sums.owner >= 0) flush(sums);
-    __syncthreads();
+    __syncwarp();  // the tables are reused
   }
+  flush();
   for (int o = 16; o > 0; o >>= 1) new_vertices += __shfl_xor_sync(0xffffffffu, new_vertices, o);
   if (lane == 0 && new_vertices) atomicAdd(counter, new_vertices);
 }
@@ -881,21 +910,21 @@ struct BcBackArgs {
 
 // Chunk bounds of a level list's merge path, the list's size and edge count
 // read from *fpacked (its scan S[0..q) does not store S[q]): cb[c] = the
-// members whose end marker S[i + 1] + i lies before c * kMbChunk,
+// members whose end marker S[i + 1] + i lies before c * kMbWarpChunk,
 // cb[nchunks] = q. One thread per chunk; threads past the list's chunks
 // return.
 __global__ void k_list_bounds(const int32_t *S, const unsigned long long *fpacked, int32_t *cb) {
   const unsigned long long fp = *fpacked;
   const int32_t q = (int32_t)(fp & 0xFFFFFFFFull);
   const int32_t qe = (int32_t)(fp >> 32);
-  const long long nchunks = ((long long)q + qe + kMbChunk - 1) / kMbChunk;
+  const long long nchunks = ((long long)q + qe + kMbWarpChunk - 1) / kMbWarpChunk;
   const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (c > nchunks) return;
   if (c == nchunks) {
     cb[c] = q;
     return;
   }
-  const long long d = c * kMbChunk;
+  const long long d = c * kMbWarpChunk;
   int32_t lo = 0, hi = q;  // first member whose end marker is not before d
   while (lo < hi) {
     const int32_t mid = (int32_t)(((long long)lo + hi) >> 1);
@@ -916,52 +945,54 @@ constexpr int kBcBackBlocksPerSm = 4;
 // visited, so the whole backward pass reads every edge about once instead of
 // once per level.
 
-__global__ void __launch_bounds__(kMbThreads, kBcBackBlocksPerSm) k_bc_backward(BcBackArgs a, const int32_t *Q,
-                                                             const int32_t *S,
-                                                             const unsigned long long *fpacked,
-                                                             const int32_t *cb) {
-  __shared__ int32_t s_off[kMbChunk + 1];
-  __shared__ int32_t s_row[kMbChunk + 1];
-  __shared__ int32_t s_v[kMbChunk + 1];
-  __shared__ unsigned long long s_A[kMbChunk + 1];
-  __shared__ LaneBuf s_lanes[kMbThreads / 32];
+struct BcBackWarp {  // a warp's chunk: its vertices' list scan, row starts, ids, lanes
+  int32_t off[kMbWarpChunk + 1];
+  int32_t row[kMbWarpChunk + 1];
+  int32_t v[kMbWarpChunk + 1];
+  unsigned long long A[kMbWarpChunk + 1];
+  LaneBuf lanes;
+};
+
+__global__ void __launch_bounds__(kMbThreads, kBcBackBlocksPerSm) k_bc_backward(
+    BcBackArgs a, const int32_t *Q, const int32_t *S, const unsigned long long *fpacked,
+    const int32_t *cb) {
+  __shared__ BcBackWarp s_warp[kMbThreads / 32];
+  BcBackWarp &sm = s_warp[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
   const unsigned long long fp = *fpacked;
   const int32_t q = (int32_t)(fp & 0xFFFFFFFFull);
   const int32_t qe = (int32_t)(fp >> 32);
   const long long total = (long long)q + qe;
-  const long long nchunks = (total + kMbChunk - 1) / kMbChunk;
-  auto add = [](double x, double y) { return x + y; };
-  LaneBuf &buf = s_lanes[threadIdx.x >> 5];
+  const long long nchunks = (total + kMbWarpChunk - 1) / kMbWarpChunk;
   auto flush = [&](const LaneSums<double> &s) {
     double *qv = a.q + (int64_t)s.owner * 64;
 #pragma unroll
     for (int h = 0; h < 2; ++h)
       if (s.acc[h] != 0.0) atomicAdd(qv + s.src[h], s.acc[h]);
   };
-  for (long long chunk = blockIdx.x; chunk < nchunks; chunk += gridDim.x) {
-    const long long d0 = chunk * kMbChunk;
-    const long long d1 = min(d0 + kMbChunk, total);
+  LaneSums<double> sums = {};
+  sums.owner = -1;
+  const long long warps = (long long)gridDim.x * (kMbThreads / 32);
+  for (long long chunk = (long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; chunk < nchunks;
+       chunk += warps) {
+    const long long d0 = chunk * kMbWarpChunk;
+    const long long d1 = min(d0 + kMbWarpChunk, total);
     const int32_t i0 = cb[chunk], i1 = cb[chunk + 1];  // k_list_bounds
     const long long j0 = d0 - i0, j1 = d1 - i1;
     const int32_t nv = (i0 <= q - 1) ? (min(i1, q - 1) - i0 + 1) : 0;
-    for (int32_t k = threadIdx.x; k < nv; k += kMbThreads) {
+    for (int32_t k = lane; k < nv; k += 32) {
       const int32_t i = i0 + k;
       const int32_t v = GR_IN(i, a.n + 1, 220) ? Q[i] : 0;
       const bool ok = GR_IN(v, a.n, 221);
-      s_off[k] = S[i];
-      s_v[k] = ok ? v : -1;
-      s_row[k] = ok ? a.R[v] : 0;
-      s_A[k] = ok ? a.lv[v] : 0ull;
+      sm.off[k] = S[i];
+      sm.v[k] = ok ? v : -1;
+      sm.row[k] = ok ? a.R[v] : 0;
+      sm.A[k] = ok ? a.lv[v] : 0ull;
     }
-    __syncthreads();
+    __syncwarp();
     const int32_t ne = (int32_t)(j1 - j0);
-    int32_t w0, w1;
-    chunk_windows(ne, &w0, &w1);
-    LaneSums<double> sums = {};
-    sums.owner = -1;
-    for (int32_t win = w0; win < w1; ++win) {
-      const int32_t k = win * 32 + lane;
+    for (int32_t kb = 0; kb < ne; kb += 32) {
+      const int32_t k = kb + lane;
       int32_t owner = -1, w = 0;
       unsigned long long bits = 0ull, A = 0ull;
       if (k < ne) {
@@ -969,23 +1000,23 @@ __global__ void __launch_bounds__(kMbThreads, kBcBackBlocksPerSm) k_bc_backward(
         int32_t lo = 0, hi = nv - 1;
         while (lo < hi) {
           const int32_t mid = (lo + hi + 1) >> 1;
-          if (s_off[mid] <= er) lo = mid;
+          if (sm.off[mid] <= er) lo = mid;
           else hi = mid - 1;
         }
-        owner = s_v[lo];
-        const long long e = (long long)s_row[lo] + (er - s_off[lo]);
-        A = s_A[lo];
+        owner = sm.v[lo];
+        const long long e = (long long)sm.row[lo] + (er - sm.off[lo]);
+        A = sm.A[lo];
         if (owner >= 0 && A && GR_IN(e, a.m, 222)) {
           w = a.C[e];
           bits = GR_IN(w, a.n, 223) ? (A & a.lw[w]) : 0ull;
         }
       }
       __syncwarp();
-      lane_window<false>(sums, buf, owner, w, bits, A, (const double *)a.q, add, flush);
+      lane_window(sums, sm.lanes, owner, w, bits, A, (const double *)a.q, flush);
     }
-    if (sums.owner >= 0) flush(sums);
-    __syncthreads();
+    __syncwarp();  // the tables are reused
   }
+  if (sums.owner >= 0) flush(sums);
 }
 
 // The vertices with lanes in `lv`, with their degree scan (block-wise
@@ -1119,11 +1150,11 @@ gr_status batch_ws_create(gr_graph *g, BatchWorkspace **out) {
     // level: their chunk bounds are found once
     const int32_t *R = g->row_off.as<int32_t>();
     const int32_t cp = merge_chunks(g->n, g->m, kMbPullChunk);
-    const int32_t cf = merge_chunks(g->n, g->m, kMbChunk);
+    const int32_t cf = merge_chunks(g->n, g->m, kMbWarpChunk);
     GR_TRY(ws->cb_pull.alloc(sizeof(int32_t) * ((size_t)cp + 1), "batch pull chunk bounds"));
     GR_TRY(ws->cb_fwd.alloc(sizeof(int32_t) * ((size_t)cf + 1), "BC pull chunk bounds"));
     k_chunk_bounds<<<(cp + 256) / 256, 256>>>(R, g->n, kMbPullChunk, cp, ws->cb_pull.as<int32_t>());
-    k_chunk_bounds<<<(cf + 256) / 256, 256>>>(R, g->n, kMbChunk, cf, ws->cb_fwd.as<int32_t>());
+    k_chunk_bounds<<<(cf + 256) / 256, 256>>>(R, g->n, kMbWarpChunk, cf, ws->cb_fwd.as<int32_t>());
     GR_CUDA(cudaGetLastError());
     GR_CUDA(cudaStreamSynchronize(0));
   }
@@ -1137,7 +1168,7 @@ gr_status batch_ws_create(gr_graph *g, BatchWorkspace **out) {
 
 // Most merge-path chunks a BC level list can have (n vertices, m edges).
 static long long bc_list_max_chunks(const gr_graph *g) {
-  return ((long long)g->n + g->m) / kMbChunk + 1;
+  return ((long long)g->n + g->m) / kMbWarpChunk + 1;
 }
 
 static gr_status ensure_batch_ws(gr_graph *g, BatchWorkspace **slot, bool need_bc) {
