@@ -45,12 +45,12 @@
 #include <type_traits>
 #include <vector>
 
-#include "advance.cuh"
 #include "double_single.cuh"
+#include "gather.cuh"
 
 namespace gr {
 
-constexpr int kMbThreads = 256, kMbItems = 4;
+constexpr int kMbThreads = 256, kMbItems = 2;
 // Batched BFS keeps the lane masks of its first kKeepLevels levels, each in
 // its own array, and writes their depths in one pass at the end (full
 // coalesced rows); deeper levels rotate through three arrays and write their
@@ -67,6 +67,7 @@ constexpr int kMbChunk = kMbThreads * kMbItems;
 // its warps waited for the slowest at every chunk (half of the forward's
 // stalls).
 constexpr int kMbWarpChunk = 128;
+constexpr int kMbListChunk = 1024;  // vertices per block step of k_mb_list
 // What the forward pass counts: nothing (batched BFS), path counts in uint64,
 // or path counts in FP64 (a batch whose uint64 counts overflowed).
 enum : int { kSigNone = 0, kSigU64 = 1, kSigF64 = 2 };
@@ -74,7 +75,9 @@ enum : int { kSigNone = 0, kSigU64 = 1, kSigF64 = 2 };
 
 struct BatchWorkspace {
   DevMem visit, sigma, q, counter, lmp, ctl;
-  DevMem cb_pull, cb_fwd;  // chunk bounds of the all-vertex pulls (fixed per graph)
+  GatherPlan plan;  // row structure of the batched BFS's pulls (symmetric graphs)
+  DevMem full;      // a bit per vertex: it holds every lane in use
+  DevMem cb_fwd;    // chunk bounds of BC's all-vertex pulls (fixed per graph)
   DevMem fq, fs;    // BC backward: one level's vertex list and degree scan
   DevMem fcb;       // BC backward: that list's merge-path chunk bounds
   DevMem lq[3], ls[3];  // forward: level lists (ring by level) and degree scans
@@ -128,9 +131,9 @@ struct MbArgs {
   int32_t symmetric;
   int32_t max_levels;
   MbCtl *ctl;
-  // chunk bounds of the all-vertex merge paths of the pull levels (chunks of
-  // kMbPullChunk items for the batched BFS, kMbWarpChunk for BC)
-  const int32_t *cb_pull;
+  GatherPlanArgs plan;  // batched BFS: row structure of the pull levels
+  uint32_t *full;       // batched BFS: vertices with every lane, by the last pull
+  // BC: chunk bounds of the all-vertex merge path, kMbWarpChunk items each
   const int32_t *cb_fwd;
 };
 
@@ -243,8 +246,6 @@ __global__ void k_mb_sources(MbArgs a, MbSources srcs, int32_t sk) {
 // Block-local list of the vertices a push level adds to the next level,
 // flushed per chunk with flush_scanned (one packed atomic per block and
 // chunk); a chunk of kMbChunk items adds at most kMbChunk vertices.
-constexpr int kMbPullItems = 8;
-constexpr int kMbPullChunk = kMbThreads * kMbPullItems;
 using MbEmitBuf = ScannedBuf<kMbChunk>;
 
 __device__ __forceinline__ void mb_emit(MbEmitBuf &em, const MbArgs &a, int32_t v) {
@@ -260,10 +261,6 @@ __device__ __forceinline__ unsigned long long joined(const MbArgs &a, int32_t v)
 
 // Shared memory of the level forms (one at a time).
 union MbSmem {
-  struct {
-    int32_t end[kMbPullChunk + 1];  // end marker of each vertex, chunk-local
-    unsigned long long U[kMbPullChunk + 1];  // lanes the vertex still misses
-  } pull;
   struct {  // per warp
     int32_t off[kMbWarpChunk + 1];
     unsigned long long U[kMbWarpChunk + 1];
@@ -286,115 +283,80 @@ __device__ __forceinline__ void mb_write_depth(const MbArgs &a, int32_t v, unsig
       a.depth[(int64_t)s * a.n + v] = L;
 }
 
-// A batched BFS pull level (no path counts): nxt[v] = OR over edges (v, u)
-// of cur[u] & ~seen(v), seen(v) = visit[v] | cur[v], for every vertex v.
-// Merge-based: a chunk's vertex end markers and edges form one sequence of
-// kMbThreads * kMbPullItems items; each thread finds its first item's
-// vertex with one search, then walks its kMbPullItems consecutive items.
-// The column and lane-mask loads of all its items are issued before any is
-// used, edges of vertices that already hold every lane are skipped, and the
-// OR of a vertex accumulates in a register. A vertex whose edges and end
-// marker all fall in one thread's items is written with a plain store (no
-// other thread touches it); the others with atomicOr. The vertex loader
-// folds cur into visit and, past the kept levels, writes depth L. The level
-// counts the vertices whose mask goes from empty to non-empty (and their
-// edges); it writes no list (a push level after it compacts one).
-__device__ void mb_pull_level(const MbArgs &a, MbSmem &sm, int32_t *s_red8, int32_t L,
-                              const unsigned long long *cur, unsigned long long *nxt,
-                              unsigned long long *counter) {
-  constexpr int ITEMS = kMbPullItems;
-  constexpr int CHUNK = kMbPullChunk;
+// A batched BFS pull level (no path counts) has two parts. The fold: every
+// vertex's cur goes into visit, its depths at L are written past the kept
+// levels, and the vertices that hold every lane are marked in `full`. After
+// a grid barrier the gather: nxt[v] = OR over the entries (v, u) of v's row
+// of cur[u], less visit[v], in registers (gather_reduce_tiles), the rows of
+// full vertices skipped; whole rows are stored (nxt is zero), pieces of rows
+// combined with atomicOr. It counts the vertices whose mask goes from empty
+// to non-empty, and their edges; it writes no list (a push level after it
+// compacts one). R-MAT 2^20, 64 sources, 31.4 M entries: the four pulls took
+// 192, 237, 199 and 97 us with merge-path tables in shared memory (which take
+// the masks' L1) and a lane mask looked up per edge.
+__device__ void mb_pull_fold(const MbArgs &a, int32_t L, const unsigned long long *cur) {
   const bool write_depth = a.depth && L >= a.keep;
-  const long long total = (long long)a.n + a.R[a.n];
-  const long long nchunks = (total + CHUNK - 1) / CHUNK;
-  unsigned long long new_vertices = 0;
-  for (long long chunk = blockIdx.x; chunk < nchunks; chunk += gridDim.x) {
-    const long long d0 = chunk * CHUNK;
-    const long long d1 = min(d0 + CHUNK, total);
-    const int32_t i0 = a.cb_pull[chunk], i1 = a.cb_pull[chunk + 1];
-    const long long j0 = d0 - i0;  // CSR position of the chunk's first edge
-    const int32_t nv = (i0 <= a.n - 1) ? (min(i1, a.n - 1) - i0 + 1) : 0;
-    const int32_t len = (int32_t)(d1 - d0);
-    for (int32_t kk = threadIdx.x; kk < nv; kk += kMbThreads) {
-      const int32_t v = i0 + kk;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const int64_t nr = ((int64_t)a.n + 31) & ~31ll;  // warp-uniform bound
+  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < nr; v += stride) {
+    bool all = true;
+    if (v < a.n) {
       const unsigned long long c = cur[v];
-      const unsigned long long seen = a.visit[v] | c;
+      unsigned long long seen = a.visit[v];
       if (c) {
+        seen |= c;
         a.visit[v] = seen;
-        if (write_depth) mb_write_depth(a, v, c, L);
+        if (write_depth) mb_write_depth(a, (int32_t)v, c, L);
       }
-      sm.pull.end[kk] = (int32_t)((long long)a.R[v + 1] + v - d0);
-      sm.pull.U[kk] = a.all & ~seen;
+      all = seen == a.all;
     }
-    __syncthreads();
-    const int32_t k0 = min(len, (int32_t)threadIdx.x * ITEMS);
-    const int32_t k1 = min(len, k0 + ITEMS);
-    if (k0 < k1) {
-      // chunk vertices whose end marker lies before k0
-      int32_t lo = 0, hi = nv;
-      while (lo < hi) {
-        const int32_t mid = (lo + hi) >> 1;
-        if (sm.pull.end[mid] < k0) lo = mid + 1;
-        else hi = mid;
-      }
-      // classify the items: end markers (bit i of `ends`) and edges, loading
-      // the column of each edge whose vertex still misses lanes
-      uint32_t ends = 0u;
-      int32_t u[ITEMS];
-      int32_t r = lo, e = k0 - lo;  // e: chunk-local edge index
-#pragma unroll
-      for (int i = 0; i < ITEMS; ++i) {
-        const int32_t k = k0 + i;
-        u[i] = -1;
-        if (k < k1 && r < nv) {
-          if (sm.pull.end[r] == k) {
-            ends |= 1u << i;
-            ++r;
-          } else {
-            const long long pos = j0 + e;
-            if (sm.pull.U[r] && GR_IN(pos, a.m, 202)) u[i] = (int32_t)pos;
-            ++e;
-          }
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < ITEMS; ++i) u[i] = u[i] >= 0 ? a.C[u[i]] : -1;
-      unsigned long long b[ITEMS];
-#pragma unroll
-      for (int i = 0; i < ITEMS; ++i) b[i] = (u[i] >= 0 && GR_IN(u[i], a.n, 203)) ? cur[u[i]] : 0ull;
-      // walk: OR per vertex, written at its end marker
-      r = lo;
-      unsigned long long acc = 0ull;
-      bool whole = false;  // the vertex's first edge lies in this thread's items
-#pragma unroll
-      for (int i = 0; i < ITEMS; ++i) {
-        const int32_t k = k0 + i;
-        if (k < k1 && r < nv) {
-          if ((ends >> i) & 1u) {
-            if (acc) {
-              const int32_t v = i0 + r;
-              if (whole) {
-                nxt[v] = acc;
-                new_vertices += joined(a, v);
-              } else if (!atomicOr(nxt + v, acc)) {
-                new_vertices += joined(a, v);
-              }
-            }
-            acc = 0ull;
-            whole = true;
-            ++r;
-          } else {
-            acc |= b[i] & sm.pull.U[r];
-          }
-        }
-      }
-      if (acc && r < nv && !atomicOr(nxt + (i0 + r), acc))  // continues past k1
-        new_vertices += joined(a, i0 + r);
-    }
-    __syncthreads();
+    const uint32_t b = __ballot_sync(0xffffffffu, all);
+    if ((threadIdx.x & 31) == 0) a.full[v >> 5] = b;
   }
-  for (int o = 16; o > 0; o >>= 1) new_vertices += __shfl_xor_sync(0xffffffffu, new_vertices, o);
-  if ((threadIdx.x & 31) == 0 && new_vertices) atomicAdd(counter, new_vertices);
+}
+
+struct LaneMask {
+  static constexpr bool kWeighted = false;
+  const unsigned long long *cur;
+  __device__ __forceinline__ unsigned long long operator()(int32_t u, int32_t) const {
+    return cur[u];
+  }
+};
+struct OrU64 {
+  static __device__ __forceinline__ unsigned long long identity() { return 0ull; }
+  static __device__ __forceinline__ unsigned long long op(unsigned long long x,
+                                                          unsigned long long y) {
+    return x | y;
+  }
+};
+struct SkipFull {
+  static constexpr bool kSkips = true;
+  const uint32_t *full;
+  __device__ __forceinline__ bool operator()(int32_t v) const { return test_bit(full, v); }
+};
+struct JoinLanes {
+  const MbArgs &a;
+  unsigned long long *nxt;
+  unsigned long long &count;
+  __device__ __forceinline__ void operator()(int32_t v, unsigned long long x, bool whole) const {
+    if (!x) return;
+    x &= ~a.visit[v];
+    if (!x) return;
+    if (whole) nxt[v] = x;
+    else if (atomicOr(nxt + v, x)) return;
+    count += joined(a, v);
+  }
+};
+
+__device__ __forceinline__ void mb_pull_gather(const MbArgs &a, const unsigned long long *cur,
+                                               unsigned long long *nxt,
+                                               unsigned long long *counter) {
+  unsigned long long count = 0;
+  gather_reduce_tiles<1, unsigned long long, OrU64>(
+      a.plan, a.C, nullptr, 0, (int32_t)a.m, LaneMask{cur}, JoinLanes{a, nxt, count},
+      spread_warp(), grid_warps(), SkipFull{a.full});
+  count = warp_sum(count);
+  if ((threadIdx.x & 31) == 0 && count) atomicAdd(counter, count);
 }
 
 // ------------------------------------------------------- lane-wise gathers
@@ -732,31 +694,34 @@ __device__ void mb_compact_list(const MbArgs &a, MbSmem &sm, const unsigned long
 // of one vertex are disjoint, so the level of every lane follows from bit
 // slices: slice j is the OR of the masks of the levels whose index has bit j
 // set.
-__device__ void mb_depth_pass(const MbArgs &a, int32_t levels) {
-  constexpr int kSlices = 6;  // levels < 64
+template <int SLICES>
+__device__ void mb_depth_slices(const MbArgs &a, int32_t levels) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  const int64_t nr = ((int64_t)a.n + 31) & ~31ll;  // warp-uniform bound
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < nr; v += stride) {
-    unsigned long long b[kSlices] = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull}, reached = 0ull;
-    if (v < a.n) {
-      for (int32_t L = 0; L < levels; ++L) {
-        const unsigned long long m = a.lmp[L][v];
-        reached |= m;
+  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < a.n; v += stride) {
+    unsigned long long b[SLICES], reached = 0ull;
 #pragma unroll
-        for (int j = 0; j < kSlices; ++j)
-          if ((L >> j) & 1) b[j] |= m;
-      }
+    for (int j = 0; j < SLICES; ++j) b[j] = 0ull;
+    for (int32_t L = 0; L < levels; ++L) {
+      const unsigned long long m = a.lmp[L][v];
+      reached |= m;
+#pragma unroll
+      for (int j = 0; j < SLICES; ++j)
+        if ((L >> j) & 1) b[j] |= m;
     }
-    for (int32_t s = 0; s < a.k; ++s) {
-      int32_t d = -1;
-      if ((reached >> s) & 1ull) {
-        d = 0;
+    int32_t *out = a.depth + v;
+    for (int32_t s = 0; s < a.k; ++s, out += a.n) {
+      int32_t d = 0;
 #pragma unroll
-        for (int j = 0; j < kSlices; ++j) d |= (int32_t)((b[j] >> s) & 1ull) << j;
-      }
-      if (v < a.n) a.depth[(int64_t)s * a.n + v] = d;
+      for (int j = 0; j < SLICES; ++j) d |= (int32_t)((b[j] >> s) & 1ull) << j;
+      *out = (reached >> s) & 1ull ? d : -1;
     }
   }
+}
+
+__device__ __forceinline__ void mb_depth_pass(const MbArgs &a, int32_t levels) {
+  static_assert(kKeepLevels <= 16, "four slices");
+  if (levels <= 8) mb_depth_slices<3>(a, levels);
+  else mb_depth_slices<4>(a, levels);
 }
 
 // Blocks per SM of k_mb_do: the batched BFS at 5 (48 registers; 7.48 ms
@@ -855,7 +820,9 @@ __global__ void __launch_bounds__(kMbThreads, mb_do_blocks_per_sm<SK>()) k_mb_do
       mb_push_level<SK>(a, sm, s_red8, L, cur, nxt, a.lq[L % 3], a.ls[L % 3], st.q, st.qe,
                         a.lq[(L + 1) % 3], a.ls[(L + 1) % 3], counter, ovf);
     } else if (SK == kSigNone) {
-      mb_pull_level(a, sm, s_red8, L, cur, nxt, counter);
+      mb_pull_fold(a, L, cur);
+      if (!grid_sync(&c->bar, &c->error, gen)) break;
+      mb_pull_gather(a, cur, nxt, counter);
     } else {
       mb_forward_level<SK == kSigNone ? kSigU64 : SK>(a, sm, cur, nxt, counter, ovf);
     }
@@ -1027,12 +994,12 @@ __global__ void __launch_bounds__(kMbThreads) k_mb_list(const unsigned long long
                                                          const int32_t *R, int32_t n,
                                                          int32_t *Q, int32_t *S,
                                                          unsigned long long *fpacked) {
-  __shared__ ScannedBuf<kMbChunk> buf;
+  __shared__ ScannedBuf<kMbListChunk> buf;
   if (threadIdx.x == 0) buf.cnt = 0;
   __syncthreads();
-  constexpr int PER = kMbChunk / kMbThreads;
-  for (int64_t base = (int64_t)blockIdx.x * kMbChunk; base < n;
-       base += (int64_t)gridDim.x * kMbChunk) {  // block-uniform
+  constexpr int PER = kMbListChunk / kMbThreads;
+  for (int64_t base = (int64_t)blockIdx.x * kMbListChunk; base < n;
+       base += (int64_t)gridDim.x * kMbListChunk) {  // block-uniform
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
       const int64_t v = base + j * kMbThreads + threadIdx.x;
@@ -1137,7 +1104,9 @@ size_t batch_ws_bytes(const gr_graph *g) {
   // visit masks, the level arrays of a batched BFS, the level lists
   const size_t n = (size_t)g->n;
   return sizeof(unsigned long long) * n * (1 + bfs_keep_levels(g) + 3) +
-         3 * sizeof(int32_t) * (2 * n + 3) + sizeof(MbCtl) + 4096;
+         3 * sizeof(int32_t) * (2 * n + 3) + sizeof(MbCtl) + 4096 +
+         (g->symmetric ? gather_plan_bytes(g->n, g->m) + n / 8 + 4 * ((n + (size_t)g->m) / kMbWarpChunk)
+                       : 0);
 }
 
 gr_status batch_ws_create(gr_graph *g, BatchWorkspace **out) {
@@ -1145,15 +1114,14 @@ gr_status batch_ws_create(gr_graph *g, BatchWorkspace **out) {
   GR_TRY(ws->visit.alloc(sizeof(unsigned long long) * (size_t)g->n, "lane visit masks"));
   GR_TRY(ws->counter.alloc(sizeof(unsigned long long) * 4, "batch counters"));
   GR_TRY(ws->ctl.alloc(sizeof(MbCtl), "batch control"));
-  {
-    // the pull levels' merge paths over all vertices are the same on every
-    // level: their chunk bounds are found once
+  if (g->symmetric) {  // else no level pulls
+    GR_TRY(gather_plan_build(&ws->plan, g->row_off.as<int32_t>(), g->n, g->m, 0));
+    GR_TRY(ws->full.alloc(sizeof(uint32_t) * (size_t)g->nwords, "batch full vertices"));
+    // BC's merge path over all vertices is the same on every level: its chunk
+    // bounds are found once
     const int32_t *R = g->row_off.as<int32_t>();
-    const int32_t cp = merge_chunks(g->n, g->m, kMbPullChunk);
     const int32_t cf = merge_chunks(g->n, g->m, kMbWarpChunk);
-    GR_TRY(ws->cb_pull.alloc(sizeof(int32_t) * ((size_t)cp + 1), "batch pull chunk bounds"));
     GR_TRY(ws->cb_fwd.alloc(sizeof(int32_t) * ((size_t)cf + 1), "BC pull chunk bounds"));
-    k_chunk_bounds<<<(cp + 256) / 256, 256>>>(R, g->n, kMbPullChunk, cp, ws->cb_pull.as<int32_t>());
     k_chunk_bounds<<<(cf + 256) / 256, 256>>>(R, g->n, kMbWarpChunk, cf, ws->cb_fwd.as<int32_t>());
     GR_CUDA(cudaGetLastError());
     GR_CUDA(cudaStreamSynchronize(0));
@@ -1240,7 +1208,8 @@ static MbArgs mb_args(gr_graph *g, BatchWorkspace *ws, int32_t k, int32_t *depth
   a.symmetric = g->symmetric ? 1 : 0;
   a.max_levels = max_levels;
   a.ctl = ws->ctl.as<MbCtl>();
-  a.cb_pull = ws->cb_pull.as<int32_t>();
+  a.plan = ws->plan.a;
+  a.full = ws->full.as<uint32_t>();
   a.cb_fwd = ws->cb_fwd.as<int32_t>();
   return a;
 }

@@ -83,15 +83,22 @@ struct StoreReduced {
   }
 };
 
+struct SkipNone {
+  static constexpr bool kSkips = false;
+  __device__ __forceinline__ bool operator()(int32_t) const { return false; }
+};
+
 // One warp's share (tiles gw, gw + nw, ...) of the entries [eb, ee), which
 // begin and end with whole rows. F: value_type operator()(u, weight) and
 // F::kWeighted (whether it reads w[e], then non-null). E: operator()(v,
-// value, whole), once per whole row and once per piece of the others.
-template <int G8, class T, class OP, class F, class E>
+// value, whole), once per whole row and once per piece of the others. S:
+// operator()(v), whether v's row needs no gathering (its value is then OP's
+// identity), asked for every row of a lane before its columns are loaded.
+template <int G8, class T, class OP, class F, class E, class S = SkipNone>
 __device__ __forceinline__ void gather_reduce_tiles(const GatherPlanArgs &p, const int32_t *C,
                                                     const int32_t *W, int32_t eb, int32_t ee,
                                                     const F &f, const E &emit, int64_t gw,
-                                                    int64_t nw) {
+                                                    int64_t nw, const S &skip = S()) {
   constexpr int ITEMS = 8 * G8;
   constexpr int TILE = 32 * ITEMS;
   static_assert(TILE % kGpTile == 0, "a warp's tile is whole rank_base tiles");
@@ -111,12 +118,25 @@ __device__ __forceinline__ void gather_reduce_tiles(const GatherPlanArgs &p, con
       rank = (int32_t)(p.rank_base[e0 / kGpTile] & 0x7FFFFFFFu) + (int32_t)(d0 >> 8);
       if (G8 == 2) ends |= (uint32_t)(p.desc[g + 1] & 0xFFu) << 8;
     }
-    uint32_t valid = (1u << ITEMS) - 1u;
+    uint32_t valid = (1u << ITEMS) - 1u;  // entries to gather
+    if (S::kSkips && whole) {
+      uint32_t left = ends;
+      int32_t r = rank;
+      for (int from = 0; from < ITEMS; ++r) {
+        const int to = left ? __ffs(left) : ITEMS;
+        if (skip(p.rows[r])) valid &= ~((1u << to) - (1u << from));
+        left &= left - 1u;
+        from = to;
+      }
+    }
     if (whole) {
 #pragma unroll
       for (int k = 0; k < G8; ++k) {
         int32_t x[8];
-        ld_stream8(C + e0 + 8 * k, x);
+        if (!S::kSkips || valid) ld_stream8(C + e0 + 8 * k, x);
+        else
+#pragma unroll
+          for (int i = 0; i < 8; ++i) x[i] = 0;
 #pragma unroll
         for (int i = 0; i < 8; ++i) c[8 * k + i] = x[i];
         if (F::kWeighted) {
