@@ -724,9 +724,8 @@ __device__ __forceinline__ void mb_depth_pass(const MbArgs &a, int32_t levels) {
   else mb_depth_slices<4>(a, levels);
 }
 
-// Blocks per SM of k_mb_do: the batched BFS at 5 (48 registers; 7.48 ms
-// for 64 sources on R-MAT s23 against 8.25 ms at 6), BC at 6 (116 ms
-// against 118 ms at 5).
+// Most blocks per SM of k_mb_do: 48 registers a thread for the batched BFS, 64
+// for BC's forward.
 template <int SK>
 constexpr int mb_do_blocks_per_sm() { return SK == kSigNone ? 5 : 4; }
 
@@ -1218,7 +1217,19 @@ static gr_status mb_launch(gr_graph *g, const MbArgs &a, int sk, cudaStream_t s)
   void *kern = sk == kSigU64   ? (void *)k_mb_do<kSigU64>
                : sk == kSigF64 ? (void *)k_mb_do<kSigF64>
                                : (void *)k_mb_do<kSigNone>;
-  const int want = sk == kSigNone ? mb_do_blocks_per_sm<kSigNone>() : mb_do_blocks_per_sm<kSigU64>();
+  // small graphs are bound by the grid barrier, which costs more the more
+  // blocks meet at it. Batched BFS at 1 to 5 blocks per SM, 20 lanes: R-MAT
+  // 34,000 entries 81, 88, 92, 97, 99 us; 0.24 M 81, 93, 95, 101, 102; 0.64 M
+  // 115, 112, 111, 114, 119; 1.1 M 133, 116, 115, 112, 115; 2.5 M 174, 138,
+  // 131, 130, 132; 32 lanes 5.7 M 347, 250, 222, 209, 216; 64 lanes 15 M 744,
+  // 474, 400, 366, 346. Directed, 64 lanes: 0.13 M 112, 111, 117, 120, 127;
+  // 0.34 M 150, 129, 115, 120, 115; 1.3 M 337, 224, 187, 180, 173. BC at 1 to
+  // 4: 40,000 entries 490, 505, 500, 518; 0.24 M 558, 491, 499, 499; 0.65 M
+  // 619, 539, 501, 476.
+  int want;
+  if (sk != kSigNone) want = g->m < 100'000 ? 1 : g->m < 500'000 ? 2 : mb_do_blocks_per_sm<kSigU64>();
+  else if (!g->symmetric) want = g->m < 300'000 ? 2 : mb_do_blocks_per_sm<kSigNone>();
+  else want = g->m < 400'000 ? 1 : g->m < 900'000 ? 3 : g->m < 10'000'000 ? 4 : mb_do_blocks_per_sm<kSigNone>();
   int per_sm = 1;
   GR_TRY(fit_carveout(kern, kMbThreads, want, g->device, &per_sm));
   const int blocks = per_sm * g->num_sms;
