@@ -12,11 +12,11 @@
 //               frontier once (the non-idempotent advance of Sec. 4.5).
 //   pull level  bottom-up advance (Sec. 4.5): every unvisited vertex looks
 //               for a neighbour in the frontier bitmap and stops at the first.
-//               A warp owns 32 consecutive vertices, one bitmap word, so the
-//               visited and next-frontier bitmaps are written with a ballot and
-//               a plain store: no atomics. Lanes check their first neighbours
-//               with independent loads; vertices left over with longer lists
-//               are then scanned by the whole warp, 32 neighbours at a time.
+//               A warp owns whole words of the visited bitmap, so the visited
+//               and next-frontier bitmaps are written with a ballot and a plain
+//               store: no atomics. Lanes check the unvisited vertices' first
+//               neighbours, then a few more of each, with independent loads;
+//               what is left of long lists is scanned by the whole warp.
 //
 // Both emit the next frontier together with its exclusive degree scan (the
 // "scanned edge offset queue" of Sec. 4.4): a block compacts its new
@@ -108,8 +108,8 @@ struct BfsArgs {
   int32_t low_degree;   // push-only on a graph of small maximum degree: per-thread expansion
   const int4 *adj;      // low-degree graphs: first four neighbours per vertex (low_adjacency)
   // persistent kernel: per-block segments of the vertices a pull level
-  // found (and their degrees), compacted into a queue by the next level
-  // when it pushes; null in the other drivers
+  // found (and their degrees), filled by the next level when it pushes; null
+  // in the other drivers
   int32_t *seg_v;
   int32_t *seg_d;
   unsigned long long *seg_cnt;  // per block: [31:0] vertices, [63:32] edges
@@ -122,8 +122,7 @@ constexpr int kLvItems = 4;                        // merge items per thread (pu
 constexpr int kLvChunk = kLvThreads * kLvItems;    // merge items per chunk
 constexpr int kLvWarps = kLvThreads / 32;
 // neighbours after the first a lane checks alone in a pull level, before the
-// warp scans what is left of a long list (R-MAT s22: 0.1827 ms per traversal
-// at 3, 0.1815 at 5, 0.1806 at 8, 0.1811 at 12, 0.1809 at 20)
+// warp scans what is left of a long list
 constexpr int kPullLane = 8;
 constexpr int kLvBlocksPerSm = 6;
 // On graphs of at most kLowDegreeMax push levels expand one frontier vertex
@@ -216,15 +215,27 @@ __global__ void k_bfs_init(BfsArgs a, int32_t src, int32_t *depth, int32_t *pare
   }
 }
 
+// A warp's vertices of a pull step: those still to be looked at, as positions
+// in the step's words, and a mark for each one found.
+constexpr int kPullBatch = 32;  // bitmap words a warp takes at once
+struct PullWarp {
+  uint16_t list[kPullBatch * 32];
+  uint4 mark[kPullBatch * 2];
+};
+
 // Shared memory of the level kernel: the push part's merge-path tables and
-// the emit buffer (new vertices and their degrees), which the pull part
-// reuses.
+// the emit buffer (new vertices and their degrees), or the pull part's lists.
 struct LevelSmem {
-  int32_t off[kLvChunk + 1];
-  int32_t u[kLvChunk + 1];
-  int32_t row[kLvChunk + 1];
-  int32_t out[kLvChunk];
-  int32_t deg[kLvChunk];
+  union {
+    struct {
+      int32_t off[kLvChunk + 1];
+      int32_t u[kLvChunk + 1];
+      int32_t row[kLvChunk + 1];
+      int32_t out[kLvChunk];
+      int32_t deg[kLvChunk];
+    };
+    PullWarp pull[kLvWarps];
+  };
   uint32_t red[33];
   unsigned long long red64[33];
   int32_t sred[kLvWarps];
@@ -462,11 +473,37 @@ __device__ void push_level_thread(const BfsArgs &a, BfsCtl *c, int32_t p, int32_
   }
 }
 
+// Words of the visited bitmap that one warp walks in a pull level.
+__host__ __device__ __forceinline__ int32_t pull_words_per_warp(int32_t nwords, int32_t warps) {
+  return (nwords + warps - 1) / warps;
+}
+
+// Warp g takes one word of each round of as many words as there are warps,
+// shifted from round to round: a skewed graph's unvisited vertices are not
+// spread evenly, neither over ranges of ids nor over ids a power of two apart.
+constexpr uint32_t kPullShift = 61;
+__device__ __forceinline__ int64_t pull_word(int32_t g, int32_t warps, int32_t round) {
+  return (int64_t)round * warps +
+         ((uint32_t)g + (uint32_t)round * kPullShift) % (uint32_t)warps;
+}
+
 // Pull level: no queue is written; the block counts the vertices it found
-// and their edges and adds both to the packed counter once at the end. A
-// warp owns kPullWords consecutive bitmap words per step (32 * kPullWords
-// vertices, kPullWords per lane) so several load chains are in flight.
-constexpr int kPullWords = 2;
+// and their edges and adds both to the packed counter once at the end.
+//
+// Bound by latency: a vertex costs a chain of a row offset or column from HBM
+// and a frontier bit from L2, so the lanes are kept full and their loads
+// independent. A warp loads the visited words of a step at once and lists the
+// unvisited vertices; each lane tests the first neighbour of two of them; the
+// ones that are left are listed again and looked at one per lane, four
+// neighbours at a time; what is still left of a long list is scanned by the
+// whole warp. Marks in shared memory become the next frontier's words and the
+// depths, in full lines. (With a lane per bit of the words, visited or not,
+// and one neighbour after another, the three pull levels of a search of R-MAT
+// 2^22 took 53, 34 and 22 us, the last with 4062 vertices unvisited; here 28,
+// 16 and 9, and the search 104 us instead of 166.)
+//
+// The words of the next frontier that stay empty were cleared a level ago.
+constexpr int kPullItems = 2;  // first neighbours a lane tests at once
 
 __device__ void pull_level(const BfsArgs &a, BfsCtl *c, LevelSmem &sm, int32_t L,
                            unsigned long long *counter, int32_t *maxdeg = nullptr) {
@@ -475,118 +512,149 @@ __device__ void pull_level(const BfsArgs &a, BfsCtl *c, LevelSmem &sm, int32_t L
   int32_t *depth = c->depth;
   int32_t *parent = c->parent;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const long long gw = (long long)blockIdx.x * kLvWarps + wid;
-  const long long nw = (long long)gridDim.x * kLvWarps;
-  const long long groups = (a.nwords + kPullWords - 1) / kPullWords;
+  const uint32_t below = (1u << lane) - 1u;
+  const int32_t gw = blockIdx.x * kLvWarps + wid;
+  const int32_t nw = gridDim.x * kLvWarps;
+  const int32_t per = pull_words_per_warp(a.nwords, nw);
+  PullWarp &pw = sm.pull[wid];
+  uint8_t *mark = (uint8_t *)pw.mark;
   uint32_t found_cnt = 0;
   unsigned long long found_deg = 0;
   uint32_t found_max = 0;
-  for (long long gi = gw; gi < groups; gi += nw) {  // warp-uniform loop
-    const long long w0 = gi * kPullWords;
-    uint32_t vis[kPullWords];
-    int32_t v[kPullWords], r0[kPullWords], r1[kPullWords], uf[kPullWords];
-    bool act[kPullWords], fnd[kPullWords];
-#pragma unroll
-    for (int j = 0; j < kPullWords; ++j) {
-      const long long w = w0 + j;
-      vis[j] = w < a.nwords ? a.visited[w] : 0xFFFFFFFFu;
-      v[j] = (int32_t)(w * 32 + lane);
-      act[j] = w < a.nwords && v[j] < a.n && !((vis[j] >> lane) & 1u);
-      fnd[j] = false;
-      uf[j] = -1;
-      r0[j] = r1[j] = 0;
-    }
-    // row bounds and the first neighbour (from the dense first-neighbour
-    // array: coalesced, and not waiting for the row offset) of every
-    // unvisited vertex, independent loads
-    int32_t u1[kPullWords];
-#pragma unroll
-    for (int j = 0; j < kPullWords; ++j) {
-      u1[j] = -1;
-      if (act[j]) {
-        r0[j] = a.R[v[j]];
-        r1[j] = a.R[v[j] + 1];
-        u1[j] = a.first[v[j]];
+  auto found = [&](bool f, int32_t v, int32_t o, int32_t u, int32_t d) {
+    if (!f) return;
+    mark[o] = 1;
+    if (parent) parent[v] = u;
+    ++found_cnt;
+    found_deg += (unsigned long long)d;
+    found_max = max(found_max, (uint32_t)d);
+  };
+  for (int32_t i0 = 0; i0 < per; i0 += kPullBatch) {  // warp-uniform
+    const int32_t words = min(kPullBatch, per - i0);
+    // lane i holds word i of the step: its place, its visited bits
+    int32_t w = a.nwords;
+    uint32_t vis = 0xFFFFFFFFu;
+    if (lane < words) {
+      const int64_t at = pull_word(gw, nw, i0 + lane);
+      if (at < a.nwords) {
+        w = (int32_t)at;
+        vis = a.visited[w];
+        if (w == a.nwords - 1 && (a.n & 31)) vis |= ~((1u << (a.n & 31)) - 1u);
       }
     }
+    const uint32_t todo = __ballot_sync(0xffffffffu, vis != 0xFFFFFFFFu);
+    if (!todo) continue;
+    for (int i = lane; i < kPullBatch * 2; i += 32) pw.mark[i] = make_uint4(0u, 0u, 0u, 0u);
+    int32_t total = 0;
+    for (uint32_t t = todo; t; t &= t - 1u) {
+      const int i = __ffs(t) - 1;
+      const uint32_t live = ~__shfl_sync(0xffffffffu, vis, i);
+      if ((live >> lane) & 1u) pw.list[total + __popc(live & below)] = (uint16_t)(i * 32 + lane);
+      total += __popc(live);
+    }
+    __syncwarp();
+    // first neighbours, from their dense array: coalesced, and not waiting
+    // for the row offset
+    int32_t left = 0;
+    for (int32_t k0 = 0; k0 < total; k0 += 32 * kPullItems) {
+      int32_t o[kPullItems], v[kPullItems], r0[kPullItems], r1[kPullItems], u1[kPullItems];
+      bool hit[kPullItems];
 #pragma unroll
-    for (int j = 0; j < kPullWords; ++j) {
-      if (!GR_IN(r0[j], a.m + 1, 120) || !GR_IN(r1[j], a.m + 1, 121)) {
-        r1[j] = r0[j] = 0;
+      for (int j = 0; j < kPullItems; ++j) {
+        const int32_t k = k0 + j * 32 + lane;
+        o[j] = k < total ? (int32_t)pw.list[k] : 0;
+        v[j] = __shfl_sync(0xffffffffu, w, o[j] >> 5) * 32 + (o[j] & 31);
+        r0[j] = r1[j] = 0;
         u1[j] = -1;
-      }
-      if (u1[j] >= 0 && !GR_IN(u1[j], a.n, 122)) u1[j] = -1;
-    }
-#pragma unroll
-    for (int j = 0; j < kPullWords; ++j)
-      if (u1[j] >= 0 && test_bit(F, u1[j])) {
-        fnd[j] = true;
-        uf[j] = u1[j];
-      }
-    // the rest of each list: lanes alone up to kPullLane more neighbours,
-    // then the whole warp on whatever is left, 32 neighbours at a time
-#pragma unroll
-    for (int j = 0; j < kPullWords; ++j) {
-      if (act[j] && !fnd[j]) {
-        const int32_t stop = min(r1[j], r0[j] + 1 + kPullLane);
-        for (int32_t e = r0[j] + 1; e < stop; ++e) {
-          const int32_t u = a.C[e];
-          if (GR_IN(u, a.n, 123) && test_bit(F, u)) {
-            fnd[j] = true;
-            uf[j] = u;
-            break;
-          }
+        if (k < total && GR_IN(v[j], a.n, 119)) {
+          r0[j] = a.R[v[j]];
+          r1[j] = a.R[v[j] + 1];
+          u1[j] = a.first[v[j]];
         }
       }
-      uint32_t longm =
-          __ballot_sync(0xffffffffu, act[j] && !fnd[j] && r1[j] - r0[j] > 1 + kPullLane);
+#pragma unroll
+      for (int j = 0; j < kPullItems; ++j) {
+        if (!GR_IN(r0[j], a.m + 1, 120) || !GR_IN(r1[j], a.m + 1, 121)) {
+          r1[j] = r0[j] = 0;
+          u1[j] = -1;
+        }
+        if (u1[j] >= 0 && !GR_IN(u1[j], a.n, 122)) u1[j] = -1;
+        hit[j] = u1[j] >= 0 && test_bit(F, u1[j]);
+      }
+      __syncwarp();  // the list entries above are read before any is replaced
+#pragma unroll
+      for (int j = 0; j < kPullItems; ++j) {
+        found(hit[j], v[j], o[j], u1[j], r1[j] - r0[j]);
+        const bool more = !hit[j] && r1[j] - r0[j] > 1;
+        const uint32_t mm = __ballot_sync(0xffffffffu, more);
+        if (more) pw.list[left + __popc(mm & below)] = (uint16_t)o[j];
+        left += __popc(mm);
+      }
+      __syncwarp();
+    }
+    // the rest of the lists
+    for (int32_t k0 = 0; k0 < left; k0 += 32) {
+      const int32_t k = k0 + lane;
+      const int32_t o = k < left ? (int32_t)pw.list[k] : 0;
+      const int32_t v = __shfl_sync(0xffffffffu, w, o >> 5) * 32 + (o & 31);
+      int32_t r0 = 0, r1 = 0, uf = -1;
+      if (k < left && GR_IN(v, a.n, 123)) {
+        r0 = a.R[v];
+        r1 = a.R[v + 1];
+        const int32_t stop = min(r1, r0 + 1 + kPullLane);
+        for (int32_t e = r0 + 1; e < stop && uf < 0; e += 4) {
+          int32_t u[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) u[i] = e + i < stop ? a.C[e + i] : -1;
+          uint32_t bit[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            bit[i] = (u[i] >= 0 && GR_IN(u[i], a.n, 117)) ? test_bit(F, u[i]) : 0u;
+#pragma unroll
+          for (int i = 3; i >= 0; --i)
+            if (bit[i]) uf = u[i];
+        }
+      }
+      uint32_t longm = __ballot_sync(0xffffffffu, uf < 0 && r1 - r0 > 1 + kPullLane);
       while (longm) {
         const int leader = __ffs(longm) - 1;
         longm &= longm - 1u;
-        const int32_t b0 = __shfl_sync(0xffffffffu, r0[j], leader) + 1 + kPullLane;
-        const int32_t b1 = __shfl_sync(0xffffffffu, r1[j], leader);
-        for (int32_t base = b0; base < b1; base += 32) {
-          const int32_t e = base + lane;
-          const int32_t u = e < b1 ? a.C[e] : 0;
-          const bool hit = e < b1 && GR_IN(u, a.n, 124) && test_bit(F, u);
-          const uint32_t hb = __ballot_sync(0xffffffffu, hit);
+        const int32_t b0 = __shfl_sync(0xffffffffu, r0, leader) + 1 + kPullLane;
+        const int32_t b1 = __shfl_sync(0xffffffffu, r1, leader);
+        for (int32_t base = b0; base < b1; base += 128) {
+          int32_t x = -1;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int32_t e = base + 32 * i + lane;
+            const int32_t u = e < b1 ? a.C[e] : -1;
+            if (u >= 0 && GR_IN(u, a.n, 124) && test_bit(F, u)) x = u;
+          }
+          const uint32_t hb = __ballot_sync(0xffffffffu, x >= 0);
           if (hb) {
-            const int32_t hu = __shfl_sync(0xffffffffu, u, __ffs(hb) - 1);
-            if (lane == leader) {
-              fnd[j] = true;
-              uf[j] = hu;
-            }
+            x = __shfl_sync(0xffffffffu, x, __ffs(hb) - 1);
+            if (lane == leader) uf = x;
             break;
           }
         }
       }
-      const uint32_t fm = __ballot_sync(0xffffffffu, fnd[j]);
-      const long long w = w0 + j;
-      if (w < a.nwords && lane == 0) {
-        N[w] = fm;
-        if (fm) a.visited[w] = vis[j] | fm;
-      }
-      if (fnd[j]) {
-        depth[v[j]] = L + 1;
-        if (parent) parent[v[j]] = uf[j];
-        ++found_cnt;
-        found_deg += (unsigned long long)(r1[j] - r0[j]);
-        found_max = max(found_max, (uint32_t)(r1[j] - r0[j]));
-      }
-      if (a.seg_v && fm) {  // append to this block's segment (shared-memory slot)
-        int32_t pos = 0;
-        if (lane == 0) pos = atomicAdd(&sm.segcnt, __popc(fm));
-        pos = __shfl_sync(0xffffffffu, pos, 0);
-        if (fnd[j]) {
-          const int64_t kk = pos + __popc(fm & ((1u << lane) - 1u));
-          const int64_t k = (int64_t)blockIdx.x * a.seg_cap + kk;
-          if (GR_IN(kk, a.seg_cap, 125)) {
-            a.seg_v[k] = v[j];
-            a.seg_d[k] = r1[j] - r0[j];
-          }
-        }
-      }
+      found(uf >= 0, v, o, uf, r1 - r0);
     }
+    __syncwarp();
+    // marks to bitmap words and depths
+    uint32_t fm = 0;
+    for (uint32_t t = todo; t; t &= t - 1u) {
+      const int i = __ffs(t) - 1;
+      const bool f = mark[i * 32 + lane] != 0;
+      const uint32_t b = __ballot_sync(0xffffffffu, f);
+      if (lane == i) fm = b;
+      const int32_t wi = __shfl_sync(0xffffffffu, w, i);
+      if (f) depth[wi * 32 + lane] = L + 1;
+    }
+    if (fm) {
+      N[w] = fm;
+      a.visited[w] = vis | fm;
+    }
+    __syncwarp();
   }
   if (maxdeg) {
     const uint32_t wmax = __reduce_max_sync(0xffffffffu, found_max);
@@ -599,6 +667,41 @@ __device__ void pull_level(const BfsArgs &a, BfsCtl *c, LevelSmem &sm, int32_t L
     if (packed) atomicAdd(counter, packed);
     if (a.seg_v) a.seg_cnt[blockIdx.x] = packed;
   }
+}
+
+// The vertices of the frontier F that this block's warps found in the last
+// pull level, with their degrees, into the block's segment. (Written by each
+// pull level as it found them they cost 4 of 113 us on R-MAT 2^22, and most
+// pull levels are followed by another.)
+__device__ void collect_found(const BfsArgs &a, LevelSmem &sm, const uint32_t *F) {
+  const int lane = threadIdx.x & 31;
+  const int32_t gw = blockIdx.x * kLvWarps + (threadIdx.x >> 5);
+  const int32_t nw = gridDim.x * kLvWarps;
+  const int32_t per = pull_words_per_warp(a.nwords, nw);
+  const int64_t base = (int64_t)blockIdx.x * a.seg_cap;
+  for (int32_t i0 = 0; i0 < per; i0 += 32) {  // warp-uniform
+    const int64_t at = i0 + lane < per ? pull_word(gw, nw, i0 + lane) : a.nwords;
+    const int32_t w = (int32_t)min(at, (int64_t)a.nwords);
+    const uint32_t bits = w < a.nwords ? F[w] : 0u;
+    const uint32_t incl = warp_incl_sum((uint32_t)__popc(bits));
+    const uint32_t all = __shfl_sync(0xffffffffu, incl, 31);
+    if (!all) continue;
+    int32_t at0 = 0;
+    if (lane == 0) at0 = atomicAdd(&sm.segcnt, (int32_t)all);
+    at0 = __shfl_sync(0xffffffffu, at0, 0);
+    for (uint32_t t = __ballot_sync(0xffffffffu, bits != 0u); t; t &= t - 1u) {
+      const int i = __ffs(t) - 1;
+      const uint32_t b = __shfl_sync(0xffffffffu, bits, i);
+      const int32_t k0 = at0 + (int32_t)__shfl_sync(0xffffffffu, incl, i) - __popc(b);
+      const int32_t v = __shfl_sync(0xffffffffu, w, i) * 32 + lane;
+      const int32_t k = k0 + __popc(b & ((1u << lane) - 1u));
+      if (((b >> lane) & 1u) && GR_IN(v, a.n, 125) && GR_IN(k, a.seg_cap, 116)) {
+        a.seg_v[base + k] = v;
+        a.seg_d[base + k] = a.R[v + 1] - a.R[v];
+      }
+    }
+  }
+  __syncthreads();
 }
 
 // Queue + degree scan of the vertices the last pull level found, from the
@@ -851,15 +954,18 @@ __global__ void __launch_bounds__(kLvThreads, kLvBlocksPerSm)
 
 __device__ __forceinline__ bool grid_barrier(BfsCtl *c, int32_t nblocks, int32_t &gen);
 
-// 6 blocks of 256 threads per SM (40 registers, no spills) took R-MAT s22
-// from 0.1976 to 0.1900 ms per traversal against 5 (48 registers); 7 or more
-// spill
-constexpr int kDoBlocksPerSm = 6;
+// Blocks per SM of a push-only search and of one that also pulls. Pushing
+// wants warps in flight (a directed graph of 3 M entries: 6 blocks 108 us, 4
+// blocks 111); a pull level's warps have many loads in flight each, and more of
+// them only meet at the barrier: R-MAT 2^22 113 us at 4 blocks and their 64
+// registers, 119 at 4 with 40 registers, 130 at 6.
+constexpr int kDoBlocksPerSm = 6, kPullBlocksPerSm = 4;
 // After a pull level whose found vertices all have at most this degree, each
 // block pushes its own pull segment (no grid-wide compaction).
 constexpr int32_t kSegPushMaxDeg = 1024;
 
-__global__ void __launch_bounds__(kLvThreads, kDoBlocksPerSm) k_bfs_do(BfsArgs a) {
+template <int BPS>
+__global__ void __launch_bounds__(kLvThreads, BPS) k_bfs_do(BfsArgs a) {
   BfsCtl *c = a.ctl;
   __shared__ LevelSmem sm;
   // a traversal the one-cluster driver finished, or one it hands over at
@@ -892,10 +998,12 @@ __global__ void __launch_bounds__(kLvThreads, kDoBlocksPerSm) k_bfs_do(BfsArgs a
     if (dir == kPull) {
       pull_level(a, c, sm, L, counter, &c->maxdeg3[L % 3]);
     } else if (from_bitmap && seg_maxdeg <= kSegPushMaxDeg) {
+      collect_found(a, sm, bits_of(a, L));
       push_own_segment(a, c, sm, parity, L, counter);
     } else {
       int32_t qq = q, qe = (int32_t)mf;
       if (from_bitmap) {
+        collect_found(a, sm, bits_of(a, L));
         segments_to_queue(a, sm, queue_of(a, parity), scan_of(a, parity), &qq, &qe);
         if (!grid_barrier(c, gridDim.x, gen)) break;
       }
@@ -1121,6 +1229,7 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_bfs_solo(BfsArgs a) {
 // of the unexplored ones a level, a push-only one all of them (53,000 entries:
 // 60 us here, 45 on a grid of one block per SM).
 constexpr int kSmallThreads = 1024;
+constexpr int kPullWords = 2;  // bitmap words a warp pulls at once
 constexpr int32_t kSmallMaxN = 32768;
 constexpr int64_t kSmallMaxM = 1 << 20, kSmallMaxPushM = 1 << 14;
 
@@ -1720,7 +1829,7 @@ static size_t solo_smem(const gr_graph *g) {
 size_t bfs_ws_bytes(const gr_graph *g) {
   const size_t n = (size_t)g->n;
   const size_t seg = (size_t)g->nwords * 32 +
-                     (size_t)g->num_sms * kDoBlocksPerSm * kLvWarps * kPullWords * 32;
+                     (size_t)g->num_sms * kDoBlocksPerSm * kLvWarps * 32;
   return 2 * sizeof(int32_t) * (n + 1) + 2 * sizeof(int32_t) * (n + 2) +
          4 * sizeof(uint32_t) * (size_t)g->nwords + 2 * sizeof(int32_t) * seg +
          sizeof(BfsCtl) + (solo_smem(g) ? 16 * n : 0);
@@ -1740,7 +1849,7 @@ gr_status bfs_ws_create(gr_graph *g, cudaStream_t s, BfsWorkspace **out) {
     // segment capacity for any persistent grid of num_sms .. num_sms *
     // kDoBlocksPerSm blocks (see bfs_run)
     const size_t max_blocks = (size_t)g->num_sms * kDoBlocksPerSm;
-    const size_t entries = (size_t)g->nwords * 32 + max_blocks * kLvWarps * kPullWords * 32;
+    const size_t entries = (size_t)g->nwords * 32 + max_blocks * kLvWarps * 32;
     GR_TRY(ws->seg_v.alloc(sizeof(int32_t) * entries, "pull segments"));
     GR_TRY(ws->seg_d.alloc(sizeof(int32_t) * entries, "pull segment degrees"));
     GR_TRY(ws->seg_cnt.alloc(sizeof(unsigned long long) * max_blocks, "pull segment counts"));
@@ -1910,17 +2019,14 @@ gr_status bfs_run(gr_graph *g, BfsWorkspace *ws, int32_t src, int32_t *depth, in
     GR_CUDA(cudaGraphLaunch(ws->exec[do_bitmap], s));
   } else if (mode == GR_MODE_PERSISTENT) {
     int per_sm = 0;
-    GR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bfs_do, kLvThreads, 0));
-    int bps = std::min(per_sm, kDoBlocksPerSm);
+    void *kern = do_bitmap ? (void *)k_bfs_do<kPullBlocksPerSm> : (void *)k_bfs_do<kDoBlocksPerSm>;
+    GR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kLvThreads, 0));
+    int bps = std::min(per_sm, do_bitmap ? kPullBlocksPerSm : kDoBlocksPerSm);
     const int32_t want = o.block > 0 ? o.block : g->tuned_blocks_per_sm;
     if (want > 0) bps = std::min(bps, want);
     const int blocks = std::max(1, bps) * g->num_sms;
-    // per-block segments for the pull levels: a block handles at most
-    // `rounds` groups of kPullWords words per warp
-    const long long groups = (g->nwords + kPullWords - 1) / kPullWords;
-    const long long per_round = (long long)blocks * kLvWarps;
-    const long long rounds = (groups + per_round - 1) / per_round;
-    a.seg_cap = (int32_t)(rounds * kLvWarps * kPullWords * 32);
+    // per-block segments for the pull levels
+    a.seg_cap = pull_words_per_warp(g->nwords, blocks * kLvWarps) * kLvWarps * 32;
     if ((size_t)blocks * a.seg_cap > ws->seg_v.bytes / sizeof(int32_t))
       return fail(GR_ECUDA, "pull segment buffer too small");
     a.seg_v = ws->seg_v.as<int32_t>();
@@ -1930,15 +2036,15 @@ gr_status bfs_run(gr_graph *g, BfsWorkspace *ws, int32_t src, int32_t *depth, in
     // their visited bitmap does not fit it, in one cluster first
     const size_t solo = a.low_degree ? solo_smem(g) : 0;
     if (solo) {
-      auto kern = g->max_degree > 4 ? k_bfs_solo<true> : k_bfs_solo<false>;
-      GR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)solo));
-      kern<<<1, kSoloThreads, solo, s>>>(a);
+      auto one = g->max_degree > 4 ? k_bfs_solo<true> : k_bfs_solo<false>;
+      GR_CUDA(cudaFuncSetAttribute(one, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)solo));
+      one<<<1, kSoloThreads, solo, s>>>(a);
       GR_CUDA(cudaGetLastError());
     } else if (a.low_degree) {
       GR_TRY(launch_cluster_bfs(a, s));
     }
     void *args[] = {&a};
-    GR_CUDA(cudaLaunchCooperativeKernel((void *)k_bfs_do, blocks, kLvThreads, args, 0, s));
+    GR_CUDA(cudaLaunchCooperativeKernel(kern, blocks, kLvThreads, args, 0, s));
   } else {
     // host-driven: enqueue batches of levels, then check the done flag
     BfsCtl *h = ws->h_ctl.as<BfsCtl>();

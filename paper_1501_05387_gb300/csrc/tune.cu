@@ -45,16 +45,16 @@ void tune_prior(gr_graph *g) {
   } else {
     g->tuned_direction = GR_DIR_AUTO;
     // Small graphs are bound by the grid barrier, whose cost grows with the
-    // blocks that meet at it. BFS at 1, 2, 3, 4 and 6 blocks per SM: R-MAT
-    // 2^12 (0.1 M entries) 42, 48, 48, 49, 55 us; 2^16 (1.8 M) 48, 54, 56, 59,
-    // 70; 2^18 (7.6 M) 87, 77, 78, 71, 77; 2^21 (64 M) 234, 158, 137, 123, 126;
-    // 2^22 (128 M) 426, 260, 211, 188, 180.
+    // blocks that meet at it. BFS at 1, 2, 3 and 4 blocks per SM (means of eight
+    // sources): R-MAT 1.8 M entries 47, 52, 54, 57 us; 7.6 M 58, 63, 65, 68; 15 M
+    // 66, 68, 71, 73; 24 M, ids at random, 91, 85, 85, 87; 31 M 98, 88, 85, 87;
+    // 64 M, ids at random, 160, 120, 110, 108; 128 M 162, 116, 109, 105.
     // Directed graphs push every level, which takes more of them (three graphs
     // each at 1 to 6): 0.1 M entries 51, 55, 57, 59, 61, 64 us; 0.47 M 75, 74,
     // 72, 75, 77, 80; 1 M 99, 84, 80, 80, 81, 81; 2.2 M 149, 111, 99, 95, 94, 93;
     // 3 M 190, 136, 115, 111, 106, 108.
     if (g->symmetric)
-      g->tuned_blocks_per_sm = g->m < 4'000'000 ? 1 : g->m < 96'000'000 ? 4 : 0;
+      g->tuned_blocks_per_sm = g->m < 20'000'000 ? 1 : g->m < 48'000'000 ? 3 : 4;
     else
       g->tuned_blocks_per_sm = g->m < 150'000 ? 1 : g->m < 700'000 ? 3 : g->m < 1'500'000 ? 4 : 0;
     // SSSP at 1 to 5: 2^12 101, 115, 123, 126, 141 us; 2^14 (0.4 M) 158, 143,
