@@ -70,6 +70,9 @@ __device__ __forceinline__ float u16_to_float(uint32_t p) {
 // A uint64 path count as double-single (its four 16-bit pieces, each exact
 // as a float, summed without losing more than the last of 64 bits' worth).
 __device__ __forceinline__ DS ds_from_u64(unsigned long long c) {
+  if (c >> 32 == 0ull)  // the same sum without the pieces that are 0
+    return ds_fast_two_sum(__fmul_rn(u16_to_float((uint32_t)c >> 16), 65536.f),
+                           u16_to_float((uint32_t)c & 0xFFFFu));
   DS r{__fmul_rn(u16_to_float((uint32_t)(c >> 48)), 281474976710656.f), 0.f};  // 2^48
   r = ds_add_f(r, __fmul_rn(u16_to_float((uint32_t)(c >> 32) & 0xFFFFu), 4294967296.f));
   r = ds_add_f(r, __fmul_rn(u16_to_float((uint32_t)(c >> 16) & 0xFFFFu), 65536.f));
@@ -114,9 +117,6 @@ __device__ __forceinline__ double ds_to_double(DS a) {
 __device__ __forceinline__ DS shfl_xor_ds(DS a, int o) {
   return {__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
 }
-
-// r += x, both of any sign and size.
-__device__ __forceinline__ void ds_acc(DS &r, DS x) { r = ds_add(r, x); }
 
 // |a - b| exactly, as hi + lo.
 __device__ __forceinline__ DS ds_abs_diff(float a, float b) {
