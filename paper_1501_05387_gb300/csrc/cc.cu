@@ -18,8 +18,8 @@
 //
 // Symmetric graphs store each undirected edge twice, so most edges need no
 // visit at all: the sampling form of the hooking sweep starts every vertex
-// under its first neighbour (where that has the smaller id: no cycle, and no
-// atomic), hooks it to the second and compresses, which on graphs
+// under the end of a short chain of first neighbours (each with a smaller id:
+// no cycle, and no atomic), hooks it to the second and compresses, which on graphs
 // with one giant component already places most vertices in it; the
 // component that most of a fixed sample of vertices lies in is then
 // skipped, and only the vertices outside it hook all their edges (an edge
@@ -47,12 +47,24 @@ GR_GUARD_REPORTER(guard_report_cc)
 
 namespace {
 
-// first (may be null): the vertices' first neighbours, -1 where there is none
+// first (may be null): the vertices' first neighbours, -1 where there is none.
+// A vertex starts under the end of the chain of first neighbours of ever
+// smaller ids, if that ends within kCcChain steps (on a skewed graph, at a hub),
+// and else on its own: a mesh's chains are as long as its side, a path's as the
+// graph, and trees that deep would make every later walk to the root as long
+// (linked all the way, a path of 4 M vertices took 2.7 ms).
+constexpr int kCcChain = 8;
 __global__ void k_cc_init(int32_t *label, const int32_t *first, int32_t n) {
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
        v += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t u = first ? first[v] : -1;
-    label[v] = u >= 0 && u < v ? u : (int32_t)v;
+    int32_t x = (int32_t)v;
+    bool end = !first;
+    for (int i = 0; i < kCcChain && !end; ++i) {
+      const int32_t u = first[x];
+      end = u < 0 || u >= x || !GR_IN(u, n, 404);
+      if (!end) x = u;
+    }
+    label[v] = end ? x : (int32_t)v;
   }
 }
 
@@ -100,10 +112,58 @@ struct HookF {
   }
 };
 
+// The sampling pass's form of hook. Its walks write only the entry of the
+// thread's own vertex: halving a path on the way, as find_root does, makes
+// every thread below a hub's root store to the same few entries, and an entry
+// read from a stale L1 line can put an older ancestor back (R-MAT with ids at
+// random, 2^20 vertices: the pass alone 350 us). An own entry only ever moves
+// up, and is what other walks through the vertex follow: together they double
+// their steps as halving would. Lanes that meet at one root send one CAS.
+__device__ __forceinline__ int32_t walk(const int32_t *label, int32_t x) {
+  int32_t p = label[x];
+  while (p != x) {
+    x = p;
+    p = label[x];
+  }
+  return x;
+}
+
+__device__ __forceinline__ int32_t walk_own(int32_t *label, int32_t v) {
+  int32_t p = label[v];
+  if (p == v) return v;
+  for (;;) {
+    const int32_t gp = label[p];
+    if (gp == p) return p;
+    label[v] = gp;  // v is no root: nobody else writes its entry
+    p = gp;
+  }
+}
+
+__device__ __forceinline__ void hook_own(int32_t *label, int32_t v, int32_t x) {
+  int32_t a = walk_own(label, v);
+  int32_t b = walk(label, x);
+  while (a != b) {
+    const int32_t hi = max(a, b), lo = min(a, b);
+    const uint32_t peers = __match_any_sync(__activemask(), hi);
+    const int leader = __ffs(peers) - 1;
+    int32_t prev = 0;
+    if ((threadIdx.x & 31) == leader) prev = atomicCAS(label + hi, hi, lo);
+    prev = __shfl_sync(peers, prev, leader);
+    const int32_t under = __shfl_sync(peers, lo, leader);
+    if (prev == hi) {  // hooked under the leader's root
+      if (under == lo) break;
+      prev = under;
+    }
+    a = walk(label, prev);
+    b = walk(label, lo);
+  }
+}
+
 // Each vertex hooks to its second neighbour, and to its first where
-// k_cc_init could not start it there. The trees are shallow by then and most
-// pairs share one already: R-MAT 2^22 143 us when all vertices hooked both
-// neighbours from themselves on, their roots' CASes in each other's way.
+// k_cc_init left it on its own. The trees are shallow by then and most pairs
+// share one already: R-MAT 2^22 151 us, 240 when all vertices start on their
+// own; ids at random, 2^20: 130 (350 us with halving walks), 2^18 90 (570);
+// grids 300 and 700 a side 125 and 145 (155 and 235).
 __global__ void k_cc_sample(const int32_t *R, const int32_t *C, const int32_t *first, int32_t n,
                             int32_t *label) {
   for (int64_t vv = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; vv < n;
@@ -112,10 +172,10 @@ __global__ void k_cc_sample(const int32_t *R, const int32_t *C, const int32_t *f
     const int32_t u = first[v];
     if (u < 0) continue;
     const int32_t r = R[v] + 1;
-    if (u > v) hook(label, v, u);
+    if (label[v] == v) hook_own(label, v, u);
     if (r < R[v + 1]) {
       const int32_t x = C[r];
-      if (GR_IN(x, n, 403)) hook(label, v, x);
+      if (GR_IN(x, n, 403)) hook_own(label, v, x);
     }
   }
 }
@@ -220,8 +280,10 @@ __global__ void k_cc_jump(int32_t *label, int32_t n, int32_t *num_roots) {
   int32_t roots = 0;
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
        v += (int64_t)gridDim.x * blockDim.x) {
-    // halving on the way: a mesh's chains of first neighbours are long
-    const int32_t r = find_root(label, (int32_t)v);
+    // a walk that writes nothing on the way: halving another vertex's path
+    // here could put an older ancestor back over the root it has been given
+    int32_t r = label[v];
+    while (label[r] != r) r = label[r];
     label[v] = r;
     roots += r == v;
   }

@@ -160,3 +160,20 @@ def test_pagerank_cc_rmat_s23(cuda_lib):
         lab, k = run_cc(cuda_lib, g)
         ref_l, k_ref = oracle.cc(r, c)
         assert np.array_equal(lab, ref_l) and k == k_ref
+
+
+@pytest.mark.parametrize("order", ["ascending", "descending", "random"])
+def test_cc_long_path_rows_in_any_order(cuda_lib, order):
+    # a path through all vertices in id order: every vertex starts under the
+    # one before it, a chain of 200,000, or (rows turned round) under none
+    n = 200_000
+    r, c = gg.from_edges(n, [(i, i + 1) for i in range(n - 1) if i % 70_001 != 70_000])
+    if order != "ascending":
+        rng = np.random.default_rng(2)
+        for v in np.nonzero(np.diff(r) == 2)[0]:
+            if order == "descending" or rng.random() < 0.5:
+                c[r[v]:r[v + 1]] = c[r[v]:r[v + 1]][::-1]
+    ref, k_ref = oracle.cc(r, c)
+    with cuda_lib.gr_graph_create(r, c) as g:
+        lab, k = run_cc(cuda_lib, g)
+        assert np.array_equal(lab, ref) and k == k_ref
