@@ -80,7 +80,8 @@ enum {
 typedef struct gr_opts {
   int32_t direction;  /* GR_DIR_* */
   int32_t mode;       /* GR_MODE_* */
-  int32_t block;      /* persistent BFS: blocks per SM (0: tuned) */
+  int32_t block;      /* persistent BFS: blocks per SM (0: tuned), at most
+                         those resident: 4 where it may pull, else 6 */
   int32_t chunk;      /* merge-path items per block chunk (0: tuned) */
   float alpha;        /* push->pull when frontier edges > unexplored/alpha */
   float beta;         /* pull->push when frontier vertices < n/beta */

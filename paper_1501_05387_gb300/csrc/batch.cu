@@ -5,8 +5,8 @@
 // idea of Then et al., VLDB 2014). Per vertex v a 64-bit mask lm[L][v] holds
 // the lanes whose frontier at level L contains v; visit[v] the lanes that
 // reached v at an earlier level. One level is a pull over all vertices
-// (the all-vertex frontier of the load-balanced advance, merge-path chunks,
-// lanes over edges): for an edge (v, u), bits = lm[L][u] & ~visited(v) are
+// (batched BFS: in 256-entry register tiles over the rows that miss a lane; BC:
+// in merge-path chunks, one per warp): for an edge (v, u), bits = lm[L][u] & ~visited(v) are
 // the lanes in which u is a predecessor of v, and v joins lm[L+1] in those
 // lanes. Every column index is read once per level; the 64 traversals share
 // that read.
