@@ -158,8 +158,7 @@ def _graph(case, seed):
     if "wmax" in case:
         # equal for both directions of an edge: a hash of its ends and the seed
         c = col.long()
-        salt = (seed * 7_046_029_254_386_353 + 2**63) % 2**64 - 2**63  # within int64
-        h = torch.minimum(row, c) * n + torch.maximum(row, c) + salt
+        h = torch.minimum(row, c) * n + torch.maximum(row, c) + seed * 7_046_029_254_386_353
         h = (h ^ (h >> 31)) * 0x2545F4914F6CDD1D
         h = (h ^ (h >> 29)) * 0x5851F42D4C957F2D
         w = (((h >> 33) & 0x3FFFFFFF) % case["wmax"] + 1).int()
