@@ -1265,7 +1265,7 @@ static SsspArgs sssp_args(gr_graph *g, SsspWorkspace *ws, int32_t lanes = 1) {
   a.ctl = ws->ctl.as<SsspCtl>();
   a.low_degree = g->max_degree <= kLowDegreeMax ? 1 : 0;
   a.adjw = g->adjw4.as<int4>();
-  a.plan = ws->plan.a;  // null for batched workspaces, which never pull
+  a.plan = ws->plan.a;  // null where nothing may be pulled (sssp_pull_min_edges)
   a.lowered = ws->lowered.as<uint32_t>();
   a.qcb = ws->qcb.as<int32_t>();  // null on low-degree graphs
   return a;
@@ -1273,10 +1273,14 @@ static SsspArgs sssp_args(gr_graph *g, SsspWorkspace *ws, int32_t lanes = 1) {
 
 // Smallest near-frontier edge count at which a relaxation pulls: m /
 // opts->alpha, else m / the graph's tuned alpha (0: never); GR_DIR_PUSH
-// never pulls, GR_DIR_PULL pulls every relaxation. A graph whose rows are not
-// its in-edges (weights that differ by direction among them) is only pushed.
-static long long sssp_pull_min_edges(const gr_graph *g, const gr_opts &o, int32_t lanes) {
-  if (lanes != 1 || !can_pull(g) || o.direction == GR_DIR_PUSH) return LLONG_MAX;
+// never pulls, GR_DIR_PULL pulls every relaxation. Only a single search on a
+// workspace with a plan pulls: one made for several lanes has none, whatever
+// the number of sources it is used for, nor has that of a graph whose rows are
+// not its in-edges (weights that differ by direction among them).
+static long long sssp_pull_min_edges(const gr_graph *g, const SsspWorkspace *ws, const gr_opts &o,
+                                     int32_t lanes) {
+  if (lanes != 1 || !ws->plan.a.desc || !ws->lowered.p || o.direction == GR_DIR_PUSH)
+    return LLONG_MAX;
   if (o.direction == GR_DIR_PULL) return 1;
   const double div = o.alpha > 0.f ? (double)o.alpha : (double)g->tuned_sssp_alpha;
   if (div <= 0.0) return LLONG_MAX;
@@ -1364,11 +1368,12 @@ static gr_status sssp_drive(gr_graph *g, SsspWorkspace *ws, SsspArgs a, const Ss
                             uint32_t *dist, int32_t *pred, int32_t mode, const gr_opts &o,
                             cudaStream_t s) {
   const int32_t max_iters = sssp_max_iters_of(g, o);
+  const long long pull_min_edges = sssp_pull_min_edges(g, ws, o, src.k);
   // meshes whose membership bits fit one block's shared memory: one block
   // per search, up to the frontier size where the grid takes over
   const size_t near_only = mode == GR_MODE_PERSISTENT ? solo_smem(g, false) : 0;
   k_sssp_init<<<g->num_sms * 8, 256, 0, s>>>(a, src, dist, pred, sssp_delta_of(g, o), max_iters,
-                                             sssp_pull_min_edges(g, o, src.k), near_only > 0);
+                                             pull_min_edges, near_only > 0);
   GR_CUDA(cudaGetLastError());
   if (near_only) {
     const size_t both = solo_smem(g, true), bytes = both ? both : near_only;
@@ -1381,8 +1386,8 @@ static gr_status sssp_drive(gr_graph *g, SsspWorkspace *ws, SsspArgs a, const Ss
   }
   if (mode == GR_MODE_PERSISTENT) {
     void *kern = a.low_degree ? (void *)k_sssp_do<true, false>
-                 : sssp_pull_min_edges(g, o, src.k) < LLONG_MAX ? (void *)k_sssp_do<false, true>
-                                                                : (void *)k_sssp_do<false, false>;
+                 : pull_min_edges < LLONG_MAX ? (void *)k_sssp_do<false, true>
+                                              : (void *)k_sssp_do<false, false>;
     const int32_t want = o.block > 0 ? o.block : g->tuned_sssp_blocks_per_sm;
     // the carveout fitted to the blocks that run leaves the rest to L1
     int bps = 1;
