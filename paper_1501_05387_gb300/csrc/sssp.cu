@@ -1398,14 +1398,19 @@ static gr_status sssp_drive(gr_graph *g, SsspWorkspace *ws, SsspArgs a, const Ss
     GR_CUDA(cudaLaunchCooperativeKernel(kern, std::max(1, bps) * g->num_sms,
                                         kSsspThreads, args, 0, s));
   } else if (mode == GR_MODE_LAUNCH) {
+    // the device ends the run, at its iteration limit at the latest; a pulled
+    // iteration takes two launches
     SsspCtl h;
-    int32_t enq = 0, batch = 8;
+    const long long most = 2ll * max_iters + 2;
+    long long enq = 0;
+    int32_t batch = 8;
     for (;;) {
       for (int i = 0; i < batch; ++i) GR_TRY(sssp_enqueue_iter(g, a, s, 0, 0));
       enq += batch;
       GR_CUDA(cudaMemcpyAsync(&h, a.ctl, sizeof(h), cudaMemcpyDeviceToHost, s));
       GR_CUDA(cudaStreamSynchronize(s));
-      if (h.done || enq > max_iters + 1) break;
+      if (h.done) break;
+      if (enq > most) return fail(GR_ETIMEOUT, "SSSP did not end within its iteration limit");
       batch = std::min(batch * 2, 256);
     }
   } else {

@@ -29,3 +29,30 @@ def test_one_source_after_a_larger_batch(cuda_lib, s12w, mode, direction, alpha)
     with cuda_lib.gr_graph_create(r, c, w) as g:
         for k in (1, 16, 1, 2, 1):
             ts.check_batch(cuda_lib, r, c, w, g, srcs[:k], o)
+
+
+@pytest.mark.parametrize("mode", ["launch", "persistent", "graph"])
+@pytest.mark.parametrize("direction", ["pull", "push", "auto"])
+def test_every_iteration_limit(cuda_lib, mode, direction):
+    """A search either ends within its limit, with the right distances, or
+    reports that it did not, whatever the launches an iteration takes."""
+    # a path through hubs of 20 leaves each: 40 relaxations, one bucket
+    hubs = 40
+    edges = [(i, i + 1) for i in range(hubs - 1)]
+    edges += [(i, hubs + 20 * i + j) for i in range(hubs) for j in range(20)]
+    r, c = gg.from_edges(hubs * 21, edges)
+    w = gg.weights(r, c, seed=3, wmin=1, wmax=64)
+    want = oracle.sssp(r, c, w, 0)[0]
+    o = ts.opts(cuda_lib, 0xFFFFFFFF, mode, direction, 100.0 if direction == "auto" else 0.0)
+    with cuda_lib.gr_graph_create(r, c, w) as g:
+        for limit in list(range(1, 12)) + [20, 21, 22, 23, 30, 38, 39, 40, 41, 42, 100]:
+            o.max_iters = limit
+            try:
+                d, _ = ts.run_sssp(cuda_lib, g, 0, o, with_pred=False)
+            except cuda_lib.GrError as e:
+                assert e.status == cuda_lib.GR_ETIMEOUT and limit < 42, limit
+                continue
+            assert np.array_equal(d, want), limit
+            # a push goes one step further an iteration, and finds its end in
+            # one more; a pull may go further
+            assert direction != "push" or limit >= hubs, limit
