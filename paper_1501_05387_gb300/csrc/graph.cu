@@ -413,7 +413,9 @@ gr_status gr_graph_create(int32_t n, int64_t m, const int32_t *row_off,
   g->num_isolated = hf[2];
   g->rows_sorted = !hr.unsorted;
   g->symmetric = false;
-  if (g->rows_sorted && hr.above == hr.below) {
+  // without repeated columns unequal halves cannot be partners; with them
+  // (0: [1, 1], 1: [0]) they can
+  if (g->rows_sorted && (hr.repeated || hr.above == hr.below)) {
     k_symmetric<<<grid * 2, 256, 0, s>>>(g->row_off.as<int32_t>(), g->col.as<int32_t>(),
                                           w ? g->w.as<uint32_t>() : nullptr, n, !hr.repeated,
                                           f + 4);
