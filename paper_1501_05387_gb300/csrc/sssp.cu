@@ -1180,13 +1180,18 @@ __global__ void k_sssp_pred_fin(int32_t *pred, int32_t n, int32_t src) {
 
 }  // namespace
 
+// Dynamic shared memory k_sssp_solo may take: the compiler rounds its SoloState
+// up (to 48 bytes).
+constexpr size_t kSoloSmemMax = kBlockSmemMax - 64;
+static_assert(sizeof(SoloState) <= 64, "the state does not fit beside the bits");
+
 // Shared memory k_sssp_solo needs on this graph with the far pile's bits in
 // it or not; 0 where the graph is not a mesh or does not fit.
 static size_t solo_smem(const gr_graph *g, bool far_bits) {
   if (g->max_degree > kLowDegreeMax) return 0;
   const size_t bytes = sizeof(int32_t) * (2 * (size_t)kSoloQueue +
                                           (size_t)g->nwords * (far_bits ? 2 : 1));
-  return bytes + sizeof(SoloState) <= kBlockSmemMax ? bytes : 0;
+  return bytes <= kSoloSmemMax ? bytes : 0;
 }
 
 // Whether a single search may pull: a row holds the in-edges and their
