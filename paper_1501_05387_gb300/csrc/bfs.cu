@@ -1818,12 +1818,15 @@ __global__ void __launch_bounds__(kPersThreads) k_bfs_persistent(BfsArgs a) {
 }  // namespace
 
 // ---------------------------------------------------------------- host
+// Dynamic shared memory k_bfs_solo may take (64 bytes left to its counters).
+constexpr size_t kSoloSmemMax = kBlockSmemMax - 64;
+
 // Shared memory the one-block driver needs on this graph, 0 where the graph
 // is not a mesh or does not fit.
 static size_t solo_smem(const gr_graph *g) {
   if (g->max_degree > kLowDegreeMax) return 0;
   const size_t bytes = sizeof(int32_t) * (2 * (size_t)kSoloQueue + (size_t)g->nwords + 32);
-  return bytes + 64 <= kBlockSmemMax ? bytes : 0;
+  return bytes <= kSoloSmemMax ? bytes : 0;
 }
 
 size_t bfs_ws_bytes(const gr_graph *g) {
@@ -2004,8 +2007,7 @@ gr_status bfs_run(gr_graph *g, BfsWorkspace *ws, int32_t src, int32_t *depth, in
   if (mode == GR_MODE_PERSISTENT && !a.low_degree && o.block == 0 && policy != GR_DIR_PULL &&
       g->n <= kSmallMaxN && g->m <= (policy == GR_DIR_PUSH ? kSmallMaxPushM : kSmallMaxM)) {
     const size_t bytes = small_smem_bytes(g->n);
-    GR_CUDA(cudaFuncSetAttribute(k_bfs_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)bytes));
+    GR_TRY(allow_smem(k_bfs_small, small_smem_bytes(kSmallMaxN)));
     k_bfs_small<<<1, kSmallThreads, bytes, s>>>(a, src, depth, parent, policy, alpha, beta,
                                                 max_levels, (g->symmetric && do_bitmap) ? 1 : 0);
     GR_CUDA(cudaGetLastError());
@@ -2037,7 +2039,7 @@ gr_status bfs_run(gr_graph *g, BfsWorkspace *ws, int32_t src, int32_t *depth, in
     const size_t solo = a.low_degree ? solo_smem(g) : 0;
     if (solo) {
       auto one = g->max_degree > 4 ? k_bfs_solo<true> : k_bfs_solo<false>;
-      GR_CUDA(cudaFuncSetAttribute(one, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)solo));
+      GR_TRY(allow_smem(one, kSoloSmemMax));
       one<<<1, kSoloThreads, solo, s>>>(a);
       GR_CUDA(cudaGetLastError());
     } else if (a.low_degree) {

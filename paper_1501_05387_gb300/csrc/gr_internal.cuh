@@ -168,6 +168,15 @@ constexpr int32_t kLowDegreeMax = 16;
 // Shared memory one block may take.
 constexpr size_t kBlockSmemMax = 232448;
 
+// Lets a kernel take `most` bytes of dynamic shared memory, always the same
+// for that kernel: the limit belongs to the kernel, not to a launch, and
+// another thread may be about to launch it on a larger graph.
+template <class K>
+gr_status allow_smem(K kern, size_t most) {
+  GR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
+  return GR_OK;
+}
+
 // Builds g->adj4 (g->adjw4 if weighted) on `s` unless it is there already.
 // The caller synchronises `s` before another stream may read it.
 gr_status low_adjacency(gr_graph *g, bool weighted, cudaStream_t s);

@@ -1385,7 +1385,7 @@ static gr_status sssp_drive(gr_graph *g, SsspWorkspace *ws, SsspArgs a, const Ss
     const bool longer = g->max_degree > 4;
     auto kern = both ? (longer ? k_sssp_solo<true, true> : k_sssp_solo<false, true>)
                      : (longer ? k_sssp_solo<true, false> : k_sssp_solo<false, false>);
-    GR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    GR_TRY(allow_smem(kern, kSoloSmemMax));
     kern<<<src.k, kSoloThreads, bytes, s>>>(a, src);
     GR_CUDA(cudaGetLastError());
   }
