@@ -110,21 +110,27 @@ gr_status gather_plan_build(GatherPlan *p, const int32_t *R, int32_t n, int64_t 
   uint32_t *rank_base = desc2 + words;
   int32_t *rows = (int32_t *)(rank_base + tiles);
   int32_t *part = rows + n;
-  p->a = {(const uint16_t *)desc2, rank_base, rows};
+  const GatherPlanArgs a = {(const uint16_t *)desc2, rank_base, rows};
   if (m > 0) {
     const int grid = (int)std::min<int64_t>(((int64_t)n + 255) / 256, 4096);
-    GR_CUDA(cudaMemsetAsync(desc2, 0, sizeof(uint32_t) * (size_t)words, s));
-    k_gp_ends<<<grid, 256, 0, s>>>(R, n, desc2);
-    k_gp_sums<<<(unsigned)blocks, kGpThreads, 0, s>>>(desc2, words, part);
-    k_gp_parts<<<1, 1024, 0, s>>>(part, (int32_t)blocks);
-    k_gp_apply<<<(unsigned)blocks, kGpThreads, 0, s>>>(desc2, words, part, rank_base);
-    k_gp_rows<<<grid, 256, 0, s>>>(R, n, p->a.desc, rank_base, rows);
-    const cudaError_t e = cudaGetLastError();
+    cudaError_t e = cudaMemsetAsync(desc2, 0, sizeof(uint32_t) * (size_t)words, s);
+    if (e == cudaSuccess) {
+      k_gp_ends<<<grid, 256, 0, s>>>(R, n, desc2);
+      k_gp_sums<<<(unsigned)blocks, kGpThreads, 0, s>>>(desc2, words, part);
+      k_gp_parts<<<1, 1024, 0, s>>>(part, (int32_t)blocks);
+      k_gp_apply<<<(unsigned)blocks, kGpThreads, 0, s>>>(desc2, words, part, rank_base);
+      k_gp_rows<<<grid, 256, 0, s>>>(R, n, a.desc, rank_base, rows);
+      e = cudaGetLastError();
+    }
+    // a later call on another stream, or one after this call has failed, finds
+    // the plan finished; a stream that is being captured is refused here
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
       p->mem.reset();  // not a plan
       return cuda_fail(e, "gather plan");
     }
   }
+  p->a = a;
   return GR_OK;
 }
 

@@ -59,7 +59,7 @@ inline size_t gather_plan_bytes(int32_t n, int64_t m) {
 }
 
 // Builds the plan of the CSR row offsets R (n vertices, m entries) on `s`
-// unless it is there already; nothing is synchronised. In gather.cu.
+// unless it is there already, and waits for it. In gather.cu.
 gr_status gather_plan_build(GatherPlan *p, const int32_t *R, int32_t n, int64_t m, cudaStream_t s);
 
 #ifdef __CUDACC__

@@ -177,8 +177,8 @@ gr_status allow_smem(K kern, size_t most) {
   return GR_OK;
 }
 
-// Builds g->adj4 (g->adjw4 if weighted) on `s` unless it is there already.
-// The caller synchronises `s` before another stream may read it.
+// Builds g->adj4 (g->adjw4 if weighted) on `s` unless it is there already,
+// and waits for it.
 gr_status low_adjacency(gr_graph *g, bool weighted, cudaStream_t s);
 
 // Internal primitive entry points with explicit workspaces (device outputs,

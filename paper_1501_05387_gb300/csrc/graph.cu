@@ -24,6 +24,7 @@ gr_status fail(gr_status st, const std::string &msg) {
 gr_status cuda_fail(cudaError_t e, const char *what) {
   std::string msg = std::string(what) + ": " + cudaGetErrorName(e) + " (" +
                     cudaGetErrorString(e) + ")";
+  cudaGetLastError();  // reported here: the next call's launches are not to find it
   set_error(msg);
   return e == cudaErrorMemoryAllocation ? GR_ENOMEM : GR_ECUDA;
 }
@@ -282,7 +283,9 @@ gr_status low_adjacency(gr_graph *g, bool weighted, cudaStream_t s) {
   k_low_adjacency<<<g->num_sms * 8, 256, 0, s>>>(
       g->row_off.as<int32_t>(), g->col.as<int32_t>(), weighted ? g->w.as<uint32_t>() : nullptr,
       g->n, m.as<int4>());
-  const cudaError_t e = cudaGetLastError();
+  // finished when a later call finds it, whatever becomes of this one
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) {
     m.reset();
     return cuda_fail(e, "low-degree adjacency");
