@@ -192,6 +192,9 @@ gr_status bfs_read_ctl_error(BfsWorkspace *ws, cudaStream_t s);
 // lanes > 1: buffers for that many lane-major copies (sssp_batch_run)
 gr_status sssp_ws_create(gr_graph *g, cudaStream_t s, SsspWorkspace **out, int32_t lanes = 1);
 size_t sssp_ws_bytes(const gr_graph *g, int32_t lanes = 1);
+// what each lane adds to a workspace (what a graph or a single search has once
+// is not part of it)
+size_t sssp_lane_bytes(const gr_graph *g);
 // most sources one batched SSSP run on this graph may take
 int32_t sssp_batch_max_lanes(const gr_graph *g);
 // blocks per SM the persistent SSSP kernel starts out with on m entries

@@ -333,7 +333,7 @@ gr_status gr_server_add_graph(gr_server *srv, gr_graph *g, int32_t batchable,
   e.n = g->n;
   e.min_batch = batchable;
   if (g->has_weights) {
-    const size_t per_lane = sssp_ws_bytes(g, 1) + sizeof(uint32_t) * (size_t)g->n;
+    const size_t per_lane = sssp_lane_bytes(g) + sizeof(uint32_t) * (size_t)g->n;
     const size_t by_mem = std::max<size_t>(1, kSsspBatchBytes / per_lane);
     e.sssp_lanes = (int32_t)std::min<size_t>(by_mem, (size_t)sssp_batch_max_lanes(g));
   }

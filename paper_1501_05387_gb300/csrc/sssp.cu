@@ -1200,16 +1200,27 @@ static bool can_pull(const gr_graph *g) {
   return g->weights_symmetric && g->max_degree > kLowDegreeMax && g->m > 0;
 }
 
+// Most merge-path chunks a near frontier of `lanes` copies can have: n vertices
+// of each and their edges.
+static size_t sssp_max_chunks(const gr_graph *g, int32_t lanes) {
+  const int items = lanes == 1 && can_pull(g) ? kSsspPullItems : kSsspItems;
+  return (size_t)lanes * ((size_t)g->n + (size_t)g->m) / (kSsspThreads * items) + 2;
+}
+
 size_t sssp_ws_bytes(const gr_graph *g, int32_t lanes) {
-  const size_t n = (size_t)g->n * (size_t)std::max(lanes, 1);
-  const size_t qcb = g->max_degree > kLowDegreeMax
-                         ? sizeof(int32_t) * ((n + (size_t)std::max(lanes, 1) * (size_t)g->m) /
-                                                  (kSsspThreads * kSsspPullItems) + 3)
-                         : 0;
-  return 4 * sizeof(int32_t) * (n + 1) + 2 * sizeof(int32_t) * (n + 2) +
-         2 * sizeof(int32_t) * n + sizeof(SsspCtl) + qcb +
+  return (size_t)lanes * sssp_lane_bytes(g) + sizeof(SsspCtl) +
          (solo_smem(g, false) ? 32 * (size_t)g->n : 0) +
-         (lanes == 1 && can_pull(g) ? gather_plan_bytes(g->n, g->m) + 4 * (size_t)g->nwords : 0);
+         (lanes == 1 && can_pull(g) ? gather_plan_bytes(g->n, g->m) + 4 * (size_t)g->nwords +
+                                          4 * sssp_max_chunks(g, 1)
+                                    : 0);
+}
+
+size_t sssp_lane_bytes(const gr_graph *g) {
+  const size_t n = (size_t)g->n;
+  return 4 * sizeof(int32_t) * (n + 1) + 2 * sizeof(int32_t) * (n + 2) + 2 * sizeof(int32_t) * n +
+         (g->max_degree > kLowDegreeMax
+              ? sizeof(int32_t) * ((n + (size_t)g->m) / (kSsspThreads * kSsspItems) + 3)
+              : 0);
 }
 
 int32_t sssp_batch_max_lanes(const gr_graph *g) {
@@ -1236,10 +1247,8 @@ gr_status sssp_ws_create(gr_graph *g, cudaStream_t s, SsspWorkspace **out, int32
   GR_TRY(ws->far_stamp.alloc(sizeof(int32_t) * n, "SSSP far stamps"));
   GR_TRY(ws->ctl.alloc(sizeof(SsspCtl), "SSSP control"));
   if (g->max_degree > kLowDegreeMax) {
-    // a frontier holds at most n vertices of each lane and their edges
-    const long long chunks = ((long long)n + (long long)lanes * g->m) /
-                                 (kSsspThreads * kSsspPullItems) + 2;
-    GR_TRY(ws->qcb.alloc(sizeof(int32_t) * ((size_t)chunks + 1), "SSSP frontier chunk bounds"));
+    GR_TRY(ws->qcb.alloc(sizeof(int32_t) * (sssp_max_chunks(g, lanes) + 1),
+                         "SSSP frontier chunk bounds"));
   }
   if (lanes == 1 && can_pull(g)) {
     GR_TRY(gather_plan_build(&ws->plan, g->row_off.as<int32_t>(), g->n, g->m, s));
