@@ -124,4 +124,45 @@ __device__ __forceinline__ DS ds_abs_diff(float a, float b) {
   return d.hi < 0.f ? DS{-d.hi, -d.lo} : d;
 }
 
+// A sum of floats as three floats: what an addition rounds off at one goes to
+// the next, so only the last one rounds, below 2^-72 of the sum (FP64: 2^-53).
+struct TripleSum {
+  float a, b, c;
+};
+
+__device__ __forceinline__ void ts_add(TripleSum &s, float x) {
+  const DS p = ds_two_sum(s.a, x), q = ds_two_sum(s.b, p.lo);
+  s.a = p.hi;
+  s.b = q.hi;
+  s.c = __fadd_rn(s.c, q.lo);
+}
+
+// Rare cases in FP64 are calls: inlined, their few instructions are issued for
+// every warp, predicated off, and hold the FP64 pipe all the same (87 cycles a
+// vertex in PageRank's update, 27-90 us of it instead of 17 at R-MAT 2^21).
+static __device__ __noinline__ double add_f32_to_f64(double r, float c) { return r + (double)c; }
+static __device__ __noinline__ float fma_rounded_once_more(double x, float d, float s) {
+  return __double2float_rn(fma((double)d, (double)s, x));
+}
+
+__device__ __forceinline__ double ts_to_double(const TripleSum &s) {
+  const double r = ds_to_double({s.a, s.b});
+  return s.c != 0.f ? add_f32_to_f64(r, s.c) : r;
+}
+
+// (float)(x + d * s) as FP64 arithmetic gives it, for x = xh + xl to 48 bits
+// and finite, non-negative values. The product and the sums are taken apart
+// into exact parts; what is rounded off on the way, under 2^-47 of the result,
+// matters only where the exact sum lies as near to the middle of two floats,
+// and there (2^-20 of half a unit on either side, once in 200,000) FP64 decides.
+__device__ __forceinline__ float fma_f64_to_f32(double x, float xh, float xl, float d, float s) {
+  const float p = __fmul_rn(d, s);  // p + e = d * s exactly
+  const float e = __fmaf_rn(d, s, -p);
+  const DS t = ds_two_sum(xh, p);
+  const DS r = ds_two_sum(t.hi, __fadd_rn(t.lo, __fadd_rn(e, xl)));
+  if (__fadd_rn(r.hi, __fmul_rn(r.lo, 1.f + 0x1p-20f)) != r.hi)
+    return fma_rounded_once_more(x, d, s);
+  return r.hi;
+}
+
 }  // namespace gr

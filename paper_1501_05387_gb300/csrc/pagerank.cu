@@ -8,9 +8,9 @@
 //   gather  sum[v] = sum over edges (v, u) of contrib[u], contrib[u] =
 //           rank[u] / deg(u), FP32 (gather_reduce_tiles)
 //   update  rank'[v] = (1 - d)/n + d * (sum[v] + D/n), D = rank mass on
-//           degree-0 vertices; writes contrib' and clears sum; the dangling
-//           mass of rank' and the L1 change sum |rank' - rank| are reduced
-//           in double-single and FP64
+//           degree-0 vertices, as FP64 rounds it; writes contrib' and
+//           clears sum; the dangling mass of rank' and the L1 change
+//           sum |rank' - rank| are reduced in three floats and FP64
 //
 // k_pr_do runs the whole iteration loop as one cooperative kernel, a grid
 // barrier after each of the two; every block takes the same stop decision
@@ -118,31 +118,49 @@ __device__ __forceinline__ double pr_base(float damping, int32_t n, double dangl
 }
 
 // New ranks from the sums, their contributions, the block's share of the L1
-// change (red[0]) and of the dangling mass (red[1]). base + d * sum is formed
-// in double-single and rounded once: the FP64 form (two conversions and an
-// FMA per vertex, two more operations for the change, and the base's
-// divisions in every thread) kept the FP64 pipe busy for 50 us of a 245 us
-// iteration at R-MAT 2^21.
+// change (red[0]) and of the dangling mass (red[1]): what FP64 gives or better,
+// from FP32 instructions. A rank is the FP64 sum's, rounded once
+// (fma_f64_to_f32); the change and the dangling mass are summed in three floats
+// a thread and in FP64 from there. In FP64 throughout (two conversions and an
+// FMA per vertex, two more operations for the change, and the base's divisions
+// in every thread) the FP64 pipe was busy for 50 us of a 245 us iteration at
+// R-MAT 2^21; so the update takes 17 us. A thread loads two vertices at once
+// (three spill).
+constexpr int kPrUpdateItems = 2;
+
 __device__ __forceinline__ void pr_update(const PrArgs &a, float *rank, float damping, double base,
                                           double *smem, double *red) {
   const float bh = (float)base, bl = (float)(base - (double)bh);
-  DS dang{0.f, 0.f}, delta{0.f, 0.f};
-  const int lane = threadIdx.x & 31;
-  for (int64_t v = spread_warp() * 32 + lane; v < a.n; v += grid_warps() * 32) {
-    const float s = a.sum[v], ro = rank[v];
-    const int32_t dg = a.deg[v];
-    const float p = __fmul_rn(damping, s);  // p + e = damping * s exactly
-    const float e = __fmaf_rn(damping, s, -p);
-    const DS t = ds_two_sum(bh, p);
-    const float rn = __fadd_rn(t.hi, __fadd_rn(t.lo, __fadd_rn(e, bl)));
-    rank[v] = rn;
-    a.contrib[v] = dg ? rn / (float)dg : 0.0f;
-    a.sum[v] = 0.0f;
-    if (!dg) dang = ds_add_f(dang, rn);
-    delta = ds_add(delta, ds_abs_diff(rn, ro));
+  TripleSum dang{0.f, 0.f, 0.f}, delta{0.f, 0.f, 0.f};
+  const int64_t step = grid_warps() * 32;
+  for (int64_t v0 = spread_warp() * 32 + (threadIdx.x & 31); v0 < a.n; v0 += kPrUpdateItems * step) {
+    float s[kPrUpdateItems], ro[kPrUpdateItems];
+    int32_t dg[kPrUpdateItems];
+#pragma unroll
+    for (int j = 0; j < kPrUpdateItems; ++j) {
+      const int64_t v = v0 + j * step;
+      if (v < a.n) {
+        s[j] = a.sum[v];
+        ro[j] = rank[v];
+        dg[j] = a.deg[v];
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < kPrUpdateItems; ++j) {
+      const int64_t v = v0 + j * step;
+      if (v >= a.n) break;
+      const float rn = fma_f64_to_f32(base, bh, bl, damping, s[j]);
+      rank[v] = rn;
+      a.contrib[v] = dg[j] ? rn / (float)dg[j] : 0.0f;
+      a.sum[v] = 0.0f;
+      if (!dg[j]) ts_add(dang, rn);
+      const DS diff = ds_abs_diff(rn, ro[j]);
+      ts_add(delta, diff.hi);
+      if (diff.lo != 0.f) ts_add(delta, diff.lo);  // ranks more than a factor of two apart
+    }
   }
-  block_add_f64<kPrThreads>(ds_to_double(delta), smem, red);
-  block_add_f64<kPrThreads>(ds_to_double(dang), smem, red + 1);
+  block_add_f64<kPrThreads>(ts_to_double(delta), smem, red);
+  block_add_f64<kPrThreads>(ts_to_double(dang), smem, red + 1);
 }
 
 __device__ __forceinline__ double read_f64(const double *p) { return *(const volatile double *)p; }
