@@ -215,13 +215,19 @@ gr_status gr_cc(gr_graph *g, int32_t *label, int32_t *num_components,
  * r[u]/deg(u) + D/n), D = sum of r[u] over vertices of out-degree 0,
  * starting from r = 1/n. Stops after max_iter iterations or once
  * sum |r' - r| < tol. rank[n] (float) receives the ranks; *iters (host, may
- * be NULL) the iterations run (asking for it synchronises). damping must lie
- * in (0, 1), max_iter >= 0, tol >= 0. A directed CSR is transposed once on
+ * be NULL) the iterations run (asking for it synchronises; without it
+ * gr_pagerank_stats tells later whether the call ran to its end). damping must
+ * lie in (0, 1), max_iter >= 0, tol >= 0. A directed CSR is transposed once on
  * the device for the in-neighbour gather. opts->mode GR_MODE_LAUNCH runs
  * host-driven batches instead of the device-side loop. */
 gr_status gr_pagerank(gr_graph *g, float damping, int32_t max_iter, double tol,
                       float *rank, int32_t *iters, const gr_opts *opts,
                       void *stream);
+
+/* Iterations of the last completed gr_pagerank on this graph (host scalar, may
+ * be NULL; synchronises). GR_ETIMEOUT when a device-side wait of it gave up:
+ * its ranks are then unfinished. */
+gr_status gr_pagerank_stats(gr_graph *g, int32_t *iters);
 
 /* Batched BFS from k in [1, 64] sources at once (one bit lane per source).
  * A level whose frontier (over all lanes) has fewer than m/16 edges pushes

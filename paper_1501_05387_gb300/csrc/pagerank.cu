@@ -264,6 +264,7 @@ static gr_status ensure_pr_ws(gr_graph *g, cudaStream_t s) {
     GR_TRY(ws->contrib.alloc(sizeof(float) * (size_t)g->n, "PageRank contributions"));
     GR_TRY(ws->sum.alloc(sizeof(float) * (size_t)g->n, "PageRank sums"));
     GR_TRY(ws->ctl.alloc(sizeof(PrCtl), "PageRank control"));
+    GR_CUDA(cudaMemsetAsync(ws->ctl.p, 0, sizeof(PrCtl), s));
     int per_sm = 1;
     GR_TRY(fit_carveout(k_pr_gather, kPrThreads, kPrBlocksPerSm, g->device, &per_sm));
     GR_TRY(fit_carveout(k_pr_do, kPrThreads, kPrBlocksPerSm, g->device, &per_sm));
@@ -368,6 +369,20 @@ gr_status gr_pagerank(gr_graph *g, float damping, int32_t max_iter, double tol, 
     *iters = h.iter;
   }
   GR_TRY(end_call(g, s));
+  return GR_OK;
+}
+
+gr_status gr_pagerank_stats(gr_graph *g, int32_t *iters) {
+  clear_error();
+  if (!g) return fail(GR_EINVAL, "graph must not be NULL");
+  std::lock_guard<std::mutex> lock(g->mu);
+  if (!g->pr) return fail(GR_EINVAL, "no PageRank has run on this graph");
+  GR_CUDA(cudaSetDevice(g->device));
+  if (g->has_last) GR_CUDA(cudaEventSynchronize(g->last_done));
+  PrCtl h;
+  GR_CUDA(cudaMemcpy(&h, g->pr->ctl.p, sizeof(PrCtl), cudaMemcpyDeviceToHost));
+  if (h.error == kDevTimeout) return fail(GR_ETIMEOUT, "a device-side wait timed out");
+  if (iters) *iters = h.iter;
   return GR_OK;
 }
 

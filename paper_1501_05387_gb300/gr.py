@@ -100,6 +100,7 @@ _sig("gr_ppr", [_vp, _vp, _i32, ctypes.c_double, _i32, ctypes.c_double, _vp, _P(
 _sig("gr_cc", [_vp, _vp, _P(_i32), _P(gr_opts), _vp])
 _sig("gr_pagerank", [_vp, ctypes.c_float, _i32, ctypes.c_double, _vp, _P(_i32),
                      _P(gr_opts), _vp])
+_sig("gr_pagerank_stats", [_vp, _P(_i32)])
 
 
 def _check(status: int, where: str):
@@ -401,6 +402,14 @@ def gr_pagerank(g: Graph, rank, damping=0.85, max_iter=50, tol=1e-7, opts=None,
                             _ptr(rank, np.float32), ctypes.byref(it) if count else None,
                             _opts(opts), _stream(stream)), "gr_pagerank")
     return it.value if count else None
+
+
+def gr_pagerank_stats(g: Graph) -> int:
+    """Iterations of the last gr_pagerank on g; raises GR_ETIMEOUT if a
+    device-side wait of it gave up. Synchronises."""
+    it = _i32()
+    _check(_lib.gr_pagerank_stats(g.handle, ctypes.byref(it)), "gr_pagerank_stats")
+    return it.value
 
 
 def gr_autotune(g: Graph, srcs, what: int = 1, stream=None):
