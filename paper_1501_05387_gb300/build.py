@@ -35,7 +35,7 @@ def sources():
 
 
 def _headers():
-    hs = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h"))]
+    hs = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h", ".hpp"))]
     hs += [os.path.join(INCLUDE, f) for f in os.listdir(INCLUDE)]
     return hs
 

@@ -9,8 +9,9 @@
 //     traversal and a small persistent grid (cheap barriers for thousands of
 //     levels); skewed graphs get direction-optimising traversal on the full
 //     GPU;
-//   * gr_autotune measures candidate settings on sample sources with CUDA
-//     events and keeps the fastest: BFS level-loop driver, persistent grid
+//   * gr_autotune measures the graph's present settings and candidates for
+//     others (tune_core.hpp) on sample sources with CUDA events and keeps the
+//     fastest: BFS level-loop driver, persistent grid
 //     size, push->pull / pull->push thresholds (alpha, beta), and the SSSP
 //     near/far bucket width. The results are stored in the graph and used
 //     whenever the caller's options leave a field at 0.
@@ -21,6 +22,7 @@
 #include <vector>
 
 #include "gr_internal.cuh"
+#include "tune_core.hpp"
 
 namespace gr {
 
@@ -123,24 +125,14 @@ gr_status gr_autotune(gr_graph *g, const int32_t *srcs, int32_t k, int32_t what,
   Timer t;
   if (what & GR_TUNE_BFS) {
     if (!g->bfs) GR_TRY(bfs_ws_create(g, s, &g->bfs));
-    struct Cand {
-      int32_t mode, bps, dir;
-      float alpha, beta;
-    };
-    std::vector<Cand> cands;
-    const int32_t bpss[] = {1, 2, 0};
-    auto add = [&](int32_t dir, float al, float be) {
-      for (int32_t bps : bpss) cands.push_back({GR_MODE_PERSISTENT, bps, dir, al, be});
-      cands.push_back({GR_MODE_GRAPH, 0, dir, al, be});
-    };
-    add(GR_DIR_PUSH, 14.f, 24.f);  // thresholds unused without pull
-    if (g->symmetric)
-      for (float al : {4.f, 10.f, 14.f, 40.f})
-        for (float be : {8.f, 24.f, 64.f}) add(GR_DIR_AUTO, al, be);
+    const std::vector<BfsSetting> cands =
+        bfs_settings({g->tuned_mode, g->tuned_blocks_per_sm, g->tuned_direction, g->tuned_alpha,
+                      g->tuned_beta},
+                     g->symmetric);
     float best = FLT_MAX;
-    Cand pick = cands[0];
+    BfsSetting pick = cands[0];
     const int32_t saved_bps = g->tuned_blocks_per_sm;
-    for (const Cand &c : cands) {
+    for (const BfsSetting &c : cands) {
       gr_opts o = default_opts();
       o.mode = c.mode;
       o.alpha = c.alpha;
@@ -176,34 +168,13 @@ gr_status gr_autotune(gr_graph *g, const int32_t *srcs, int32_t k, int32_t what,
   }
   if (what & GR_TUNE_SSSP) {
     if (!g->sssp) GR_TRY(sssp_ws_create(g, s, &g->sssp));
-    struct SCand {
-      int32_t mode, bps;
-      uint32_t delta;
-      float alpha;  // relaxations pull at m / alpha frontier edges (0: never)
-    };
-    std::vector<SCand> cands;
-    const double mw = std::max(1.0, g->mean_weight);
-    std::vector<uint32_t> deltas;
-    for (double f : {0.5, 1.0, 2.0, 4.0, 8.0, 32.0, 64.0})
-      deltas.push_back((uint32_t)std::max(1.0, std::min(4.0e9, f * mw)));
-    deltas.push_back(UINT32_MAX);
-    // pull thresholds to try where the graph can pull (in-edges in the rows,
-    // not mesh-like): the frontier holding half or a sixth of the edges
-    std::vector<float> alphas = {0.f};
-    if (g->weights_symmetric && g->max_degree > kLowDegreeMax) {
-      alphas.push_back(2.f);
-      alphas.push_back(6.f);
-    }
-    for (uint32_t d : deltas)
-      for (float al : alphas) {
-        cands.push_back({GR_MODE_GRAPH, 0, d, al});
-        cands.push_back({GR_MODE_PERSISTENT, 1, d, al});
-        cands.push_back({GR_MODE_PERSISTENT, 0, d, al});
-      }
+    const std::vector<SsspSetting> cands = sssp_settings(
+        {g->tuned_sssp_mode, g->tuned_sssp_blocks_per_sm, g->sssp_delta, g->tuned_sssp_alpha},
+        g->mean_weight, g->weights_symmetric && g->max_degree > kLowDegreeMax);
     float best = FLT_MAX;
-    SCand pick = cands[0];
+    SsspSetting pick = cands[0];
     const int32_t saved_sbps = g->tuned_sssp_blocks_per_sm;
-    for (const SCand &c : cands) {
+    for (const SsspSetting &c : cands) {
       gr_opts o = default_opts();
       o.delta = c.delta;
       o.mode = c.mode;
