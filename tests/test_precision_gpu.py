@@ -24,3 +24,26 @@ def test_pagerank_rounds_the_fp64_rank(cuda_lib, n, damping, k):
     share = np.float64((np.float32(1) / np.float32(n)) / np.float32(k))
     assert np.all(got[1:k + 1] == np.float32(base + d * share))
     assert got[0] == np.float32(base) and np.all(got[k + 1:] == np.float32(base))
+
+
+@pytest.mark.parametrize("hubs", [1, 3, 1000])
+def test_ppr_divides_by_the_degree(cuda_lib, hubs):
+    """One iteration from `hubs` seeds of degrees 1, 2, ... (a star each): a leaf
+    of degree one gets damping times what its hub's rank over its degree is, which
+    the kernel forms from the degree's reciprocal."""
+    import torch
+    gr = cuda_lib
+    deg = np.arange(1, hubs + 1)
+    leaves = int(deg.sum())
+    n = hubs + leaves
+    hub_of = np.repeat(np.arange(hubs), deg)
+    r = np.zeros(n + 1, np.int32)
+    r[1:hubs + 1] = np.cumsum(deg)
+    r[hubs + 1:] = leaves + np.arange(1, leaves + 1)
+    c = np.concatenate([np.arange(hubs, n), hub_of]).astype(np.int32)
+    rank = torch.empty(n, dtype=torch.float64, device="cuda")
+    for damping in (0.85, 0.3):
+        with gr.gr_graph_create(r, c) as g:
+            gr.gr_ppr(g, list(range(hubs)), rank, damping, 1, 0.0)
+        want = damping * ((1.0 / hubs) / deg)[hub_of]
+        assert np.array_equal(rank.cpu().numpy()[hubs:], want)
