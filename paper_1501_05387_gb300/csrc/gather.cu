@@ -101,6 +101,11 @@ __global__ void k_gp_rows(const int32_t *R, int32_t n, const uint16_t *desc,
 gr_status gather_plan_build(GatherPlan *p, const int32_t *R, int32_t n, int64_t m,
                             cudaStream_t s) {
   if (p->mem.p) return GR_OK;
+  // kernels that only go into a graph would leave a plan on paper
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  GR_CUDA(cudaStreamIsCapturing(s, &capture));
+  if (capture != cudaStreamCaptureStatusNone)
+    return fail(GR_ECUDA, "a graph's first call cannot be captured: it builds a plan");
   // a warp's tile may take two rank_base tiles: an even number of them
   const int64_t tiles = 2 * ((m + 2 * kGpTile - 1) / (2 * kGpTile));
   const int64_t words = tiles * kGpWords;
@@ -122,9 +127,6 @@ gr_status gather_plan_build(GatherPlan *p, const int32_t *R, int32_t n, int64_t 
       k_gp_rows<<<grid, 256, 0, s>>>(R, n, a.desc, rank_base, rows);
       e = cudaGetLastError();
     }
-    // a later call on another stream, or one after this call has failed, finds
-    // the plan finished; a stream that is being captured is refused here
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
       p->mem.reset();  // not a plan
       return cuda_fail(e, "gather plan");
@@ -132,6 +134,14 @@ gr_status gather_plan_build(GatherPlan *p, const int32_t *R, int32_t n, int64_t 
   }
   p->a = a;
   return GR_OK;
+}
+
+gr_status gather_plan_of_call(gr_graph *g, GatherPlan *p, const int32_t *R, cudaStream_t s) {
+  if (p->mem.p) return GR_OK;
+  GR_TRY(gather_plan_build(p, R, g->n, g->m, s));
+  const gr_status st = end_call(g, s);
+  if (st != GR_OK) p->mem.reset();
+  return st;
 }
 
 }  // namespace gr

@@ -59,8 +59,14 @@ inline size_t gather_plan_bytes(int32_t n, int64_t m) {
 }
 
 // Builds the plan of the CSR row offsets R (n vertices, m entries) on `s`
-// unless it is there already, and waits for it. In gather.cu.
+// unless it is there already; a stream that is being captured is refused.
+// Nothing is synchronised: the caller does, or orders what may use the plan on
+// another stream. In gather.cu.
 gr_status gather_plan_build(GatherPlan *p, const int32_t *R, int32_t n, int64_t m, cudaStream_t s);
+
+// The same inside a public call on g, after begin_call: whatever becomes of the
+// call, the next one, on any stream, comes after the plan's kernels.
+gr_status gather_plan_of_call(gr_graph *g, GatherPlan *p, const int32_t *R, cudaStream_t s);
 
 #ifdef __CUDACC__
 

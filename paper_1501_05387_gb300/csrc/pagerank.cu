@@ -291,7 +291,7 @@ static gr_status ensure_pr_ws(gr_graph *g, cudaStream_t s) {
     ws->has_transpose = true;
   }
   const int32_t *R = g->symmetric ? g->row_off.as<int32_t>() : ws->tr_off.as<int32_t>();
-  return gather_plan_build(&ws->plan, R, g->n, g->m, s);
+  return gather_plan_of_call(g, &ws->plan, R, s);
 }
 
 static PrArgs pr_args(gr_graph *g) {

@@ -439,7 +439,7 @@ static gr_status rank_ws(gr_graph *g, bool by_degree, RankWorkspace **out) {
 // left to L1.
 template <class T, class OP, class G>
 static gr_status nr_launch_all(gr_graph *g, RankWorkspace *ws, cudaStream_t s, G gf, T *out) {
-  GR_TRY(gather_plan_build(&ws->plan, g->row_off.as<int32_t>(), g->n, g->m, s));
+  GR_TRY(gather_plan_of_call(g, &ws->plan, g->row_off.as<int32_t>(), s));
   auto kern = k_nr_all<T, OP, G>;
   int per_sm = 1;
   GR_TRY(fit_carveout(kern, kRgThreads, range_blocks<T>(), g->device, &per_sm));
@@ -514,7 +514,7 @@ static gr_status bipartite_run(gr_graph *g, int kind, int32_t n_left, int32_t ma
   }
   bool host = false;
   GR_TRY(output_on_host(g, score, &host));
-  GR_TRY(gather_plan_build(&ws->plan, g->row_off.as<int32_t>(), g->n, g->m, s));
+  GR_TRY(gather_plan_of_call(g, &ws->plan, g->row_off.as<int32_t>(), s));
   RankArgs a;
   std::memset(&a, 0, sizeof(a));
   a.R = g->row_off.as<int32_t>();
@@ -681,7 +681,7 @@ gr_status gr_ppr(gr_graph *g, const int32_t *seeds, int32_t num_seeds, double da
                           cudaMemcpyHostToDevice, s));
   bool host = false;
   GR_TRY(output_on_host(g, rank, &host));
-  GR_TRY(gather_plan_build(&ws->plan, g->row_off.as<int32_t>(), g->n, g->m, s));
+  GR_TRY(gather_plan_of_call(g, &ws->plan, g->row_off.as<int32_t>(), s));
   RankArgs a;
   std::memset(&a, 0, sizeof(a));
   a.R = g->row_off.as<int32_t>();
