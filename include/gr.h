@@ -70,7 +70,7 @@ enum {
   GR_MODE_PERSISTENT = 3  /* one cooperative kernel runs every level with a
                              bounded-spin grid barrier between levels; on a
                              graph of maximum degree <= 16 one thread block
-                             (above 1.58 M vertices, for a BFS, one
+                             (above 1,595,904 vertices, for a BFS, one
                              thread-block cluster) runs the levels first and
                              hands a frontier of more than 4096 (32768)
                              vertices to that kernel */

@@ -60,8 +60,6 @@ constexpr int32_t kKeepLevels = 16;
 // A batched BFS level pushes when its frontier has fewer than m / kPushDiv
 // edges, and pulls over every vertex otherwise.
 constexpr long long kPushDiv = 16;
-// Graphs of at most this maximum degree (meshes) keep no level's masks.
-constexpr int32_t kLowDegreeMaxBatch = 16;
 constexpr int kMbChunk = kMbThreads * kMbItems;
 // BC's gathers take chunks of this many items per warp: with one per block
 // its warps waited for the slowest at every chunk (half of the forward's
@@ -1138,7 +1136,7 @@ __global__ void k_mb_resume(MbCtl *c) {
 
 // Levels of a batched BFS kept in their own mask arrays on this graph.
 static int32_t bfs_keep_levels(const gr_graph *g) {
-  return g->max_degree <= kLowDegreeMaxBatch ? 0 : kKeepLevels;
+  return g->max_degree <= kLowDegreeMax ? 0 : kKeepLevels;
 }
 
 size_t batch_ws_bytes(const gr_graph *g) {

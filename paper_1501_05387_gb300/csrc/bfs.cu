@@ -1069,7 +1069,7 @@ __global__ void __launch_bounds__(kLvThreads, BPS) k_bfs_do(BfsArgs a) {
 // were no better. One SM takes about one random L2 access per clock, two a
 // vertex here: that bounds the large levels, instruction latency the small.
 //
-// n is limited by the bitmap (1.58 M vertices). A frontier of more than
+// n is limited by the bitmap (1,595,904 vertices). A frontier of more than
 // kSoloHandoff vertices goes to the grid kernel, with the bitmap and the list
 // in global memory, as from the cluster driver.
 constexpr int kSoloThreads = 768;

@@ -144,6 +144,8 @@ __device__ __forceinline__ void hook_own(int32_t *label, int32_t v, int32_t x) {
   int32_t b = walk(label, x);
   while (a != b) {
     const int32_t hi = max(a, b), lo = min(a, b);
+    // whichever threads are here together: each of them gets the same mask and
+    // takes part in what names it, and any such group may share one CAS
     const uint32_t peers = __match_any_sync(__activemask(), hi);
     const int leader = __ffs(peers) - 1;
     int32_t prev = 0;

@@ -40,8 +40,13 @@ void tune_prior(gr_graph *g) {
     g->tuned_sssp_mode = GR_MODE_PERSISTENT;
     g->tuned_sssp_blocks_per_sm = 1;
     // six mean weights a bucket: one block's search (k_sssp_solo) of grids of
-    // 64 to 1024 a side, weights to 16, 64 and 1000, took 1.0-1.2 times its
-    // best there, 1.1-1.7 times at two mean weights, 1.0-1.3 at twelve
+    // 64 to 1024 a side, weights to 16, 64 and 1000, took 1.0-1.1 times its
+    // best there, 1.1-1.5 times at two mean weights, 1.0-1.1 at twelve; the grid
+    // kernel at two, six and twelve: 1400 a side 41.6, 29.2, 25.1 ms, 4096 a side
+    // 147, 104, 89 ms. Random graphs of degree 20 and 28, which run merge-path
+    // chunks, at two, six and eight: 20,000 vertices, weights to 16 and 64, 186,
+    // 194, 189 and 248, 257, 253 us; 300,000 vertices 513, 497, 488 and 940, 680,
+    // 672 us, of degree 28 744, 623, 611 and 964, 799, 776 us
     if (g->has_weights)
       g->sssp_delta = (uint32_t)std::max(1.0, std::min(6.0 * g->mean_weight, 4.0e9));
   } else {
