@@ -1071,10 +1071,17 @@ __global__ void __launch_bounds__(kLvThreads, BPS) k_bfs_do(BfsArgs a) {
 //
 // n is limited by the bitmap (1,595,904 vertices). A frontier of more than
 // kSoloHandoff vertices goes to the grid kernel, with the bitmap and the list
-// in global memory, as from the cluster driver.
+// in global memory, as from the cluster driver. Longer rows mean more claims a
+// vertex and wider frontiers; from some size on the cluster's SMs are the better
+// place for them (kSoloLongWork, entries times largest degree): 3D grids of 30,
+// 40 and 50 a side 178, 321 and 505 us here, 345, 487 and 461 there; random
+// graphs of degree 8, 400,000 entries, 83 and 86; of degree 16, 160,000 and
+// 320,000 entries, 63 and 82 here, 65 and 77 there; a 15-ary tree of 400,000
+// entries 172 and 144.
 constexpr int kSoloThreads = 768;
 constexpr int32_t kSoloQueue = 4096;  // frontier vertices kept in shared memory, per parity
 constexpr int32_t kSoloHandoff = kSoloQueue;
+constexpr int64_t kSoloLongWork = 3'000'000;
 
 // LONG: the graph has rows of more than four entries (the code for them costs
 // the others instruction fetches on every level)
@@ -1822,9 +1829,10 @@ __global__ void __launch_bounds__(kPersThreads) k_bfs_persistent(BfsArgs a) {
 constexpr size_t kSoloSmemMax = kBlockSmemMax - 64;
 
 // Shared memory the one-block driver needs on this graph, 0 where the graph
-// is not a mesh or does not fit.
+// is not a mesh, does not fit or has too many long rows.
 static size_t solo_smem(const gr_graph *g) {
   if (g->max_degree > kLowDegreeMax) return 0;
+  if (g->max_degree > 4 && g->m * g->max_degree > kSoloLongWork) return 0;
   const size_t bytes = sizeof(int32_t) * (2 * (size_t)kSoloQueue + (size_t)g->nwords + 32);
   return bytes <= kSoloSmemMax ? bytes : 0;
 }

@@ -44,3 +44,23 @@ def test_bfs_sizes(cuda_lib, n):
     r, c = strip(n)
     with cuda_lib.gr_graph_create(r, c) as g:
         tb.check(cuda_lib, r, c, g, n // 3)
+
+
+def grid3(s):
+    at = np.arange(s ** 3).reshape(s, s, s)
+    u = np.concatenate([at[:-1].ravel(), at[:, :-1].ravel(), at[:, :, :-1].ravel()])
+    v = np.concatenate([at[1:].ravel(), at[:, 1:].ravel(), at[:, :, 1:].ravel()])
+    key = np.sort(np.concatenate([u * s ** 3 + v, v * s ** 3 + u]))
+    r = np.zeros(s ** 3 + 1, np.int32)
+    r[1:] = np.cumsum(np.bincount(key // s ** 3, minlength=s ** 3))
+    return r, (key % s ** 3).astype(np.int32)
+
+
+# rows of six entries: 500,000 entries in all are where the cluster takes over
+@pytest.mark.parametrize("side", [43, 44, 45])
+def test_bfs_of_3d_grids(cuda_lib, side):
+    r, c = grid3(side)
+    assert (c.size * 6 <= 3_000_000) == (side < 45)
+    with cuda_lib.gr_graph_create(r, c) as g:
+        for src in (0, side ** 3 // 2):
+            tb.check(cuda_lib, r, c, g, src)
