@@ -103,7 +103,9 @@ struct gr_graph {
   bool weights_symmetric = false;  // and (u, v) weighs what (v, u) does
   bool rows_sorted = false;
   bool has_weights = false;
-  uint32_t sssp_delta = 1;    // tuned near/far bucket width
+  // tuned near/far bucket widths: on frontiers of few vertices and, in the grid
+  // kernels, of many
+  uint32_t sssp_delta = 1, sssp_delta_thick = 1;
   float tuned_alpha = 14.f;   // push -> pull threshold (see gr_autotune)
   float tuned_beta = 24.f;    // pull -> push threshold
   int32_t tuned_mode = GR_MODE_AUTO;

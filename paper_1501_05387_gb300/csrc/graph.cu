@@ -440,7 +440,7 @@ gr_status gr_graph_create(int32_t n, int64_t m, const int32_t *row_off,
     // near/far bucket width: a few mean edge weights keeps the near
     // frontier wide enough to fill the GPU
     double d = 2.0 * g->mean_weight;
-    g->sssp_delta = (uint32_t)std::max(1.0, std::min(d, 4.0e9));
+    g->sssp_delta = g->sssp_delta_thick = (uint32_t)std::max(1.0, std::min(d, 4.0e9));
   }
   tune_prior(g.get());
   *out = g.release();

@@ -33,7 +33,9 @@
 // loop when both piles are empty.
 //
 // T starts at delta and grows by delta per phase (delta = UINT32_MAX: one
-// bucket, i.e. plain frontier relaxation). Distances do not depend on delta.
+// bucket, i.e. plain frontier relaxation); on graphs of small maximum degree
+// the graph's own width is one for meshes' thin frontiers and one for others
+// (sssp_delta, sssp_delta_thick). Distances do not depend on delta.
 // An optional last pass fills pred[v] with the smallest u that has an edge
 // (u, v) with dist[u] + w = dist[v].
 //
@@ -89,6 +91,8 @@ struct SsspCtl {
   long long pull_min_edges;
   int32_t pulls;          // relaxations run in pull form (statistics)
   int32_t pad2_;
+  // persistent kernel: bucket width while frontiers are thick (delta: thin)
+  unsigned long long delta_thick;
   // persistent kernel: counter rings and grid barrier
   unsigned long long ring_near[3];
   int32_t ring_far[3];
@@ -111,6 +115,7 @@ struct SsspArgs {
   SsspCtl *ctl;
   int32_t low_degree;  // graph of small maximum degree: per-thread relaxation
   const int4 *adjw;    // four (neighbour, weight) pairs per vertex (low_adjacency)
+  int32_t solo_handoff;  // frontier size up to which k_sssp_solo goes on
   GatherPlanArgs plan;  // row structure of the pull relaxation
   uint32_t *lowered;    // marks of the vertices a pull lowered (zero between pulls)
   int32_t *qcb;        // room for the chunk bounds of a dense near frontier (or null)
@@ -131,14 +136,18 @@ constexpr int kSsspBoundsChunksPerBlock = 4;
 // Most sources one batched run takes.
 constexpr int32_t kSsspMaxLanes = 64;
 // k_sssp_solo: threads of the block that runs a search, frontier vertices it
-// keeps in shared memory per parity, and the frontier size from which the
-// search goes on as k_sssp_do. A block expands a vertex in 5 ns, so 4096 take
-// it twice as long as a grid barrier and their expansion on all SMs (9 us);
-// but the grid keeps the search once it has it, and meshes pass 2560 for a
-// few iterations only (700 x 700, 12 mean weights: 7.6 ms handed over there).
+// keeps in shared memory per parity, and the frontier's edges from which the
+// search goes on as k_sssp_do. A block expands a vertex of four edges in 5 ns,
+// so 4096 take it twice as long as a grid barrier and their expansion on all
+// SMs (9 us); but the grid keeps the search once it has it, and meshes pass 2560
+// for a few iterations only (700 x 700, 12 mean weights: 7.6 ms handed over
+// there).
 constexpr int kSoloThreads = 1024;
 constexpr int32_t kSoloQueue = 4096;
-constexpr int32_t kSoloHandoff = 4096;
+constexpr int32_t kSoloHandoffEdges = 16384;
+// k_sssp_do: the share of the expanded vertices below which the far pile is that
+// of a mesh (bucket width).
+constexpr int32_t kSsspFarShare = 2;
 
 struct SsspWorkspace {
   int32_t lanes = 1;  // copies of the graph the buffers hold (batched form)
@@ -174,10 +183,11 @@ struct SsspSources {
 };
 
 // solo: k_sssp_solo runs the searches from their sources; the control block
-// then starts out as what its lanes hand over: nothing.
+// then starts out as what its lanes hand over: nothing. The grid's first bucket
+// is of the thick width.
 __global__ void k_sssp_init(SsspArgs a, SsspSources src, uint32_t *dist, int32_t *pred,
-                            unsigned long long delta, int32_t max_iters,
-                            long long pull_min_edges, int32_t solo) {
+                            unsigned long long delta, unsigned long long delta_thick,
+                            int32_t max_iters, long long pull_min_edges, int32_t solo) {
   const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t v = tid; v < a.nv; v += stride) {
@@ -220,7 +230,8 @@ __global__ void k_sssp_init(SsspArgs a, SsspSources src, uint32_t *dist, int32_t
     c->far_min_next = 0xFFFFFFFFu;
     c->near_next_packed = 0ull;
     c->delta = delta;
-    c->T = solo ? ~0ull : delta;
+    c->delta_thick = delta_thick;
+    c->T = delta_thick;
     c->T_old = 0;
     c->near_edges = solo ? 0 : edges;
     c->relaxations = 0;
@@ -809,10 +820,13 @@ __global__ void __launch_bounds__(kSsspThreads, kSsspBlocksPerSm)
 // did so before that read, everybody else finds it clear and puts the vertex
 // on the next frontier, and no barrier stands between the two.
 //
-// A lane whose frontier outgrows kSoloHandoff vertices writes it and its far
-// pile to the control block's queues (parity 0) and stops; k_sssp_do, next on
-// the stream, goes on with all lanes handed over, under the smallest of their
-// thresholds (a far entry is never below its own lane's, so none is dropped).
+// A lane whose frontier outgrows kSoloHandoffEdges edges (at the graph's largest
+// degree) writes it and what is left of its far pile to the grid's far pile and
+// stops; k_sssp_do, next on the stream, goes on with all lanes handed over, by
+// a split in its own bucket width: a graph on which the frontier grows so fast
+// is no mesh, and a bucket as wide as a mesh's would hold most of it (random
+// graphs of degree 8 and 16, 500,000 vertices: 0.77 and 1.61 ms in six mean
+// weights from the first bucket on, 0.69 and 0.94 on the grid alone in two).
 // Per lane, the ids [lane * n, (lane + 1) * n) of nearq[1] hold what the
 // shared-memory queue cannot, and those of nearS[0] and nearS[1] the far pile
 // by parity (both are free: per-thread relaxations use no degree scan).
@@ -820,7 +834,7 @@ struct SoloState {
   int32_t near[3];   // frontier sizes, ring by iteration
   int32_t far[2];    // far pile sizes by parity
   uint32_t far_min;  // lower bound of the far pile's distances
-  int32_t near_at, far_at;  // hand-over positions
+  int32_t near_at;   // hand-over position
   unsigned long long relaxed;
 };
 
@@ -864,7 +878,8 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_sssp_solo(SsspArgs a, SsspS
   int32_t *near_g = a.nearq[1] + base;
   int32_t *far_stamp = a.far_stamp + base;  // -1: not in the far pile (without FAR_BITS)
   int32_t *far0 = a.nearS[0] + base, *far1 = a.nearS[1] + base;
-  const unsigned long long delta = c->delta;
+  const unsigned long long delta = c->delta, delta_thick = c->delta_thick;
+  const int32_t handoff_at = LONG ? a.solo_handoff : kSoloQueue;
   const int32_t max_iters = c->max_iters;
   const int lane = threadIdx.x & 31;
   const int32_t s0 = src.s[blockIdx.x];
@@ -878,7 +893,8 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_sssp_solo(SsspArgs a, SsspS
     st.far_min = 0xFFFFFFFFu;
     st.relaxed = 0ull;
   }
-  unsigned long long T = delta;
+  unsigned long long T = LONG ? delta_thick : delta;
+  int64_t expanded = 0;  // LONG: vertices so far
   int32_t fp = 0, iter = 0, ring = 0, phases = 0;
   uint32_t relaxed = 0u;
   __syncthreads();
@@ -886,12 +902,13 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_sssp_solo(SsspArgs a, SsspS
     const int32_t next = ring == 2 ? 0 : ring + 1, after = next == 2 ? 0 : next + 1;
     const int32_t q = st.near[ring], len = st.far[fp];
     const bool split = q == 0;
-    if ((split && len == 0) || q > kSoloHandoff || iter >= max_iters) break;
+    if ((split && len == 0) || q > handoff_at || iter >= max_iters) break;
     if (threadIdx.x == 0) st.near[after] = 0;  // last read an iteration ago
     const int32_t *Q = iter & 1 ? q1 : q0;
     int32_t *Qn = iter & 1 ? q0 : q1;
     int32_t *far = fp ? far1 : far0;
     uint32_t local_min = 0xFFFFFFFFu;
+    if (LONG) expanded += q;
     if (!split) {
       // nd < T, for distances below 0xFFFFFFFF
       const uint32_t T32 = (uint32_t)min(T, 0xFFFFFFFFull);
@@ -947,7 +964,9 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_sssp_solo(SsspArgs a, SsspS
     } else {
       // the far pile by the raised threshold; entries that fell below the
       // old one were expanded already
-      const unsigned long long T_old = T, t = T + delta, b = bucket_end(st.far_min, delta);
+      const unsigned long long width =
+          LONG && (int64_t)len * kSsspFarShare > expanded ? delta_thick : delta;
+      const unsigned long long T_old = T, t = T + width, b = bucket_end(st.far_min, width);
       T = t > b ? t : b;
       int32_t *far_n = fp ? far0 : far1;
       __syncthreads();  // every thread has read far_min
@@ -994,35 +1013,42 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_sssp_solo(SsspArgs a, SsspS
   __syncthreads();
   const int32_t q = st.near[ring], len = st.far[fp];
   const bool over = (q > 0 || len > 0) && iter >= max_iters;
-  const bool handoff = !over && q > kSoloHandoff;
+  const bool handoff = !over && q > handoff_at;
   if (threadIdx.x == 0) {
     atomicMax(&c->iter, iter);
     atomicMax(&c->phases, phases);
     atomicAdd((unsigned long long *)&c->relaxations, st.relaxed);
     if (over) atomicExch(&c->error, kDevOverflow);
-    if (handoff) {
-      st.near_at = atomicAdd(&c->near_len, q);
-      st.far_at = atomicAdd(&c->far_len, len);
-      atomicMin(&c->far_min, st.far_min);
-      atomicMin(&c->T, T);
-    }
+    if (handoff) st.near_at = atomicAdd(&c->far_len, q);
   }
   __syncthreads();
   if (!handoff) return;
   const int32_t *Q = iter & 1 ? q1 : q0;
   const int32_t *far = fp ? far1 : far0;
-  long long edges = 0;
+  uint32_t lowest = 0xFFFFFFFFu;
   for (int32_t i = threadIdx.x; i < q; i += kSoloThreads) {
     const int32_t v = i < kSoloQueue ? Q[i] : near_g[i];
-    a.nearq[0][st.near_at + i] = base + v;
-    edges += a.R[v + 1] - a.R[v];
+    a.farq[0][st.near_at + i] = base + v;
+    lowest = min(lowest, __ldcg(dist + v));
   }
-  edges = warp_sum(edges);
-  if (lane == 0 && edges) atomicAdd((unsigned long long *)&c->near_edges, (unsigned long long)edges);
-  for (int32_t i = threadIdx.x; i < len; i += kSoloThreads) {
-    a.farq[0][st.far_at + i] = base + far[i];
-    far_stamp[far[i]] = 0;  // k_sssp_do's first far epoch
+  // of the far pile what has not fallen below T: the rest is on the frontier or
+  // expanded already. (far_stamp says nothing of the grid's pile, whose epochs
+  // begin at 0: its first step splits all of it into epoch 1.)
+  for (int32_t i = threadIdx.x; i - lane < len; i += kSoloThreads) {  // warp-uniform
+    const int32_t v = i < len ? far[i] : 0;
+    const uint32_t d = i < len ? __ldcg(dist + v) : 0u;
+    const bool keep = i < len && (unsigned long long)d >= T;
+    const uint32_t kb = __ballot_sync(0xffffffffu, keep);
+    int32_t at = 0;
+    if (lane == 0 && kb) at = atomicAdd(&c->far_len, __popc(kb));
+    at = __shfl_sync(0xffffffffu, at, 0) + __popc(kb & ((1u << lane) - 1u));
+    if (keep) {
+      a.farq[0][at] = base + v;
+      lowest = min(lowest, d);
+    }
   }
+  lowest = __reduce_min_sync(0xffffffffu, lowest);
+  if (lane == 0) atomicMin(&c->far_min, lowest);
 }
 
 // Persistent form: the whole SSSP in one cooperative kernel, one grid
@@ -1044,16 +1070,27 @@ __global__ void __launch_bounds__(kSsspThreads, kSsspBlocksPerSm) k_sssp_do(Sssp
   uint32_t *dist = c->dist;
   const unsigned long long delta = c->delta;
   const int32_t max_iters = c->max_iters;
-  // the sources, or what k_sssp_solo handed over (no near frontier: it
-  // finished every search)
+  // the sources, or the pile that k_sssp_solo handed over (nothing: it finished
+  // every search)
   int32_t mode = kSsspRelax, near_parity = 0, far_parity = 0, near_len = c->near_len,
           far_len = c->far_len;
-  if (near_len == 0) return;
+  if (near_len == 0 && far_len == 0) return;
+  // Bucket width: a mesh's thin frontiers wait for the barrier whatever their
+  // size, so wide buckets save iterations (4096 x 4096: 147 ms at two mean
+  // weights, 104 at six); where an iteration has more than a vertex per thread,
+  // relaxing vertices again costs more (random graph of degree 16, 2 M vertices:
+  // 2.8 and 5.5 ms). Each split goes by the iterations since the last.
+  const unsigned long long delta_thick = c->delta_thick;
+  long long expanded = 0;
   long long near_edges = c->near_edges, relaxations = c->relaxations;
   const long long pull_min_edges = c->pull_min_edges;
   int32_t iter = c->iter, far_epoch = 0, phases = c->phases, gen = 0, pulls = 0;
   uint32_t far_min = c->far_min;
   unsigned long long T = c->T, T_old = 0;
+  if (LOW && near_len == 0) {
+    mode = kSsspSplit;
+    T = bucket_end(far_min, delta_thick);
+  }
   for (;;) {
     const int32_t slot = iter % 3, clear = (iter + 1) % 3;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -1109,6 +1146,7 @@ __global__ void __launch_bounds__(kSsspThreads, kSsspBlocksPerSm) k_sssp_do(Sssp
       pulls += mode == kSsspPull;
       far_len += fcnt;
       far_min = min(far_min, fmin);
+      if (LOW) expanded += near_len;
     } else {
       far_len = fcnt;
       far_parity ^= 1;
@@ -1126,8 +1164,10 @@ __global__ void __launch_bounds__(kSsspThreads, kSsspBlocksPerSm) k_sssp_do(Sssp
     } else if (far_len > 0) {
       mode = kSsspSplit;
       T_old = T;
-      const unsigned long long t = T + delta;
-      const unsigned long long j = bucket_end(far_min, delta);
+      unsigned long long width = delta;
+      if (LOW && (long long)far_len * kSsspFarShare > expanded) width = delta_thick;
+      const unsigned long long t = T + width;
+      const unsigned long long j = bucket_end(far_min, width);
       T = t > j ? t : j;
     } else {
       done = true;
@@ -1279,6 +1319,7 @@ static SsspArgs sssp_args(gr_graph *g, SsspWorkspace *ws, int32_t lanes = 1) {
   a.ctl = ws->ctl.as<SsspCtl>();
   a.low_degree = g->max_degree <= kLowDegreeMax ? 1 : 0;
   a.adjw = g->adjw4.as<int4>();
+  a.solo_handoff = std::min(kSoloQueue, kSoloHandoffEdges / std::max(g->max_degree, 4));
   a.plan = ws->plan.a;  // null where nothing may be pulled (sssp_pull_min_edges)
   a.lowered = ws->lowered.as<uint32_t>();
   a.qcb = ws->qcb.as<int32_t>();  // null on low-degree graphs
@@ -1367,8 +1408,10 @@ int32_t sssp_prior_blocks(int64_t m) {
   return m < 150'000 ? 1 : m < 4'000'000 ? 3 : m < 16'000'000 ? 4 : 0;
 }
 
-static unsigned long long sssp_delta_of(const gr_graph *g, const gr_opts &o) {
-  return o.delta == UINT32_MAX ? (1ull << 40) : (o.delta ? o.delta : g->sssp_delta);
+// Bucket width of thin or of thick frontiers: the caller's, or the graph's own.
+static unsigned long long sssp_delta_of(const gr_graph *g, const gr_opts &o, bool thick) {
+  if (o.delta == UINT32_MAX) return 1ull << 40;
+  return o.delta ? o.delta : thick ? g->sssp_delta_thick : g->sssp_delta;
 }
 
 static int32_t sssp_max_iters_of(const gr_graph *g, const gr_opts &o) {
@@ -1386,8 +1429,10 @@ static gr_status sssp_drive(gr_graph *g, SsspWorkspace *ws, SsspArgs a, const Ss
   // meshes whose membership bits fit one block's shared memory: one block
   // per search, up to the frontier size where the grid takes over
   const size_t near_only = mode == GR_MODE_PERSISTENT ? solo_smem(g, false) : 0;
-  k_sssp_init<<<g->num_sms * 8, 256, 0, s>>>(a, src, dist, pred, sssp_delta_of(g, o), max_iters,
-                                             pull_min_edges, near_only > 0);
+  // the other drivers know one width
+  k_sssp_init<<<g->num_sms * 8, 256, 0, s>>>(
+      a, src, dist, pred, sssp_delta_of(g, o, mode != GR_MODE_PERSISTENT),
+      sssp_delta_of(g, o, true), max_iters, pull_min_edges, near_only > 0);
   GR_CUDA(cudaGetLastError());
   if (near_only) {
     const size_t both = solo_smem(g, true), bytes = both ? both : near_only;

@@ -39,15 +39,14 @@ void tune_prior(gr_graph *g) {
     // thousands of thin iterations: one kernel with a cheap grid barrier
     g->tuned_sssp_mode = GR_MODE_PERSISTENT;
     g->tuned_sssp_blocks_per_sm = 1;
-    // six mean weights a bucket: one block's search (k_sssp_solo) of grids of
-    // 64 to 1024 a side, weights to 16, 64 and 1000, took 1.0-1.1 times its
-    // best there, 1.1-1.5 times at two mean weights, 1.0-1.1 at twelve; the grid
-    // kernel at two, six and twelve: 1400 a side 41.6, 29.2, 25.1 ms, 4096 a side
-    // 147, 104, 89 ms. Random graphs of degree 20 and 28, which run merge-path
-    // chunks, at two, six and eight: 20,000 vertices, weights to 16 and 64, 186,
-    // 194, 189 and 248, 257, 253 us; 300,000 vertices 513, 497, 488 and 940, 680,
-    // 672 us, of degree 28 744, 623, 611 and 964, 799, 776 us
-    if (g->has_weights)
+    // Thin frontiers, six mean weights a bucket: one block's search
+    // (k_sssp_solo) of grids of 64 to 1024 a side, weights to 16, 64 and 1000,
+    // took 1.0-1.1 times its best there, 1.1-1.5 times at two mean weights,
+    // 1.0-1.1 at twelve; the grid kernel at two, six and twelve: 1400 a side 41.6,
+    // 29.2, 25.1 ms, 4096 a side 147, 104, 89 ms. Thick ones, and merge-path
+    // chunks (degrees 17 to 32), keep two: random graphs of degree 18 to 28 and
+    // 0.4 to 1.2 M entries 250-490 us at two, 4-18 % more at six.
+    if (g->has_weights && g->max_degree <= kLowDegreeMax)
       g->sssp_delta = (uint32_t)std::max(1.0, std::min(6.0 * g->mean_weight, 4.0e9));
   } else {
     g->tuned_direction = GR_DIR_AUTO;
@@ -74,7 +73,8 @@ void tune_prior(gr_graph *g) {
     // 1.60 so; 2^16: 432 and 315 us)
     g->tuned_sssp_mode = GR_MODE_PERSISTENT;
     if (g->has_weights)
-      g->sssp_delta = (uint32_t)std::max(1.0, std::min(8.0 * g->mean_weight, 4.0e9));
+      g->sssp_delta = g->sssp_delta_thick =
+          (uint32_t)std::max(1.0, std::min(8.0 * g->mean_weight, 4.0e9));
   }
   // A frontier with a third of the edges is relaxed in pull form where its
   // 256-entry tiles fill the GPU: R-MAT 2^21 0.95 ms (1.60 pushed; 0.95 from
@@ -208,7 +208,7 @@ gr_status gr_autotune(gr_graph *g, const int32_t *srcs, int32_t k, int32_t what,
       }
     }
     // UINT32_MAX selects "one bucket"; it is stored as is
-    g->sssp_delta = pick.delta;
+    g->sssp_delta = g->sssp_delta_thick = pick.delta;
     g->tuned_sssp_alpha = pick.alpha;
     g->tuned_sssp_mode = pick.mode;
     g->tuned_sssp_blocks_per_sm = pick.mode == GR_MODE_PERSISTENT ? pick.bps : saved_sbps;

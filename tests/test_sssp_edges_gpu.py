@@ -56,3 +56,49 @@ def test_every_iteration_limit(cuda_lib, mode, direction):
             # a push goes one step further an iteration, and finds its end in
             # one more; a pull may go further
             assert direction != "push" or limit >= hubs, limit
+
+
+def regular(n, half, seed):
+    """`half` random permutations and their inverses: degrees up to 2 * half."""
+    rng = np.random.default_rng(seed)
+    u, v = np.tile(np.arange(n), half), np.concatenate([rng.permutation(n) for _ in range(half)])
+    key = np.unique(np.concatenate([u * n + v, v * n + u]))
+    key = key[key // n != key % n]
+    r = np.zeros(n + 1, np.int32)
+    r[1:] = np.cumsum(np.bincount(key // n, minlength=n))
+    return r, (key % n).astype(np.int32)
+
+
+# frontiers that outgrow a block at once; the far pile's bits in shared memory or
+# not, rows of four and of more entries
+@pytest.mark.parametrize("n,half", [(30_000, 2), (30_000, 3), (30_000, 8), (900_000, 2),
+                                    (900_000, 4)])
+def test_hand_over_of_random_graphs(cuda_lib, n, half):
+    r, c = regular(n, half, half)
+    w = gg.weights(r, c, seed=3, wmin=0, wmax=64)
+    srcs = [int(x) for x in gg.sources(r, 3, seed=4)]
+    with cuda_lib.gr_graph_create(r, c, w) as g:
+        for delta in (0, 1, 200, 0xFFFFFFFF):
+            o = ts.opts(cuda_lib, delta, "persistent")
+            ts.check(cuda_lib, r, c, w, g, srcs[0], o)
+        ts.check_batch(cuda_lib, r, c, w, g, srcs)
+
+
+def test_wide_buckets_are_for_thin_frontiers(cuda_lib):
+    """A search of a random graph of degree 16 expands about as many edges in the
+    graph's own bucket widths as in two mean weights; a mesh takes fewer
+    iterations."""
+    r, c = regular(100_000, 8, 1)
+    w = gg.weights(r, c, seed=3, wmin=1, wmax=64)
+    with cuda_lib.gr_graph_create(r, c, w) as g:
+        ts.run_sssp(cuda_lib, g, 5, with_pred=False)
+        own = cuda_lib.gr_sssp_stats(g)[2]
+        ts.run_sssp(cuda_lib, g, 5, ts.opts(cuda_lib, 65, "persistent"), with_pred=False)
+        assert own < 1.25 * cuda_lib.gr_sssp_stats(g)[2]
+    r, c = gg.grid(200, p_del=0.05, seed=4)
+    w = gg.weights(r, c, seed=3, wmin=1, wmax=64)
+    with cuda_lib.gr_graph_create(r, c, w) as g:
+        ts.run_sssp(cuda_lib, g, 5, with_pred=False)
+        own = cuda_lib.gr_sssp_stats(g)[0]
+        ts.run_sssp(cuda_lib, g, 5, ts.opts(cuda_lib, 65, "persistent"), with_pred=False)
+        assert own < 0.95 * cuda_lib.gr_sssp_stats(g)[0]
