@@ -82,6 +82,13 @@ void tune_prior(gr_graph *g) {
   // vertices 0.42 ms (0.55), but 2^16 and 1.4 M entries 326 us (321), 2^13
   // 128 us (115).
   g->tuned_sssp_alpha = g->m >= (int64_t)g->num_sms * 10240 ? 3.f : 0.f;
+  // Degrees 17 to 32 run one block per SM, with which a pull can take longer than
+  // the push; at two, pushed at one and pulled at one and two: Erdos-Renyi of
+  // mean degree 8 and 1 M vertices 1282, 1543, 1045 us, 3 M 3079, 3404, 2114;
+  // random of degree 20, 1.5 M vertices 3899, 5277, 2952; of degree 28, 300,000
+  // vertices 1547, 946, 671; a mesh of 1000 a side with hubs 16.7, 14.3, 16.1 ms.
+  if (g->tuned_sssp_alpha > 0.f && g->max_degree > kLowDegreeMax && g->max_degree <= 32)
+    g->tuned_sssp_blocks_per_sm = 2;
   g->tuned_mode = GR_MODE_AUTO;
 }
 
