@@ -50,7 +50,12 @@
 
 namespace gr {
 
-constexpr int kMbThreads = 256, kMbItems = 2;
+// Items per thread of a push level's chunk: two leave the pulls' gathers more of
+// the L1; the batched BFS of a directed graph of kMbPushOnlyM entries or more, which
+// only pushes, takes four (R-MAT 2^20, 15.7 M entries, 16 lanes: 1053 us at two,
+// 867 at four; 2^18, 3.8 M, 247 and 233; 2^16, 0.9 M, 131 and 137).
+constexpr int kMbThreads = 256, kMbItems = 2, kMbPushOnlyItems = 4;
+constexpr int64_t kMbPushOnlyM = 3'000'000;
 // Batched BFS keeps the lane masks of its first kKeepLevels levels, each in
 // its own array, and writes their depths in one pass at the end (full
 // coalesced rows); deeper levels rotate through three arrays and write their
@@ -60,7 +65,6 @@ constexpr int32_t kKeepLevels = 16;
 // A batched BFS level pushes when its frontier has fewer than m / kPushDiv
 // edges, and pulls over every vertex otherwise.
 constexpr long long kPushDiv = 16;
-constexpr int kMbChunk = kMbThreads * kMbItems;
 // BC's gathers take chunks of this many items per warp: with one per block
 // its warps waited for the slowest at every chunk (half of the forward's
 // stalls).
@@ -243,10 +247,9 @@ __global__ void k_mb_sources(MbArgs a, MbSources srcs, int32_t sk) {
 
 // Block-local list of the vertices a push level adds to the next level,
 // flushed per chunk with flush_scanned (one packed atomic per block and
-// chunk); a chunk of kMbChunk items adds at most kMbChunk vertices.
-using MbEmitBuf = ScannedBuf<kMbChunk>;
-
-__device__ __forceinline__ void mb_emit(MbEmitBuf &em, const MbArgs &a, int32_t v) {
+// chunk); a chunk adds at most as many vertices as it has items.
+template <int CHUNK>
+__device__ __forceinline__ void mb_emit(ScannedBuf<CHUNK> &em, const MbArgs &a, int32_t v) {
   const int32_t k = atomicAdd(&em.cnt, 1);
   em.out[k] = v;
   em.deg[k] = a.R[v + 1] - a.R[v];
@@ -258,19 +261,21 @@ __device__ __forceinline__ unsigned long long joined(const MbArgs &a, int32_t v)
 }
 
 // Shared memory of the level forms (one at a time).
+template <int ITEMS>
 union MbSmem {
+  static constexpr int kChunk = kMbThreads * ITEMS;  // items of a push level's chunk
   struct {  // per warp
     int32_t off[kMbWarpChunk + 1];
     unsigned long long U[kMbWarpChunk + 1];
   } fwd[kMbThreads / 32];
   struct {
-    int32_t off[kMbChunk + 1];
-    int32_t row[kMbChunk + 1];
-    unsigned long long cur[kMbChunk + 1];
-    int32_t u[kMbChunk + 1];
-    MbEmitBuf em;
+    int32_t off[kChunk + 1];
+    int32_t row[kChunk + 1];
+    unsigned long long cur[kChunk + 1];
+    int32_t u[kChunk + 1];
+    ScannedBuf<kChunk> em;
   } push;
-  MbEmitBuf list;  // compaction of a pulled level into its list
+  ScannedBuf<kChunk> list;  // compaction of a pulled level into its list
 };
 
 // Lanes of `c` at vertex v reach their depth at level L.
@@ -468,8 +473,8 @@ __device__ __forceinline__ void lane_window(LaneSums<T> &s, LaneBuf &b, int32_t 
 // all four loaded before any is added (dealing the threads to the lanes in
 // use, as the backward does, was slower: 1.79 against 1.48 ms on R-MAT 2^18
 // with 64 sources, before the chunks became the warps' own).
-template <int SK>
-__device__ void mb_forward_level(const MbArgs &a, MbSmem &sm, const unsigned long long *cur,
+template <int SK, class SMEM>
+__device__ void mb_forward_level(const MbArgs &a, SMEM &sm, const unsigned long long *cur,
                                  unsigned long long *nxt, unsigned long long *counter, bool &ovf) {
   using T = CountT<SK>;
   const int lane = threadIdx.x & 31;
@@ -586,8 +591,8 @@ __device__ void mb_forward_level(const MbArgs &a, MbSmem &sm, const unsigned lon
 // path counts to v's, the warp serving such edges one at a time. The
 // loader folds each listed vertex's cur into visit and, past the kept
 // levels, writes its depths.
-template <int SK>
-__device__ void mb_push_level(const MbArgs &a, MbSmem &sm, int32_t *s_red8, int32_t L,
+template <int SK, class SMEM>
+__device__ void mb_push_level(const MbArgs &a, SMEM &sm, int32_t *s_red8, int32_t L,
                               const unsigned long long *cur,
                               unsigned long long *nxt, const int32_t *Q, const int32_t *S,
                               int32_t q, int32_t qe, int32_t *Qn, int32_t *Sn,
@@ -597,16 +602,17 @@ __device__ void mb_push_level(const MbArgs &a, MbSmem &sm, int32_t *s_red8, int3
   const bool write_depth = a.depth && L >= a.keep;
   const int lane = threadIdx.x & 31;
   const long long total = (long long)q + qe;
-  const long long nchunks = (total + kMbChunk - 1) / kMbChunk;
+  constexpr int CHUNK = SMEM::kChunk;
+  const long long nchunks = (total + CHUNK - 1) / CHUNK;
   // the emission buffer shares its storage with the other level forms: its
   // count starts at zero here
   if (threadIdx.x == 0) sm.push.em.cnt = 0;
   __syncthreads();
   for (long long chunk = blockIdx.x; chunk < nchunks; chunk += gridDim.x) {
-    const long long d0 = chunk * kMbChunk;
-    const long long d1 = min(d0 + kMbChunk, total);
+    const long long d0 = chunk * CHUNK;
+    const long long d1 = min(d0 + CHUNK, total);
     int32_t i0, i1;
-    block_chunk_bounds<kMbThreads>(S, q, qe, d0, d1, kMbChunk, s_red8, &i0, &i1);
+    block_chunk_bounds<kMbThreads>(S, q, qe, d0, d1, CHUNK, s_red8, &i0, &i1);
     const long long j0 = d0 - i0, j1 = d1 - i1;
     const int32_t nv = (i0 <= q - 1) ? (min(i1, q - 1) - i0 + 1) : 0;
     for (int32_t k = threadIdx.x; k < nv; k += kMbThreads) {
@@ -667,15 +673,16 @@ __device__ void mb_push_level(const MbArgs &a, MbSmem &sm, int32_t *s_red8, int3
 
 // The list of a level reached by a pull (the vertices with lanes in cur,
 // with their degree scan), for the push level that expands it.
-__device__ void mb_compact_list(const MbArgs &a, MbSmem &sm, const unsigned long long *cur,
+template <class SMEM>
+__device__ void mb_compact_list(const MbArgs &a, SMEM &sm, const unsigned long long *cur,
                                 int32_t *Q, int32_t *S, unsigned long long *counter) {
-  constexpr int PER = kMbChunk / kMbThreads;
+  constexpr int CHUNK = SMEM::kChunk, PER = CHUNK / kMbThreads;
   // the list buffer shares its storage with the level forms: its count
   // starts at zero here
   if (threadIdx.x == 0) sm.list.cnt = 0;
   __syncthreads();
-  for (int64_t base = (int64_t)blockIdx.x * kMbChunk; base < a.n;
-       base += (int64_t)gridDim.x * kMbChunk) {  // block-uniform
+  for (int64_t base = (int64_t)blockIdx.x * CHUNK; base < a.n;
+       base += (int64_t)gridDim.x * CHUNK) {  // block-uniform
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
       const int64_t v = base + j * kMbThreads + threadIdx.x;
@@ -746,10 +753,11 @@ struct MbLoop {
   int32_t L, push, q, qe, q_prev, listed, prev_listed;
 };
 
-template <int SK>
+// PULL: the graph is symmetric (else every level pushes)
+template <int SK, bool PULL = true>
 __global__ void __launch_bounds__(kMbThreads, mb_do_blocks_per_sm<SK>()) k_mb_do(MbArgs a) {
   MbCtl *c = a.ctl;
-  __shared__ MbSmem sm;
+  __shared__ MbSmem<PULL ? kMbItems : kMbPushOnlyItems> sm;
   __shared__ int32_t s_red8[kMbThreads / 32];
   __shared__ MbLoop st;
   if (threadIdx.x == 0) {
@@ -788,7 +796,7 @@ __global__ void __launch_bounds__(kMbThreads, mb_do_blocks_per_sm<SK>()) k_mb_do
     }
     const unsigned long long *cur = a.lmp[mb_slot(a, L)];
     unsigned long long *nxt = a.lmp[mb_slot(a, L + 1)];
-    if (st.push && !st.listed) {
+    if (PULL && st.push && !st.listed) {
       mb_compact_list(a, sm, cur, a.lq[L % 3], a.ls[L % 3], &c->cnt_list);
       if (!grid_sync(&c->bar, &c->error, gen)) break;
       if (threadIdx.x == 0) st.listed = 1;
@@ -813,7 +821,7 @@ __global__ void __launch_bounds__(kMbThreads, mb_do_blocks_per_sm<SK>()) k_mb_do
       }
     }
     unsigned long long *counter = &c->cnt3[(L + 1) % 3];
-    if (st.push) {
+    if (!PULL || st.push) {
       mb_push_level<SK>(a, sm, s_red8, L, cur, nxt, a.lq[L % 3], a.ls[L % 3], st.q, st.qe,
                         a.lq[(L + 1) % 3], a.ls[(L + 1) % 3], counter, ovf);
     } else if (SK == kSigNone) {
@@ -1273,7 +1281,8 @@ static MbArgs mb_args(gr_graph *g, BatchWorkspace *ws, int32_t k, int32_t *depth
 static gr_status mb_launch(gr_graph *g, const MbArgs &a, int sk, cudaStream_t s) {
   void *kern = sk == kSigU64   ? (void *)k_mb_do<kSigU64>
                : sk == kSigF64 ? (void *)k_mb_do<kSigF64>
-                               : (void *)k_mb_do<kSigNone>;
+               : !g->symmetric && g->m >= kMbPushOnlyM ? (void *)k_mb_do<kSigNone, false>
+                                                       : (void *)k_mb_do<kSigNone>;
   // small graphs are bound by the grid barrier, which costs more the more
   // blocks meet at it. Batched BFS at 1 to 5 blocks per SM, 20 lanes: R-MAT
   // 34,000 entries 81, 88, 92, 97, 99 us; 0.24 M 81, 93, 95, 101, 102; 0.64 M
