@@ -2032,7 +2032,13 @@ gr_status bfs_run(gr_graph *g, BfsWorkspace *ws, int32_t src, int32_t *depth, in
     void *kern = do_bitmap ? (void *)k_bfs_do<kPullBlocksPerSm> : (void *)k_bfs_do<kDoBlocksPerSm>;
     GR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kLvThreads, 0));
     int bps = std::min(per_sm, do_bitmap ? kPullBlocksPerSm : kDoBlocksPerSm);
-    const int32_t want = o.block > 0 ? o.block : g->tuned_blocks_per_sm;
+    // the graph's own grid is for the direction it runs by itself: pushing all of
+    // a graph that would pull takes more blocks (R-MAT 2^18, 3.9 M entries: 235 us
+    // at one, 2^19, 29.7 M: 475 at three; 124 and 329 at all)
+    const bool push_asked = !do_bitmap && g->symmetric && g->tuned_direction != GR_DIR_PUSH;
+    const int32_t want = o.block > 0 ? o.block
+                         : push_asked ? bfs_push_blocks(g->m)
+                                      : g->tuned_blocks_per_sm;
     if (want > 0) bps = std::min(bps, want);
     const int blocks = std::max(1, bps) * g->num_sms;
     // per-block segments for the pull levels

@@ -219,6 +219,9 @@ gr_status bfs_batch_run(gr_graph *g, BatchWorkspace *ws, const int32_t *h_srcs, 
 // GR_ETIMEOUT when the last batched BFS on ws stopped at a device-side limit
 gr_status batch_read_ctl_error(BatchWorkspace *ws, cudaStream_t s);
 
+// Blocks per SM (0: all) of a BFS that pushes every level of a skewed graph with
+// m entries, measured in tune_prior.
+int32_t bfs_push_blocks(int64_t m);
 // Degree-statistics prior of the tuned settings (set at graph creation).
 void tune_prior(gr_graph *g);
 

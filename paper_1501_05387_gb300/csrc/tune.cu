@@ -26,6 +26,10 @@
 
 namespace gr {
 
+int32_t bfs_push_blocks(int64_t m) {
+  return m < 150'000 ? 1 : m < 700'000 ? 3 : m < 1'500'000 ? 4 : 0;
+}
+
 void tune_prior(gr_graph *g) {
   // push -> pull once the frontier's edges exceed a tenth of the unexplored
   // ones: on R-MAT s22 (16 sources, 6 blocks per SM) alpha 8-10 took 0.1875
@@ -62,7 +66,7 @@ void tune_prior(gr_graph *g) {
     if (g->symmetric)
       g->tuned_blocks_per_sm = g->m < 20'000'000 ? 1 : g->m < 48'000'000 ? 3 : 4;
     else
-      g->tuned_blocks_per_sm = g->m < 150'000 ? 1 : g->m < 700'000 ? 3 : g->m < 1'500'000 ? 4 : 0;
+      g->tuned_blocks_per_sm = bfs_push_blocks(g->m);
     // SSSP at 1 to 5: 2^12 101, 115, 123, 126, 141 us; 2^14 (0.4 M) 158, 143,
     // 133, 141, 151; 2^16 195, 181, 181, 186, 198; 2^18 422, 292, 262, 243, 251;
     // 2^20 (31 M) 1552, 914, 726, 629, 607.
