@@ -1224,8 +1224,8 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_bfs_solo(BfsArgs a) {
 // On a graph of a few thousand vertices a traversal is a handful of levels,
 // each a grid barrier (4-7 us) around a microsecond of work, after an init
 // kernel and a cooperative launch. Here one block does all of it in one
-// launch: depths, parents and the visited bits live in shared memory (16-bit:
-// at most 32768 vertices), so do the vertices in the order of their discovery,
+// launch: depths, parents and the visited bits live in shared memory (16-bit
+// each), so do the vertices in the order of their discovery,
 // in which a level is a range; the outputs are written once, in full rows.
 // Pushes deal the frontier's edges to the threads by a scan of its degrees
 // (1024 frontier vertices at a time); pulls give a warp a word of vertices, as
@@ -1234,11 +1234,15 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_bfs_solo(BfsArgs a) {
 // One SM takes about one random access a clock, so the edges it may have to
 // push are limited: a direction-optimising traversal pushes at most a tenth
 // of the unexplored ones a level, a push-only one all of them (53,000 entries:
-// 60 us here, 45 on a grid of one block per SM).
+// 60 us here, 45 on a grid of one block per SM). So are the vertices it may have
+// to pull, by what the grid takes with one block per SM: R-MAT of 8,192 vertices
+// 24-29 us here, 37-46 there, 16,384 40-45 and 43-54, 19,660 45-57 and 44-52,
+// 32,768 47-83 and 46-58; Erdos-Renyi, 16,000 vertices, 0.4 M entries 48 and 42,
+// 0.77 M 97 and 47.
 constexpr int kSmallThreads = 1024;
 constexpr int kPullWords = 2;  // bitmap words a warp pulls at once
-constexpr int32_t kSmallMaxN = 32768;
-constexpr int64_t kSmallMaxM = 1 << 20, kSmallMaxPushM = 1 << 14;
+constexpr int32_t kSmallMaxN = 16384;
+constexpr int64_t kSmallMaxM = 1 << 19, kSmallMaxPushM = 1 << 14;
 
 __host__ __device__ __forceinline__ size_t small_smem_bytes(int32_t n) {
   return 3 * sizeof(uint16_t) * (size_t)((n + 31) & ~31) + sizeof(uint32_t) * (size_t)((n + 31) / 32);
