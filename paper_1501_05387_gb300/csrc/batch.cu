@@ -881,13 +881,15 @@ struct BcBackArgs {
 };
 
 // Items per warp of the backward pass over a list of `total` items: kMbWarpChunk,
-// and fewer where that would leave warps without a chunk. A warp serves the
+// and fewer where that would leave three quarters of the warps without a chunk
+// (with all of them busy the chunks' own cost shows: R-MAT of 0.1 M vertices 1275
+// us, 1263 so). A warp serves the
 // vertices of its chunk one after another, each with the latency of its
 // children's rows: a level of 32 vertices with two edges each took 18.7 us in
 // one warp (a path of 1000 vertices, 16 sources: 46.3 ms; 39.4 with 512 items to a
 // block of eight warps).
 __device__ __forceinline__ int32_t list_chunk(long long total, int32_t warps) {
-  const long long share = (total + warps - 1) / warps;
+  const long long share = (4 * total + warps - 1) / warps;
   return (int32_t)min((long long)kMbWarpChunk, (share + 7) / 8 * 8);
 }
 
