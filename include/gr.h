@@ -70,10 +70,11 @@ enum {
   GR_MODE_PERSISTENT = 3  /* one cooperative kernel runs every level with a
                              bounded-spin grid barrier between levels; on a
                              graph of maximum degree <= 16 one thread block
-                             (above 1,595,904 vertices, for a BFS, one
-                             thread-block cluster) runs the levels first and
-                             hands a frontier of more than 4096 (32768)
-                             vertices to that kernel */
+                             (for a BFS above 1,595,904 vertices, or of
+                             degree > 4 and more than 3 M entries times
+                             degree, one thread-block cluster) runs the
+                             levels first and hands a frontier of more than
+                             4096 (32768) vertices to that kernel */
 };
 
 /* Options; pass NULL for tuned defaults. Zero in a field means "tuned". */
@@ -160,8 +161,10 @@ gr_status gr_bfs_stats(gr_graph *g, int32_t *levels, int32_t *pull_levels);
  * (symmetric CSR only, else GR_EINVAL) pulls every relaxation that can be.
  * On a graph of maximum degree <= 16 the persistent mode runs a search by one
  * thread block (a batch's by one each) and hands a near frontier of more than
- * 4096 vertices to the grid. Distances do not depend on
- * the direction. */
+ * 16384 edges (counted at the maximum degree, at least 4) to the grid. Such a
+ * graph's tuned bucket width is the one of thin frontiers; while frontiers grow
+ * fast the search takes a narrower one of its own, unless opts->delta sets it.
+ * Distances do not depend on the direction or the width. */
 gr_status gr_sssp(gr_graph *g, int32_t src, uint32_t *dist, int32_t *pred,
                   const gr_opts *opts, void *stream);
 
